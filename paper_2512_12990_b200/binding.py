@@ -1,6 +1,7 @@
-"""Thin ctypes binding over libslicemoe.so: argument marshalling only.
+"""Thin binding over libslicemoe.so: argument marshalling only.
 
-Function names and argument order follow include/slicemoe.h.  Device buffers are torch CUDA
+Function names and argument order follow include/slicemoe.h.  The calls of a decode or prefill loop marshal their
+arguments in native code (csrc/marshal.cpp, built as _marshal.so); everything else goes through ctypes.  Device buffers are torch CUDA
 tensors (torch is used for device memory and streams, nothing else); every step of the path
 runs in the library's kernels.  There is no fallback: if the library is missing or a call
 fails, an exception is raised.
@@ -14,6 +15,7 @@ from ctypes import (POINTER, Structure, c_char_p, c_double, c_float, c_int, c_in
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libslicemoe.so")
 _lib = None
+_m = None   # the _marshal extension: the same entry points with the per-call work in native code
 
 OK = 0
 E_INVALID_ARG, E_UNSUPPORTED, E_CUDA, E_NOMEM = -1, -2, -3, -4
@@ -154,6 +156,19 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+def _marshal():
+    """Loads the library and the native marshalling module (built beside it) on first use; raises if either is
+    missing.  The module gets the addresses of the library's entry points, so both sides use one library."""
+    global _m
+    if _m is None:
+        L = lib()
+        import torch  # noqa: F401  (its libraries are what the module links to)
+        from . import _marshal as m
+        m.setup(SliceMoEError, {n: ctypes.cast(getattr(L, n), c_void_p).value for n in EXPORTS})
+        _m = m
+    return _m
+
+
 def strerror(code: int) -> str:
     return lib().slicemoe_strerror(code).decode()
 
@@ -207,13 +222,7 @@ def slicemoe_pack(W, group: int, b_high: int = 8, b_low: int = 4, stream=None, o
     assert W.is_cuda and W.dtype == torch.float32 and W.is_contiguous() and W.dim() == 2
     N, K = W.shape
     if out is None:
-        nb = max(int(slicemoe_plane_bytes(N, K)), 1)
-        nm = max(int(slicemoe_meta_count(N, K, group)) if group > 0 else 1, 1)
-        out = PackedMat(N, K, group,
-                        torch.empty(nb, dtype=torch.uint8, device=W.device),
-                        torch.empty(nb, dtype=torch.uint8, device=W.device),
-                        torch.empty(nm, dtype=torch.int16, device=W.device),
-                        torch.empty(nm, dtype=torch.uint8, device=W.device))
+        return PackedMat(N, K, group, *(_m or _marshal()).pack_new(W, group, b_high, b_low, stream))
     rc = lib().slicemoe_pack(_ptr(W), N, K, group, b_high, b_low, _ptr(out.msb), _ptr(out.lsb), _ptr(out.scale),
                              _ptr(out.zp), _stream(stream))
     _check(rc, "slicemoe_pack")
@@ -242,17 +251,7 @@ def slicemoe_unpack_meta(scale, zp, N: int, K: int, group: int, stream=None):
 def slicemoe_route_topk(logits, k: int, bias=None, renorm: bool = False, tau: float = 2.0, rank_high: int = 0,
                         want_prec: bool = True, stream=None):
     """logits CUDA float32 [T, E].  Returns (ids int32 [T,k], weights float32 [T,k], prec_req uint8 [T,k] | None)."""
-    import torch
-    assert logits.is_cuda and logits.dtype == torch.float32 and logits.is_contiguous() and logits.dim() == 2
-    T, E = logits.shape
-    kk = max(k, 1)
-    ids = torch.empty((T, kk), dtype=torch.int32, device=logits.device)
-    w = torch.empty((T, kk), dtype=torch.float32, device=logits.device)
-    pr = torch.empty((T, kk), dtype=torch.uint8, device=logits.device) if want_prec else None
-    rc = lib().slicemoe_route_topk(_ptr(logits), T, E, k, _ptr(bias), 1 if renorm else 0, tau, rank_high,
-                                   _ptr(ids), _ptr(w), _ptr(pr), _stream(stream))
-    _check(rc, "slicemoe_route_topk")
-    return ids, w, pr
+    return (_m or _marshal()).route_topk(logits, k, bias, renorm, tau, rank_high, want_prec, stream)
 
 
 # ---- workspace -----------------------------------------------------------------------------------
@@ -296,14 +295,7 @@ def expert_table(experts, device="cuda"):
 # ---- FFN -----------------------------------------------------------------------------------------
 def slicemoe_expert_ffn(shape: Shape, experts_tbl, x, ids, prec, weights, ws, y=None, stream=None):
     """x CUDA bf16 [T, hidden]; ids int32, prec uint8, weights float32 [T, k].  Returns y float32 [T, hidden]."""
-    import torch
-    T = x.shape[0]
-    if y is None:
-        y = torch.empty((T, shape.hidden), dtype=torch.float32, device=x.device)
-    rc = lib().slicemoe_expert_ffn(ctypes.byref(shape), _ptr(experts_tbl), _ptr(x), T, _ptr(ids), _ptr(prec),
-                                   _ptr(weights), _ptr(y), _ptr(ws), ws.numel(), _stream(stream))
-    _check(rc, "slicemoe_expert_ffn")
-    return y
+    return (_m or _marshal()).expert_ffn(shape, experts_tbl, x, ids, prec, weights, ws, y, stream)
 
 
 LISTS_RESIDENT = 1
@@ -313,21 +305,8 @@ COOPERATIVE = 2
 def slicemoe_layer(shape: Shape, experts_tbl, shared_tbl, shared_gate_vec, x, ids, prec, weights, ws, y=None,
                    stream=None, flags=0):
     """flags = 0 calls slicemoe_layer, anything else slicemoe_layer_flags."""
-    import torch
-    T = x.shape[0]
-    if y is None:
-        y = torch.empty((T, shape.hidden), dtype=torch.float32, device=x.device)
-    if flags:
-        rc = lib().slicemoe_layer_flags(ctypes.byref(shape), _ptr(experts_tbl), _ptr(shared_tbl), _ptr(shared_gate_vec),
-                                        _ptr(x), T, _ptr(ids), _ptr(prec), _ptr(weights), _ptr(y), _ptr(ws),
-                                        ws.numel(), flags, _stream(stream))
-        _check(rc, "slicemoe_layer_flags")
-        return y
-    rc = lib().slicemoe_layer(ctypes.byref(shape), _ptr(experts_tbl), _ptr(shared_tbl), _ptr(shared_gate_vec),
-                              _ptr(x), T, _ptr(ids), _ptr(prec), _ptr(weights), _ptr(y), _ptr(ws), ws.numel(),
-                              _stream(stream))
-    _check(rc, "slicemoe_layer")
-    return y
+    return (_m or _marshal()).layer(shape, experts_tbl, shared_tbl, shared_gate_vec, x, ids, prec, weights, ws, y, stream,
+                                    flags)
 
 
 def slicemoe_stream_probe(shape: Shape, experts_tbl, shared_tbl, ids, prec, dependent=True, bytes_out=None,
@@ -343,30 +322,15 @@ def slicemoe_layer_static(shape: Shape, experts_tbl, shared_tbl, shared_gate_vec
     """slicemoe_layer without a caller workspace: the library's built-in scratch array is used.  `y` (CUDA
     float32 [T, hidden]) is required, because nothing may be allocated on this path - not by the library and
     not by this binding."""
-    rc = lib().slicemoe_layer_static(ctypes.byref(shape), _ptr(experts_tbl), _ptr(shared_tbl), _ptr(shared_gate_vec),
-                                     _ptr(x), x.shape[0], _ptr(ids), _ptr(prec), _ptr(weights), _ptr(y),
-                                     _stream(stream))
-    _check(rc, "slicemoe_layer_static")
-    return y
+    return (_m or _marshal()).layer_static(shape, experts_tbl, shared_tbl, shared_gate_vec, x, ids, prec, weights, y, stream)
 
 
 def slicemoe_layer_routed(shape: Shape, experts_tbl, shared_tbl, shared_gate_vec, x, logits, ws, bias=None, renorm=False,
                           tau=2.0, rank_high=0, y=None, want_lists=True, stream=None):
     """Routing and layer in one launch per token.  Returns (y, ids, prec, weights); the lists are None unless
     want_lists."""
-    import torch
-    T = x.shape[0]
-    k = shape.top_k
-    if y is None:
-        y = torch.empty((T, shape.hidden), dtype=torch.float32, device=x.device)
-    ids = torch.empty((T, k), dtype=torch.int32, device=x.device) if want_lists else None
-    prec = torch.empty((T, k), dtype=torch.uint8, device=x.device) if want_lists else None
-    w = torch.empty((T, k), dtype=torch.float32, device=x.device) if want_lists else None
-    rc = lib().slicemoe_layer_routed(ctypes.byref(shape), _ptr(experts_tbl), _ptr(shared_tbl), _ptr(shared_gate_vec),
-                                     _ptr(x), T, _ptr(logits), _ptr(bias), 1 if renorm else 0, tau, rank_high, _ptr(ids),
-                                     _ptr(prec), _ptr(w), _ptr(y), _ptr(ws), ws.numel(), _stream(stream))
-    _check(rc, "slicemoe_layer_routed")
-    return y, ids, prec, w
+    return (_m or _marshal()).layer_routed(shape, experts_tbl, shared_tbl, shared_gate_vec, x, logits, ws, bias, renorm, tau,
+                                           rank_high, y, want_lists, stream)
 
 
 def slicemoe_decode_step_host(shape: Shape, experts_tbl, shared_tbl, shared_gate_vec, x_host, logits_host, y_host,
@@ -374,13 +338,8 @@ def slicemoe_decode_step_host(shape: Shape, experts_tbl, shared_tbl, shared_gate
     """x_host: pinned CPU bf16 [hidden]; logits_host: pinned CPU float32 [E], or None when x_host is one pinned
     byte buffer holding x (bf16 [hidden]) and then the logits (float32 [E]); y_host: pinned CPU float32
     [hidden] (written).  Synchronises the stream."""
-    rc = lib().slicemoe_decode_step_host(ctypes.byref(shape), _ptr(experts_tbl), _ptr(shared_tbl),
-                                         _ptr(shared_gate_vec), c_void_p(x_host.data_ptr()),
-                                         None if logits_host is None else c_void_p(logits_host.data_ptr()), _ptr(bias), 1 if renorm else 0, tau,
-                                         rank_high, c_void_p(y_host.data_ptr()), _ptr(ws), ws.numel(),
-                                         _stream(stream))
-    _check(rc, "slicemoe_decode_step_host")
-    return y_host
+    return (_m or _marshal()).decode_step_host(shape, experts_tbl, shared_tbl, shared_gate_vec, x_host, logits_host, y_host, ws,
+                                               bias, renorm, tau, rank_high, stream)
 
 
 def slicemoe_prefill_workspace_bytes(shape: Shape, T: int) -> int:
@@ -399,17 +358,8 @@ def slicemoe_prefill_layer(shape: Shape, experts_tbl, shared_tbl, shared_gate_ve
                            y=None, status=None, stream=None):
     """x: CUDA bf16 [T, hidden]; ids/weights: CUDA [T, k]; expert_prec: CUDA uint8 [E].  Returns (y, status) with
     status a CUDA int32 [1] tensor (read it after synchronising)."""
-    import torch
-    T = x.shape[0]
-    if y is None:
-        y = torch.empty((T, shape.hidden), dtype=torch.float32, device=x.device)
-    if status is None:
-        status = torch.empty(1, dtype=torch.int32, device=x.device)
-    rc = lib().slicemoe_prefill_layer(ctypes.byref(shape), _ptr(experts_tbl), _ptr(shared_tbl), _ptr(shared_gate_vec),
-                                      _ptr(x), T, _ptr(ids), _ptr(weights), _ptr(expert_prec), _ptr(y), _ptr(ws),
-                                      ws.numel(), _ptr(status), _stream(stream))
-    _check(rc, "slicemoe_prefill_layer")
-    return y, status
+    return (_m or _marshal()).prefill_layer(shape, experts_tbl, shared_tbl, shared_gate_vec, x, ids, weights, expert_prec, ws,
+                                            y, status, stream)
 
 
 # ---- host DBSC -------------------------------------------------------------------------------------
@@ -448,8 +398,7 @@ class Dbsc:
         ids = np.ascontiguousarray(ids, dtype=np.int32)
         prec_req = np.ascontiguousarray(prec_req, dtype=np.uint8)
         out = np.empty(ids.shape, dtype=np.uint8)
-        rc = lib().slicemoe_dbsc_assign(self._h, step, layer, ids.ctypes.data_as(c_void_p),
-                                        prec_req.ctypes.data_as(c_void_p), ids.size, out.ctypes.data_as(c_void_p))
+        rc = lib().slicemoe_dbsc_assign(self._h, step, layer, ids.ctypes.data, prec_req.ctypes.data, ids.size, out.ctypes.data)
         _check(rc, "slicemoe_dbsc_assign")
         return out
 

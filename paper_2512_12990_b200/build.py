@@ -1,4 +1,4 @@
-"""Builds libslicemoe.so (the C-ABI library) in-tree with nvcc for sm_100a.
+"""Builds libslicemoe.so (the C-ABI library, nvcc for sm_100a) and _marshal.so (binding.py's native part) in-tree.
 
     python -m paper_2512_12990_b200.build [--force] [--verbose]
 """
@@ -17,8 +17,13 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 
 
+# the native argument marshalling of binding.py: a Python extension module against torch's headers
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
+MARSHAL = os.path.join(PKG, "_marshal.so")
+
+
 def _newest_source_mtime() -> float:
-    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "slicemoe.h")]
+    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "marshal.cpp"] + [os.path.join(ROOT, "include", "slicemoe.h")]
     return max(os.path.getmtime(f) for f in files)
 
 
@@ -29,6 +34,38 @@ def build(force: bool = False, verbose: bool = False, trace: bool = False) -> st
     """trace=True builds libslicemoe_trace.so: the same library with the decode kernel's time stamps compiled in
     (-DSLICEMOE_TRACE); the ordinary library is not touched."""
     lib = LIB_TRACE if trace else LIB
+    marshal = None if trace else _start_marshal(force)
+    if marshal is not None:
+        try:
+            _build_library(lib, force, verbose, trace)
+        finally:
+            out, _ = marshal.communicate()
+        if marshal.returncode != 0:
+            sys.stderr.write(out)
+            raise RuntimeError("the compiler failed on marshal.cpp")
+        os.replace(MARSHAL + ".new", MARSHAL)
+        return lib
+    return _build_library(lib, force, verbose, trace)
+
+
+def _start_marshal(force: bool):
+    """Starts the compiler on marshal.cpp when _marshal.so is older than its sources."""
+    deps = (MARSHAL_SRC, os.path.join(ROOT, "include", "slicemoe.h"))
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(map(os.path.getmtime, deps)):
+        return None
+    import sysconfig
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", os.path.join(ROOT, "include"),
+           "-isystem", os.path.join(t, "include"), "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"),
+           "-isystem", cuda, "-isystem", sysconfig.get_paths()["include"], MARSHAL_SRC, "-o", MARSHAL + ".new",
+           "-L", os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+
+
+def _build_library(lib: str, force: bool, verbose: bool, trace: bool) -> str:
     if not force and os.path.exists(lib) and os.path.getmtime(lib) >= _newest_source_mtime():
         return lib
     nvcc = os.environ.get("NVCC", "nvcc")

@@ -1,0 +1,424 @@
+// _marshal: what binding.py does per call, in native code - tensor and shape arguments to pointers, outputs from
+// torch's allocator, the current stream - for the entry points that a decode or prefill loop calls per token.  No
+// arithmetic and no CUDA call of its own: it calls the library's entry points, whose addresses binding.py hands over
+// (so there is one library, whichever file it was loaded from).
+//
+// Why: a decode step is 16 us of GPU time and two calls, and in Python a call cost more than that.  Measured on the
+// B200 machine's host (us per call, the launch itself 2.4): slicemoe_route_topk 17.9 in Python (three torch.empty at 2.4,
+// torch.cuda.current_stream 3.2, ctypes conversions), slicemoe_layer with a given y 9.5.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <ATen/cuda/EmptyTensor.h>
+#include <ATen/ops/empty.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <algorithm>
+
+#include "slicemoe.h"
+
+namespace {
+
+struct Entry {
+  decltype(&slicemoe_pack) pack;
+  decltype(&slicemoe_plane_bytes) plane_bytes;
+  decltype(&slicemoe_meta_count) meta_count;
+  decltype(&slicemoe_route_topk) route_topk;
+  decltype(&slicemoe_expert_ffn) expert_ffn;
+  decltype(&slicemoe_layer_flags) layer_flags;
+  decltype(&slicemoe_layer_routed) layer_routed;
+  decltype(&slicemoe_layer_static) layer_static;
+  decltype(&slicemoe_decode_step_host) decode_step_host;
+  decltype(&slicemoe_prefill_layer) prefill_layer;
+} lib;
+PyObject* error_type = nullptr;  // binding.SliceMoEError(code, where)
+PyObject* s_data_ptr = nullptr;
+PyObject* s_cuda_stream = nullptr;
+
+struct Failed {};  // a Python error is set
+
+// A tensor's (or any data_ptr()-bearing object's) address; None is a null pointer.
+void* address(PyObject* o) {
+  if (o == Py_None) return nullptr;
+  if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
+  PyObject* v = PyObject_CallMethodNoArgs(o, s_data_ptr);
+  if (!v) throw Failed();
+  void* p = PyLong_AsVoidPtr(v);
+  Py_DECREF(v);
+  if (!p && PyErr_Occurred()) throw Failed();
+  return p;
+}
+const at::Tensor& tensor(PyObject* o, const char* name) {
+  if (!THPVariable_Check(o)) {
+    PyErr_Format(PyExc_TypeError, "%s: a tensor is wanted, got %s", name, Py_TYPE(o)->tp_name);
+    throw Failed();
+  }
+  return THPVariable_Unpack(o);
+}
+void* stream_of(PyObject* o) {
+  if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+  PyObject* v = PyObject_GetAttr(o, s_cuda_stream);
+  if (!v) throw Failed();
+  void* p = PyLong_AsVoidPtr(v);
+  Py_DECREF(v);
+  if (!p && PyErr_Occurred()) throw Failed();
+  return p;
+}
+int64_t integer(PyObject* o) {
+  PyObject* idx = PyNumber_Index(o);
+  if (!idx) throw Failed();
+  const int64_t v = PyLong_AsLongLong(idx);
+  Py_DECREF(idx);
+  if (v == -1 && PyErr_Occurred()) throw Failed();
+  return v;
+}
+// ctypes takes the low 32 bits of an int argument
+int integer32(PyObject* o) { return (int)(uint32_t)(uint64_t)integer(o); }
+float real(PyObject* o) {
+  const double v = PyFloat_AsDouble(o);
+  if (v == -1.0 && PyErr_Occurred()) throw Failed();
+  return (float)v;
+}
+int truth(PyObject* o) {
+  const int v = PyObject_IsTrue(o);
+  if (v < 0) throw Failed();
+  return v;
+}
+// The ctypes Structure binding.Shape: its bytes are the struct.
+struct ShapeArg {
+  Py_buffer b;
+  explicit ShapeArg(PyObject* o) {
+    if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) throw Failed();
+    if (b.len != (Py_ssize_t)sizeof(slicemoe_shape)) {
+      PyBuffer_Release(&b);
+      PyErr_SetString(PyExc_TypeError, "shape: a binding.Shape is wanted");
+      throw Failed();
+    }
+  }
+  ~ShapeArg() { PyBuffer_Release(&b); }
+  ShapeArg(const ShapeArg&) = delete;
+  const slicemoe_shape* get() const { return static_cast<const slicemoe_shape*>(b.buf); }
+};
+at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type, at::Device dev) {
+  if (dev.is_cuda()) return at::Tensor(at::detail::empty_cuda(sizes, type, dev, std::nullopt));
+  return at::empty(sizes, at::TensorOptions().dtype(type).device(dev));
+}
+PyObject* wrap(const at::Tensor& t) {
+  PyObject* o = THPVariable_Wrap(t);
+  if (!o) throw Failed();
+  return o;
+}
+PyObject* wrap_or_none(const at::Tensor& t) {
+  if (t.defined()) return wrap(t);
+  return Py_NewRef(Py_None);
+}
+PyObject* tuple_of(std::initializer_list<const at::Tensor*> ts) {
+  PyObject* r = PyTuple_New((Py_ssize_t)ts.size());
+  if (!r) throw Failed();
+  Py_ssize_t i = 0;
+  for (const at::Tensor* t : ts) {
+    PyObject* o = nullptr;
+    try {
+      o = wrap_or_none(*t);
+    } catch (...) {
+      Py_DECREF(r);
+      throw;
+    }
+    PyTuple_SET_ITEM(r, i++, o);
+  }
+  return r;
+}
+void check(int rc, const char* where) {
+  if (rc == SLICEMOE_OK) return;
+  PyObject* e = PyObject_CallFunction(error_type, "is", rc, where);
+  if (e) {
+    PyErr_SetObject(error_type, e);
+    Py_DECREF(e);
+  }
+  throw Failed();
+}
+// Calls the library without the interpreter lock, as ctypes does: a launch may wait for room in the stream's queue.
+template <class F>
+int unlocked(F&& f) {
+  int rc;
+  Py_BEGIN_ALLOW_THREADS rc = f();
+  Py_END_ALLOW_THREADS return rc;
+}
+void want(Py_ssize_t n, Py_ssize_t k) {
+  if (n == k) return;
+  PyErr_Format(PyExc_TypeError, "%zd arguments are wanted, got %zd", k, n);
+  throw Failed();
+}
+template <class F>
+PyObject* guarded(F&& f) {
+  try {
+    return f();
+  } catch (const Failed&) {
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+  }
+  return nullptr;
+}
+// y, or a new float32 [T, hidden] on x's device
+at::Tensor output(PyObject* y, const at::Tensor& x, const slicemoe_shape* s, PyObject** given) {
+  if (y != Py_None) {
+    *given = y;
+    return at::Tensor();
+  }
+  *given = nullptr;
+  return empty({x.size(0), s->hidden}, at::kFloat, x.device());
+}
+
+#define SM_ARGS PyObject *, PyObject *const *a, Py_ssize_t n
+
+PyObject* py_setup(SM_ARGS) {  // (error type, dict name -> address)
+  return guarded([&]() -> PyObject* {
+    want(n, 2);
+    auto load = [&](const char* name, auto& fn) {
+      PyObject* v = PyDict_GetItemString(a[1], name);
+      if (!v) {
+        PyErr_Format(PyExc_KeyError, "%s", name);
+        throw Failed();
+      }
+      fn = reinterpret_cast<std::decay_t<decltype(fn)>>(PyLong_AsVoidPtr(v));
+    };
+    load("slicemoe_pack", lib.pack);
+    load("slicemoe_plane_bytes", lib.plane_bytes);
+    load("slicemoe_meta_count", lib.meta_count);
+    load("slicemoe_route_topk", lib.route_topk);
+    load("slicemoe_expert_ffn", lib.expert_ffn);
+    load("slicemoe_layer_flags", lib.layer_flags);
+    load("slicemoe_layer_routed", lib.layer_routed);
+    load("slicemoe_layer_static", lib.layer_static);
+    load("slicemoe_decode_step_host", lib.decode_step_host);
+    load("slicemoe_prefill_layer", lib.prefill_layer);
+    Py_XSETREF(error_type, Py_NewRef(a[0]));
+    Py_RETURN_NONE;
+  });
+}
+
+PyObject* py_pack_new(SM_ARGS) {  // W, group, b_high, b_low, stream -> (msb, lsb, scale, zp)
+  return guarded([&]() -> PyObject* {
+    want(n, 5);
+    const at::Tensor& W = tensor(a[0], "W");
+    const int N = (int)W.size(0), K = (int)W.size(1), group = integer32(a[1]);
+    const int64_t nb = std::max<int64_t>((int64_t)lib.plane_bytes(N, K), 1);
+    const int64_t nm = std::max<int64_t>(group > 0 ? (int64_t)lib.meta_count(N, K, group) : 1, 1);
+    const at::Device dev = W.device();
+    const at::Tensor msb = empty({nb}, at::kByte, dev), lsb = empty({nb}, at::kByte, dev);
+    const at::Tensor scale = empty({nm}, at::kShort, dev), zp = empty({nm}, at::kByte, dev);
+    const int bh = integer32(a[2]), bl = integer32(a[3]);
+    void* st = stream_of(a[4]);
+    check(unlocked([&] {
+            return lib.pack(static_cast<const float*>(W.data_ptr()), N, K, group, bh, bl, msb.data_ptr(), lsb.data_ptr(),
+                            static_cast<uint16_t*>(scale.data_ptr()), static_cast<uint8_t*>(zp.data_ptr()), st);
+          }),
+          "slicemoe_pack");
+    return tuple_of({&msb, &lsb, &scale, &zp});
+  });
+}
+
+PyObject* py_route_topk(SM_ARGS) {  // logits, k, bias, renorm, tau, rank_high, want_prec, stream -> (ids, weights, prec)
+  return guarded([&]() -> PyObject* {
+    want(n, 8);
+    const at::Tensor& logits = tensor(a[0], "logits");
+    if (!(logits.is_cuda() && logits.scalar_type() == at::kFloat && logits.is_contiguous() && logits.dim() == 2)) {
+      PyErr_SetString(PyExc_AssertionError, "logits: a contiguous CUDA float32 matrix is wanted");
+      throw Failed();
+    }
+    const int64_t T = logits.size(0), E = logits.size(1);
+    const int k = integer32(a[1]), kk = std::max(k, 1);
+    const at::Device dev = logits.device();
+    const at::Tensor ids = empty({T, kk}, at::kInt, dev), w = empty({T, kk}, at::kFloat, dev);
+    at::Tensor prec;
+    if (truth(a[6])) prec = empty({T, kk}, at::kByte, dev);
+    const float* bias = static_cast<const float*>(address(a[2]));
+    const int renorm = truth(a[3]), rank_high = integer32(a[5]);
+    const float tau = real(a[4]);
+    void* st = stream_of(a[7]);
+    check(unlocked([&] {
+            return lib.route_topk(static_cast<const float*>(logits.data_ptr()), (int)T, (int)E, k, bias, renorm, tau, rank_high,
+                                  static_cast<int32_t*>(ids.data_ptr()), static_cast<float*>(w.data_ptr()),
+                                  prec.defined() ? static_cast<uint8_t*>(prec.data_ptr()) : nullptr, st);
+          }),
+          "slicemoe_route_topk");
+    return tuple_of({&ids, &w, &prec});
+  });
+}
+
+PyObject* py_expert_ffn(SM_ARGS) {  // shape, experts, x, ids, prec, weights, ws, y, stream -> y
+  return guarded([&]() -> PyObject* {
+    want(n, 9);
+    const ShapeArg s(a[0]);
+    const at::Tensor &x = tensor(a[2], "x"), &ws = tensor(a[6], "ws");
+    PyObject* given;
+    const at::Tensor y = output(a[7], x, s.get(), &given);
+    const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
+    const auto* ids = static_cast<const int32_t*>(address(a[3]));
+    const auto* prec = static_cast<const uint8_t*>(address(a[4]));
+    const auto* w = static_cast<const float*>(address(a[5]));
+    float* yp = static_cast<float*>(given ? address(given) : y.data_ptr());
+    void* st = stream_of(a[8]);
+    check(unlocked([&] {
+            return lib.expert_ffn(s.get(), ex, x.data_ptr(), (int)x.size(0), ids, prec, w, yp, ws.data_ptr(),
+                                  (size_t)ws.numel(), st);
+          }),
+          "slicemoe_expert_ffn");
+    return given ? Py_NewRef(given) : wrap(y);
+  });
+}
+
+PyObject* py_layer(SM_ARGS) {  // shape, experts, shared, gate_vec, x, ids, prec, weights, ws, y, stream, flags -> y
+  return guarded([&]() -> PyObject* {
+    want(n, 12);
+    const ShapeArg s(a[0]);
+    const at::Tensor &x = tensor(a[4], "x"), &ws = tensor(a[8], "ws");
+    PyObject* given;
+    const at::Tensor y = output(a[9], x, s.get(), &given);
+    const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
+    const auto* sh = static_cast<const slicemoe_expert*>(address(a[2]));
+    const auto* gv = static_cast<const float*>(address(a[3]));
+    const auto* ids = static_cast<const int32_t*>(address(a[5]));
+    const auto* prec = static_cast<const uint8_t*>(address(a[6]));
+    const auto* w = static_cast<const float*>(address(a[7]));
+    float* yp = static_cast<float*>(given ? address(given) : y.data_ptr());
+    void* st = stream_of(a[10]);
+    const unsigned flags = (unsigned)integer32(a[11]);
+    check(unlocked([&] {
+            return lib.layer_flags(s.get(), ex, sh, gv, x.data_ptr(), (int)x.size(0), ids, prec, w, yp, ws.data_ptr(),
+                                   (size_t)ws.numel(), flags, st);
+          }),
+          flags ? "slicemoe_layer_flags" : "slicemoe_layer");
+    return given ? Py_NewRef(given) : wrap(y);
+  });
+}
+
+PyObject* py_layer_static(SM_ARGS) {  // shape, experts, shared, gate_vec, x, ids, prec, weights, y, stream -> y
+  return guarded([&]() -> PyObject* {
+    want(n, 10);
+    const ShapeArg s(a[0]);
+    const at::Tensor& x = tensor(a[4], "x");
+    const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
+    const auto* sh = static_cast<const slicemoe_expert*>(address(a[2]));
+    const auto* gv = static_cast<const float*>(address(a[3]));
+    const auto* ids = static_cast<const int32_t*>(address(a[5]));
+    const auto* prec = static_cast<const uint8_t*>(address(a[6]));
+    const auto* w = static_cast<const float*>(address(a[7]));
+    float* yp = static_cast<float*>(address(a[8]));
+    void* st = stream_of(a[9]);
+    check(unlocked([&] { return lib.layer_static(s.get(), ex, sh, gv, x.data_ptr(), (int)x.size(0), ids, prec, w, yp, st); }),
+          "slicemoe_layer_static");
+    return Py_NewRef(a[8]);
+  });
+}
+
+// shape, experts, shared, gate_vec, x, logits, ws, bias, renorm, tau, rank_high, y, want_lists, stream -> (y, ids, prec, weights)
+PyObject* py_layer_routed(SM_ARGS) {
+  return guarded([&]() -> PyObject* {
+    want(n, 14);
+    const ShapeArg s(a[0]);
+    const at::Tensor &x = tensor(a[4], "x"), &ws = tensor(a[6], "ws");
+    PyObject* given;
+    const at::Tensor y = output(a[11], x, s.get(), &given);
+    const int64_t T = x.size(0), k = s.get()->top_k;
+    at::Tensor ids, prec, w;
+    if (truth(a[12])) {
+      ids = empty({T, k}, at::kInt, x.device());
+      prec = empty({T, k}, at::kByte, x.device());
+      w = empty({T, k}, at::kFloat, x.device());
+    }
+    const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
+    const auto* sh = static_cast<const slicemoe_expert*>(address(a[2]));
+    const auto* gv = static_cast<const float*>(address(a[3]));
+    const auto* logits = static_cast<const float*>(address(a[5]));
+    const auto* bias = static_cast<const float*>(address(a[7]));
+    const int renorm = truth(a[8]), rank_high = integer32(a[10]);
+    const float tau = real(a[9]);
+    float* yp = static_cast<float*>(given ? address(given) : y.data_ptr());
+    void* st = stream_of(a[13]);
+    auto ptr = [](const at::Tensor& t) -> void* { return t.defined() ? t.data_ptr() : nullptr; };
+    check(unlocked([&] {
+            return lib.layer_routed(s.get(), ex, sh, gv, x.data_ptr(), (int)T, logits, bias, renorm, tau, rank_high,
+                                    static_cast<int32_t*>(ptr(ids)), static_cast<uint8_t*>(ptr(prec)),
+                                    static_cast<float*>(ptr(w)), yp, ws.data_ptr(), (size_t)ws.numel(), st);
+          }),
+          "slicemoe_layer_routed");
+    if (!given) return tuple_of({&y, &ids, &prec, &w});
+    PyObject* r = tuple_of({&y, &ids, &prec, &w});  // y undefined: a place holder
+    PyTuple_SetItem(r, 0, Py_NewRef(given));
+    return r;
+  });
+}
+
+// shape, experts, shared, gate_vec, x_host, logits_host, y_host, ws, bias, renorm, tau, rank_high, stream -> y_host
+PyObject* py_decode_step_host(SM_ARGS) {
+  return guarded([&]() -> PyObject* {
+    want(n, 13);
+    const ShapeArg s(a[0]);
+    const at::Tensor& ws = tensor(a[7], "ws");
+    const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
+    const auto* sh = static_cast<const slicemoe_expert*>(address(a[2]));
+    const auto* gv = static_cast<const float*>(address(a[3]));
+    const void* x = address(a[4]);
+    const auto* logits = static_cast<const float*>(address(a[5]));
+    float* y = static_cast<float*>(address(a[6]));
+    const auto* bias = static_cast<const float*>(address(a[8]));
+    const int renorm = truth(a[9]), rank_high = integer32(a[11]);
+    const float tau = real(a[10]);
+    void* st = stream_of(a[12]);
+    check(unlocked([&] {
+            return lib.decode_step_host(s.get(), ex, sh, gv, x, logits, bias, renorm, tau, rank_high, y, ws.data_ptr(),
+                                        (size_t)ws.numel(), st);
+          }),
+          "slicemoe_decode_step_host");
+    return Py_NewRef(a[6]);
+  });
+}
+
+// shape, experts, shared, gate_vec, x, ids, weights, expert_prec, ws, y, status, stream -> (y, status)
+PyObject* py_prefill_layer(SM_ARGS) {
+  return guarded([&]() -> PyObject* {
+    want(n, 12);
+    const ShapeArg s(a[0]);
+    const at::Tensor &x = tensor(a[4], "x"), &ws = tensor(a[8], "ws");
+    PyObject* given;
+    const at::Tensor y = output(a[9], x, s.get(), &given);
+    at::Tensor status;
+    if (a[10] == Py_None) status = empty({1}, at::kInt, x.device());
+    const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
+    const auto* sh = static_cast<const slicemoe_expert*>(address(a[2]));
+    const auto* gv = static_cast<const float*>(address(a[3]));
+    const auto* ids = static_cast<const int32_t*>(address(a[5]));
+    const auto* w = static_cast<const float*>(address(a[6]));
+    const auto* prec = static_cast<const uint8_t*>(address(a[7]));
+    float* yp = static_cast<float*>(given ? address(given) : y.data_ptr());
+    int* sp = static_cast<int*>(status.defined() ? status.data_ptr() : address(a[10]));
+    void* st = stream_of(a[11]);
+    check(unlocked([&] {
+            return lib.prefill_layer(s.get(), ex, sh, gv, x.data_ptr(), (int)x.size(0), ids, w, prec, yp, ws.data_ptr(),
+                                     (size_t)ws.numel(), sp, st);
+          }),
+          "slicemoe_prefill_layer");
+    PyObject* r = tuple_of({&y, &status});
+    if (given) PyTuple_SetItem(r, 0, Py_NewRef(given));
+    if (!status.defined()) PyTuple_SetItem(r, 1, Py_NewRef(a[10]));
+    return r;
+  });
+}
+
+#define SM_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_##name)), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {SM_METHOD(setup),        SM_METHOD(pack_new),         SM_METHOD(route_topk),
+                         SM_METHOD(expert_ffn),   SM_METHOD(layer),            SM_METHOD(layer_static),
+                         SM_METHOD(layer_routed), SM_METHOD(decode_step_host), SM_METHOD(prefill_layer),
+                         {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__marshal() {
+  s_data_ptr = PyUnicode_InternFromString("data_ptr");
+  s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+  if (!s_data_ptr || !s_cuda_stream) return nullptr;
+  return PyModule_Create(&module);
+}
