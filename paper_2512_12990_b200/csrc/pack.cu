@@ -14,11 +14,19 @@
 
 namespace slicemoe {
 
-__device__ __forceinline__ int quantise_one(float w, float s, int z, int qmax) {
-  float r = rintf(__fdiv_rn(w, s));
-  r = fminf(fmaxf(r, -1.0e9f), 1.0e9f);
-  int q = (int)r + z;
-  return min(max(q, 0), qmax);
+// clamp(rint(w / s) + z, 0, qmax) with the IEEE quotient.  w times the rounded reciprocal r is within 2^-22 of the
+// quotient, relatively, so wherever the product is below 1024 in size and farther than 2^-10 from a half-integer its
+// nearest integer is the quotient's; the others (one weight in five hundred, and whatever is not a number) divide.
+__device__ __forceinline__ int quantise_one(float w, float s, float r, int z, int qmax) {
+  const float t = w * r;
+  const float big = t + 12582912.f;  // 1.5 x 2^23: the sum's unit is 1, so it is rounded to the nearest even integer
+  const float frac = fabsf(t - (big - 12582912.f));
+  int n = __float_as_int(big) - 0x4b400000;
+  if (!(fabsf(t) < 1024.f && frac < 0.5f - 0.0009765625f)) {
+    const float d = fminf(fmaxf(rintf(__fdiv_rn(w, s)), -1.0e9f), 1.0e9f);
+    n = (int)d;
+  }
+  return min(max(n + z, 0), qmax);
 }
 
 // Smallest / largest of the float over the lanes of `mask` (which all call it); NaNs lose, as in fminf / fmaxf.
@@ -34,58 +42,83 @@ __device__ __forceinline__ float lanes_max(unsigned mask, float v) {
 }
 
 constexpr int kPackThreads = 256;  // eight warps: the row pairs (g, g + 8) of one 16-row block
+constexpr int kPackBlocks = 2;     // 128-column blocks of a warp, their loads in flight together
 template <int G>
 __global__ void __launch_bounds__(kPackThreads) pack_kernel(const float* __restrict__ W, int K, int qmax, int shift,
                                                             uint32_t* __restrict__ msb, uint32_t* __restrict__ lsb,
                                                             uint16_t* __restrict__ scale, uint8_t* __restrict__ zp) {
   const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int kblocks = K >> 7;
-  const int rb = (int)(blockIdx.x / (unsigned)kblocks), kb = (int)(blockIdx.x % (unsigned)kblocks);
+  const int kblocks = K >> 7, per_row = (kblocks + kPackBlocks - 1) / kPackBlocks;
+  const int rb = (int)(blockIdx.x / (unsigned)per_row), kb0 = (int)(blockIdx.x % (unsigned)per_row) * kPackBlocks;
   constexpr int kLanes = G / 4;  // lanes of a group
   const unsigned mask = kLanes == 32 ? 0xffffffffu : ((1u << (kLanes & 31)) - 1u) << (lane & ~(kLanes - 1));
-  float4 v[2];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // W may be the work of the kernel before
+  float4 v[kPackBlocks][2];
 #pragma unroll
-  for (int hi = 0; hi < 2; ++hi)
-    v[hi] = __ldcs(reinterpret_cast<const float4*>(W + (size_t)(rb * 16 + g + 8 * hi) * K + kb * 128) + lane);
-  const int grp = kb * (128 / G) + lane / kLanes;
-  uint32_t mw = 0, lw = 0;
+  for (int i = 0; i < kPackBlocks; ++i)
 #pragma unroll
-  for (int hi = 0; hi < 2; ++hi) {
-    const float vals[4] = {v[hi].x, v[hi].y, v[hi].z, v[hi].w};
-    float lo = 0.0f, top = 0.0f;  // the range always contains zero
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      lo = fminf(lo, vals[j]);
-      top = fmaxf(top, vals[j]);
+    for (int hi = 0; hi < 2; ++hi)
+    {
+      v[i][hi] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (kb0 + i < kblocks)
+        v[i][hi] = __ldcs(reinterpret_cast<const float4*>(W + (size_t)(rb * 16 + g + 8 * hi) * K + (kb0 + i) * 128) + lane);
     }
-    lo = lanes_min(mask, lo);
-    top = lanes_max(mask, top);
-    __half s16 = __float2half_rn(__fdiv_rn(__fsub_rn(top, lo), (float)qmax));
-    float s = __half2float(s16);
-    int z = 0;
-    if ((top == lo) || (s == 0.0f) || isinf(s) || isnan(s)) {  // degenerate
-      s16 = __float2half_rn(1.0f);
-      s = 1.0f;
-    } else {
-      z = (int)fminf(fmaxf(rintf(__fdiv_rn(-lo, s)), 0.0f), (float)qmax);
-    }
-    if (lane % kLanes == 0) {
-      const size_t idx = ((size_t)rb * (K / G) + grp) * 16 + g + 8 * hi;  // meta_index
-      scale[idx] = __half_as_ushort(s16);
-      zp[idx] = (uint8_t)z;
-    }
+  // The range of every (block, row)'s group in all of its lanes; then lane l works out scale and zero-point for
+  // combination l % 4 alone (every four consecutive lanes share a group), and the four take each other's results.
+  static_assert(kPackBlocks == 2, "four combinations, one per lane of four");
+  float lo_of = 0.f, top_of = 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int q = quantise_one(vals[j], s, z, qmax);
-      const int pos = 2 * j + hi;
-      mw |= (uint32_t)(q >> shift) << (4 * pos);  // a slice narrower than 4 bits sits in the low bits of its nibble
-      lw |= (uint32_t)(q & ((1 << shift) - 1)) << (4 * pos);
+  for (int c = 0; c < 4; ++c) {
+    const float4 w = v[c >> 1][c & 1];
+    const float lo = lanes_min(mask, fminf(fminf(0.f, w.x), fminf(fminf(0.f, w.y), fminf(fminf(0.f, w.z), fminf(0.f, w.w)))));
+    const float top = lanes_max(mask, fmaxf(fmaxf(0.f, w.x), fmaxf(fmaxf(0.f, w.y), fmaxf(fmaxf(0.f, w.z), fmaxf(0.f, w.w)))));
+    if ((lane & 3) == c) {
+      lo_of = lo;
+      top_of = top;
     }
   }
-  // column 4 lane of the 128 is tile lane / 16, word (lane / 4) % 4 of plane lane 4 g + lane % 4
-  const size_t word = plane_word_index(K, rb, 2 * kb + (lane >> 4), 4 * g + (lane & 3), (lane >> 2) & 3);
-  msb[word] = mw;
-  lsb[word] = lw;
+  __half s16_of = __float2half_rn(__fdiv_rn(__fsub_rn(top_of, lo_of), (float)qmax));
+  float s_of = __half2float(s16_of);
+  int z_of = 0;
+  if ((top_of == lo_of) || (s_of == 0.0f) || isinf(s_of) || isnan(s_of)) {  // degenerate
+    s16_of = __float2half_rn(1.0f);
+    s_of = 1.0f;
+  } else {
+    z_of = (int)fminf(fmaxf(rintf(__fdiv_rn(-lo_of, s_of)), 0.0f), (float)qmax);
+  }
+  const float r_of = __frcp_rn(s_of);
+  if (lane % kLanes < 4) {
+    const int c = lane & 3, kb = kb0 + (c >> 1);
+    if (kb < kblocks) {
+      const size_t idx = ((size_t)rb * (K / G) + kb * (128 / G) + lane / kLanes) * 16 + g + 8 * (c & 1);  // meta_index
+      scale[idx] = __half_as_ushort(s16_of);
+      zp[idx] = (uint8_t)z_of;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kPackBlocks; ++i) {
+    const int kb = kb0 + i;
+    if (kb >= kblocks) break;
+    uint32_t code[2];  // four codes of a row, one per byte
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+      const int from = (lane & ~3) + 2 * i + hi;
+      const float s = __shfl_sync(0xffffffffu, s_of, from), r = __shfl_sync(0xffffffffu, r_of, from);
+      const int z = __shfl_sync(0xffffffffu, z_of, from);
+      const float vals[4] = {v[i][hi].x, v[i][hi].y, v[i][hi].z, v[i][hi].w};
+      uint32_t q[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) q[j] = (uint32_t)quantise_one(vals[j], s, r, z, qmax);
+      code[hi] = q[0] | q[1] << 8 | q[2] << 16 | q[3] << 24;
+    }
+    // a slice narrower than 4 bits sits in the low bits of its nibble; the codes have no bits beyond theirs
+    const uint32_t low = ((1u << shift) - 1u) * 0x01010101u;
+    // column 4 lane of the 128 is tile lane / 16, word (lane / 4) % 4 of plane lane 4 g + lane % 4
+    const size_t word = plane_word_index(K, rb, 2 * kb + (lane >> 4), 4 * g + (lane & 3), (lane >> 2) & 3);
+    msb[word] = ((code[0] & ~low) >> shift) | ((code[1] & ~low) >> shift << 4);
+    lsb[word] = (code[0] & low) | (code[1] & low) << 4;
+  }
 }
 
 __global__ void unpack_plane_kernel(const uint32_t* __restrict__ plane, int N, int K,
@@ -166,12 +199,20 @@ extern "C" int slicemoe_pack(const float* W, int N, int K, int group, int b_high
   const int rc = check_dims(N, K, group);
   if (rc != SLICEMOE_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  const long long blocks = (long long)(N / 16) * (K / 128);
+  const long long blocks = (long long)(N / 16) * ((K / 128 + kPackBlocks - 1) / kPackBlocks);
   if (blocks > 0x7fffffffll) return SLICEMOE_E_INVALID_ARG;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(kPackThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // the next matrix' launch overlaps this one's end
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   auto* kernel = group == 128 ? pack_kernel<128> : group == 64 ? pack_kernel<64> : pack_kernel<32>;
-  kernel<<<(unsigned)blocks, kPackThreads, 0, st>>>(W, K, qmax, shift, reinterpret_cast<uint32_t*>(msb),
-                                                    reinterpret_cast<uint32_t*>(lsb), scale, zp);
-  SM_LAUNCH_CHECK();
+  SM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, W, K, qmax, shift, reinterpret_cast<uint32_t*>(msb),
+                                 reinterpret_cast<uint32_t*>(lsb), scale, zp));
   return SLICEMOE_OK;
 }
 

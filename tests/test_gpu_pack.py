@@ -147,3 +147,28 @@ def test_dense_storage_of_narrow_slices(N, K, b_high, b_low):
         back = B.slicemoe_expand_plane(c, N, K, bits)
         torch.cuda.synchronize()
         assert torch.equal(back, plane.view(torch.uint8).reshape(-1))
+
+
+@pytest.mark.parametrize("group", [32, 64, 128])
+@pytest.mark.parametrize("b_high,b_low", [(8, 4), (6, 3), (4, 2)])
+def test_pack_bit_exact_at_half_integers(group, b_high, b_low):
+    """Quotients on and one float beside every half-integer (where the rounding turns), scales from subnormal to large,
+    an odd number of 128-column blocks, an infinity in one row."""
+    N, K = 32, 384
+    Q = (1 << b_high) - 1
+    rng = np.random.default_rng(group * 100 + b_high)
+    W = np.empty((N, K), dtype=np.float32)
+    for n in range(N):
+        for g0 in range(0, K, group):
+            # lo and hi fix s = fp16((hi - lo) / Q); the others are half-integer multiples of it, nudged by one float or not
+            s = np.float32(np.float16(2.0 ** rng.integers(-24, 7) * (1 + rng.integers(0, 1024) / 1024.0)))
+            z = int(rng.integers(0, Q + 1))
+            half = (rng.integers(-2 * z - 1, 2 * (Q - z) + 2, size=group) * np.float32(0.5)).astype(np.float32)
+            v = (half * s).astype(np.float32)
+            nudge = rng.integers(-1, 2, size=group)
+            v = np.where(nudge == 0, v, np.nextafter(v, np.where(nudge > 0, np.float32(np.inf), np.float32(-np.inf)))).astype(np.float32)
+            v[0], v[1] = -z * s, (Q - z) * s
+            W[n, g0:g0 + group] = v
+    W[5, 7] = np.inf
+    with np.errstate(all="ignore"):
+        _check(W, group, b_high, b_low)
