@@ -4,10 +4,11 @@
 // holds columns 4 l .. 4 l + 3 of both rows, which are the eight weights of one 32-bit word of each plane, and the
 // groups are 8, 16 or 32 consecutive lanes, so that the range of a group is two warp reductions and the codes never
 // leave the registers.  The eight warps of a block (g = 0 .. 7) fill whole 512-byte plane blocks.  Bound: HBM, 5
-// bytes per weight.  All arithmetic that decides an integer uses IEEE division and rint (no fast-math, no
-// reciprocal), so the codes are bit-exact against a float32 CPU evaluation.
+// bytes per weight.  Every integer is that of IEEE division and rint (a reciprocal only where it provably
+// rounds to the same integer, see quantise_one), so the codes are bit-exact against a float32 CPU evaluation.
 // Measured on a 1408 x 2048 matrix, G 128 (14.5 MB, 2.2 us at the copy rate): two kernels - range and meta first, then
-// planes from a second read of W - 16 us; this one PACK_US us.
+// planes from a second read of W - 16 us; this one 5.8 us back to back (load latency, the chain of reductions and
+// divides, and the hand-over from launch to launch; a larger matrix comes closer to the rate).
 #include <cuda_fp16.h>
 
 #include "common.cuh"
