@@ -3,18 +3,18 @@
 // that prefill wants high-bit computation; the per-expert precision flag here is this library's generalisation
 // (an expert can also be run from its MSB slice alone), which the mixed-precision prefill benchmark uses.
 //
-// Steps, all on the device:
-//   1. count the tokens of every routed expert, lay the experts' token rows out one after the other
-//      (each expert padded to a multiple of 128 rows), list the 128-row tiles;
+// Steps, all on the device, five launches chained by programmatic dependent launch:
+//   1. plan: count the tokens of every routed expert, give every (token, expert) pair a row - the experts' rows one
+//      after the other, without padding - and sort the experts by their number of tokens;
 //   2. gather x (bf16) into that order as fp16 (exact for every bf16 value in fp16's normal range);
 //   3. grouped GEMM 1: per tile  H = silu(X Wg^T) * (X Wu^T)  (fp16 out);
 //   4. grouped GEMM 2: per tile  Yrow = H Wd^T  (fp32 out, one row per (token, expert) pair);
 //   5. combine: y[t] = sum_j w[t,j] Yrow[pos(t,j)] + shared experts, in list order (deterministic).
-// In both GEMMs the weight tile is dequantised on the fly from the nibble planes - s * (q - zp) from both
-// slices, 16 s * (q_msb - (zp >> 4)) from the MSB slice alone - straight into tensor memory and multiplied on
-// the 5th-generation tensor cores (tcgen05.mma, fp16 x fp16 -> fp32).  A dequantised weight needs about 20
-// significant bits, fp16 holds 11: every weight is therefore kept as the exact sum of two fp16 numbers and
-// multiplied in two MMAs.
+// In both GEMMs the weight tile is brought from the nibble planes to fp16 on the fly - the integer q - zp from both
+// slices, 2^shift (q_msb - (zp >> shift)) from the MSB slice alone, both exact in fp16 - straight into tensor memory
+// and multiplied on the 5th-generation tensor cores (tcgen05.mma, fp16 x fp16 -> fp32).  The scale belongs to a
+// quantisation group: a group's sums are read from tensor memory and added to fp32 registers with one
+// multiply-add by the scale.  No weight is rounded anywhere.
 #include <cuda.h>  // CUtensorMap (types only; the encoder is fetched through the runtime)
 #include <cuda_fp16.h>
 
@@ -22,208 +22,345 @@
 
 namespace slicemoe {
 
-constexpr int kPfTileM = 128;  // token rows per tile
+constexpr int kPfTileN = 192;  // most token rows of a tile
 constexpr int kPfTileB = 128;  // weight rows per tile: 64 gate + 64 up columns of h (GEMM 1), 128 columns of y (GEMM 2)
-constexpr int kPfChunkK = 64;  // contraction columns per pipeline step (one plane block)
+constexpr int kPfChunkK = 128;  // contraction columns per pipeline step (two plane blocks; every width is a multiple)
+
+// An expert with tokens, as the GEMMs see it; sorted, the longest work items first.
+struct PfRun {
+  int expert;             // routed: 0 .. E - 1, shared: E ..
+  int count, tiles;       // tokens; tiles of equal width (up to 16) they are cut into
+  int in_row, out_row;    // first row in the gathered x; first row of h and of the result rows
+  int items1, items2;     // work items before this run's in GEMM 1 and GEMM 2
+  int pad_;
+};
+struct PfHead {
+  int runs;
+  int items1, items2;     // work items in all
+  int next1, next2;       // next work item to hand out
+};
 
 // ---- workspace layout (host and device agree through this one function) --------------------------------
 struct PfLayout {
-  size_t counts, cursor, offsets, tile_expert, tile_row0, item_start, ntiles, row_token, posmap, gate, xs, h, yrow, total;
-  int rmax, max_tiles, nexp_all;
+  size_t head, counts, offsets, cursor, runs, row_token, posmap, gate, xs, h, yrow, total;
+  int in_rows, out_rows, nexp_all;
 };
 __host__ __device__ inline size_t pf_align(size_t v) { return (v + 255) & ~(size_t)255; }
 __host__ __device__ inline PfLayout pf_layout(int T, int E, int k, int n_shared, int hidden, int inter, int shared_inter) {
   PfLayout L;
   L.nexp_all = E + n_shared;
-  // routed rows: T*k plus at most 127 rows of padding per expert; shared: T rows each, padded
-  const int tpad = (T + kPfTileM - 1) / kPfTileM * kPfTileM;
-  L.rmax = (T * k + E * (kPfTileM - 1) + kPfTileM - 1) / kPfTileM * kPfTileM + n_shared * tpad;
-  L.max_tiles = L.rmax / kPfTileM;
+  L.in_rows = T * k + (n_shared ? T : 0);  // the shared experts read the same rows
+  L.out_rows = T * (k + n_shared);
   const int wide = inter > shared_inter ? inter : shared_inter;
   size_t o = 0;
+  L.head = o;         o = pf_align(o + sizeof(PfHead));
   L.counts = o;       o = pf_align(o + sizeof(int) * L.nexp_all);
+  L.offsets = o;      o = pf_align(o + sizeof(int) * L.nexp_all);
   L.cursor = o;       o = pf_align(o + sizeof(int) * L.nexp_all);
-  L.offsets = o;      o = pf_align(o + sizeof(int) * (L.nexp_all + 1));
-  L.tile_expert = o;  o = pf_align(o + sizeof(int) * L.max_tiles);
-  L.tile_row0 = o;    o = pf_align(o + sizeof(int) * L.max_tiles);
-  L.item_start = o;   o = pf_align(o + sizeof(int) * (L.max_tiles + 1));
-  L.ntiles = o;       o = pf_align(o + sizeof(int) * 4);
-  L.row_token = o;    o = pf_align(o + sizeof(int) * L.rmax);
+  L.runs = o;         o = pf_align(o + sizeof(PfRun) * L.nexp_all);
+  L.row_token = o;    o = pf_align(o + sizeof(int) * (size_t)T * k);
   L.posmap = o;       o = pf_align(o + sizeof(int) * (size_t)T * (k + n_shared));
   L.gate = o;         o = pf_align(o + sizeof(float) * T);
-  L.xs = o;           o = pf_align(o + sizeof(__half) * (size_t)L.rmax * hidden);
-  L.h = o;            o = pf_align(o + sizeof(__half) * (size_t)L.rmax * wide);
-  L.yrow = o;         o = pf_align(o + sizeof(float) * (size_t)L.rmax * hidden);
+  L.xs = o;           o = pf_align(o + sizeof(__half) * (size_t)L.in_rows * hidden);
+  L.h = o;            o = pf_align(o + sizeof(__half) * (size_t)L.out_rows * wide);
+  L.yrow = o;         o = pf_align(o + sizeof(float) * (size_t)L.out_rows * hidden);
   L.total = o;
   return L;
 }
 
-// ---- step 1: token rows per expert -----------------------------------------------------------------------
-__global__ void pf_count_kernel(const int32_t* __restrict__ ids, int n, int E, int* __restrict__ counts,
-                                unsigned* __restrict__ status) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int e = ids[i];
-  if (e < 0 || e >= E) {
-    atomicOr(status, (unsigned)SLICEMOE_STATUS_BAD_EXPERT_ID);
-    return;
-  }
-  atomicAdd(&counts[e], 1);
-}
+__device__ __forceinline__ void pf_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pf_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// One warp: padded offsets of every expert (routed, then shared with T rows each) and the tile list.  Lane l takes
-// the experts l, l + 32, ...; warp scans turn the experts' tile and item counts into each tile's place in the lists.
-__global__ void pf_scan_kernel(const int* __restrict__ counts, int E, int n_shared, int T, int inter, int shared_inter,
-                               int* __restrict__ offsets, int* __restrict__ tile_expert, int* __restrict__ tile_row0,
-                               int* __restrict__ item_start, int* __restrict__ ntiles) {
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x >= 32) return;
-  const int n = E + n_shared;
-  int nt = 0, items = 0, nt_routed = 0;  // tiles / first-GEMM work items / routed experts' tiles so far
-  for (int e0 = 0; e0 < n; e0 += 32) {
-    const int e = e0 + lane;
-    const int c = e < n ? (e < E ? counts[e] : T) : 0;
-    const int tiles = (c + kPfTileM - 1) / kPfTileM;
-    const int per = (e < E ? inter : shared_inter) / 64;  // first GEMM: 64 columns of h per work item
-    int tin = tiles, iin = tiles * per;                    // inclusive scans
+// ---- step 1: rows and work items ---------------------------------------------------------------------------
+// One block: the whole plan is a few passes over T k expert ids, and one block needs no grid barrier between them.
+// Counters sit in shared memory up to kPfSmemExperts experts, in the workspace beyond.  Which row a pair gets depends
+// on the order of the atomics, the values computed for it do not.
+constexpr int kPfPlanThreads = 1024;
+constexpr int kPfSmemExperts = 2048;
+struct PfPlanParams {
+  const int32_t* ids;
+  int T, k, E, n_shared;
+  int per1_routed, per1_shared, per2;  // work items per tile: GEMM 1 of a routed / shared expert, GEMM 2
+  PfHead* head;
+  int *counts, *offsets, *cursor;
+  PfRun* runs;
+  int *row_token, *posmap;
+  unsigned* status;
+};
+__device__ __forceinline__ int pf_tiles_of(int count) { return (count + kPfTileN - 1) / kPfTileN; }
+// Exclusive block-wide scan of one value per thread; *total gets the sum.
+__device__ int pf_block_scan(int v, int* warp_sums, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int inc = v;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int a = __shfl_up_sync(0xffffffffu, tin, off), b = __shfl_up_sync(0xffffffffu, iin, off);
-      if (lane >= off) {
-        tin += a;
-        iin += b;
-      }
-    }
-    const int routed = __reduce_add_sync(0xffffffffu, e < E ? tiles : 0);
-    if (e < n) {
-      const int first = nt + tin - tiles;  // the expert's first tile; rows are padded to whole tiles
-      offsets[e] = first * kPfTileM;
-      for (int r = 0; r < tiles; ++r) {
-        tile_expert[first + r] = e;
-        tile_row0[first + r] = (first + r) * kPfTileM;
-        item_start[first + r] = items + iin - tiles * per + r * per;
-      }
-    }
-    nt += __shfl_sync(0xffffffffu, tin, 31);
-    items += __shfl_sync(0xffffffffu, iin, 31);
-    nt_routed += routed;
+  for (int off = 1; off < 32; off <<= 1) {
+    const int a = __shfl_up_sync(0xffffffffu, inc, off);
+    if (lane >= off) inc += a;
   }
-  if (lane == 0) {
-    offsets[n] = nt * kPfTileM;
-    item_start[nt] = items;
-    ntiles[0] = nt;
-    ntiles[1] = nt * kPfTileM;
-    ntiles[2] = items;
-    ntiles[3] = n_shared > 0 ? nt_routed : nt;  // tiles of routed experts: they come first and have inter / 64 items each
+  __syncthreads();  // the previous scan's sums have been read
+  if (lane == 31) warp_sums[warp] = inc;
+  __syncthreads();
+  int before = 0, sum = 0;
+  const int w = warp_sums[lane];
+  static_assert(kPfPlanThreads == 1024, "one warp sum per lane");
+  before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0);
+  sum = __reduce_add_sync(0xffffffffu, w);
+  *total = sum;
+  return before + inc - v;
+}
+__global__ void __launch_bounds__(kPfPlanThreads) pf_plan_kernel(const PfPlanParams p) {
+  __shared__ int s_counts[kPfSmemExperts], s_offsets[kPfSmemExperts], s_cursor[kPfSmemExperts];
+  __shared__ int s_sums[32];
+  const int tid = threadIdx.x;
+  const int n = p.E + p.n_shared;
+  const bool fits = n <= kPfSmemExperts;
+  int* counts = fits ? s_counts : p.counts;
+  int* offsets = fits ? s_offsets : p.offsets;
+  int* cursor = fits ? s_cursor : p.cursor;
+  pf_dep_launch();
+  pf_dep_wait();  // the ids may be the work of the kernel before, which may also still read what is now the workspace
+  for (int e = tid; e < n; e += kPfPlanThreads) {
+    counts[e] = e < p.E ? 0 : p.T;
+    cursor[e] = 0;
+  }
+  if (tid == 0) {
+    *p.status = 0u;
+    p.head->next1 = p.head->next2 = 0;
+  }
+  __syncthreads();
+  const int npairs = p.T * p.k;
+  bool bad = false;
+  for (int i = tid; i < npairs; i += kPfPlanThreads) {
+    const int e = p.ids[i];
+    if (e >= 0 && e < p.E) atomicAdd(&counts[e], 1);
+    else bad = true;
+  }
+  if (bad) atomicOr(p.status, (unsigned)SLICEMOE_STATUS_BAD_EXPERT_ID);
+  __syncthreads();
+  // rows: the routed experts' one after the other
+  int base = 0;
+  for (int e0 = 0; e0 < p.E; e0 += kPfPlanThreads) {
+    const int e = e0 + tid;
+    int total;
+    const int before = pf_block_scan(e < p.E ? counts[e] : 0, s_sums, &total);
+    if (e < p.E) offsets[e] = base + before;
+    base += total;
+  }
+  __syncthreads();
+  for (int i = tid; i < npairs; i += kPfPlanThreads) {
+    const int e = p.ids[i], t = i / p.k;
+    int pos = -1;
+    if (e >= 0 && e < p.E) {
+      pos = offsets[e] + atomicAdd(&cursor[e], 1);
+      p.row_token[pos] = t;
+    }
+    p.posmap[t * (p.k + p.n_shared) + (i - t * p.k)] = pos;
+  }
+  for (int i = tid; i < p.T * p.n_shared; i += kPfPlanThreads) {
+    const int t = i / p.n_shared, j = i - t * p.n_shared;
+    p.posmap[t * (p.k + p.n_shared) + p.k + j] = npairs + j * p.T + t;
+  }
+  // runs: experts with tokens, shared ones first (their contraction in GEMM 2 is usually the longest), then by
+  // falling number of tokens: handed out in this order, the longest items do not come last.  rank = number of
+  // experts that come before.
+  __syncthreads();
+  for (int e = tid; e < n; e += kPfPlanThreads) {
+    const int c = counts[e];
+    if (c == 0) continue;
+    int rank = 0;
+    if (e >= p.E) {
+      rank = e - p.E;
+    } else {
+      rank = p.n_shared;
+      for (int o = 0; o < p.E; ++o) rank += counts[o] > c || (counts[o] == c && o < e);
+    }
+    PfRun r;
+    r.expert = e;
+    r.count = c;
+    r.tiles = pf_tiles_of(c);
+    r.in_row = e < p.E ? offsets[e] : npairs;
+    r.out_row = e < p.E ? offsets[e] : npairs + (e - p.E) * p.T;
+    r.items1 = r.items2 = r.pad_ = 0;
+    p.runs[rank] = r;
+  }
+  __syncthreads();
+  int live = 0, base1 = 0, base2 = 0;
+  for (int r0 = 0; r0 < n; r0 += kPfPlanThreads) {
+    // an expert's rank is below the number of experts with tokens: count them, and scan the runs' work items
+    const int e = r0 + tid;
+    int total;
+    pf_block_scan(e < n && counts[e] > 0 ? 1 : 0, s_sums, &total);
+    live += total;
+  }
+  for (int r0 = 0; r0 < live; r0 += kPfPlanThreads) {
+    const int r = r0 + tid;
+    int v1 = 0, v2 = 0, t1, t2;
+    if (r < live) {
+      const PfRun run = p.runs[r];
+      v1 = run.tiles * (run.expert < p.E ? p.per1_routed : p.per1_shared);
+      v2 = run.tiles * p.per2;
+    }
+    const int b1 = pf_block_scan(v1, s_sums, &t1);
+    const int b2 = pf_block_scan(v2, s_sums, &t2);
+    if (r < live) {
+      p.runs[r].items1 = base1 + b1;
+      p.runs[r].items2 = base2 + b2;
+    }
+    base1 += t1;
+    base2 += t2;
+  }
+  if (tid == 0) {
+    p.head->runs = live;
+    p.head->items1 = base1;
+    p.head->items2 = base2;
   }
 }
 
-// Every (token, slot) pair takes a row of its expert; shared experts take row t.  Which row a pair gets
-// depends on the order of the atomics, the values computed for it do not.
-__global__ void pf_scatter_kernel(const int32_t* __restrict__ ids, int T, int k, int E, int n_shared,
-                                  const int* __restrict__ offsets, int* __restrict__ cursor, int* __restrict__ row_token,
-                                  int* __restrict__ posmap) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int slots = k + n_shared;
-  if (i >= T * slots) return;
-  const int t = i / slots, j = i % slots;
-  int pos = -1;
-  if (j < k) {
-    const int e = ids[t * k + j];
-    if (e >= 0 && e < E) pos = offsets[e] + atomicAdd(&cursor[e], 1);
-  } else {
-    pos = offsets[E + (j - k)] + t;
-  }
-  posmap[i] = pos;
-  if (pos >= 0) row_token[pos] = t;
-}
-
-// ---- step 2: gather x into expert order, bf16 -> fp16; padding rows are zero ----------------------------
-// With a gated shared expert the rows of the first shared expert - one per token - also give the token's gate
-// sigmoid(gate_vec . x): the row is being read anyway.  `shared_row0` points at the first shared expert's offset.
-__global__ void pf_gather_kernel(const uint16_t* __restrict__ x, int hidden, const int* __restrict__ row_token,
-                                 const int* __restrict__ ntiles, __half* __restrict__ xs,
-                                 const float* __restrict__ gate_vec, const int* __restrict__ shared_row0, int T,
-                                 float* __restrict__ gate) {
-  const int row = blockIdx.x;
-  if (row >= ntiles[1]) return;
-  const int t = row_token[row];
-  __half2* dst = reinterpret_cast<__half2*>(xs + (size_t)row * hidden);
-  if (t < 0) {
-    for (int i = threadIdx.x; i < hidden / 2; i += blockDim.x) dst[i] = __floats2half2_rn(0.f, 0.f);
-    return;
-  }
-  const bool gated = gate_vec != nullptr && row >= shared_row0[0] && row < shared_row0[0] + T;
+// ---- step 2: gather x into expert order, bf16 -> fp16 ----------------------------------------------------
+// A warp per row, 16 bytes per lane and step (4 where x is not 16-byte aligned).  With a gated shared expert the last
+// T rows - the tokens in their own order - also give the token's gate sigmoid(gate_vec . x): the row is being read
+// anyway.
+constexpr int kPfGatherThreads = 256;
+template <int WORDS>
+__global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const uint16_t* __restrict__ x, int hidden, int T,
+                                                                     const int* __restrict__ row_token, int routed_rows,
+                                                                     int rows, __half* __restrict__ xs,
+                                                                     const float* __restrict__ gate_vec,
+                                                                     float* __restrict__ gate) {
+  const int row = (int)(blockIdx.x * (kPfGatherThreads / 32) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  pf_dep_launch();
+  pf_dep_wait();
+  if (row >= rows) return;
+  const int t = row < routed_rows ? row_token[row] : row - routed_rows;
+  if ((unsigned)t >= (unsigned)T) return;  // ids out of range leave rows at the end of the routed ones without a token
   const uint32_t* src = reinterpret_cast<const uint32_t*>(x + (size_t)t * hidden);
+  uint32_t* dst = reinterpret_cast<uint32_t*>(xs + (size_t)row * hidden);
+  const bool gated = gate_vec != nullptr && row >= routed_rows;
   float dot = 0.f;
-  for (int i = threadIdx.x; i < hidden / 2; i += blockDim.x) {
-    const uint32_t raw = src[i];
-    const float lo = __uint_as_float(raw << 16), hi = __uint_as_float(raw & 0xffff0000u);
-    dst[i] = __floats2half2_rn(lo, hi);
-    if (gated) {
-      const float2 gv = *reinterpret_cast<const float2*>(gate_vec + 2 * i);
-      dot = fmaf(gv.x, lo, dot);
-      dot = fmaf(gv.y, hi, dot);
+#pragma unroll 4
+  for (int i = lane * WORDS; i < hidden / 2; i += 32 * WORDS) {
+    uint32_t in[WORDS], out[WORDS];
+    if (WORDS == 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(src + i);
+      in[0] = v.x; in[WORDS / 4] = v.y; in[WORDS / 2] = v.z; in[WORDS - 1] = v.w;
+    } else {
+      in[0] = src[i];
     }
+#pragma unroll
+    for (int j = 0; j < WORDS; ++j) {
+      const float lo = __uint_as_float(in[j] << 16), hi = __uint_as_float(in[j] & 0xffff0000u);
+      const __half2 h = __floats2half2_rn(lo, hi);
+      out[j] = *reinterpret_cast<const uint32_t*>(&h);
+      if (gated) {
+        const float2 gv = *reinterpret_cast<const float2*>(gate_vec + 2 * (i + j));
+        dot = fmaf(gv.x, lo, dot);
+        dot = fmaf(gv.y, hi, dot);
+      }
+    }
+    if (WORDS == 4) *reinterpret_cast<uint4*>(dst + i) = make_uint4(out[0], out[WORDS / 4], out[WORDS / 2], out[WORDS - 1]);
+    else dst[i] = out[0];
   }
-  if (gated) {  // block sum in a fixed order: lanes by butterfly, then the warps one after the other
-    __shared__ float part[32];
+  if (gated) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = dot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float sum = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += part[w];
-      gate[t] = 1.f / (1.f + expf(-sum));
-    }
+    if (lane == 0) gate[t] = 1.f / (1.f + expf(-dot));
   }
 }
 
 // ---- steps 3 and 4: the grouped GEMM on the 5th-generation tensor cores ---------------------------------
-// One persistent CTA per SM walks work items (128 weight rows x 128 token rows) and computes the transposed
-// product D[weight row, token].  Per 64-column step of the contraction:
-//   - the load warp brings the token tile (rows of x or h, fp16) into shared memory with one TMA tiled copy,
-//     128-byte swizzle: the B operand;
-//   - the dequantisation warps (sets of four, taking the steps in turn) build from the nibble planes and
-//     zero-points the integer d = q - zp (or 16 (q_msb - (zp >> 4))), exact in fp16, and multiply it by the
-//     group's scale normalised by a power of two per weight row: the product is kept as p + e with p the
-//     rounded fp16 product and e = fma(d, f, -p) the exact remainder, and both halves go straight into tensor
-//     memory with tcgen05.st: the A operands, one weight row per lane.  Weights never pass through shared
-//     memory as fp16;
-//   - the MMA warp issues eight tcgen05.mma (M 128, N 128, K 16): leading parts and remainders against the
-//     same tokens, all accumulating into one of two fp32 accumulators in tensor memory.
-// When an item's contraction is complete its accumulator is handed to eight epilogue warps, which read it with
-// tcgen05.ld and multiply each row by its power of two; meanwhile the next item accumulates in the other
-// buffer.  No weight is ever rounded: p + e equals s 2^n (q - zp) exactly.  Every wait is bounded; a wait that
-// runs out sets SLICEMOE_STATUS_WAIT_TIMEOUT and the CTA winds down (tensor memory is freed on every path).
-constexpr int kUSets = 2;           // dequantisation sets of four warps; the steps go round them
-constexpr int kUWarpTma = 8 + 4 * kUSets, kUWarpMma = kUWarpTma + 1;
-constexpr int kUThreads = 32 * (kUWarpMma + 1);  // warps 0-7 epilogue, then the dequantisation sets, loads, MMA issue
-constexpr int kUStages = 4;
-constexpr int kUTileBytes = kPfTileM * kPfChunkK * 2;  // 16,384: the token tile of a step
-constexpr int kUScaleSlots = 4;     // ring of per-item row scales: dequantisation is less than 4 items ahead of the epilogue
-constexpr int kUScaleBytes = kUScaleSlots * kPfTileB * 4;
-constexpr int kURawDepth = 3;       // steps of raw plane words each dequantisation warp keeps in flight (cp.async)
-constexpr int kURawBytes = 4 * kUSets * kURawDepth * 2048;  // per warp and step: 2 blocks x 512 bytes MSB, the same of LSB
-constexpr int kUXchBytes = 4 * 64 * 32 * 4;        // silu(gate) on its way from the gate warps to the up warps
-constexpr int kUSmemBytes =
-    kUStages * kUTileBytes + kURawBytes + kUXchBytes + kUScaleBytes + 1024 /* alignment slack */ + 256 /* barriers */;
-constexpr int kUAccCols = 256;      // two accumulators of 128 fp32 columns (tokens)
-constexpr int kUWCols = 64;         // a step's weights: 64 fp16 per row, twice (leading part, remainder)
-constexpr int kUTmemCols = 512;     // accumulators + kUStages weight stages, rounded up to a power of two
-constexpr long long kUWaitCycles = 2000000000ll;
+// One persistent CTA per SM takes work items (128 weight rows x up to 192 token rows) from a counter and computes the
+// transposed product D[weight row, token].  Per 128-column step of the contraction:
+//   - the token warp brings the token tile (rows of x or h, fp16) into shared memory with TMA tiled copies of 32
+//     rows, 128-byte swizzle: the B operand;
+//   - the weight warps (two sets of four, taking the steps in turn) turn nibbles into fp16 integers d = q - zp (or
+//     2^shift (q_msb - (zp >> shift))) and store them to tensor memory with tcgen05.st, one weight row per lane: the A
+//     operand.  Weights never pass through shared memory as fp16;
+//   - the MMA warp issues tcgen05.mma (M 128, K 16) for one quantisation group at a time, into one of two fp32
+//     accumulators in tensor memory.  A tile wider than 96 tokens is cut into two halves with an accumulator each; a
+//     narrower one uses them for alternate groups.  Either way one accumulator is read while the other is written;
+//   - the sum warps (two warpgroups) read a group's sums with tcgen05.ld and add them, times the weight row's scale of
+//     that group, to fp32 registers: 96 tokens per warpgroup, one weight row per lane.
+// After the last group the sum warps hold the item's result and write it: SwiGLU between gate and up rows (GEMM 1,
+// exchanged through shared memory), fp32 rows (GEMM 2).  A scheduler warp fetches items ahead and leaves their
+// description in a ring in shared memory.
+//
+// Why integers and a read-out per group: the dequantised weight s (q - zp) has up to 20 significant bits.  Kept as the
+// exact sum of two fp16 numbers (the version before this one) every product is issued twice and the conversion is twice
+// as long; the read-out costs half an instruction per value with packed multiply-adds.  Why 192 tokens: the conversion of a
+// weight tile is shared by all its tokens, and 96 sums per lane leave registers (61,440 at launch) for eight weight
+// warps, without which a tile of few tokens is bound by one set's latency.
+// Every wait is bounded; a wait that runs out sets SLICEMOE_STATUS_WAIT_TIMEOUT and the CTA winds down (tensor memory is
+// freed on every path).
+constexpr int kUSumWarps = 8;                 // two warpgroups
+constexpr int kUSets = 2;                     // sets of four weight warps; the steps go round them
+constexpr int kUWarpTok = kUSumWarps + 4 * kUSets, kUWarpMma = kUWarpTok + 1, kUWarpSched = kUWarpTok + 2,
+              kUWarpMeta = kUWarpTok + 3;
+constexpr int kUThreads = 32 * (kUWarpTok + 4);
+// registers per thread at launch 96 (640 threads); the split's sum is the launch's: 256 x 152 + 256 x 72 + 128 x 32
+constexpr int kURegsSum = 152, kURegsWeight = 72, kURegsRest = 32;
+static_assert(256 * kURegsSum + 256 * kURegsWeight + 128 * kURegsRest <= kUThreads * 96, "register split");
+constexpr int kUStages = 3;                   // steps in flight: tokens in shared, weights in tensor memory
+constexpr int kUBoxRows = 32, kUBoxCols = 64; // token rows and columns of one TMA copy (128 bytes: the swizzle's span)
+constexpr int kUBoxBytes = kUBoxRows * kUBoxCols * 2;
+constexpr int kUPanelBytes = kPfTileN * kUBoxCols * 2;  // half of a step's tile: 64 columns of all tokens
+constexpr int kUTileBytes = 2 * kUPanelBytes;
+constexpr int kURawDepth = 2;                 // steps of raw plane words each weight warp keeps in flight (cp.async)
+constexpr int kURawStep = 4096;               // of a warp and step: [plane][block][half] x 512 bytes
+constexpr int kURawBytes = 4 * kUSets * kURawDepth * kURawStep;
+constexpr int kUItemSlots = 8;
+// Scales and zero-points of 16 quantisation groups at a time: [8 row blocks][16 groups][16 rows], 512 + 256 bytes each
+constexpr int kUMetaGroups = 16, kUMetaStages = 2;
+constexpr int kUMetaScale = kUMetaGroups * 32, kUMetaZp = kUMetaGroups * 16;
+constexpr int kUMetaBytes = 8 * (kUMetaScale + kUMetaZp);
+constexpr int kUHalfMax = kPfTileN / 2;       // tokens per warpgroup
+constexpr int kUAccCols = 128;                // tensor-memory columns between the two accumulators
+constexpr int kUWCol0 = 256, kUWCols = 64;    // weight stages: 128 fp16 per row
+constexpr int kUTmemCols = 512;
+constexpr uint32_t kUWaitCycles = 2000000000u;
+constexpr uint32_t kUCopyCycles = 2000000u;  // a millisecond: far more than any copy takes
+
+// What a work item is.  [0] gate, [1] up in GEMM 1; both down in GEMM 2.  Pointers are at the item's first row block.
+struct __align__(16) PfItem {
+  const uint8_t* msb[2];
+  const uint8_t* lsb[2];
+  const uint16_t* scale[2];
+  const uint8_t* zp[2];
+  int nk;        // steps
+  int n, n0;     // tokens of the tile, up to a multiple of 16; of the first warpgroup
+  int halves;    // accumulators of a group: 2 when the tile is cut in two
+  int count;     // tokens that are there
+  int in_row, out_row;
+  int col;       // first column of h or of y
+  int prec;      // both slices (else the MSB slice alone)
+  int stop;      // no more items
+};
+
+struct USmem {
+  static constexpr int tok = 0;
+  static constexpr int raw = tok + kUStages * kUTileBytes;
+  static constexpr int meta = raw + kURawBytes;
+  static constexpr int items = meta + kUMetaStages * kUMetaBytes;
+  static constexpr int bars = items + kUItemSlots * (int)sizeof(PfItem);
+  // barriers: tokens and weights of a step in / step done / sums there [accumulator] / sums read [accumulator] / item
+  // there, item read / scales and zero-points in, read / drained
+  static constexpr int full = 0, done = full + kUStages, acc_full = done + kUStages, acc_free = acc_full + 2,
+                       item_full = acc_free + 2, item_free = item_full + kUItemSlots, meta_full = item_free + kUItemSlots,
+                       meta_free = meta_full + kUMetaStages, drain = meta_free + kUMetaStages, nbars = drain + 1;
+  static constexpr int tail = bars + nbars * 8;  // tensor-memory address, abort flag
+  static constexpr int total = tail + 16;
+};
+static_assert(USmem::bars % 8 == 0 && USmem::items % 16 == 0, "alignment");
+constexpr int kUSmemBytes = USmem::total + 1024 /* alignment slack */;
+static_assert(kUSmemBytes <= 227 * 1024, "shared memory budget");
 
 struct PfGemmParams {
   const slicemoe_expert* experts;  // routed
   const slicemoe_expert* shared;
   const uint8_t* expert_prec;      // per routed expert: 1 = both slices, 0 = MSB slice only
-  const int* tile_expert;
-  const int* tile_row0;
-  const int* item_start;           // phase 1: first work item of every tile (prefix sum of its n-tiles)
-  const int* ntiles;               // [0] tiles, [1] rows, [2] phase-1 work items
-  __half* h;                       // phase 1 output, phase 2 A operand [rows, ldh]
-  float* yrow;                     // phase 2 output [rows, hidden]
+  const PfRun* runs;
+  PfHead* head;
+  __half* h;                       // GEMM 1 output, GEMM 2 token operand [rows, ldh]
+  float* yrow;                     // GEMM 2 output [rows, hidden]
   unsigned* status;
   int E, hidden, inter, shared_inter, ldh;
   int shift;  // b_high - b_low
@@ -248,16 +385,24 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
                : "memory");
   return ok != 0;
 }
-__device__ __noinline__ bool mbar_wait_slow(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  const long long t0 = clock64();
-  for (;;) {
-    if (mbar_try(b, parity)) return true;
-    if (*abort_flag || clock64() - t0 > kUWaitCycles) return false;
-  }
+// The same, but the hardware may hold the thread for up to 10 ms while the phase is not there: a waiting warp then takes
+// no issue slots from the others.
+__device__ __forceinline__ bool mbar_try_long(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
+               : "=r"(ok)
+               : "r"(smem_u32(b)), "r"(parity), "r"(10000000u)
+               : "memory");
+  return ok != 0;
 }
+// By a whole warp; every lane gets the same answer.  (No call: the sum warps have no registers to set aside for one.)
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try(b, parity)) return true;  // the common case costs one instruction
-  return mbar_wait_slow(b, parity, abort_flag);
+  if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;  // the common case costs one instruction
+  const uint32_t t0 = (uint32_t)clock64();
+  for (;;) {
+    if (__all_sync(0xffffffffu, mbar_try_long(b, parity))) return true;
+    if (__any_sync(0xffffffffu, *abort_flag != 0 || (uint32_t)clock64() - t0 > kUWaitCycles)) return false;
+  }
 }
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
@@ -280,19 +425,29 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
   d |= (uint64_t)2 << 61;                   // 128-byte swizzle
   return d;
 }
-// Instruction descriptor: fp16 x fp16 -> fp32, both operands K-major, M 128, N 128.
-constexpr uint32_t kUmmaIdesc = (1u << 4) | ((uint32_t)(kPfTileB >> 3) << 17) | ((uint32_t)(kPfTileM >> 4) << 24);
+// Instruction descriptor: fp16 x fp16 -> fp32, both operands K-major, M 128, N tokens (a multiple of 16).
+__device__ __forceinline__ uint32_t umma_idesc(int n) { return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kPfTileB >> 4) << 24); }
+
+// One lane of a converged warp.  The compiler knows that a branch on it is taken by one thread: what the branch computes
+// stays on the uniform datapath, where the tensor instructions take their operands from.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0;
+}
 
 // D (tensor memory) (+)= A (tensor memory: lane = row, 32-bit column = two consecutive k) x B (shared memory).
-__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b), "r"(kUmmaIdesc), "r"(acc)
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+// 16 rows x 32 columns: lane 4 g + c gives row g, columns 8 i + 2 c and the next, in registers 4 i and 4 i + 1, and row
+// g + 8, the same columns, in registers 4 i + 2 and 4 i + 3.
+__device__ __forceinline__ void tmem_st_16x32(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
       "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
@@ -301,74 +456,37 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// With the wait in the same statement: nothing that uses the registers can come between.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Two fp32 multiply-adds in one instruction: acc += v * s, s in both halves of ss.
+__device__ __forceinline__ void fma2(uint64_t& acc, uint32_t v0, uint32_t v1, uint64_t ss) {
+  asm("{\n .reg .b64 v;\n mov.b64 v, {%1, %2};\n fma.rn.f32x2 %0, v, %3, %0;\n}" : "+l"(acc) : "r"(v0), "r"(v1), "l"(ss));
+}
+__device__ __forceinline__ float half_of(uint64_t v, int i) { return __uint_as_float((uint32_t)(v >> (32 * i))); }
 
-// Byte offset of element (row, k) in a swizzled [128][64] fp16 tile (k a multiple of 4 here).
-__device__ __forceinline__ uint32_t swz128(int row, int k) {
-  return (uint32_t)(row * 128 + ((((k >> 3) ^ (row & 7)) << 4) | ((k & 7) << 1)));
-}
-
-// What a work item is: which tile of token rows, which 128 weight rows of which expert.
-struct UItem {
-  const slicemoe_expert* ex;
-  int row0, nt, K;
-  bool prec;     // both slices (else the MSB slice alone)
-  bool missing;  // both slices were asked for but the LSB planes are absent
-};
+// The run that a work item belongs to: the last one whose first item is not above it.  Whole warp, 32 runs a step.
 template <int PHASE>
-__device__ __forceinline__ int u_item_count(const PfGemmParams& p) {
-  return PHASE == 1 ? p.ntiles[2] : p.ntiles[0] * (p.hidden / 128);
-}
-template <int PHASE>
-__device__ __forceinline__ UItem u_item(const PfGemmParams& p, int item) {
-  int tile, nt;
-  if (PHASE == 1) {
-    // routed tiles first, inter / 64 items each, then the shared experts' tiles with shared_inter / 64 items each
-    const int per_r = p.inter / 64, routed_items = p.ntiles[3] * per_r;
-    if (item < routed_items) {
-      tile = item / per_r;
-      nt = item - tile * per_r;
-    } else {
-      const int per_s = p.shared_inter / 64, rest = item - routed_items;
-      tile = p.ntiles[3] + rest / per_s;
-      nt = rest - (rest / per_s) * per_s;
-    }
-  } else {
-    const int per = p.hidden / 128;
-    tile = item / per;
-    nt = item - tile * per;
+__device__ __forceinline__ int u_find_run(const PfRun* runs, int n, int item, int lane) {
+  int lo = 0;  // the answer is in [lo, n)
+  int step = 1;
+  while (step * 32 < n) step *= 32;
+  for (; step >= 1; step >>= 5) {
+    const int r = lo + lane * step;
+    const bool below = r < n && (PHASE == 1 ? runs[r].items1 : runs[r].items2) <= item;
+    lo += (__popc(__ballot_sync(0xffffffffu, below)) - 1) * step;
+    if (step == 1) break;
   }
-  UItem it;
-  const int e = p.tile_expert[tile];
-  const bool is_shared = e >= p.E;
-  it.ex = is_shared ? p.shared + (e - p.E) : p.experts + e;
-  it.row0 = p.tile_row0[tile];
-  it.nt = nt;
-  it.K = PHASE == 1 ? p.hidden : (is_shared ? p.shared_inter : p.inter);
-  it.prec = is_shared ? true : (p.expert_prec[e] != 0);
-  const bool has_lsb = PHASE == 1 ? (it.ex->gate.lsb && it.ex->up.lsb) : (it.ex->down.lsb != nullptr);
-  it.missing = it.prec && !has_lsb;
-  if (it.missing) it.prec = false;
-  return it;
-}
-// Weight row block (16 rows) that row block rbk (0..7) of an item's 128 weight rows holds.  First GEMM: rows
-// [0,64) are gate rows of h columns [64 nt, 64 nt + 64), rows [64,128) the up rows of the same columns.
-template <int PHASE>
-__device__ __forceinline__ const slicemoe_mat& u_block_mat(const UItem& it, int rbk, int* rb) {
-  if (PHASE == 1) {
-    *rb = it.nt * 4 + (rbk & 3);
-    return rbk < 4 ? it.ex->gate : it.ex->up;
-  }
-  *rb = it.nt * 8 + rbk;
-  return it.ex->down;
+  return lo;
 }
 
 template <int G, int PHASE>
@@ -376,35 +494,36 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   constexpr int LG = G == 128 ? 7 : (G == 64 ? 6 : 5);
   extern __shared__ uint8_t u_smem_raw[];
   uint8_t* smem = u_smem_raw + ((1024 - (smem_u32(u_smem_raw) & 1023)) & 1023);
-  uint8_t* raw_ring = smem + kUStages * kUTileBytes;
-  float(*xch)[64][32] = reinterpret_cast<float(*)[64][32]>(raw_ring + kURawBytes);  // [pair][token][row]
-  float(*row_scale)[kPfTileB] = reinterpret_cast<float(*)[kPfTileB]>(raw_ring + kURawBytes + kUXchBytes);  // [item % 4][row]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(raw_ring + kURawBytes + kUXchBytes + kUScaleBytes);
-  uint64_t* full = bars;                    // [stage]: tokens landed (TMA) and weights stored (8 warps)
-  uint64_t* empty = bars + kUStages;        // [stage]: the MMAs that read the stage have completed
-  uint64_t* acc_full = bars + 2 * kUStages;       // [2]: an item's sums are complete in the accumulator
-  uint64_t* acc_empty = bars + 2 * kUStages + 2;  // [2]: the epilogue warps have read it
-  uint64_t* xch_full = bars + 2 * kUStages + 4;   // [4]: silu(gate) of a warp pair is in shared memory
-  uint64_t* xch_empty = bars + 2 * kUStages + 8;  // [4]: it has been consumed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kUStages + 12);
+  PfItem* items = reinterpret_cast<PfItem*>(smem + USmem::items);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + USmem::bars);
+  uint64_t *full = bars + USmem::full, *done = bars + USmem::done, *acc_full = bars + USmem::acc_full,
+           *acc_free = bars + USmem::acc_free, *item_full = bars + USmem::item_full, *item_free = bars + USmem::item_free,
+           *meta_full = bars + USmem::meta_full, *meta_free = bars + USmem::meta_free, *drain = bars + USmem::drain;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + USmem::tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   // the warp index by way of a shuffle: the compiler then knows that it is uniform across the warp, and keeps
   // the role branches and what they compute (addresses, descriptors, counters) on the uniform datapath
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  pf_dep_launch();
   if (tid == 0) {
     for (int s = 0; s < kUStages; ++s) {
-      mbar_init(&full[s], 5);  // the set's four dequantisation warps and the load warp
-      mbar_init(&empty[s], 1);
+      mbar_init(&full[s], 1 + 4);  // the token warp (and its copies' bytes) and a set's four warps
+      mbar_init(&done[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 8);
+      mbar_init(&acc_free[a], 8);  // the eight sum warps once each, or one warpgroup's four twice each
     }
-    for (int a = 0; a < 4; ++a) {
-      mbar_init(&xch_full[a], 1);
-      mbar_init(&xch_empty[a], 1);
+    for (int s = 0; s < kUItemSlots; ++s) {
+      mbar_init(&item_full[s], 1);
+      mbar_init(&item_free[s], kUSumWarps + 4 * kUSets + 3);
     }
+    for (int s = 0; s < kUMetaStages; ++s) {
+      mbar_init(&meta_full[s], 1);
+      mbar_init(&meta_free[s], kUSumWarps + 4 * kUSets);
+    }
+    mbar_init(drain, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -417,284 +536,451 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int n_items = u_item_count<PHASE>(p);
   bool alive = true;
+  pf_dep_wait();  // the plan, the token rows and the counters are the work of the kernels before
 
-  if (warp == kUWarpTma) {
-    // ---- token tiles: one TMA copy per step ----
-    if (lane == 0) {
-      uint32_t s = 0, ph = 0;
-      // the next item's description is fetched while this item's copies go out
-      UItem w{};
-      if ((int)blockIdx.x < n_items) w = u_item<PHASE>(p, blockIdx.x);
-      for (int item = blockIdx.x; item < n_items && alive; item += gridDim.x) {
-        UItem wn = w;
-        if (item + (int)gridDim.x < n_items) wn = u_item<PHASE>(p, item + gridDim.x);
-        const int nk = w.K / kPfChunkK;
+  if (warp >= kUWarpTok) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kURegsRest));
+    if (warp == kUWarpTok) {
+      // ---- token tiles: TMA copies of 32 rows x 64 columns, a lane each ----
+      uint32_t st = 0, par = 1;  // stage; parity of the use before (the first one waits for nothing)
+      const int box = lane % (kPfTileN / kUBoxRows), panel = lane / (kPfTileN / kUBoxRows);
+      for (uint32_t ni = 0;; ++ni) {
+        const PfItem& it = items[ni % kUItemSlots];
+        if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
+        if (it.stop) break;
+        const int nk = it.nk, boxes = (it.n + kUBoxRows - 1) / kUBoxRows, row = it.in_row + box * kUBoxRows;
+        // released at once, as by everybody: the next item's description must not depend on this one's progress (the
+        // weight warps want it while they have steps of this one to deliver)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
         for (int kc = 0; kc < nk; ++kc) {
-          if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { alive = false; break; }
-          mbar_expect_tx(&full[s], kUTileBytes);
-          asm volatile(
-              "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-                  smem_u32(smem + s * kUTileBytes)),
-              "l"(&tm_tok), "r"(smem_u32(&full[s])), "r"(kc * kPfChunkK), "r"(w.row0)
-              : "memory");
-          if (++s == kUStages) { s = 0; ph ^= 1; }
+          if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
+          if (lane == 0) mbar_expect_tx(&full[st], 2 * boxes * kUBoxBytes);
+          __syncwarp();
+          if (box < boxes && panel < 2)
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+                    smem_u32(smem + USmem::tok + st * kUTileBytes + panel * kUPanelBytes + box * kUBoxBytes)),
+                "l"(&tm_tok), "r"(smem_u32(&full[st])), "r"(kc * kPfChunkK + panel * kUBoxCols), "r"(row)
+                : "memory");
+          if (++st == kUStages) { st = 0; par ^= 1; }
         }
-        w = wn;
+        if (!alive) break;
       }
-    }
-  } else if (warp == kUWarpMma) {
-    // ---- MMA issue: D[weight row, token] += W[weight row, k] (tensor memory) x X[token, k] (shared memory) ----
-    // The whole warp walks the loop (waits included) so that its bookkeeping stays uniform; lane 0 issues.
-    uint32_t st = 0, ph = 0, ni = 0;  // stage, its parity, items issued so far
-    uint64_t* last_empty = nullptr;
-    uint32_t last_ph = 0;
-    const uint64_t bd0 = umma_desc(smem_u32(smem));
-    UItem w{};
-      if ((int)blockIdx.x < n_items) w = u_item<PHASE>(p, blockIdx.x);
-    for (int item = blockIdx.x; item < n_items && alive; item += gridDim.x, ++ni) {
-      UItem wn = w;
-      if (item + (int)gridDim.x < n_items) wn = u_item<PHASE>(p, item + gridDim.x);
-      const int nk = w.K / kPfChunkK;
-      const uint32_t ab = ni & 1;
-      // the accumulator must have been read out (the item before the previous one used it)
-      if (!__all_sync(0xffffffffu, mbar_wait(&acc_empty[ab], ((ni >> 1) & 1) ^ 1, abort_flag))) { alive = false; break; }
-      tc_fence_after();
-      for (int kc = 0; kc < nk; ++kc) {
-        if (!__all_sync(0xffffffffu, mbar_wait(&full[st], ph, abort_flag))) { alive = false; break; }
-        tc_fence_after();
-        const uint64_t bd = bd0 + (uint64_t)(st * (kUTileBytes >> 4));
-        const uint32_t a_tmem = tmem + kUAccCols + st * kUWCols;
-        if (lane == 0) {
+      // No copy may still be on its way into shared memory when the CTA ends (only after a time-out can one be): the
+      // step's barrier also counts the weight warps, so it cannot tell; the longest a copy can take is waited out.
+      if (!alive) {
+        const uint32_t t0 = (uint32_t)clock64();
+        while ((uint32_t)clock64() - t0 < kUCopyCycles) {}
+      }
+    } else if (warp == kUWarpMma) {
+      // ---- MMA issue: D[weight row, token] += W[weight row, k] (tensor memory) x X[token, k] (shared memory) ----
+      // The whole warp walks the loop, so that its state stays on the uniform datapath, where the tensor instructions take
+      // their operands from; one elected lane issues.  (All of it in one lane: twice the time per step.)
+      uint32_t st = 0, par = 0;  // stage and parity of its use
+      uint32_t free0 = 1, free1 = 1;  // parity to wait for before an accumulator is written again (at first it is free)
+      bool issued = false;
+      const uint64_t bd0 = umma_desc(smem_u32(smem + USmem::tok));
+      constexpr int kGroups = 128 / G, kKs = G / 16;  // quantisation groups of a step, K 16 slices of a group
+      for (uint32_t ni = 0; alive; ++ni) {
+        const PfItem& it = items[ni % kUItemSlots];
+        if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
+        if (__shfl_sync(0xffffffffu, it.stop, 0)) break;
+        const int nk = __shfl_sync(0xffffffffu, it.nk, 0), halves = __shfl_sync(0xffffffffu, it.halves, 0),
+                  n0 = __shfl_sync(0xffffffffu, it.n0, 0), n = __shfl_sync(0xffffffffu, it.n, 0);
+        __syncwarp();
+        if (elect_one()) mbar_arrive(&item_free[ni % kUItemSlots]);
+        const uint32_t id_first = umma_idesc(halves == 2 ? n0 : n), id_second = umma_idesc(n - n0);
+        uint32_t alt = 0;  // narrow tiles: the accumulator whose turn it is
+        for (int kc = 0; kc < nk && alive; ++kc) {
+          if (!mbar_wait(&full[st], par, abort_flag)) { alive = false; break; }
+          const uint64_t bd_step = bd0 + (uint64_t)((st * kUTileBytes) >> 4);
+          const uint32_t a_step = tmem + kUWCol0 + st * kUWCols;
 #pragma unroll
-          for (int ks = 0; ks < kPfChunkK / 16; ++ks) {
-            // leading part and remainder of the weights against the same tokens
-            umma_f16_ts(tmem + ab * kPfTileM, a_tmem + 8 * ks, bd + 2 * ks, (kc | ks) ? 1u : 0u);
-            umma_f16_ts(tmem + ab * kPfTileM, a_tmem + 32 + 8 * ks, bd + 2 * ks, 1u);
+          for (int grp = 0; grp < kGroups; ++grp) {
+            for (int half = 0; half < halves; ++half) {
+              const uint32_t buf = halves == 2 ? (uint32_t)half : alt;
+              if (!mbar_wait(&acc_free[buf], buf ? free1 : free0, abort_flag)) { alive = false; break; }
+              if (buf) free1 ^= 1u;
+              else free0 ^= 1u;
+              tc_fence_after();
+              const uint32_t d = tmem + buf * kUAccCols, id = half ? id_second : id_first;
+              const uint64_t bd = bd_step + (half ? (uint64_t)(n0 * 8) : 0ull);
+              if (elect_one()) {
+#pragma unroll
+                for (int ks = 0; ks < kKs; ++ks) {
+                  const int k16 = grp * kKs + ks;  // within the step; four to a panel
+                  umma_f16_ts(d, a_step + 8 * k16, bd + (uint64_t)((k16 >> 2) * (kUPanelBytes >> 4) + 2 * (k16 & 3)), id, ks ? 1u : 0u);
+                }
+                if (grp == kGroups - 1 && half == halves - 1) umma_commit(&done[st]);
+                umma_commit(&acc_full[buf]);
+              }
+              issued = true;
+              __syncwarp();
+            }
+            alt ^= 1u;
+            if (!alive) break;
           }
-          umma_commit(&empty[st]);
+          if (++st == kUStages) { st = 0; par ^= 1; }
+        }
+      }
+      // the last commits must have arrived before shared and tensor memory go away
+      if (issued) {
+        if (elect_one()) umma_commit(drain);
+        __syncwarp();
+        const uint32_t t0 = (uint32_t)clock64();
+        while (!mbar_try(drain, 0) && (uint32_t)clock64() - t0 < kUWaitCycles) {}
+        __syncwarp();
+      }
+    } else if (warp == kUWarpSched) {
+      // ---- scheduler: takes items from the counter and describes them ----
+      int* next = PHASE == 1 ? &p.head->next1 : &p.head->next2;
+      const int n_runs = p.head->runs, n_items = PHASE == 1 ? p.head->items1 : p.head->items2;
+      // How far ahead: one item where an item is long (its successor is fetched when the sums of the item itself have
+      // begun, and no CTA sits on items that another could take), else as many as the ring holds.
+      constexpr int kLongItem = 8, kAheadShort = 6;
+      static_assert(kAheadShort <= kUItemSlots && 2 * kURawDepth < kAheadShort, "items between the copies and their use");
+      int ahead = kAheadShort;
+      for (uint32_t ni = 0;; ++ni) {
+        if (ni >= (uint32_t)ahead) {
+          const uint32_t j = ni - ahead;
+          if (!mbar_wait(&item_free[j % kUItemSlots], (j / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
+        }
+        int item = 0;
+        if (lane == 0) item = atomicAdd(next, 1);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        PfItem& it = items[ni % kUItemSlots];
+        PfRun r{};
+        bool prec = true;
+        int in_run = 0;
+        const slicemoe_expert* ex = nullptr;
+        const void* ptr = nullptr;
+        if (item < n_items) {
+          const int run = u_find_run<PHASE>(p.runs, n_runs, item, lane);
+          r = p.runs[run];
+          in_run = item - (PHASE == 1 ? r.items1 : r.items2);
+          const bool is_shared = r.expert >= p.E;
+          ex = is_shared ? p.shared + (r.expert - p.E) : p.experts + r.expert;
+          prec = is_shared || p.expert_prec[r.expert] != 0;
+          // lanes 0 .. 7: MSB, LSB, scales, zero-points of the first and of the second matrix
+          const slicemoe_mat* m = PHASE == 1 ? ((lane & 1) ? &ex->up : &ex->gate) : &ex->down;
+          const int what = (lane >> 1) & 3;
+          ptr = what == 0 ? m->msb : what == 1 ? m->lsb : what == 2 ? (const void*)m->scale : (const void*)m->zp;
+          const bool no_lsb = __any_sync(0xffffffffu, what == 1 && ptr == nullptr);
+          if (prec && no_lsb) {  // both slices were asked for but the LSB planes are absent
+            if (lane == 0) atomicOr(p.status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
+            prec = false;
+          }
+        }
+        if (item < n_items) {
+          // items of a run: weight tile by weight tile, its token tiles next to one another (they share the weights)
+          const int nt = in_run / r.tiles, tile = in_run - nt * r.tiles;
+          const bool is_shared = r.expert >= p.E;
+          const int K = PHASE == 1 ? p.hidden : (is_shared ? p.shared_inter : p.inter);
+          ahead = K / kPfChunkK >= kLongItem ? 1 : kAheadShort;
+          const int width = ((r.count + r.tiles - 1) / r.tiles + 15) & ~15;  // the tiles are equally wide, the last may be shorter
+          const int t0 = tile * width, count = max(0, min(width, r.count - t0)), n = (count + 15) & ~15;
+          // the item's first row block: 4 of gate and of up per 64 columns of h, or 8 of down
+          const size_t rb = (size_t)nt * (PHASE == 1 ? 4 : 8), blocks = rb * (K / 64), entries = rb * (K >> LG) * 16;
+          const int what = (lane >> 1) & 3;
+          if (lane < 8) {
+            const uint8_t* b = reinterpret_cast<const uint8_t*>(ptr);
+            if (what == 0) it.msb[lane & 1] = b + blocks * 512;
+            else if (what == 1) it.lsb[lane & 1] = b ? b + blocks * 512 : b;
+            else if (what == 2) it.scale[lane & 1] = reinterpret_cast<const uint16_t*>(b) + entries;
+            else it.zp[lane & 1] = b + entries;
+          }
+          if (lane == 0) {
+            it.nk = K / kPfChunkK;
+            it.n = n;
+            it.halves = n > kUHalfMax ? 2 : 1;
+            // two accumulators: halves of a multiple of 16; one: the first warpgroup reads whole 32-column pieces
+            it.n0 = n > kUHalfMax ? ((n / 2 + 15) & ~15) : min(n, 32 * ((n + 63) / 64));
+            it.count = count;
+            it.in_row = (PHASE == 1 ? r.in_row : r.out_row) + t0;
+            it.out_row = r.out_row + t0;
+            it.col = nt * (PHASE == 1 ? 64 : 128);
+            it.prec = prec ? 1 : 0;
+            it.stop = 0;
+          }
+        } else if (lane == 0) {
+          it.stop = 1;
         }
         __syncwarp();
-        last_empty = &empty[st];
-        last_ph = ph;
-        if (++st == kUStages) { st = 0; ph ^= 1; }
+        if (lane == 0) mbar_arrive(&item_full[ni % kUItemSlots]);
+        if (item >= n_items) break;
       }
-      if (!alive) break;
-      if (lane == 0) umma_commit(&acc_full[ab]);
-      __syncwarp();
-      w = wn;
+    } else {
+      // ---- scales and zero-points: a row block's are contiguous over the groups, so lanes 0 .. 7 copy a row block's
+      // scales of up to 16 groups each and lanes 8 .. 15 its zero-points.  (Fetched by their users one group ahead, they
+      // cost a trip to memory per group.) ----
+      uint32_t m = 0;  // stages so far
+      static_assert((kUMetaStages & (kUMetaStages - 1)) == 0, "stage and parity by mask and shift");
+      for (uint32_t ni = 0; alive; ++ni) {
+        const PfItem& it = items[ni % kUItemSlots];
+        if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
+        if (it.stop) break;
+        const int ngroups = (it.nk * kPfChunkK) >> LG;
+        const int rbk = lane & 7, mat = PHASE == 1 ? rbk & 1 : 0, rb = PHASE == 1 ? rbk >> 1 : rbk;
+        const bool zps = lane >= 8;
+        const uint8_t* src = (zps ? it.zp[mat] : reinterpret_cast<const uint8_t*>(it.scale[mat])) + (size_t)rb * ngroups * (zps ? 16 : 32);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
+        const bool aligned = __all_sync(0xffffffffu, lane >= 16 || (reinterpret_cast<uintptr_t>(src) & 15) == 0);
+        for (int g0 = 0; g0 < ngroups; g0 += kUMetaGroups, ++m) {
+          const uint32_t ms = m % kUMetaStages;
+          if (m >= kUMetaStages && !mbar_wait(&meta_free[ms], ((m / kUMetaStages) & 1) ^ 1, abort_flag)) { alive = false; break; }
+          const int gs = min(kUMetaGroups, ngroups - g0), bytes = gs * (zps ? 16 : 32);
+          uint8_t* dst = smem + USmem::meta + ms * kUMetaBytes + (zps ? 8 * kUMetaScale + rbk * kUMetaZp : rbk * kUMetaScale);
+          const uint8_t* from = src + (size_t)g0 * (zps ? 16 : 32);
+          if (aligned) {
+            if (lane == 0) mbar_expect_tx(&meta_full[ms], gs * 8 * 48);
+            __syncwarp();
+            if (lane < 16)
+              asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                               smem_u32(dst)),
+                           "l"(from), "r"(bytes), "r"(smem_u32(&meta_full[ms]))
+                           : "memory");
+          } else {  // a caller's array that does not start on 16 bytes: byte by byte
+            if (lane < 16)
+              for (int i = 0; i < bytes; ++i) dst[i] = from[i];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&meta_full[ms]);
+          }
+        }
+      }
+      for (uint32_t i = m > kUMetaStages ? m - kUMetaStages : 0; i < m && !alive; ++i) {  // as for the token tiles
+        const uint32_t t0 = (uint32_t)clock64();
+        while (!mbar_try(&meta_full[i % kUMetaStages], (i / kUMetaStages) & 1) && (uint32_t)clock64() - t0 < kUWaitCycles) {}
+      }
     }
-    // the last commit must have arrived before shared memory goes away
-    if (alive && last_empty && !__all_sync(0xffffffffu, mbar_wait(last_empty, last_ph, abort_flag))) alive = false;
-  } else if (warp >= 8) {
-    // ---- dequantisation: sets of four warps take the 64-column steps in turn; thread (q, lane) of a set owns
-    // weight row 32 q + lane and stores the row's 64 values of the step, as leading parts and remainders,
-    // into the stage's tensor-memory columns ----
-    const int q = warp & 3, set = (warp - 8) >> 2;
-    const int blk = lane >> 4, g = lane & 7, sh = ((lane >> 3) & 1) * 4;  // row = 16 (2 q + blk) + g + 8 (sh / 4)
+  } else if (warp >= kUSumWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kURegsWeight));
+    // ---- weights: sets of four warps take the 64-column steps in turn; warp q of a set owns tensor-memory lanes
+    // [32 q, 32 q + 32), two row blocks, and stores their integers of the step into the stage's columns.  The planes are laid
+    // out as the fragments of a 16-row store: plane lane 4 g + c holds rows g and g + 8, columns 16 w + 4 c + j, which
+    // is what lane 4 g + c of tcgen05.st.16x256b gives.  So a lane copies, converts and stores the same 16 bytes
+    // of a plane: both nibbles of every byte are used, and no lane reads what another copied. ----
+    const int q = warp & 3, set = (warp - kUSumWarps) >> 2;
+    const int g = lane >> 2;
     constexpr int kGpc = G == 32 ? 2 : 1;  // quantisation groups in a step
-    // Raw plane words run kURawDepth of the warp's steps ahead of their use, across work items.  Per step the
-    // warp needs two 16-row blocks of 512 bytes per plane; lane l copies the 16 bytes of plane lane l of both
-    // blocks with cp.async into the warp's ring (16-byte pieces XOR-swizzled against bank conflicts), and
-    // after a warp barrier every lane reads the four pieces of its row.
-    uint8_t* raw = raw_ring + (warp - 8) * (kURawDepth * 2048);
-    const int wr_piece = (lane ^ (lane >> 3)) * 16;  // plane lane l = 4 g' + c: low two bits XOR (g' >> 1)
-    // Step c of the CTA (counted over all its items) belongs to set c mod kUSets and to stage c mod kUStages.
-    auto first_kc = [&](uint32_t base) { return (int)((set + kUSets - base % kUSets) % kUSets); };
-    uint32_t i_base = 0;  // steps of the items before the one the copies are in
-    int i_item = blockIdx.x, i_kc = set, i_nk = 0;
-    const uint8_t *i_mp = nullptr, *i_lp = nullptr;
-    bool i_prec = false;
+    // Raw plane words run kURawDepth of the warp's steps ahead of their use, across work items: per step two row blocks
+    // of 1024 bytes per plane, twice 16 bytes a lane, copied with cp.async into the warp's ring.
+    uint8_t* raw = smem + USmem::raw + (warp - kUSumWarps) * (kURawDepth * kURawStep) + lane * 16;
+    // the copies' place in the work: item number, step, addresses
+    // (Steps are counted over all items; those of the set's parity are its own.  An item of one step has none for one set.)
+    uint32_t i_ni = 0;
+    int i_left = 0;            // steps from the next own one to the item's end
+    uint32_t i_skip = set;     // steps of the next item before its first own one
+    bool i_more = true, i_prec = false;
+    const uint8_t *i_mp0 = nullptr, *i_mp1 = nullptr, *i_lp0 = nullptr, *i_lp1 = nullptr;
+    // An item is opened when its first step is to be copied, not before: the copies are then at most 2 kURawDepth items
+    // ahead, which is what the ring of descriptions holds.
     auto i_open = [&]() {
-      if (i_item >= n_items) return;
-      const UItem w = u_item<PHASE>(p, i_item);
-      int rb;
-      const slicemoe_mat& m = u_block_mat<PHASE>(w, 2 * q, &rb);  // blocks 2 q and 2 q + 1 are neighbours in one matrix
-      i_nk = w.K / kPfChunkK;
-      i_prec = w.prec;
-      i_mp = reinterpret_cast<const uint8_t*>(m.msb) + (size_t)rb * i_nk * 512 + lane * 16;
-      i_lp = w.prec ? reinterpret_cast<const uint8_t*>(m.lsb) + (size_t)rb * i_nk * 512 + lane * 16 : i_mp;
+      const PfItem& it = items[i_ni % kUItemSlots];
+      if (!mbar_wait(&item_full[i_ni % kUItemSlots], (i_ni / kUItemSlots) & 1, abort_flag)) { i_more = false; return; }
+      if (it.stop) { i_more = false; return; }
+      const int nk = it.nk;
+      i_prec = it.prec != 0;
+      // row blocks: gate and up of 16 columns of h, or two neighbours of down; a block's steps are 1024 bytes apart
+      const size_t o0 = (size_t)(PHASE == 1 ? q : 2 * q) * nk * 1024 + i_skip * 1024 + lane * 16, o1 = PHASE == 1 ? o0 : o0 + (size_t)nk * 1024;
+      i_mp0 = it.msb[0] + o0;
+      i_mp1 = it.msb[1] + o1;
+      if (i_prec) {
+        i_lp0 = it.lsb[0] + o0;
+        i_lp1 = it.lsb[1] + o1;
+      }
+      i_left = nk - (int)i_skip;
+      i_skip = (uint32_t)(i_skip + nk) & 1u;  // own steps are those with an even distance
+      ++i_ni;
     };
-    auto i_issue = [&](int slot) {
-      if (i_item < n_items) {
-        uint8_t* dst = raw + slot * 2048 + wr_piece;
-        const size_t o = (size_t)i_kc * 512, o1 = o + (size_t)i_nk * 512;
-        cp_async16(dst, i_mp + o);
-        cp_async16(dst + 512, i_mp + o1);
-        if (i_prec) {
-          cp_async16(dst + 1024, i_lp + o);
-          cp_async16(dst + 1536, i_lp + o1);
+    auto i_issue = [&](uint8_t* dst) {
+      while (i_more && i_left <= 0) i_open();
+      if (i_more) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          cp_async16(dst + 512 * h, i_mp0 + 512 * h);
+          cp_async16(dst + 1024 + 512 * h, i_mp1 + 512 * h);
+          if (i_prec) {
+            cp_async16(dst + 2048 + 512 * h, i_lp0 + 512 * h);
+            cp_async16(dst + 3072 + 512 * h, i_lp1 + 512 * h);
+          }
         }
-        i_kc += kUSets;
-        if (i_kc >= i_nk) {
-          i_base += i_nk;
-          i_item += gridDim.x;
-          i_kc = first_kc(i_base);
-          i_open();
-        }
+        i_mp0 += 1024 * kUSets;
+        i_mp1 += 1024 * kUSets;
+        i_lp0 += 1024 * kUSets;
+        i_lp1 += 1024 * kUSets;
+        i_left -= kUSets;
       }
       cp_async_commit();
     };
-    i_open();
-    for (int j = 0; j < kURawDepth; ++j) i_issue(j);
-    uint32_t base = 0, slot = 0, ni = 0;  // steps of the items so far; ring slot of the raw words; items so far
-    for (int item = blockIdx.x; item < n_items && alive; item += gridDim.x, ++ni) {
-      const UItem w = u_item<PHASE>(p, item);
-      int rb;
-      const slicemoe_mat& m = u_block_mat<PHASE>(w, 2 * q + blk, &rb);
-      if (w.missing && warp == 8 && lane == 0) atomicOr(p.status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
-      const int nk = w.K / kPfChunkK, ngroups = w.K >> LG;
-      const size_t meta = (size_t)rb * ngroups * 16 + g + 2 * sh;  // the row's entry of group 0
-      const uint8_t* zp = m.zp + meta;
-      const uint16_t* sc = m.scale + meta;
-      // The row's weights are normalised by a power of two, 2^(emax - 15) with emax the largest exponent field
-      // among the row's fp16 scales: every factor f = s 2^(15 - emax) is below 2, so |(q - zp) f| < 512 sits in
-      // the middle of fp16's range for the leading part and its remainder alike.  The epilogue multiplies the
-      // row's sums by 2^(emax - 15).
-      unsigned emax = 0;
-      for (int grp = 0; grp < ngroups; ++grp) emax = max(emax, ((unsigned)__ldg(sc + grp * 16) >> 10) & 31u);
-      const float rnorm = exp2f(15.f - (float)emax);
-      if (set == 0) row_scale[ni % kUScaleSlots][32 * q + lane] = exp2f((float)emax - 15.f);
-      // zero-points and scales of the groups of the warp's next step
-      const int kc0 = first_kc(base);
-      int z_next[kGpc];
-      uint16_t s_next[kGpc];
+    for (int j = 0; j < kURawDepth; ++j) i_issue(raw + j * kURawStep);
+    const int shift = p.shift;
+    // row g's codes: MSB nibble at bit `shift`, LSB nibble below; row g + 8's the same from the high nibbles.  A slice
+    // narrower than four bits leaves the top of its nibble zero, so what the second mask lets through beyond it is zero.
+    const uint32_t mask = 0x0f0f0f0fu << shift;
+    const int back = 4 - shift;
+    uint8_t* slot = raw;
+    uint32_t st = set, par = 1, m = 0, skip = set;  // stage of the next own step, parity of its use before; scale and zero-point stages
+    static_assert(kUSets < kUStages, "a set's next stage is at most once round the ring away");
+    for (uint32_t ni = 0; alive; ++ni) {
+      const PfItem& it = items[ni % kUItemSlots];
+      if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
+      if (it.stop) break;
+      const int nk = it.nk;
+      const bool prec = it.prec != 0;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
+      int kc = (int)skip;
+      skip = (uint32_t)(skip + nk) & 1u;
+      constexpr int kMetaSteps = kUMetaGroups * G / 128;  // steps of a scale and zero-point stage
+      for (int k0 = 0; k0 < nk && alive; k0 += kMetaSteps, ++m) {
+        const uint32_t ms = m % kUMetaStages;
+        if (!mbar_wait(&meta_full[ms], (m / kUMetaStages) & 1, abort_flag)) { alive = false; break; }
+        const uint8_t* zp_stage = smem + USmem::meta + ms * kUMetaBytes + 8 * kUMetaScale + 2 * q * kUMetaZp + g;
+        const int k_end = min(nk, k0 + kMetaSteps);
+        for (; kc < k_end; kc += kUSets) {
+          cp_async_wait_but<kURawDepth - 1>();  // this lane's own copies: nobody else reads them
+          const uint8_t* zp = zp_stage + (kc - k0) * (128 / G * 16);
+          if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
+          tc_fence_after();
+          const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + kUWCol0 + st * kUWCols;
 #pragma unroll
-      for (int i = 0; i < kGpc; ++i) {
-        const int grp = ((kc0 * kPfChunkK) >> LG) + i;
-        z_next[i] = __ldg(zp + grp * 16);
-        s_next[i] = __ldg(sc + grp * 16);
-      }
-      for (int kc = kc0; kc < nk; kc += kUSets) {
-        const uint32_t st = (base + kc) % kUStages, ph = ((base + kc) / kUStages) & 1;
-        cp_async_wait_but<kURawDepth - 1>();
-        __syncwarp();
-        const uint8_t* src = raw + slot * 2048 + blk * 512 + g * 64;
-        const int rsw = (g >> 1) * 16;  // piece c sits at 16 (c ^ (g >> 1))
-        uint32_t mws[16], lws[16];      // [4 c + w]: word w of plane lane 4 g + c: k = 16 w + 4 c + j
+          for (int b = 0; b < 2; ++b) {
+            __half2 off[128 / G][2];  // 1024 + zero-point, rows g and g + 8, twice
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint4 mv = *reinterpret_cast<const uint4*>(src + ((16 * c) ^ rsw));
-          mws[4 * c] = mv.x; mws[4 * c + 1] = mv.y; mws[4 * c + 2] = mv.z; mws[4 * c + 3] = mv.w;
-          uint4 lv = make_uint4(0, 0, 0, 0);
-          if (w.prec) lv = *reinterpret_cast<const uint4*>(src + 1024 + ((16 * c) ^ rsw));
-          lws[4 * c] = lv.x; lws[4 * c + 1] = lv.y; lws[4 * c + 2] = lv.z; lws[4 * c + 3] = lv.w;
-        }
-        __half2 off[kGpc], fac[kGpc];
+            for (int i = 0; i < 128 / G; ++i)
 #pragma unroll
-        for (int i = 0; i < kGpc; ++i) {
-          off[i] = __half2half2(__int2half_rn(1024 + (w.prec ? z_next[i] : ((z_next[i] >> p.shift) << p.shift))));
-          fac[i] = __half2half2(__float2half_rn(__half2float(__ushort_as_half(s_next[i])) * rnorm));  // exact: a power of two
-        }
-        if (kc + kUSets < nk) {
+              for (int hi = 0; hi < 2; ++hi) {
+                uint32_t z = zp[b * kUMetaZp + 16 * i + 8 * hi];
+                if (!prec) z = z >> shift << shift;
+                z = z * 0x00010001u + 0x64006400u;
+                off[i][hi] = *reinterpret_cast<__half2*>(&z);
+              }
 #pragma unroll
-          for (int i = 0; i < kGpc; ++i) {
-            const int grp = (((kc + kUSets) * kPfChunkK) >> LG) + i;
-            z_next[i] = __ldg(zp + grp * 16);
-            s_next[i] = __ldg(sc + grp * 16);
-          }
-        }
-        if (!__all_sync(0xffffffffu, mbar_wait(&empty[st], ph ^ 1, abort_flag))) { alive = false; break; }
-        tc_fence_after();
-        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + kUAccCols + st * kUWCols;
+            for (int h = 0; h < 2; ++h) {
+              const uint4 mv = *reinterpret_cast<const uint4*>(slot + 1024 * b + 512 * h);
+              uint4 lv = make_uint4(0, 0, 0, 0);
+              if (prec) lv = *reinterpret_cast<const uint4*>(slot + 2048 + 1024 * b + 512 * h);
+              const uint32_t mw[4] = {mv.x, mv.y, mv.z, mv.w}, lw[4] = {lv.x, lv.y, lv.z, lv.w};
+              uint32_t out[16];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t rh[16], rl[16];  // column 8 (w & 1) + 2 c + jj holds k = 16 w + 4 c + 2 jj, + 1 for w = 2 half, 2 half + 1
+              for (int w = 0; w < 4; ++w) {
+                // four codes a row, one per byte
+                const uint32_t code[2] = {((mw[w] << shift) & mask) | (lw[w] & ~mask), ((mw[w] >> back) & mask) | ((lw[w] >> 4) & ~mask)};
 #pragma unroll
-          for (int wi = 0; wi < 2; ++wi) {
-            const int wd = 2 * half + wi;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const uint32_t m0 = mws[4 * c + wd] >> sh, l0 = lws[4 * c + wd] >> sh;
-              // both slices: the whole code; MSB slice alone: 2^shift x its code (the factor of the low-bit
-              // dequantisation, exact in fp16).  shift = 4 for 8-bit codes; narrower slices sit in the low bits
-              // of their nibbles, so a code never exceeds a byte
-              const uint32_t qv = ((m0 & 0x0f0f0f0fu) << p.shift) | (l0 & 0x0f0f0f0fu);
-              // bytes -> fp16 1024 + code, minus (1024 + zero-point): the integer d = q - zp, exact
-              uint32_t h01 = __byte_perm(qv, 0x64646464u, 0x4140), h23 = __byte_perm(qv, 0x64646464u, 0x4342);
-              const __half2 o = off[kGpc == 2 ? (wd >> 1) : 0], f = fac[kGpc == 2 ? (wd >> 1) : 0];
-              const __half2 d01 = __hsub2(*reinterpret_cast<__half2*>(&h01), o);
-              const __half2 d23 = __hsub2(*reinterpret_cast<__half2*>(&h23), o);
-              // d f as an unevaluated sum of two fp16: the rounded product and, by one fused multiply-add, what
-              // the rounding dropped (at most 10 significant bits, so it is exact)
-              const __half2 p01 = __hmul2(d01, f), p23 = __hmul2(d23, f);
-              const __half2 e01 = __hfma2(d01, f, __hneg2(p01)), e23 = __hfma2(d23, f, __hneg2(p23));
-              rh[8 * wi + 2 * c] = *reinterpret_cast<const uint32_t*>(&p01);
-              rh[8 * wi + 2 * c + 1] = *reinterpret_cast<const uint32_t*>(&p23);
-              rl[8 * wi + 2 * c] = *reinterpret_cast<const uint32_t*>(&e01);
-              rl[8 * wi + 2 * c + 1] = *reinterpret_cast<const uint32_t*>(&e23);
+                for (int hi = 0; hi < 2; ++hi) {
+                  // bytes -> fp16 1024 + code, minus (1024 + zero-point): exact integers
+                  uint32_t h01 = __byte_perm(code[hi], 0x64646464u, 0x4140), h23 = __byte_perm(code[hi], 0x64646464u, 0x4342);
+                  const __half2 o = off[(h * 64 + w * 16) / G][hi];
+                  const __half2 d01 = __hsub2(*reinterpret_cast<__half2*>(&h01), o), d23 = __hsub2(*reinterpret_cast<__half2*>(&h23), o);
+                  out[4 * w + 2 * hi] = *reinterpret_cast<const uint32_t*>(&d01);
+                  out[4 * w + 2 * hi + 1] = *reinterpret_cast<const uint32_t*>(&d23);
+                }
+              }
+              tmem_st_16x32(ta + ((uint32_t)(16 * b) << 16) + 32 * h, out);
             }
           }
-          tmem_st16(ta + 16 * half, rh);
-          tmem_st16(ta + 32 + 16 * half, rl);
+          i_issue(slot);
+          slot = slot == raw ? raw + kURawStep : raw;
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[st]);
+          st += kUSets;
+          if (st >= kUStages) {
+            st -= kUStages;
+            par ^= 1;
+          }
         }
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&full[st]);
-        i_issue(slot);  // after the step's words were consumed by every lane: the slot is free
-        if (++slot == kURawDepth) slot = 0;
+        if (alive && lane == 0) mbar_arrive(&meta_free[ms]);
       }
-      base += nk;
     }
     cp_async_wait_but<0>();
   } else {
-    // ---- epilogue: warp (q, hh) owns weight rows [32 q, 32 q + 32) x tokens [64 hh, 64 hh + 64) ----
-    const int q = warp & 3, hh = warp >> 2;
-    uint32_t n_done = 0;
-    for (int item = blockIdx.x; item < n_items && alive; item += gridDim.x, ++n_done) {
-      const UItem w = u_item<PHASE>(p, item);
-      const uint32_t ab = n_done & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], (n_done >> 1) & 1, abort_flag))) { alive = false; break; }
-      tc_fence_after();
-      const float rs = row_scale[n_done % kUScaleSlots][32 * q + lane];  // 2^(emax - 15) of the lane's weight row
-      const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + ab * kPfTileM + 64 * hh;
-      float tot[64];
-      {
-        uint32_t r0[16], r1[16];
-        tmem_ld16(ta, r0);
-        tmem_ld16(ta + 16, r1);
-        tmem_ld_wait();
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kURegsSum));
+    // ---- sums: warp (q, wg) owns weight rows [32 q, 32 q + 32) x the warpgroup's tokens, in fp32 registers ----
+    const int q = warp & 3, wg = warp >> 2;
+    uint32_t used = 0;  // bit per accumulator: parity of the times it has been filled
+    uint32_t m = 0;     // scale stages so far
+    for (uint32_t ni = 0; alive; ++ni) {
+      const PfItem& it = items[ni % kUItemSlots];
+      if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
+      if (it.stop) break;
+      const int halves = it.halves, n0 = it.n0;
+      const int cols = wg == 0 ? n0 : it.n - n0;  // tokens of this warpgroup
+      const int ngroups = (it.nk * kPfChunkK) >> LG;
+      const int count = wg == 0 ? min(it.count, n0) : it.count - n0, out_row = it.out_row + (wg == 0 ? 0 : n0), col = it.col;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
+      const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16) + (halves == 1 && wg ? n0 : 0);
+      uint64_t acc[kUHalfMax / 2];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) tot[j] = rs * __uint_as_float(r0[j]);
+      for (int i = 0; i < kUHalfMax / 2; ++i) acc[i] = 0ull;
+      uint32_t alt = 0;  // narrow tiles: the accumulator whose turn it is
+      for (int g0 = 0; g0 < ngroups && alive; g0 += kUMetaGroups, ++m) {
+        const uint32_t ms = m % kUMetaStages;
+        if (!mbar_wait(&meta_full[ms], (m / kUMetaStages) & 1, abort_flag)) { alive = false; break; }
+        const uint8_t* sc = smem + USmem::meta + ms * kUMetaBytes + (2 * q + (lane >> 4)) * kUMetaScale + (lane & 15) * 2;
+        for (int gi = min(kUMetaGroups, ngroups - g0); gi > 0; --gi, sc += 32) {
+          const float s = __half2float(*reinterpret_cast<const __half*>(sc));
+          const uint64_t ss = ((uint64_t)__float_as_uint(s) << 32) | __float_as_uint(s);
+          // (with two accumulators the other warpgroup's one is filled and read without this one)
+          const uint32_t buf = halves == 2 ? (uint32_t)wg : alt;
+          if (!mbar_wait(&acc_full[buf], (used >> buf) & 1u, abort_flag)) { alive = false; break; }
+          used ^= halves == 2 ? 3u : 1u << buf;
+          alt ^= 1u;
+          tc_fence_after();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) tot[16 + j] = rs * __uint_as_float(r1[j]);
-        tmem_ld16(ta + 32, r0);
-        tmem_ld16(ta + 48, r1);
-        tmem_ld_wait();
-        tc_fence_before();
+          for (int c = 0; c < kUHalfMax / 32; ++c) {
+            if (32 * c < cols) {
+              uint32_t v[32];
+              tmem_ld32(lane_base + buf * kUAccCols + 32 * c, v);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) fma2(acc[16 * c + i], v[2 * i], v[2 * i + 1], ss);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(&acc_free[buf]);
+            if (halves == 2) mbar_arrive(&acc_free[buf]);
+          }
+        }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[ab]);  // the accumulator is free for the item after the next
-#pragma unroll
-        for (int j = 0; j < 16; ++j) tot[32 + j] = rs * __uint_as_float(r0[j]);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) tot[48 + j] = rs * __uint_as_float(r1[j]);
+        if (alive && lane == 0) mbar_arrive(&meta_free[ms]);
       }
       if (!alive) break;
-      const int tok0 = w.row0 + 64 * hh;
       if (PHASE == 1) {
-        // rows [0,64) hold gate, rows [64,128) up: warp (q, hh) with q < 2 hands silu(gate) to warp (q + 2, hh)
-        // through shared memory; that warp multiplies and writes h
-        const int pair = 2 * hh + (q & 1);
-        if (q < 2) {
-          if (!__all_sync(0xffffffffu, mbar_wait(&xch_empty[pair], (n_done & 1) ^ 1, abort_flag))) { alive = false; break; }
+        // lanes 0 .. 15 hold gate rows, lanes 16 .. 31 the up rows of the same 16 columns of h.  Of two tokens the gate lane
+        // finishes the first and the up lane the second: one exchange each.
+        const bool up = lane >= 16;
+        __half* dst = p.h + (size_t)(out_row + (up ? 1 : 0)) * p.ldh + col + 16 * q + (lane & 15);
+        const size_t two_rows = 2 * (size_t)p.ldh;
 #pragma unroll
-          for (int j = 0; j < 64; ++j) xch[pair][j][lane] = tot[j] / (1.f + __expf(-tot[j]));
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&xch_full[pair]);
-        } else {
-          if (!__all_sync(0xffffffffu, mbar_wait(&xch_full[pair], n_done & 1, abort_flag))) { alive = false; break; }
-          __half* dst = p.h + (size_t)tok0 * p.ldh + 64 * w.nt + 32 * (q & 1) + lane;
-#pragma unroll
-          for (int j = 0; j < 64; ++j) dst[(size_t)j * p.ldh] = __float2half_rn(xch[pair][j][lane] * tot[j]);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&xch_empty[pair]);
+        for (int i = 0; i < kUHalfMax / 2; ++i) {
+          if (2 * i < count) {
+            const float v0 = half_of(acc[i], 0), v1 = half_of(acc[i], 1);
+            const float got = __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 16);
+            const float gate = up ? got : v0, upv = up ? v1 : got;
+            // silu: g / (1 + e^-g), the quotient by the reciprocal and one step of Newton's iteration.  Below -80 the
+            // result is zero in fp16 either way; the bound keeps 1 + e^-g finite.
+            const float t = 1.f + __expf(fminf(-gate, 80.f));
+            float r;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+            r = fmaf(r, fmaf(-t, r, 1.f), r);
+            if (2 * i + (up ? 1 : 0) < count) *dst = __float2half_rn(gate * r * upv);
+            dst += two_rows;
+          }
         }
       } else {
-        float* dst = p.yrow + (size_t)tok0 * p.hidden + 128 * w.nt + 32 * q + lane;
+        float* dst = p.yrow + (size_t)out_row * p.hidden + col + 32 * q + lane;
 #pragma unroll
-        for (int j = 0; j < 64; ++j) dst[(size_t)j * p.hidden] = tot[j];
+        for (int i = 0; i < kUHalfMax / 2; ++i) {
+          if (2 * i < count) dst[(size_t)(2 * i) * p.hidden] = half_of(acc[i], 0);
+          if (2 * i + 1 < count) dst[(size_t)(2 * i + 1) * p.hidden] = half_of(acc[i], 1);
+        }
       }
     }
   }
@@ -711,22 +997,42 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
 }
 
 // ---- step 5: weighted combine in list order ---------------------------------------------------------------
-__global__ void pf_combine_kernel(const float* __restrict__ yrow, const int* __restrict__ posmap,
-                                  const float* __restrict__ weights, const float* __restrict__ gate, int T, int k,
-                                  int n_shared, int hidden, float* __restrict__ y) {
+// A block per token: the token's rows and weights are read once into shared memory, then four slots' rows at a time are in
+// flight.
+constexpr int kPfMaxSlots = SLICEMOE_MAX_TOP_K + SLICEMOE_MAX_SHARED;
+__global__ void __launch_bounds__(256) pf_combine_kernel(const float* __restrict__ yrow, const int* __restrict__ posmap,
+                                                         const float* __restrict__ weights, const float* __restrict__ gate, int k,
+                                                         int n_shared, int hidden, float* __restrict__ y) {
+  __shared__ int s_pos[kPfMaxSlots];
+  __shared__ float s_w[kPfMaxSlots];
   const int t = blockIdx.x;
   const int slots = k + n_shared;
+  pf_dep_launch();
+  pf_dep_wait();
+  if (threadIdx.x < slots) {
+    const int j = threadIdx.x, pos = posmap[t * slots + j];
+    const float w = j < k ? weights[t * k + j] : (gate ? gate[t] : 1.f);
+    s_pos[j] = pos;
+    s_w[j] = w;
+  }
+  __syncthreads();
   for (int col = threadIdx.x * 4; col < hidden; col += blockDim.x * 4) {
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j = 0; j < slots; ++j) {
-      const int pos = posmap[t * slots + j];
-      if (pos < 0) continue;
-      const float w = j < k ? weights[t * k + j] : (gate ? gate[t] : 1.f);
-      const float4 v = *reinterpret_cast<const float4*>(yrow + (size_t)pos * hidden + col);
-      a.x = fmaf(w, v.x, a.x);
-      a.y = fmaf(w, v.y, a.y);
-      a.z = fmaf(w, v.z, a.z);
-      a.w = fmaf(w, v.w, a.w);
+    for (int j0 = 0; j0 < slots; j0 += 4) {
+      float4 v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j0 + j < slots && s_pos[j0 + j] >= 0)
+          v[j] = __ldcs(reinterpret_cast<const float4*>(yrow + (size_t)s_pos[j0 + j] * hidden + col));
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j0 + j >= slots || s_pos[j0 + j] < 0) continue;
+        const float w = s_w[j0 + j];
+        a.x = fmaf(w, v[j].x, a.x);
+        a.y = fmaf(w, v[j].y, a.y);
+        a.z = fmaf(w, v[j].z, a.z);
+        a.w = fmaf(w, v[j].w, a.w);
+      }
     }
     *reinterpret_cast<float4*>(y + (size_t)t * hidden + col) = a;
   }
@@ -736,7 +1042,7 @@ typedef CUresult (*PfEncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor map of a row-major fp16 matrix [rows, cols] for 128-row x 64-column tiles with 128-byte swizzle.
+// Tensor map of a row-major fp16 matrix [rows, cols] for 32-row x 64-column tiles with 128-byte swizzle.
 static int pf_tensor_map(CUtensorMap* tm, const __half* base, int rows, int cols) {
   static PfEncodeTiled encode = nullptr;
   if (!encode) {
@@ -748,7 +1054,7 @@ static int pf_tensor_map(CUtensorMap* tm, const __half* base, int rows, int cols
   }
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)cols * sizeof(__half)};
-  const cuuint32_t box[2] = {(cuuint32_t)kPfChunkK, (cuuint32_t)kPfTileM};
+  const cuuint32_t box[2] = {(cuuint32_t)kUBoxCols, (cuuint32_t)kUBoxRows};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base), dims, strides, box, estr,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -756,8 +1062,25 @@ static int pf_tensor_map(CUtensorMap* tm, const __half* base, int rows, int cols
   return r == CUDA_SUCCESS ? SLICEMOE_OK : SLICEMOE_E_INVALID_ARG;
 }
 
+// Every kernel of a step starts while the one before it is still running and waits for it itself (pf_dep_wait).
+template <class... Args>
+static int pf_launch(void (*kernel)(Args...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return SLICEMOE_OK;
+}
+
 template <int G>
-static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int rmax, cudaStream_t st) {
+static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int in_rows, int out_rows, cudaStream_t st) {
   static bool attr_set[64];
   static int sm_count[64];
   int dev = 0;
@@ -770,16 +1093,14 @@ static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int rmax, cu
     attr_set[dev] = true;
   }
   CUtensorMap tm_x, tm_h;
-  int rc = pf_tensor_map(&tm_x, xs, rmax, p.hidden);
+  int rc = pf_tensor_map(&tm_x, xs, in_rows, p.hidden);
   if (rc != SLICEMOE_OK) return rc;
-  rc = pf_tensor_map(&tm_h, p.h, rmax, p.ldh);
+  rc = pf_tensor_map(&tm_h, p.h, out_rows, p.ldh);
   if (rc != SLICEMOE_OK) return rc;
-  // one persistent CTA per SM (shared memory admits one); each walks its share of the work items
-  pf_umma_kernel<G, 1><<<sm_count[dev], kUThreads, kUSmemBytes, st>>>(p, tm_x);
-  SM_LAUNCH_CHECK();
-  pf_umma_kernel<G, 2><<<sm_count[dev], kUThreads, kUSmemBytes, st>>>(p, tm_h);
-  SM_LAUNCH_CHECK();
-  return SLICEMOE_OK;
+  // one persistent CTA per SM (shared memory admits one); each takes work items until there are none
+  rc = pf_launch(pf_umma_kernel<G, 1>, (unsigned)sm_count[dev], kUThreads, kUSmemBytes, st, p, tm_x);
+  if (rc != SLICEMOE_OK) return rc;
+  return pf_launch(pf_umma_kernel<G, 2>, (unsigned)sm_count[dev], kUThreads, kUSmemBytes, st, p, tm_h);
 }
 
 static int pf_check(const slicemoe_shape* s, int T) {
@@ -823,47 +1144,45 @@ extern "C" int slicemoe_prefill_layer(const slicemoe_shape* s, const slicemoe_ex
     return SLICEMOE_E_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
-  int* counts = reinterpret_cast<int*>(ws + L.counts);
-  int* cursor = reinterpret_cast<int*>(ws + L.cursor);
-  int* offsets = reinterpret_cast<int*>(ws + L.offsets);
-  int* tile_expert = reinterpret_cast<int*>(ws + L.tile_expert);
-  int* tile_row0 = reinterpret_cast<int*>(ws + L.tile_row0);
-  int* item_start = reinterpret_cast<int*>(ws + L.item_start);
-  int* ntiles = reinterpret_cast<int*>(ws + L.ntiles);
-  int* row_token = reinterpret_cast<int*>(ws + L.row_token);
-  int* posmap = reinterpret_cast<int*>(ws + L.posmap);
-  float* gate = reinterpret_cast<float*>(ws + L.gate);
+  const bool gated = nsh > 0 && s->shared_sigmoid_gate;
   __half* xs = reinterpret_cast<__half*>(ws + L.xs);
-  __half* h = reinterpret_cast<__half*>(ws + L.h);
+  float* gate = reinterpret_cast<float*>(ws + L.gate);
   float* yrow = reinterpret_cast<float*>(ws + L.yrow);
 
-  // counters start at zero, unused rows are marked -1
-  SM_CUDA_TRY(cudaMemsetAsync(ws + L.counts, 0, L.offsets - L.counts, st));
-  SM_CUDA_TRY(cudaMemsetAsync(row_token, 0xff, sizeof(int) * (size_t)L.rmax, st));
-  SM_CUDA_TRY(cudaMemsetAsync(status_out_device, 0, sizeof(int), st));
-  const int npairs = T * k;
-  pf_count_kernel<<<(npairs + 255) / 256, 256, 0, st>>>(ids, npairs, E, counts, reinterpret_cast<unsigned*>(status_out_device));
-  SM_LAUNCH_CHECK();
-  pf_scan_kernel<<<1, 32, 0, st>>>(counts, E, nsh, T, s->inter, shared_inter, offsets, tile_expert, tile_row0, item_start, ntiles);
-  SM_LAUNCH_CHECK();
-  const int nslots = T * (k + nsh);
-  pf_scatter_kernel<<<(nslots + 255) / 256, 256, 0, st>>>(ids, T, k, E, nsh, offsets, cursor, row_token, posmap);
-  SM_LAUNCH_CHECK();
-  const bool gated = nsh > 0 && s->shared_sigmoid_gate;
-  pf_gather_kernel<<<L.rmax, 256, 0, st>>>(reinterpret_cast<const uint16_t*>(x), s->hidden, row_token, ntiles, xs,
-                                           gated ? shared_gate_vec : nullptr, offsets + E, T, gate);
-  SM_LAUNCH_CHECK();
+  PfPlanParams pp;
+  pp.ids = ids;
+  pp.T = T;
+  pp.k = k;
+  pp.E = E;
+  pp.n_shared = nsh;
+  pp.per1_routed = s->inter / 64;
+  pp.per1_shared = shared_inter / 64;
+  pp.per2 = s->hidden / 128;
+  pp.head = reinterpret_cast<PfHead*>(ws + L.head);
+  pp.counts = reinterpret_cast<int*>(ws + L.counts);
+  pp.offsets = reinterpret_cast<int*>(ws + L.offsets);
+  pp.cursor = reinterpret_cast<int*>(ws + L.cursor);
+  pp.runs = reinterpret_cast<PfRun*>(ws + L.runs);
+  pp.row_token = reinterpret_cast<int*>(ws + L.row_token);
+  pp.posmap = reinterpret_cast<int*>(ws + L.posmap);
+  pp.status = reinterpret_cast<unsigned*>(status_out_device);
+  rc = pf_launch(pf_plan_kernel, 1u, (unsigned)kPfPlanThreads, 0, st, (PfPlanParams)pp);
+  if (rc != SLICEMOE_OK) return rc;
+  constexpr int kRowsPerBlock = kPfGatherThreads / 32;
+  rc = pf_launch((reinterpret_cast<uintptr_t>(x) & 15) ? pf_gather_kernel<1> : pf_gather_kernel<4>,
+                 (unsigned)((L.in_rows + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)kPfGatherThreads, 0, st,
+                 reinterpret_cast<const uint16_t*>(x), (int)s->hidden, (int)T, (const int*)pp.row_token, (int)(T * k), (int)L.in_rows, xs,
+                 gated ? shared_gate_vec : (const float*)nullptr, gate);
+  if (rc != SLICEMOE_OK) return rc;
   PfGemmParams p;
   p.experts = experts;
   p.shared = shared;
   p.expert_prec = expert_prec;
-  p.tile_expert = tile_expert;
-  p.tile_row0 = tile_row0;
-  p.item_start = item_start;
-  p.ntiles = ntiles;
-  p.h = h;
+  p.runs = pp.runs;
+  p.head = pp.head;
+  p.h = reinterpret_cast<__half*>(ws + L.h);
   p.yrow = yrow;
-  p.status = reinterpret_cast<unsigned*>(status_out_device);
+  p.status = pp.status;
   p.E = E;
   p.hidden = s->hidden;
   p.inter = s->inter;
@@ -871,14 +1190,13 @@ extern "C" int slicemoe_prefill_layer(const slicemoe_shape* s, const slicemoe_ex
   p.ldh = s->inter > shared_inter ? s->inter : shared_inter;
   p.shift = s->b_high - s->b_low;
   if (s->group == 128) {
-    rc = pf_launch_gemms<128>(p, xs, L.rmax, st);
+    rc = pf_launch_gemms<128>(p, xs, L.in_rows, L.out_rows, st);
   } else if (s->group == 64) {
-    rc = pf_launch_gemms<64>(p, xs, L.rmax, st);
+    rc = pf_launch_gemms<64>(p, xs, L.in_rows, L.out_rows, st);
   } else {
-    rc = pf_launch_gemms<32>(p, xs, L.rmax, st);
+    rc = pf_launch_gemms<32>(p, xs, L.in_rows, L.out_rows, st);
   }
   if (rc != SLICEMOE_OK) return rc;
-  pf_combine_kernel<<<T, 256, 0, st>>>(yrow, posmap, weights, gated ? gate : nullptr, T, k, nsh, s->hidden, y);
-  SM_LAUNCH_CHECK();
-  return SLICEMOE_OK;
+  return pf_launch(pf_combine_kernel, (unsigned)T, 256u, 0, st, (const float*)yrow, (const int*)pp.posmap, weights,
+                   gated ? (const float*)gate : (const float*)nullptr, (int)k, (int)nsh, (int)s->hidden, y);
 }
