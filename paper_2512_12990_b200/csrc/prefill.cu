@@ -300,22 +300,24 @@ constexpr int kUThreads = 32 * (kUWarpTok + 4);
 constexpr int kURegsSum = 152, kURegsWeight = 72, kURegsRest = 32;
 static_assert(256 * kURegsSum + 256 * kURegsWeight + 128 * kURegsRest <= kUThreads * 96, "register split");
 constexpr int kUStages = 3;                   // steps in flight: tokens in shared, weights in tensor memory
-constexpr int kUBoxRows = 32, kUBoxCols = 64; // token rows and columns of one TMA copy (128 bytes: the swizzle's span)
-constexpr int kUBoxBytes = kUBoxRows * kUBoxCols * 2;
+constexpr int kUBoxRows = 32, kUBoxCols = 64; // a TMA copy brings a multiple of 32 token rows x 64 columns (128 bytes: the swizzle's span)
+constexpr int kUBoxes = kPfTileN / kUBoxRows; // heights a copy can have: a tensor map each
 constexpr int kUPanelBytes = kPfTileN * kUBoxCols * 2;  // half of a step's tile: 64 columns of all tokens
 constexpr int kUTileBytes = 2 * kUPanelBytes;
-constexpr int kURawDepth = 2;                 // steps of raw plane words each weight warp keeps in flight (cp.async)
-constexpr int kURawStep = 4096;               // of a warp and step: [plane][block][half] x 512 bytes
-constexpr int kURawBytes = 4 * kUSets * kURawDepth * kURawStep;
+constexpr int kURawStages = 4;                // steps of raw plane words in shared memory or on their way to it
+constexpr int kURawBlock = 1024;              // a row block's bytes of a step in one plane
+constexpr int kURawStep = 16 * kURawBlock;    // [plane][row block]
+constexpr int kURawBytes = kURawStages * kURawStep;
 constexpr int kUItemSlots = 8;
 // Scales and zero-points of 16 quantisation groups at a time: [8 row blocks][16 groups][16 rows], 512 + 256 bytes each
 constexpr int kUMetaGroups = 16, kUMetaStages = 2;
 constexpr int kUMetaScale = kUMetaGroups * 32, kUMetaZp = kUMetaGroups * 16;
 constexpr int kUMetaBytes = 8 * (kUMetaScale + kUMetaZp);
 constexpr int kUHalfMax = kPfTileN / 2;       // tokens per warpgroup
-constexpr int kUAccCols = 128;                // tensor-memory columns between the two accumulators
-constexpr int kUWCol0 = 256, kUWCols = 64;    // weight stages: 128 fp16 per row
+constexpr int kUAccs = 3, kUAccCols = 96;     // accumulators, tensor-memory columns of one
+constexpr int kUWCol0 = kUAccs * kUAccCols, kUWCols = 64;  // weight stages: 128 fp16 per row
 constexpr int kUTmemCols = 512;
+static_assert(kUWCol0 + kUStages * kUWCols <= kUTmemCols && kUHalfMax <= kUAccCols, "tensor memory");
 constexpr uint32_t kUWaitCycles = 2000000000u;
 constexpr uint32_t kUCopyCycles = 2000000u;  // a millisecond: far more than any copy takes
 
@@ -342,10 +344,11 @@ struct USmem {
   static constexpr int items = meta + kUMetaStages * kUMetaBytes;
   static constexpr int bars = items + kUItemSlots * (int)sizeof(PfItem);
   // barriers: tokens and weights of a step in / step done / sums there [accumulator] / sums read [accumulator] / item
-  // there, item read / scales and zero-points in, read / drained
-  static constexpr int full = 0, done = full + kUStages, acc_full = done + kUStages, acc_free = acc_full + 2,
-                       item_full = acc_free + 2, item_free = item_full + kUItemSlots, meta_full = item_free + kUItemSlots,
-                       meta_free = meta_full + kUMetaStages, drain = meta_free + kUMetaStages, nbars = drain + 1;
+  // there, item read / scales and zero-points in, read / raw words in, read / drained
+  static constexpr int full = 0, done = full + kUStages, acc_full = done + kUStages, acc_free = acc_full + kUAccs,
+                       item_full = acc_free + kUAccs, item_free = item_full + kUItemSlots, meta_full = item_free + kUItemSlots,
+                       meta_free = meta_full + kUMetaStages, raw_full = meta_free + kUMetaStages, raw_free = raw_full + kURawStages,
+                       drain = raw_free + kURawStages, nbars = drain + 1;
   static constexpr int tail = bars + nbars * 8;  // tensor-memory address, abort flag
   static constexpr int total = tail + 16;
 };
@@ -353,6 +356,9 @@ static_assert(USmem::bars % 8 == 0 && USmem::items % 16 == 0, "alignment");
 constexpr int kUSmemBytes = USmem::total + 1024 /* alignment slack */;
 static_assert(kUSmemBytes <= 227 * 1024, "shared memory budget");
 
+struct PfMaps {
+  CUtensorMap rows[kUBoxes];  // [i]: copies of 32 (i + 1) rows
+};
 struct PfGemmParams {
   const slicemoe_expert* experts;  // routed
   const slicemoe_expert* shared;
@@ -404,13 +410,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
     if (__any_sync(0xffffffffu, *abort_flag != 0 || (uint32_t)clock64() - t0 > kUWaitCycles)) return false;
   }
 }
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_but() {  // all but the N most recent groups have landed
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+// The calling thread's cp.async so far arrive at the barrier when they have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* b) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -489,8 +499,20 @@ __device__ __forceinline__ int u_find_run(const PfRun* runs, int n, int item, in
   return lo;
 }
 
+// One plane of an item's eight row blocks for one step, 1024 bytes each, by one warp: `first` and `second` are the lane's place
+// in the first block of gate and up (whose blocks alternate) or of down, `stride` the bytes from one block to the next.
+template <int PHASE>
+__device__ __forceinline__ void u_copy_raw(uint32_t dst, const uint8_t* first, const uint8_t* second, uint32_t stride) {
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const uint8_t* src = PHASE == 1 ? (b & 1 ? second : first) + (size_t)(b >> 1) * stride : first + (size_t)b * stride;
+    cp_async16(dst + b * kURawBlock, src);
+    cp_async16(dst + b * kURawBlock + 512, src + 512);
+  }
+}
+
 template <int G, int PHASE>
-__global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParams p, const __grid_constant__ CUtensorMap tm_tok) {
+__global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParams p, const __grid_constant__ PfMaps maps) {
   constexpr int LG = G == 128 ? 7 : (G == 64 ? 6 : 5);
   extern __shared__ uint8_t u_smem_raw[];
   uint8_t* smem = u_smem_raw + ((1024 - (smem_u32(u_smem_raw) & 1023)) & 1023);
@@ -498,7 +520,8 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + USmem::bars);
   uint64_t *full = bars + USmem::full, *done = bars + USmem::done, *acc_full = bars + USmem::acc_full,
            *acc_free = bars + USmem::acc_free, *item_full = bars + USmem::item_full, *item_free = bars + USmem::item_free,
-           *meta_full = bars + USmem::meta_full, *meta_free = bars + USmem::meta_free, *drain = bars + USmem::drain;
+           *meta_full = bars + USmem::meta_full, *meta_free = bars + USmem::meta_free,
+           *raw_full = bars + USmem::raw_full, *raw_free = bars + USmem::raw_free, *drain = bars + USmem::drain;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + USmem::tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -511,7 +534,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       mbar_init(&full[s], 1 + 4);  // the token warp (and its copies' bytes) and a set's four warps
       mbar_init(&done[s], 1);
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < kUAccs; ++a) {
       mbar_init(&acc_full[a], 1);
       mbar_init(&acc_free[a], 8);  // the eight sum warps once each, or one warpgroup's four twice each
     }
@@ -522,6 +545,10 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
     for (int s = 0; s < kUMetaStages; ++s) {
       mbar_init(&meta_full[s], 1);
       mbar_init(&meta_free[s], kUSumWarps + 4 * kUSets);
+    }
+    for (int s = 0; s < kURawStages; ++s) {
+      mbar_init(&raw_full[s], 64);  // the lanes of the two warps that copy, one plane each
+      mbar_init(&raw_free[s], 4);  // the four warps of the set that takes the step
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -542,32 +569,46 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   if (warp >= kUWarpTok) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kURegsRest));
     if (warp == kUWarpTok) {
-      // ---- token tiles: TMA copies of 32 rows x 64 columns, a lane each ----
+      // ---- token tiles: two TMA copies of the tile's rows x 64 columns; and the raw LSB planes ----
       uint32_t st = 0, par = 1;  // stage; parity of the use before (the first one waits for nothing)
-      const int box = lane % (kPfTileN / kUBoxRows), panel = lane / (kPfTileN / kUBoxRows);
+      uint32_t rs = 0, rpar = 1;
       for (uint32_t ni = 0;; ++ni) {
         const PfItem& it = items[ni % kUItemSlots];
         if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
         if (it.stop) break;
-        const int nk = it.nk, boxes = (it.n + kUBoxRows - 1) / kUBoxRows, row = it.in_row + box * kUBoxRows;
+        const int nk = it.nk, box = (it.n + kUBoxRows - 1) / kUBoxRows, row = it.in_row;
+        const bool prec = it.prec != 0;
+        const uint8_t *p0 = it.lsb[0] + lane * 16, *p1 = it.lsb[1] + lane * 16;
         // released at once, as by everybody: the next item's description must not depend on this one's progress (the
         // weight warps want it while they have steps of this one to deliver)
         __syncwarp();
         if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
         for (int kc = 0; kc < nk; ++kc) {
+          if (!mbar_wait(&raw_free[rs], rpar, abort_flag)) { alive = false; break; }
+          if (prec) {
+            u_copy_raw<PHASE>(smem_u32(smem + USmem::raw + rs * kURawStep + 8 * kURawBlock + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
+            p0 += kURawBlock;
+            p1 += kURawBlock;
+          }
+          cp_async_arrive(&raw_full[rs]);
+          if (++rs == kURawStages) { rs = 0; rpar ^= 1; }
           if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
-          if (lane == 0) mbar_expect_tx(&full[st], 2 * boxes * kUBoxBytes);
+          if (elect_one()) {
+            mbar_expect_tx(&full[st], 2 * box * (kUBoxRows * kUBoxCols * 2));
+#pragma unroll
+            for (int panel = 0; panel < 2; ++panel)
+              asm volatile(
+                  "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+                      smem_u32(smem + USmem::tok + st * kUTileBytes + panel * kUPanelBytes)),
+                  "l"(&maps.rows[box - 1]), "r"(smem_u32(&full[st])), "r"(kc * kPfChunkK + panel * kUBoxCols), "r"(row)
+                  : "memory");
+          }
           __syncwarp();
-          if (box < boxes && panel < 2)
-            asm volatile(
-                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-                    smem_u32(smem + USmem::tok + st * kUTileBytes + panel * kUPanelBytes + box * kUBoxBytes)),
-                "l"(&tm_tok), "r"(smem_u32(&full[st])), "r"(kc * kPfChunkK + panel * kUBoxCols), "r"(row)
-                : "memory");
           if (++st == kUStages) { st = 0; par ^= 1; }
         }
         if (!alive) break;
       }
+      asm volatile("cp.async.wait_all;" ::: "memory");
       // No copy may still be on its way into shared memory when the CTA ends (only after a time-out can one be): the
       // step's barrier also counts the weight warps, so it cannot tell; the longest a copy can take is waited out.
       if (!alive) {
@@ -579,7 +620,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       // The whole warp walks the loop, so that its state stays on the uniform datapath, where the tensor instructions take
       // their operands from; one elected lane issues.  (All of it in one lane: twice the time per step.)
       uint32_t st = 0, par = 0;  // stage and parity of its use
-      uint32_t free0 = 1, free1 = 1;  // parity to wait for before an accumulator is written again (at first it is free)
+      uint32_t buf = 0, bpar = 1;  // accumulator of the next unit, parity of its use before
       bool issued = false;
       const uint64_t bd0 = umma_desc(smem_u32(smem + USmem::tok));
       constexpr int kGroups = 128 / G, kKs = G / 16;  // quantisation groups of a step, K 16 slices of a group
@@ -592,7 +633,6 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         __syncwarp();
         if (elect_one()) mbar_arrive(&item_free[ni % kUItemSlots]);
         const uint32_t id_first = umma_idesc(halves == 2 ? n0 : n), id_second = umma_idesc(n - n0);
-        uint32_t alt = 0;  // narrow tiles: the accumulator whose turn it is
         for (int kc = 0; kc < nk && alive; ++kc) {
           if (!mbar_wait(&full[st], par, abort_flag)) { alive = false; break; }
           const uint64_t bd_step = bd0 + (uint64_t)((st * kUTileBytes) >> 4);
@@ -600,10 +640,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
 #pragma unroll
           for (int grp = 0; grp < kGroups; ++grp) {
             for (int half = 0; half < halves; ++half) {
-              const uint32_t buf = halves == 2 ? (uint32_t)half : alt;
-              if (!mbar_wait(&acc_free[buf], buf ? free1 : free0, abort_flag)) { alive = false; break; }
-              if (buf) free1 ^= 1u;
-              else free0 ^= 1u;
+              if (!mbar_wait(&acc_free[buf], bpar, abort_flag)) { alive = false; break; }
               tc_fence_after();
               const uint32_t d = tmem + buf * kUAccCols, id = half ? id_second : id_first;
               const uint64_t bd = bd_step + (half ? (uint64_t)(n0 * 8) : 0ull);
@@ -618,8 +655,8 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
               }
               issued = true;
               __syncwarp();
+              if (++buf == kUAccs) { buf = 0; bpar ^= 1; }
             }
-            alt ^= 1u;
             if (!alive) break;
           }
           if (++st == kUStages) { st = 0; par ^= 1; }
@@ -640,7 +677,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       // How far ahead: one item where an item is long (its successor is fetched when the sums of the item itself have
       // begun, and no CTA sits on items that another could take), else as many as the ring holds.
       constexpr int kLongItem = 8, kAheadShort = 6;
-      static_assert(kAheadShort <= kUItemSlots && 2 * kURawDepth < kAheadShort, "items between the copies and their use");
+      static_assert(kAheadShort <= kUItemSlots, "items between the copies and their use");
       int ahead = kAheadShort;
       for (uint32_t ni = 0;; ++ni) {
         if (ni >= (uint32_t)ahead) {
@@ -712,124 +749,83 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         if (item >= n_items) break;
       }
     } else {
-      // ---- scales and zero-points: a row block's are contiguous over the groups, so lanes 0 .. 7 copy a row block's
-      // scales of up to 16 groups each and lanes 8 .. 15 its zero-points.  (Fetched by their users one group ahead, they
-      // cost a trip to memory per group.) ----
-      uint32_t m = 0;  // stages so far
-      static_assert((kUMetaStages & (kUMetaStages - 1)) == 0, "stage and parity by mask and shift");
+      // ---- raw MSB planes (cp.async); scales and zero-points (bulk copies): a row block's are contiguous over the groups, so
+      // for up to 16 groups at a time lanes 0 .. 7 copy a block's scales and lanes 8 .. 15 its zero-points.  (Planes by bulk
+      // copies of a row block's 1024 bytes each: a warp issues those lane by lane, 60 cycles each.) ----
+      uint32_t m = 0, rs = 0, rpar = 1;  // scale stages so far; raw stage, parity of its use before
+      const int rbk = lane & 7, mat = PHASE == 1 ? rbk & 1 : 0, rb = PHASE == 1 ? rbk >> 1 : rbk;
+      const bool second = lane >= 8;  // zero-points
+      constexpr int kMetaSteps = kUMetaGroups * G / 128;  // steps of a scale and zero-point stage
       for (uint32_t ni = 0; alive; ++ni) {
         const PfItem& it = items[ni % kUItemSlots];
         if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
         if (it.stop) break;
-        const int ngroups = (it.nk * kPfChunkK) >> LG;
-        const int rbk = lane & 7, mat = PHASE == 1 ? rbk & 1 : 0, rb = PHASE == 1 ? rbk >> 1 : rbk;
-        const bool zps = lane >= 8;
-        const uint8_t* src = (zps ? it.zp[mat] : reinterpret_cast<const uint8_t*>(it.scale[mat])) + (size_t)rb * ngroups * (zps ? 16 : 32);
+        const int nk = it.nk, ngroups = (nk * kPfChunkK) >> LG;
+        const uint8_t* src = (second ? it.zp[mat] : reinterpret_cast<const uint8_t*>(it.scale[mat])) + (size_t)rb * ngroups * (second ? 16 : 32);
+        const uint8_t *p0 = it.msb[0] + lane * 16, *p1 = it.msb[1] + lane * 16;
         __syncwarp();
         if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
         const bool aligned = __all_sync(0xffffffffu, lane >= 16 || (reinterpret_cast<uintptr_t>(src) & 15) == 0);
-        for (int g0 = 0; g0 < ngroups; g0 += kUMetaGroups, ++m) {
-          const uint32_t ms = m % kUMetaStages;
-          if (m >= kUMetaStages && !mbar_wait(&meta_free[ms], ((m / kUMetaStages) & 1) ^ 1, abort_flag)) { alive = false; break; }
-          const int gs = min(kUMetaGroups, ngroups - g0), bytes = gs * (zps ? 16 : 32);
-          uint8_t* dst = smem + USmem::meta + ms * kUMetaBytes + (zps ? 8 * kUMetaScale + rbk * kUMetaZp : rbk * kUMetaScale);
-          const uint8_t* from = src + (size_t)g0 * (zps ? 16 : 32);
-          if (aligned) {
-            if (lane == 0) mbar_expect_tx(&meta_full[ms], gs * 8 * 48);
-            __syncwarp();
-            if (lane < 16)
-              asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                               smem_u32(dst)),
-                           "l"(from), "r"(bytes), "r"(smem_u32(&meta_full[ms]))
-                           : "memory");
-          } else {  // a caller's array that does not start on 16 bytes: byte by byte
-            if (lane < 16)
-              for (int i = 0; i < bytes; ++i) dst[i] = from[i];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&meta_full[ms]);
+        for (int kc = 0; kc < nk; ++kc) {
+          if (kc % kMetaSteps == 0) {
+            const uint32_t ms = m % kUMetaStages;
+            if (!mbar_wait(&meta_free[ms], ((m / kUMetaStages) & 1) ^ 1, abort_flag)) { alive = false; break; }
+            const int g0 = (kc * kPfChunkK) >> LG, gs = min(kUMetaGroups, ngroups - g0), bytes = gs * (second ? 16 : 32);
+            uint8_t* dst = smem + USmem::meta + ms * kUMetaBytes + (second ? 8 * kUMetaScale + rbk * kUMetaZp : rbk * kUMetaScale);
+            const uint8_t* from = src + (size_t)g0 * (second ? 16 : 32);
+            if (aligned) {
+              if (lane == 0) mbar_expect_tx(&meta_full[ms], gs * 8 * 48);
+              __syncwarp();
+              if (lane < 16) bulk_copy(dst, from, bytes, &meta_full[ms]);
+            } else {  // a caller's array that does not start on 16 bytes: byte by byte
+              if (lane < 16)
+                for (int i = 0; i < bytes; ++i) dst[i] = from[i];
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&meta_full[ms]);
+            }
+            ++m;
           }
+          if (!mbar_wait(&raw_free[rs], rpar, abort_flag)) { alive = false; break; }
+          u_copy_raw<PHASE>(smem_u32(smem + USmem::raw + rs * kURawStep + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
+          p0 += kURawBlock;
+          p1 += kURawBlock;
+          cp_async_arrive(&raw_full[rs]);
+          if (++rs == kURawStages) { rs = 0; rpar ^= 1; }
         }
       }
-      for (uint32_t i = m > kUMetaStages ? m - kUMetaStages : 0; i < m && !alive; ++i) {  // as for the token tiles
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      for (uint32_t i = m > kUMetaStages ? m - kUMetaStages : 0; i < m && !alive; ++i) {  // no copy on its way when the CTA ends
         const uint32_t t0 = (uint32_t)clock64();
         while (!mbar_try(&meta_full[i % kUMetaStages], (i / kUMetaStages) & 1) && (uint32_t)clock64() - t0 < kUWaitCycles) {}
       }
     }
   } else if (warp >= kUSumWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kURegsWeight));
-    // ---- weights: sets of four warps take the 64-column steps in turn; warp q of a set owns tensor-memory lanes
+    // ---- weights: sets of four warps take the steps in turn; warp q of a set owns tensor-memory lanes
     // [32 q, 32 q + 32), two row blocks, and stores their integers of the step into the stage's columns.  The planes are laid
     // out as the fragments of a 16-row store: plane lane 4 g + c holds rows g and g + 8, columns 16 w + 4 c + j, which
-    // is what lane 4 g + c of tcgen05.st.16x256b gives.  So a lane copies, converts and stores the same 16 bytes
-    // of a plane: both nibbles of every byte are used, and no lane reads what another copied. ----
+    // is what lane 4 g + c of tcgen05.st.16x256b gives.  So a lane reads 16 bytes of a plane block, converts and stores
+    // them: both nibbles of every byte are used, and nothing is exchanged. ----
     const int q = warp & 3, set = (warp - kUSumWarps) >> 2;
     const int g = lane >> 2;
-    constexpr int kGpc = G == 32 ? 2 : 1;  // quantisation groups in a step
-    // Raw plane words run kURawDepth of the warp's steps ahead of their use, across work items: per step two row blocks
-    // of 1024 bytes per plane, twice 16 bytes a lane, copied with cp.async into the warp's ring.
-    uint8_t* raw = smem + USmem::raw + (warp - kUSumWarps) * (kURawDepth * kURawStep) + lane * 16;
-    // the copies' place in the work: item number, step, addresses
-    // (Steps are counted over all items; those of the set's parity are its own.  An item of one step has none for one set.)
-    uint32_t i_ni = 0;
-    int i_left = 0;            // steps from the next own one to the item's end
-    uint32_t i_skip = set;     // steps of the next item before its first own one
-    bool i_more = true, i_prec = false;
-    const uint8_t *i_mp0 = nullptr, *i_mp1 = nullptr, *i_lp0 = nullptr, *i_lp1 = nullptr;
-    // An item is opened when its first step is to be copied, not before: the copies are then at most 2 kURawDepth items
-    // ahead, which is what the ring of descriptions holds.
-    auto i_open = [&]() {
-      const PfItem& it = items[i_ni % kUItemSlots];
-      if (!mbar_wait(&item_full[i_ni % kUItemSlots], (i_ni / kUItemSlots) & 1, abort_flag)) { i_more = false; return; }
-      if (it.stop) { i_more = false; return; }
-      const int nk = it.nk;
-      i_prec = it.prec != 0;
-      // row blocks: gate and up of 16 columns of h, or two neighbours of down; a block's steps are 1024 bytes apart
-      const size_t o0 = (size_t)(PHASE == 1 ? q : 2 * q) * nk * 1024 + i_skip * 1024 + lane * 16, o1 = PHASE == 1 ? o0 : o0 + (size_t)nk * 1024;
-      i_mp0 = it.msb[0] + o0;
-      i_mp1 = it.msb[1] + o1;
-      if (i_prec) {
-        i_lp0 = it.lsb[0] + o0;
-        i_lp1 = it.lsb[1] + o1;
-      }
-      i_left = nk - (int)i_skip;
-      i_skip = (uint32_t)(i_skip + nk) & 1u;  // own steps are those with an even distance
-      ++i_ni;
-    };
-    auto i_issue = [&](uint8_t* dst) {
-      while (i_more && i_left <= 0) i_open();
-      if (i_more) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          cp_async16(dst + 512 * h, i_mp0 + 512 * h);
-          cp_async16(dst + 1024 + 512 * h, i_mp1 + 512 * h);
-          if (i_prec) {
-            cp_async16(dst + 2048 + 512 * h, i_lp0 + 512 * h);
-            cp_async16(dst + 3072 + 512 * h, i_lp1 + 512 * h);
-          }
-        }
-        i_mp0 += 1024 * kUSets;
-        i_mp1 += 1024 * kUSets;
-        i_lp0 += 1024 * kUSets;
-        i_lp1 += 1024 * kUSets;
-        i_left -= kUSets;
-      }
-      cp_async_commit();
-    };
-    for (int j = 0; j < kURawDepth; ++j) i_issue(raw + j * kURawStep);
+    const uint8_t* raw = smem + USmem::raw + 2 * q * kURawBlock + lane * 16;
     const int shift = p.shift;
     // row g's codes: MSB nibble at bit `shift`, LSB nibble below; row g + 8's the same from the high nibbles.  A slice
     // narrower than four bits leaves the top of its nibble zero, so what the second mask lets through beyond it is zero.
     const uint32_t mask = 0x0f0f0f0fu << shift;
     const int back = 4 - shift;
-    uint8_t* slot = raw;
-    uint32_t st = set, par = 1, m = 0, skip = set;  // stage of the next own step, parity of its use before; scale and zero-point stages
-    static_assert(kUSets < kUStages, "a set's next stage is at most once round the ring away");
+    // (Steps are counted over all items; those of the set's parity are its own.)
+    uint32_t st = set, par = 1, m = 0, skip = set;  // stage of the next own step, parity of its use before; scale and zero-point
+                                                    // stages; steps of the item before the first own one
+    uint32_t rs = set, rpar = 0;                    // raw stage of the next own step, parity of this use
+    static_assert(kUSets < kUStages && kURawStages % kUSets == 0, "a set's next stage is at most once round the rings away");
     for (uint32_t ni = 0; alive; ++ni) {
       const PfItem& it = items[ni % kUItemSlots];
       if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
       if (it.stop) break;
       const int nk = it.nk;
       const bool prec = it.prec != 0;
+      const uint32_t zmask = prec ? 0xffu : 0xffu << shift;  // from the MSB slice alone: 2^shift (zp >> shift)
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
       int kc = (int)skip;
@@ -841,8 +837,14 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         const uint8_t* zp_stage = smem + USmem::meta + ms * kUMetaBytes + 8 * kUMetaScale + 2 * q * kUMetaZp + g;
         const int k_end = min(nk, k0 + kMetaSteps);
         for (; kc < k_end; kc += kUSets) {
-          cp_async_wait_but<kURawDepth - 1>();  // this lane's own copies: nobody else reads them
           const uint8_t* zp = zp_stage + (kc - k0) * (128 / G * 16);
+          if (!mbar_wait(&raw_full[rs], rpar, abort_flag)) { alive = false; break; }
+          const uint8_t* slot = raw + rs * kURawStep;
+          uint4 mv[4], lv[4];  // [2 block + half]
+#pragma unroll
+          for (int i = 0; i < 4; ++i) mv[i] = *reinterpret_cast<const uint4*>(slot + 512 * i);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) lv[i] = prec ? *reinterpret_cast<const uint4*>(slot + 8 * kURawBlock + 512 * i) : make_uint4(0, 0, 0, 0);
           if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
           tc_fence_after();
           const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + kUWCol0 + st * kUWCols;
@@ -854,16 +856,13 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
 #pragma unroll
               for (int hi = 0; hi < 2; ++hi) {
                 uint32_t z = zp[b * kUMetaZp + 16 * i + 8 * hi];
-                if (!prec) z = z >> shift << shift;
-                z = z * 0x00010001u + 0x64006400u;
+                z = (z & zmask) * 0x00010001u + 0x64006400u;
                 off[i][hi] = *reinterpret_cast<__half2*>(&z);
               }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-              const uint4 mv = *reinterpret_cast<const uint4*>(slot + 1024 * b + 512 * h);
-              uint4 lv = make_uint4(0, 0, 0, 0);
-              if (prec) lv = *reinterpret_cast<const uint4*>(slot + 2048 + 1024 * b + 512 * h);
-              const uint32_t mw[4] = {mv.x, mv.y, mv.z, mv.w}, lw[4] = {lv.x, lv.y, lv.z, lv.w};
+              const uint32_t mw[4] = {mv[2 * b + h].x, mv[2 * b + h].y, mv[2 * b + h].z, mv[2 * b + h].w},
+                             lw[4] = {lv[2 * b + h].x, lv[2 * b + h].y, lv[2 * b + h].z, lv[2 * b + h].w};
               uint32_t out[16];
 #pragma unroll
               for (int w = 0; w < 4; ++w) {
@@ -882,11 +881,15 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
               tmem_st_16x32(ta + ((uint32_t)(16 * b) << 16) + 32 * h, out);
             }
           }
-          i_issue(slot);
-          slot = slot == raw ? raw + kURawStep : raw;
           tmem_st_wait();
           tc_fence_before();
           __syncwarp();
+          if (lane == 0) mbar_arrive(&raw_free[rs]);
+          rs += kUSets;
+          if (rs >= kURawStages) {
+            rs -= kURawStages;
+            rpar ^= 1;
+          }
           if (lane == 0) mbar_arrive(&full[st]);
           st += kUSets;
           if (st >= kUStages) {
@@ -897,12 +900,11 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         if (alive && lane == 0) mbar_arrive(&meta_free[ms]);
       }
     }
-    cp_async_wait_but<0>();
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kURegsSum));
     // ---- sums: warp (q, wg) owns weight rows [32 q, 32 q + 32) x the warpgroup's tokens, in fp32 registers ----
     const int q = warp & 3, wg = warp >> 2;
-    uint32_t used = 0;  // bit per accumulator: parity of the times it has been filled
+    uint32_t buf = 0, bpar = 0;  // accumulator of the next unit (a group's sums for the tile or half of it), parity of its use
     uint32_t m = 0;     // scale stages so far
     for (uint32_t ni = 0; alive; ++ni) {
       const PfItem& it = items[ni % kUItemSlots];
@@ -915,10 +917,12 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
       const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16) + (halves == 1 && wg ? n0 : 0);
+      auto next_unit = [&]() {
+        if (++buf == kUAccs) { buf = 0; bpar ^= 1; }
+      };
       uint64_t acc[kUHalfMax / 2];
 #pragma unroll
       for (int i = 0; i < kUHalfMax / 2; ++i) acc[i] = 0ull;
-      uint32_t alt = 0;  // narrow tiles: the accumulator whose turn it is
       for (int g0 = 0; g0 < ngroups && alive; g0 += kUMetaGroups, ++m) {
         const uint32_t ms = m % kUMetaStages;
         if (!mbar_wait(&meta_full[ms], (m / kUMetaStages) & 1, abort_flag)) { alive = false; break; }
@@ -926,11 +930,9 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         for (int gi = min(kUMetaGroups, ngroups - g0); gi > 0; --gi, sc += 32) {
           const float s = __half2float(*reinterpret_cast<const __half*>(sc));
           const uint64_t ss = ((uint64_t)__float_as_uint(s) << 32) | __float_as_uint(s);
-          // (with two accumulators the other warpgroup's one is filled and read without this one)
-          const uint32_t buf = halves == 2 ? (uint32_t)wg : alt;
-          if (!mbar_wait(&acc_full[buf], (used >> buf) & 1u, abort_flag)) { alive = false; break; }
-          used ^= halves == 2 ? 3u : 1u << buf;
-          alt ^= 1u;
+          // (a tile in two halves has a unit for each warpgroup; the other one's is filled and read without this one)
+          if (halves == 2 && wg == 1) next_unit();
+          if (!mbar_wait(&acc_full[buf], bpar, abort_flag)) { alive = false; break; }
           tc_fence_after();
 #pragma unroll
           for (int c = 0; c < kUHalfMax / 32; ++c) {
@@ -947,6 +949,8 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
             mbar_arrive(&acc_free[buf]);
             if (halves == 2) mbar_arrive(&acc_free[buf]);
           }
+          next_unit();
+          if (halves == 2 && wg == 0) next_unit();
         }
         __syncwarp();
         if (alive && lane == 0) mbar_arrive(&meta_free[ms]);
@@ -958,28 +962,37 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         const bool up = lane >= 16;
         __half* dst = p.h + (size_t)(out_row + (up ? 1 : 0)) * p.ldh + col + 16 * q + (lane & 15);
         const size_t two_rows = 2 * (size_t)p.ldh;
+        // 16 tokens at a time, with a branch per 16: within them the chains of shuffle, exponential and reciprocal overlap
 #pragma unroll
-        for (int i = 0; i < kUHalfMax / 2; ++i) {
-          if (2 * i < count) {
-            const float v0 = half_of(acc[i], 0), v1 = half_of(acc[i], 1);
-            const float got = __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 16);
-            const float gate = up ? got : v0, upv = up ? v1 : got;
-            // silu: g / (1 + e^-g), the quotient by the reciprocal and one step of Newton's iteration.  Below -80 the
-            // result is zero in fp16 either way; the bound keeps 1 + e^-g finite.
-            const float t = 1.f + __expf(fminf(-gate, 80.f));
-            float r;
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
-            r = fmaf(r, fmaf(-t, r, 1.f), r);
-            if (2 * i + (up ? 1 : 0) < count) *dst = __float2half_rn(gate * r * upv);
-            dst += two_rows;
+        for (int i0 = 0; i0 < kUHalfMax / 2; i0 += 8) {
+          if (2 * i0 < count) {
+#pragma unroll
+            for (int i = i0; i < i0 + 8; ++i) {
+              const float v0 = half_of(acc[i], 0), v1 = half_of(acc[i], 1);
+              const float got = __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 16);
+              const float gate = up ? got : v0, upv = up ? v1 : got;
+              // silu: g / (1 + e^-g), the quotient by the reciprocal and one step of Newton's iteration.  Below -80 the
+              // result is zero in fp16 either way; the bound keeps 1 + e^-g finite.
+              const float t = 1.f + __expf(fminf(-gate, 80.f));
+              float r;
+              asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+              r = fmaf(r, fmaf(-t, r, 1.f), r);
+              if (2 * i + (up ? 1 : 0) < count) *dst = __float2half_rn(gate * r * upv);
+              dst += two_rows;
+            }
           }
         }
       } else {
         float* dst = p.yrow + (size_t)out_row * p.hidden + col + 32 * q + lane;
 #pragma unroll
-        for (int i = 0; i < kUHalfMax / 2; ++i) {
-          if (2 * i < count) dst[(size_t)(2 * i) * p.hidden] = half_of(acc[i], 0);
-          if (2 * i + 1 < count) dst[(size_t)(2 * i + 1) * p.hidden] = half_of(acc[i], 1);
+        for (int i0 = 0; i0 < kUHalfMax / 2; i0 += 8) {
+          if (2 * i0 < count) {
+#pragma unroll
+            for (int i = 2 * i0; i < 2 * i0 + 16; ++i) {
+              if (i < count) *dst = half_of(acc[i >> 1], i & 1);
+              dst += p.hidden;
+            }
+          }
         }
       }
     }
@@ -1042,8 +1055,8 @@ typedef CUresult (*PfEncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor map of a row-major fp16 matrix [rows, cols] for 32-row x 64-column tiles with 128-byte swizzle.
-static int pf_tensor_map(CUtensorMap* tm, const __half* base, int rows, int cols) {
+// Tensor maps of a row-major fp16 matrix [rows, cols] for tiles of 32, 64, ... rows x 64 columns with 128-byte swizzle.
+static int pf_tensor_maps(PfMaps* maps, const __half* base, int rows, int cols) {
   static PfEncodeTiled encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q;
@@ -1054,12 +1067,15 @@ static int pf_tensor_map(CUtensorMap* tm, const __half* base, int rows, int cols
   }
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)cols * sizeof(__half)};
-  const cuuint32_t box[2] = {(cuuint32_t)kUBoxCols, (cuuint32_t)kUBoxRows};
   const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base), dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? SLICEMOE_OK : SLICEMOE_E_INVALID_ARG;
+  for (int i = 0; i < kUBoxes; ++i) {
+    const cuuint32_t box[2] = {(cuuint32_t)kUBoxCols, (cuuint32_t)(kUBoxRows * (i + 1))};
+    const CUresult r = encode(&maps->rows[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base), dims, strides, box,
+                              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return SLICEMOE_E_INVALID_ARG;
+  }
+  return SLICEMOE_OK;
 }
 
 // Every kernel of a step starts while the one before it is still running and waits for it itself (pf_dep_wait).
@@ -1092,10 +1108,10 @@ static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int in_rows,
     SM_CUDA_TRY(cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev));
     attr_set[dev] = true;
   }
-  CUtensorMap tm_x, tm_h;
-  int rc = pf_tensor_map(&tm_x, xs, in_rows, p.hidden);
+  PfMaps tm_x, tm_h;
+  int rc = pf_tensor_maps(&tm_x, xs, in_rows, p.hidden);
   if (rc != SLICEMOE_OK) return rc;
-  rc = pf_tensor_map(&tm_h, p.h, out_rows, p.ldh);
+  rc = pf_tensor_maps(&tm_h, p.h, out_rows, p.ldh);
   if (rc != SLICEMOE_OK) return rc;
   // one persistent CTA per SM (shared memory admits one); each takes work items until there are none
   rc = pf_launch(pf_umma_kernel<G, 1>, (unsigned)sm_count[dev], kUThreads, kUSmemBytes, st, p, tm_x);
