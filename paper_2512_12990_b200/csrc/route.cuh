@@ -4,7 +4,10 @@
 //
 // Each lane keeps E/32 (<= 16) logits in registers; the softmax uses fp32 expf; selection runs k rounds of a
 // warp arg-max on key = logit + bias (one fp32 add, NaN -> -inf) with ties broken towards the lower expert
-// index, so the ids are a pure function of the keys.
+// index, so the ids are a pure function of the keys.  A decode step waits for this, so what counts is the length of the
+// dependent chain: a key is mapped to an integer of the same order, a round is two warp reductions (largest key, lowest
+// index that has it), and the k probabilities are worked out side by side at the end.  (Rounds of five shuffle steps
+// on (key, index) pairs with the probability in between made a decode step of two launches 20.8 us; this way 19.6.)
 #pragma once
 
 #include <math_constants.h>
@@ -26,26 +29,26 @@ template <int VPT>
 __device__ __forceinline__ RouteSel route_warp_vpt(const float* __restrict__ row, int E, int k,
                                                    const float* __restrict__ bias, int renorm, float tau, int rank_high,
                                                    int lane) {
-  float key[VPT];
+  uint32_t key[VPT];  // ordered like the float keys; 0: no such expert, or taken
   float val[VPT];
   float vmax = -CUDART_INF_F;
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
     const int e = v * 32 + lane;
-    float l = -CUDART_INF_F, kk = -CUDART_INF_F;
+    float l = -CUDART_INF_F;
+    key[v] = 0u;
     if (e < E) {
-      l = row[e];
-      if (isnan(l)) l = -CUDART_INF_F;
-      kk = row[e];
-      if (bias) kk = __fadd_rn(kk, bias[e]);
+      const float raw = row[e];
+      l = isnan(raw) ? -CUDART_INF_F : raw;
+      float kk = bias ? __fadd_rn(raw, bias[e]) : raw;
       if (isnan(kk)) kk = -CUDART_INF_F;
+      const uint32_t b = __float_as_uint(kk + 0.0f);  // both zeros are one key
+      key[v] = b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
     }
     val[v] = l;
-    key[v] = kk;
     vmax = fmaxf(vmax, l);
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, off));
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(vmax) : "f"(vmax));
   float sum = 0.0f;
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
@@ -56,54 +59,38 @@ __device__ __forceinline__ RouteSel route_warp_vpt(const float* __restrict__ row
   for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
   const float inv_sum = 1.0f / sum;
 
-  uint32_t taken = 0;  // bit v: this lane's value v was already selected
-  float wsel = 0.0f;   // lane j keeps the weight of selection j (k <= 16 < 32)
-  int idsel = 0;
-  float wtotal = 0.0f;
+  int idsel = 0;  // lane j keeps selection j (k <= 16 < 32)
   for (int j = 0; j < k; ++j) {
-    float best = -CUDART_INF_F;
-    int best_e = 0x7fffffff;
+    uint32_t best = key[0];
+    int bv = 0;
 #pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      const int e = v * 32 + lane;
-      if (e < E && !((taken >> v) & 1u)) {
-        if (best_e == 0x7fffffff || key[v] > best) {  // ascending e within a lane: strict > keeps the lower index
-          best = key[v];
-          best_e = e;
-        }
+    for (int v = 1; v < VPT; ++v) {
+      if (key[v] > best) {  // ascending e within a lane: strict > keeps the lower index
+        best = key[v];
+        bv = v;
       }
     }
+    const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+    const int e = (int)__reduce_min_sync(0xffffffffu, best == top ? (uint32_t)(bv * 32 + lane) : 0xffffffffu);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const float ob = __shfl_xor_sync(0xffffffffu, best, off);
-      const int oe = __shfl_xor_sync(0xffffffffu, best_e, off);
-      const bool other_wins = (oe != 0x7fffffff) && (best_e == 0x7fffffff || ob > best || (ob == best && oe < best_e));
-      if (other_wins) {
-        best = ob;
-        best_e = oe;
-      }
-    }
-    // every lane now agrees on best_e; its owner marks it and provides the probability
-    const int owner = best_e & 31, ov = best_e >> 5;
-    float p = 0.0f;
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      if (v == ov && lane == owner) {
-        taken |= 1u << v;
-        p = expf(val[v] - vmax) * inv_sum;
-      }
-    }
-    p = __shfl_sync(0xffffffffu, p, owner);
-    wtotal += p;
-    if (lane == j) {
-      wsel = p;
-      idsel = best_e;
-    }
+    for (int v = 0; v < VPT; ++v)
+      if (e == v * 32 + lane) key[v] = 0u;
+    if (lane == j) idsel = e;
+  }
+  float p = 0.0f;
+  if (lane < k) {
+    const float raw = row[idsel];
+    p = expf((isnan(raw) ? -CUDART_INF_F : raw) - vmax) * inv_sum;
+  }
+  float total = 1.0f;
+  if (renorm) {  // added up in selection order
+    total = 0.0f;
+    for (int j = 0; j < k; ++j) total += __shfl_sync(0xffffffffu, p, j);
   }
   RouteSel sel;
   sel.id = idsel;
-  sel.w = renorm ? wsel / wtotal : wsel;
-  sel.prec_req = (uint8_t)((wsel >= tau || lane < rank_high) ? 1 : 0);
+  sel.w = renorm ? p / total : p;
+  sel.prec_req = (uint8_t)((p >= tau || lane < rank_high) ? 1 : 0);
   return sel;
 }
 
