@@ -1355,6 +1355,40 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
   }
 }
 
+// ---- inputs in host memory ---------------------------------------------------------------------------
+// A decode step whose x and logits sit in device-mapped host memory: one block reads them over the bus, side by side, routes
+// (so that the layer kernel, whose every CTA would otherwise work out the list for itself, just reads it) and leaves x and
+// the list in the workspace.  The layer kernel's launch overlaps it.  Bound: one trip over the bus, about 2 us.  Against
+// two copies and the layer kernel with the routing in its prologue - copies cannot overlap the launch, and the prologue
+// is 3 us longer - a step of the 2048-wide layer takes 34 us instead of 38.
+constexpr int kStageThreads = 256;
+__global__ void __launch_bounds__(kStageThreads) stage_step_kernel(const uint32_t* x_host, const float* logits_host, int hidden, int E,
+                                                                   int k, const float* bias, int renorm, float tau, int rank_high,
+                                                                   uint32_t* x, int32_t* ids, float* weights, uint8_t* prec) {
+  __shared__ float row[32 * ROUTE_MAX_VPT];
+  const int tid = threadIdx.x, lane = tid & 31;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the work ahead may be what writes the host buffers
+  constexpr int kWords = kMaxHidden / 2 / kStageThreads;
+  uint32_t v[kWords];
+#pragma unroll
+  for (int i = 0; i < kWords; ++i)
+    if (i * kStageThreads + tid < hidden / 2) v[i] = __ldcv(x_host + i * kStageThreads + tid);
+  for (int e = tid; e < E; e += kStageThreads) row[e] = __ldcv(logits_host + e);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kWords; ++i)
+    if (i * kStageThreads + tid < hidden / 2) x[i * kStageThreads + tid] = v[i];
+  if (tid < 32) {
+    const RouteSel sel = route_warp(row, E, k, bias, renorm, tau, rank_high, lane);
+    if (lane < k) {
+      ids[lane] = sel.id;
+      weights[lane] = sel.w;
+      prec[lane] = sel.prec_req;
+    }
+  }
+}
+
 // ---- host side --------------------------------------------------------------------------------------
 static int g_num_sms[64];
 static bool g_attr_set[64][6];
@@ -1632,16 +1666,42 @@ extern "C" int slicemoe_decode_step_host(const slicemoe_shape* shape, const slic
   float* dy = reinterpret_cast<float*>(ws + kWsStY);
   // y_host in pinned (device-mapped) host memory: the kernel writes its 16 output rows per CTA straight
   // into it and the copy back falls away; otherwise y goes through the staging area.
-  bool y_direct = false;
-  {
+  auto mapped = [](const void* host, unsigned align) -> void* {
     cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, y_host) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer &&
-        (reinterpret_cast<uintptr_t>(attr.devicePointer) & 15) == 0) {
-      dy = reinterpret_cast<float*>(attr.devicePointer);
-      y_direct = true;
-    } else {
-      (void)cudaGetLastError();  // an unregistered pointer is not an error here
-    }
+    if (cudaPointerGetAttributes(&attr, host) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer &&
+        (reinterpret_cast<uintptr_t>(attr.devicePointer) & (align - 1)) == 0)
+      return attr.devicePointer;
+    (void)cudaGetLastError();  // an unregistered pointer is not an error here
+    return nullptr;
+  };
+  void* y_mapped = mapped(y_host, 16);
+  const bool y_direct = y_mapped != nullptr;
+  if (y_direct) dy = reinterpret_cast<float*>(y_mapped);
+  // x and the logits likewise are read where they are
+  const void* x_mapped = mapped(x_host, 4);
+  const float* logits_mapped = x_mapped == nullptr ? nullptr
+                                                  : reinterpret_cast<const float*>(mapped(
+                                                        logits_host ? static_cast<const void*>(logits_host)
+                                                                    : static_cast<const uint8_t*>(x_host) + 2 * (size_t)shape->hidden, 4));
+  if (logits_mapped) {
+    if (!experts || (shape->n_shared > 0 && (!shared || (shape->shared_sigmoid_gate && !shared_gate_vec)))) return SLICEMOE_E_INVALID_ARG;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(kStageThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SM_CUDA_TRY(cudaLaunchKernelEx(&cfg, stage_step_kernel, reinterpret_cast<const uint32_t*>(x_mapped), logits_mapped, (int)shape->hidden,
+                                   (int)shape->n_experts, (int)shape->top_k, bias, renorm, tau, rank_high,
+                                   reinterpret_cast<uint32_t*>(dx), dids, dw, dprec));
+    rc = slicemoe_layer(shape, experts, shared, shared_gate_vec, dx, 1, dids, dprec, dw, dy, workspace, workspace_bytes, stream);
+    if (rc != SLICEMOE_OK) return rc;
+    if (!y_direct) SM_CUDA_TRY(cudaMemcpyAsync(y_host, dy, 4 * (size_t)shape->hidden, cudaMemcpyDeviceToHost, st));
+    SM_CUDA_TRY(cudaStreamSynchronize(st));
+    return SLICEMOE_OK;
   }
   if (logits_host) {
     SM_CUDA_TRY(cudaMemcpyAsync(dx, x_host, 2 * (size_t)shape->hidden, cudaMemcpyHostToDevice, st));
