@@ -33,7 +33,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "batch.cuh"
 #include "common.cuh"
+#include "decode_common.cuh"
 #include "route.cuh"
 
 namespace slicemoe {
@@ -60,9 +62,6 @@ constexpr int kMaxHidden = 4096;
 constexpr int kHCap = 12288;  // sum of intermediate widths over all slots of a layer
 constexpr int kMaxMine = 32;   // phase-2 chunks one consumer group can have: (slots + kHCap / kChunkK) chunks per
                                // output row block, at most 4 row blocks per CTA, shared by 4 groups
-// Every device-side wait is bounded: by this many clock cycles (about 50 ms; a layer takes tens of microseconds)
-// unless the workspace header carries another limit.
-constexpr unsigned long long kWaitCycles = 100000000ull;
 
 // ---- optional time stamps ------------------------------------------------------------------------
 // A build with -DSLICEMOE_TRACE records, per CTA and for the most recent launch, when its roles passed a few
@@ -122,6 +121,14 @@ constexpr size_t kWsStW = kWsStIds + 64;
 constexpr size_t kWsStPrec = kWsStW + 64;
 constexpr size_t kWsStY = kWsStPrec + 64;
 constexpr size_t kWsBytes = kWsStY + 4 * kMaxHidden;
+// Behind that, in a workspace of slicemoe_workspace_bytes(): the batch kernels' part, then the lists of a pass that is
+// routed here: ids i32, w f32, prec u8, [kBatchTokens][SLICEMOE_MAX_TOP_K] each.
+constexpr size_t kWsBatchOff = (kWsBytes + 255) & ~(size_t)255;
+constexpr size_t kWsListEntries = (size_t)kBatchTokens * SLICEMOE_MAX_TOP_K;
+constexpr size_t kWsListBytes = kWsListEntries * 9;
+// From this many tokens on a layer call takes the batch kernels (four launches) instead of a launch of the batch-1 kernel
+// per token.  BATCH_RULE
+constexpr int kBatchMinTokens = 4;
 static_assert(sizeof(WsHeader) <= kWsHOff, "workspace header");
 static_assert(kWsStLogits + 4 * 512 <= kWsStIds, "x and the logits fit the staging area back to back too");
 
@@ -239,133 +246,22 @@ struct Bars {
 
 static_assert(Bars::count <= SmemLayout::nbars, "barrier storage");
 
-// ---- PTX helpers -------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// The CTA's wait limit sits 8 bytes behind its dead flag.
-__device__ __forceinline__ unsigned long long wait_limit(volatile int* dead) {
-  return *reinterpret_cast<volatile unsigned long long*>(dead + 2);
-}
-// Bounded wait.  Returns false (and raises the CTA's dead flag) when the limit is hit or another
-// role of this CTA already gave up.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* dead, unsigned* status) {
-  const long long t0 = clock64();
-  for (;;) {
-    for (int i = 0; i < 256; ++i)
-      if (mbar_try(bar, parity)) return true;
-    if (*dead) return false;
-    if ((unsigned long long)(clock64() - t0) > wait_limit(dead)) {
-      *dead = 1;
-      atomicOr(status, (unsigned)SLICEMOE_STATUS_WAIT_TIMEOUT);
-      return false;
-    }
-  }
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* dead, unsigned* status) {
-  if (mbar_try(bar, parity)) return true;
-  return mbar_wait_slow(bar, parity, dead, status);
-}
-// Weights are used once per token: they go through L2 marked evict-first, so that the stream does not push out
-// what every launch uses again (the kernel's own instructions, expert tables, h).
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-  uint64_t pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-  return pol;
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar), "l"(pol)
-      : "memory");
-}
-__device__ __forceinline__ void mma_u8s8(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-// d = a * b (no accumulator input: the first step of a chain)
-__device__ __forceinline__ void mma_u8s8_first(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1) {
-  const int z = 0;
-  asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-      : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(z));
-}
-// ---- fixed-point activations ---------------------------------------------------------------------
-// Byte offset, inside a digit buffer, of digit t of the four values k..k+3 (k % 4 == 0): steps of 32
-// columns, 3 digit rows of 32 bytes, and inside a row the order in which the B fragment of m16n8k32 wants
-// them: (k % 16) / 4 selects the lane quad position, (k % 32) / 16 the register.
-__device__ __forceinline__ int digit_offset(int k, int t) {
-  return (k >> 5) * 96 + t * 32 + ((k >> 2) & 3) * 8 + ((k >> 4) & 1) * 4;
-}
-
-// One warp converts one 128-element block (lane L holds elements 4L..4L+3 of the block, whose first
-// element has index k0 in its vector): fixed point X = rint(v * 2^e) with 2^e * max|v| < 2^22, split into
-// balanced base-256 digits d0 + 256 d1 + 65536 d2 (each in int8 range; the low byte of X read as a signed
-// byte is d0, and so on up), stored in B-fragment order; the weighted digit sums of every group of G
-// elements (the zero-point term of the fold) and the block's 2^-e.
+// ---- fixed-point activations (see decode_common.cuh) ----------------------------------------------------
+// One warp converts one 128-element block whose first element has index k0 in its vector: digits in B-fragment order,
+// the weighted digit sums of every group of G elements (the zero-point term of the fold) and the block's 2^-e.
 template <int G>
 __device__ __forceinline__ void block_to_digits(const float (&v)[4], int k0, int lane, uint8_t* dig, float* sumw,
                                                 float* inv) {
-  unsigned mb = 0u;  // bit pattern of max |v|: non-negative floats order like their bit patterns
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const unsigned a = __float_as_uint(v[j]) & 0x7fffffffu;
-    if (a <= 0x7f800000u) mb = max(mb, a);  // a NaN input gives an undefined result, never a fault
-  }
-  mb = __reduce_max_sync(0xffffffffu, mb);
-  const int ex = (int)(mb >> 23) - 127;  // floor(log2 max) for normal numbers
-  const int e = max(-100, min(100, 21 - ex));
-  const float scale = __uint_as_float((unsigned)(127 + e) << 23);
-  // Z = (X + 0x808080) ^ 0x808080 holds the three digits in its bytes: adding 128 to a byte and flipping its top
-  // bit back leaves the byte read as a signed digit, and the carry into the next byte is exactly what remains
-  // after taking that digit (X1 = (X + 128) >> 8, and so on up).
-  uint32_t Z[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int X = max(-4194304, min(4194304, __float2int_rn(v[j] * scale)));
-    Z[j] = (uint32_t)(X + 0x808080) ^ 0x808080u;
-  }
-  // byte i of each of the four values -> one word (value j in byte j)
-  const uint32_t d0 = __byte_perm(__byte_perm(Z[0], Z[1], 0x0040), __byte_perm(Z[2], Z[3], 0x0040), 0x5410);
-  const uint32_t d1 = __byte_perm(__byte_perm(Z[0], Z[1], 0x0051), __byte_perm(Z[2], Z[3], 0x0051), 0x5410);
-  const uint32_t d2 = __byte_perm(__byte_perm(Z[0], Z[1], 0x0062), __byte_perm(Z[2], Z[3], 0x0062), 0x5410);
+  const BlockDigits b = block_digits(v);
   const int k = k0 + 4 * lane;
-  *reinterpret_cast<uint32_t*>(dig + digit_offset(k, 0)) = d0;
-  *reinterpret_cast<uint32_t*>(dig + digit_offset(k, 1)) = d1;
-  *reinterpret_cast<uint32_t*>(dig + digit_offset(k, 2)) = d2;
-  constexpr int lanes_per_group = G / 4;  // 8, 16 or 32 consecutive lanes cover one group
-  const unsigned gmask = lanes_per_group == 32 ? 0xffffffffu
-                                               : ((1u << lanes_per_group) - 1u) << (lane & ~(lanes_per_group - 1));
-  const int s0 = __reduce_add_sync(gmask, __dp4a((int)d0, 0x01010101, 0));  // sums of the signed bytes
-  const int s1 = __reduce_add_sync(gmask, __dp4a((int)d1, 0x01010101, 0));
-  const int s2 = __reduce_add_sync(gmask, __dp4a((int)d2, 0x01010101, 0));
-  if ((lane & (lanes_per_group - 1)) == 0) {
+  store_digits(b, k, dig);
+  int s0, s1, s2;
+  group_digit_sums<G>(b, lane, s0, s1, s2);
+  if ((lane & (G / 4 - 1)) == 0) {
     sumw[(k / G) * 2 + 0] = (float)s0 + 256.f * (float)s1;
     sumw[(k / G) * 2 + 1] = 65536.f * (float)s2;
   }
-  if (lane == 0) inv[k0 >> 7] = __uint_as_float((unsigned)(127 - e) << 23);
+  if (lane == 0) inv[k0 >> 7] = b.inv;
 }
 
 // ---- schedule enumeration (identical in every role) ----------------------------------------------------
@@ -1516,6 +1412,37 @@ static int run_layer(const slicemoe_shape* shape, const slicemoe_expert* experts
   p.ids = nullptr;
   p.prec = nullptr;
   p.weights = nullptr;
+  // A small batch: every expert is streamed once for all of a pass' tokens.  (A workspace of the batch-1 kernel's size, as
+  // slicemoe_layer_static's, has no room for that: token after token then.)
+  const size_t batch_bytes = batch_workspace_bytes(shape, n_shared);
+  if (T >= kBatchMinTokens && workspace_bytes >= kWsBatchOff + batch_bytes + kWsListBytes) {
+    uint8_t* bws = reinterpret_cast<uint8_t*>(workspace) + kWsBatchOff;
+    uint8_t* lists = bws + batch_bytes;
+    const BatchControl ctl = {&p.ws->status, &p.ws->extra_arrivals, &p.ws->wait_cycles};
+    const int passes = (T + kBatchTokens - 1) / kBatchTokens, k = shape->top_k;
+    for (int i = 0; i < passes; ++i) {
+      const int t0 = (int)((long long)T * i / passes), n = (int)((long long)T * (i + 1) / passes) - t0;
+      const size_t o = (size_t)t0 * k;
+      const int32_t* pids = ids ? ids + o : nullptr;
+      const uint8_t* pprec = prec ? prec + o : nullptr;
+      const float* pw = weights ? weights + o : nullptr;
+      if (fused) {
+        int32_t* ri = fused->ids_out ? fused->ids_out + o : reinterpret_cast<int32_t*>(lists);
+        float* rw = fused->weights_out ? fused->weights_out + o : reinterpret_cast<float*>(lists) + kWsListEntries;
+        uint8_t* rp = fused->prec_out ? fused->prec_out + o : lists + 8 * kWsListEntries;
+        rc = slicemoe_route_topk(fused->logits + (size_t)t0 * shape->n_experts, n, shape->n_experts, k, fused->bias, fused->renorm, fused->tau,
+                                 fused->rank_high, ri, rw, rp, stream);
+        if (rc != SLICEMOE_OK) return rc;
+        pids = ri;
+        pprec = rp;
+        pw = rw;
+      }
+      rc = batch_layer(shape, experts, shared, n_shared, gate_vec, reinterpret_cast<const uint16_t*>(x) + (size_t)t0 * shape->hidden, n, pids,
+                       pprec, pw, y + (size_t)t0 * shape->hidden, bws, ctl, sms, stream);
+      if (rc != SLICEMOE_OK) return rc;
+    }
+    return SLICEMOE_OK;
+  }
   for (int t = 0; t < T; ++t) {
     p.x = reinterpret_cast<const uint16_t*>(x) + (size_t)t * shape->hidden;
     if (fused) {
@@ -1564,8 +1491,10 @@ extern "C" int slicemoe_trace_read(long long* out_host, int max_ctas, int* slots
 }
 
 extern "C" size_t slicemoe_workspace_bytes(const slicemoe_shape* shape) {
-  (void)shape;
-  return kWsBytes;
+  if (check_shape(shape) != SLICEMOE_OK) return kWsBytes;
+  const long long hsum = (long long)shape->top_k * shape->inter + (long long)shape->n_shared * shape->shared_inter;
+  if (hsum > kHCap) return kWsBytes;
+  return kWsBatchOff + batch_workspace_bytes(shape, shape->n_shared) + kWsListBytes;
 }
 
 extern "C" int slicemoe_workspace_init(void* workspace, size_t workspace_bytes, void* stream) {
