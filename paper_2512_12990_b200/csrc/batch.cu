@@ -13,11 +13,11 @@
 // Four groups of a producer warp and four consumer warps each take the share's row blocks in turn: the producer
 // streams the planes, scales and zero-points through the group's own ring with bulk copies, never waiting for anything but
 // space; the consumers split a row block's 128-column blocks.  The arithmetic is the batch-1 kernel's: activations
-// as 23-bit fixed point per 128-element block in three base-256 digits (int8), integer MMAs on the raw nibbles,
-// scale and zero-point once per group.  Column n of the MMA's B operand is token n, one MMA per digit: a lane ends up
-// with all digits of its two tokens, so the digits are put together in its registers and a row block's result is two
-// values per lane, row half and matrix.  A pair at MSB precision shares the run with pairs at both slices: its columns
-// leave out the LSB sums and the zero-point's low bits.
+// as 23-bit fixed point per 128-element block in three base-256 digits (int8), integer MMAs on the codes or nibbles,
+// scale and zero-point once per group.  With column n of the MMA's B operand for token n and one MMA per digit, a lane ends
+// up with all digits of its two tokens, so the digits are put together in its registers and a row block's result is two
+// values per lane, row half and matrix; up to two tokens take one MMA for all their digits.  A pair at MSB precision shares
+// the run with pairs at both slices: its columns leave out the LSB sums and the zero-point's low bits.
 //
 // Bound: HBM.  Per 16 x 128 block of both planes (2 KB, 89 cycles of an SM's share of the bandwidth) a warp issues about 125
 // instructions, 24 of them MMAs (53 cycles of the integer tensor pipe).
@@ -27,6 +27,8 @@
 // waits for data, the consumers walk through the rest of their work and the producers stop and wait for their copies.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "batch.cuh"
 #include "common.cuh"
@@ -40,26 +42,24 @@ constexpr int kBThreads = 32 * (kBConsumers + kBGroups);
 constexpr int kBChunkK = 2048;           // columns of a down projection's task; wider experts are several
 constexpr int kBPlane = 8192;            // plane bytes of a stage: 4 blocks of both slices or 8 of the MSB slice
 constexpr int kBMaxSegs = 40;            // runs that a CTA's share can touch
-constexpr int kBFixedCost = 4;           // a row block's cost besides its plane blocks, in plane blocks
 constexpr int kBPlanThreads = 256;
 static_assert(kBatchTokens * SLICEMOE_MAX_TOP_K <= kBPlanThreads, "a thread per pair");
 
-struct __align__(16) BRun {
-  int expert;          // routed: 0 .., shared: n_experts ..
-  int n;
-  unsigned high;       // bit per pair: both slices
-  int inter;
-  int hoff;            // first h of the run: [n][inter]
-  int pad_;
+// The row blocks of a run - up to eight pairs of one expert - in one projection (down: for one chunk of columns).
+struct __align__(16) BSeg {
+  unsigned start, ucost;     // cost of the segments before, cost of a row block
+  int units;                 // row blocks
+  int n;                     // pairs
+  const uint8_t* ptr[2][4];  // [gate, up / down][MSB, LSB, scales, zero-points]
+  unsigned high;             // bit per pair: both slices
+  int lsb;                   // some pair uses both slices
+  int inter, hoff;           // the run's h: [n][inter] from hoff on
+  int yrow;                  // down: first result row
+  int kb0, nkb, row_kb;      // first 128-column block, their number, blocks of a whole row
   uint8_t tok[kBRun];
-};
-struct __align__(16) BSeg {  // the row blocks of a run in one projection (down: for one chunk of columns)
-  int run, kc;
-  unsigned start, ucost;     // cost before the segment, cost of a row block
-  int units;
-  int yrow;                  // down: first result row of the segment
   int pad_[2];
 };
+static_assert(sizeof(BSeg) == 128, "a lane per word copies a segment");
 struct BHead {
   int nseg[2];
   unsigned total[2];
@@ -67,8 +67,8 @@ struct BHead {
 };
 
 struct BLayout {
-  size_t head, runs, seg1, seg2, pos, gate, h, yrow, total;
-  int kc_r, kc_s, max_runs, max_seg2;
+  size_t head, seg1, seg2, pos, gate, xdig, xsum, xinv, h, yrow, total;
+  int kc_r, kc_s;
 };
 static inline BLayout batch_layout(const slicemoe_shape* s, int n_shared) {
   BLayout L;
@@ -76,16 +76,16 @@ static inline BLayout batch_layout(const slicemoe_shape* s, int n_shared) {
   const int sint = n_shared ? s->shared_inter : 0;
   L.kc_r = (s->inter + kBChunkK - 1) / kBChunkK;
   L.kc_s = (sint + kBChunkK - 1) / kBChunkK;
-  L.max_runs = T * k + n_shared * parts;
-  L.max_seg2 = T * k * L.kc_r + n_shared * parts * L.kc_s;
   auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
   size_t o = 0;
   L.head = o; o = align(o + sizeof(BHead));
-  L.runs = o; o = align(o + sizeof(BRun) * L.max_runs);
-  L.seg1 = o; o = align(o + sizeof(BSeg) * L.max_runs);
-  L.seg2 = o; o = align(o + sizeof(BSeg) * L.max_seg2);
+  L.seg1 = o; o = align(o + sizeof(BSeg) * (size_t)(T * k + n_shared * parts));
+  L.seg2 = o; o = align(o + sizeof(BSeg) * (size_t)(T * k * L.kc_r + n_shared * parts * L.kc_s));
   L.pos = o;  o = align(o + sizeof(int2) * T * (k + n_shared));
   L.gate = o; o = align(o + sizeof(float) * T);
+  L.xdig = o; o = align(o + (size_t)T * 3 * s->hidden);
+  L.xsum = o; o = align(o + sizeof(float) * (size_t)T * 2 * (s->hidden / s->group));
+  L.xinv = o; o = align(o + sizeof(float) * (size_t)T * (s->hidden / 128));
   L.h = o;    o = align(o + sizeof(float) * (size_t)T * ((size_t)k * s->inter + (size_t)n_shared * sint));
   L.yrow = o; o = align(o + sizeof(float) * (size_t)T * ((size_t)k * L.kc_r + (size_t)n_shared * L.kc_s) * s->hidden);
   L.total = o;
@@ -103,57 +103,94 @@ struct BPlanParams {
   const uint16_t* x;
   const float* gate_vec;  // or null
   int T, k, n_experts, n_shared, hidden, inter, shared_inter, kc_r, kc_s;
+  const slicemoe_expert* experts;
+  const slicemoe_expert* shared;
   BHead* head;
-  BRun* runs;
   BSeg *seg1, *seg2;
   int2* pos;
   float* gate;
+  uint8_t* xdig;          // digits of x: [T][3 hidden]
+  float *xsum, *xinv;     // their group sums [T][hidden / G][2], block scales [T][hidden / 128]
   BatchControl ctl;
 };
-__device__ __forceinline__ unsigned b_cost1(int planes, int hidden) { return 2u * planes * (hidden >> 7) + kBFixedCost; }
+// What a 16 x 128 block of a run costs a CTA: the bytes it brings (an MSB tile 2, both slices 4) and its instructions - by
+// measurement about half as much again for up to two pairs, the same for more, twice that where pairs of either precision
+// meet.  (By bytes alone, CTAs with both-slice runs were done in 21,000 cycles and those with MSB runs in 34,000.)
+__device__ __forceinline__ unsigned b_block_cost(int n, unsigned high) {
+  const unsigned all = (1u << n) - 1u, compute = (n <= 2 ? 1u : 2u) << (high != 0u && (high & all) != all ? 1 : 0);
+  return (high ? 4u : 2u) + compute;
+}
+constexpr unsigned kBFixedCost = 12;  // a row block's own: hand-shakes and the exchange between the four warps
 __device__ __forceinline__ int b_chunk_cols(int inter, int kc) { return min(kBChunkK, inter - kc * kBChunkK); }
-__device__ __forceinline__ unsigned b_cost2(int planes, int cols) { return planes * (cols >> 7) + kBFixedCost; }
-// Block-wide exclusive scan; *total gets the sum.
-__device__ unsigned b_scan(unsigned v, unsigned* sums, unsigned* total) {
+// Block-wide exclusive scans of four values, in place; `total` gets the sums.
+__device__ void b_scan(unsigned (&v)[4], unsigned (*sums)[kBPlanThreads / 32], unsigned (&total)[4]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned inc = v;
+  unsigned inc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) inc[i] = v[i];
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
-    const unsigned a = __shfl_up_sync(0xffffffffu, inc, off);
-    if (lane >= off) inc += a;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const unsigned a = __shfl_up_sync(0xffffffffu, inc[i], off);
+      if (lane >= off) inc[i] += a;
+    }
+  }
+  if (lane == 31) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sums[i][warp] = inc[i];
   }
   __syncthreads();
-  if (lane == 31) sums[warp] = inc;
-  __syncthreads();
-  const unsigned w = lane < kBPlanThreads / 32 ? sums[lane] : 0u;
-  *total = __reduce_add_sync(0xffffffffu, w);
-  return __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + inc - v;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const unsigned w = lane < kBPlanThreads / 32 ? sums[i][lane] : 0u;
+    total[i] = __reduce_add_sync(0xffffffffu, w);
+    v[i] = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + inc[i] - v[i];
+  }
 }
-// Block 0 plans; block 1 + t, with gated shared experts, works out token t's gate.
+// Block 0 plans; block 1 + t turns token t's x into digits and, with gated shared experts, works out its gate.
+template <int G>
 __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanParams p) {
   __shared__ int s_e[kBPlanThreads];
-  __shared__ unsigned s_high[kBPlanThreads], s_index[kBPlanThreads], s_prefix[kBPlanThreads], s_sums[32];
+  __shared__ unsigned s_high[kBPlanThreads], s_index[kBPlanThreads], s_prefix[kBPlanThreads], s_sums[4][kBPlanThreads / 32];
   __shared__ uint8_t s_tok[kBPlanThreads][kBRun];
   const int tid = threadIdx.x, lane = tid & 31;
   b_dep_launch();
   b_dep_wait();
-  if (blockIdx.x > 0) {  // sigmoid(gate_vec . x[t])
-    const int t = blockIdx.x - 1;
+  if (blockIdx.x > 0) {
+    const int t = blockIdx.x - 1, nkb = p.hidden >> 7;
+    const uint16_t* x = p.x + (size_t)t * p.hidden;
     float dot = 0.f;
-    for (int i = tid; i < p.hidden / 2; i += kBPlanThreads) {
-      const uint32_t raw = *reinterpret_cast<const uint32_t*>(p.x + (size_t)t * p.hidden + 2 * i);
-      dot = fmaf(p.gate_vec[2 * i], __uint_as_float(raw << 16), dot);
-      dot = fmaf(p.gate_vec[2 * i + 1], __uint_as_float(raw & 0xffff0000u), dot);
-    }
+    for (int b = tid >> 5; b < nkb; b += kBPlanThreads / 32) {
+      const uint2 raw = *reinterpret_cast<const uint2*>(x + b * 128 + 4 * lane);
+      const float v[4] = {__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u), __uint_as_float(raw.y << 16),
+                          __uint_as_float(raw.y & 0xffff0000u)};
+      if (p.gate_vec) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    float* part = reinterpret_cast<float*>(s_sums);
-    if (lane == 0) part[tid >> 5] = dot;
-    __syncthreads();
-    if (tid == 0) {
-      float sum = 0.f;
-      for (int w = 0; w < kBPlanThreads / 32; ++w) sum += part[w];
-      p.gate[t] = 1.f / (1.f + expf(-sum));
+        for (int j = 0; j < 4; ++j) dot = fmaf(p.gate_vec[b * 128 + 4 * lane + j], v[j], dot);
+      }
+      const BlockDigits d = block_digits(v);
+      store_digits(d, b * 128 + 4 * lane, p.xdig + (size_t)t * 3 * p.hidden);
+      int s0, s1, s2;
+      group_digit_sums<G>(d, lane, s0, s1, s2);
+      if ((lane & (G / 4 - 1)) == 0) {
+        float* sum = p.xsum + ((size_t)t * (p.hidden / G) + b * (128 / G) + lane / (G / 4)) * 2;
+        sum[0] = fmaf(256.f, (float)s1, (float)s0);
+        sum[1] = 65536.f * (float)s2;
+      }
+      if (lane == 0) p.xinv[t * nkb + b] = d.inv;
+    }
+    if (p.gate_vec) {  // sigmoid(gate_vec . x[t])
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+      float* part = reinterpret_cast<float*>(s_sums[0]);
+      if (lane == 0) part[tid >> 5] = dot;
+      __syncthreads();
+      if (tid == 0) {
+        float sum = 0.f;
+        for (int w = 0; w < kBPlanThreads / 32; ++w) sum += part[w];
+        p.gate[t] = 1.f / (1.f + expf(-sum));
+      }
     }
     return;
   }
@@ -171,6 +208,25 @@ __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanPa
   }
   s_e[tid] = e;
   s_high[tid] = 0u;
+  // the expert's planes (the shared experts' for the threads that list those): asked for now, used at the end
+  const int parts = (p.T + kBRun - 1) / kBRun, n_sh = p.n_shared * parts;
+  // (the shared experts are listed by the last threads, which have a pair of their own only in the largest batches)
+  const int sid = tid - (kBPlanThreads - n_sh);
+  const slicemoe_expert* ex = e >= 0 ? p.experts + e : nullptr;
+  const slicemoe_expert* exs = sid >= 0 ? p.shared + sid / parts : nullptr;
+  const uint8_t* planes[3][4];
+  auto fetch = [&](const slicemoe_expert* x) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const slicemoe_mat& mat = m == 0 ? x->gate : m == 1 ? x->up : x->down;
+      planes[m][0] = reinterpret_cast<const uint8_t*>(mat.msb);
+      planes[m][1] = reinterpret_cast<const uint8_t*>(mat.lsb);
+      planes[m][2] = reinterpret_cast<const uint8_t*>(mat.scale);
+      planes[m][3] = mat.zp;
+    }
+  };
+  if (ex) fetch(ex);
+  else if (exs) fetch(exs);
   __syncthreads();
   int rank = 0, count = 0, first = tid;
   for (int j = 0; j < npairs; ++j) {
@@ -196,44 +252,55 @@ __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanPa
   __syncthreads();
   const bool lead = valid && leader == tid;
   const int n = lead ? min(kBRun, count - rank) : 0;
-  const int planes = lead && s_high[tid] ? 2 : 1;
-  const unsigned u1 = b_cost1(planes, p.hidden);
+  const unsigned bc = lead ? b_block_cost(n, s_high[tid]) : 0u;
+  const unsigned u1 = 2u * bc * (p.hidden >> 7) + kBFixedCost;
   unsigned c2 = 0;
-  if (lead)
-    for (int kc = 0; kc < p.kc_r; ++kc) c2 += b_cost2(planes, b_chunk_cols(p.inter, kc)) * (p.hidden / 16);
-  unsigned n_runs, n_pairs, t1, t2;
-  const unsigned index = b_scan(lead ? 1u : 0u, s_sums, &n_runs);
-  const unsigned prefix = b_scan((unsigned)n, s_sums, &n_pairs);
-  const unsigned start1 = b_scan(lead ? u1 * (p.inter / 16) : 0u, s_sums, &t1);
-  unsigned start2 = b_scan(c2, s_sums, &t2);
-  if (lead) {
-    BRun r;
-    r.expert = e;
-    r.n = n;
-    r.high = s_high[tid];
-    r.inter = p.inter;
-    r.hoff = (int)prefix * p.inter;
-    r.pad_ = 0;
-    for (int i = 0; i < kBRun; ++i) r.tok[i] = i < n ? s_tok[tid][i] : s_tok[tid][0];
-    p.runs[index] = r;
-    BSeg g;
+  if (lead) c2 = (bc * (p.inter >> 7) + kBFixedCost * p.kc_r) * (p.hidden / 16);
+  unsigned sc[4] = {lead ? 1u : 0u, (unsigned)n, lead ? u1 * (p.inter / 16) : 0u, c2}, tot[4];
+  b_scan(sc, s_sums, tot);
+  const unsigned index = sc[0], prefix = sc[1], start1 = sc[2], start2 = sc[3], n_runs = tot[0], t1 = tot[2], t2 = tot[3];
+  // a run's segments: one for gate and up, one for each chunk of down's columns
+  auto emit = [&](BSeg g, unsigned block_cost, unsigned st1, unsigned st2, BSeg* to1, BSeg* to2, int kc_n, int yrow) {
+    g.lsb = g.high != 0u;
     g.pad_[0] = g.pad_[1] = 0;
-    g.run = (int)index;
-    g.kc = 0;
-    g.start = start1;
-    g.ucost = u1;
-    g.units = p.inter / 16;
+    auto point = [&](int to, int m) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) g.ptr[to][i] = planes[m][i];
+      if (g.lsb && !g.ptr[to][1]) {  // both slices asked of an expert without LSB planes: defined garbage, reported
+        g.ptr[to][1] = g.ptr[to][0];
+        atomicOr(p.ctl.status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
+      }
+    };
+    point(0, 0);
+    point(1, 1);
+    g.start = st1;
+    g.ucost = 2u * block_cost * (p.hidden >> 7) + kBFixedCost;
+    g.units = g.inter / 16;
     g.yrow = 0;
-    p.seg1[index] = g;
+    g.kb0 = 0;
+    g.nkb = g.row_kb = p.hidden >> 7;
+    *to1 = g;
+    point(0, 2);
+    g.row_kb = g.inter >> 7;
     g.units = p.hidden / 16;
-    for (int kc = 0; kc < p.kc_r; ++kc) {
-      g.kc = kc;
-      g.start = start2;
-      g.ucost = b_cost2(planes, b_chunk_cols(p.inter, kc));
-      g.yrow = (int)prefix * p.kc_r + kc * n;
-      p.seg2[index * p.kc_r + kc] = g;
-      start2 += g.ucost * (p.hidden / 16);
+    for (int kc = 0; kc < kc_n; ++kc) {
+      g.kb0 = kc * (kBChunkK / 128);
+      g.nkb = b_chunk_cols(g.inter, kc) >> 7;
+      g.start = st2;
+      g.ucost = block_cost * g.nkb + kBFixedCost;
+      g.yrow = yrow + kc * g.n;
+      to2[kc] = g;
+      st2 += g.ucost * (p.hidden / 16);
     }
+  };
+  if (lead) {
+    BSeg g;
+    g.n = n;
+    g.high = s_high[tid];
+    g.inter = p.inter;
+    g.hoff = (int)prefix * p.inter;
+    for (int i = 0; i < kBRun; ++i) g.tok[i] = i < n ? s_tok[tid][i] : s_tok[tid][0];
+    emit(g, bc, start1, start2, p.seg1 + index, p.seg2 + index * p.kc_r, p.kc_r, (int)prefix * p.kc_r);
     s_index[tid] = (unsigned)n;
     s_prefix[tid] = prefix;
   }
@@ -242,43 +309,21 @@ __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanPa
     p.pos[(tid / p.k) * slots + tid % p.k] =
         valid ? make_int2((int)s_prefix[leader] * p.kc_r + (rank & (kBRun - 1)), (int)s_index[leader]) : make_int2(-1, 0);
   // shared experts: all tokens, both slices
-  const int parts = (p.T + kBRun - 1) / kBRun;
-  const unsigned us1 = b_cost1(2, p.hidden);
-  unsigned cs2 = 0;
-  for (int kc = 0; kc < p.kc_s; ++kc) cs2 += b_cost2(2, b_chunk_cols(p.shared_inter, kc)) * (p.hidden / 16);
-  const int n_sh = p.n_shared * parts;
-  if (tid < n_sh) {
-    const int j = tid / parts, part = tid % parts, t0 = part * kBRun, ns = min(kBRun, p.T - t0);
+  const unsigned bs = b_block_cost(min(p.T, kBRun), 0xffu);
+  const unsigned cs1 = (2u * bs * (p.hidden >> 7) + kBFixedCost) * (p.shared_inter / 16);
+  const unsigned cs2 = (bs * (p.shared_inter >> 7) + kBFixedCost * p.kc_s) * (p.hidden / 16);
+  if (sid >= 0) {
+    const int j = sid / parts, t0 = sid % parts * kBRun, ns = min(kBRun, p.T - t0);
     const int before = j * p.T + t0;  // pairs of shared experts before this run
-    BRun r;
-    r.expert = p.n_experts + j;
-    r.n = ns;
-    r.high = 0xffu;
-    r.inter = p.shared_inter;
-    r.hoff = npairs * p.inter + before * p.shared_inter;
-    r.pad_ = 0;
-    for (int i = 0; i < kBRun; ++i) r.tok[i] = (uint8_t)(t0 + (i < ns ? i : 0));
-    const int idx = (int)n_runs + tid;
-    p.runs[idx] = r;
     BSeg g;
-    g.pad_[0] = g.pad_[1] = 0;
-    g.run = idx;
-    g.kc = 0;
-    g.start = t1 + (unsigned)tid * us1 * (p.shared_inter / 16);
-    g.ucost = us1;
-    g.units = p.shared_inter / 16;
-    g.yrow = 0;
-    p.seg1[idx] = g;
-    unsigned st = t2 + (unsigned)tid * cs2;
-    g.units = p.hidden / 16;
-    for (int kc = 0; kc < p.kc_s; ++kc) {
-      g.kc = kc;
-      g.start = st;
-      g.ucost = b_cost2(2, b_chunk_cols(p.shared_inter, kc));
-      g.yrow = npairs * p.kc_r + before * p.kc_s + kc * ns;
-      p.seg2[n_runs * p.kc_r + tid * p.kc_s + kc] = g;
-      st += g.ucost * (p.hidden / 16);
-    }
+    g.n = ns;
+    g.high = 0xffu;
+    g.inter = p.shared_inter;
+    g.hoff = npairs * p.inter + before * p.shared_inter;
+    for (int i = 0; i < kBRun; ++i) g.tok[i] = (uint8_t)(t0 + (i < ns ? i : 0));
+    if (ex) fetch(exs);
+    emit(g, bs, t1 + (unsigned)sid * cs1, t2 + (unsigned)sid * cs2, p.seg1 + n_runs + sid,
+         p.seg2 + n_runs * p.kc_r + sid * p.kc_s, p.kc_s, npairs * p.kc_r + before * p.kc_s);
   }
   for (int i = tid; i < p.T * p.n_shared; i += kBPlanThreads) {
     const int t = i / p.n_shared, j = i % p.n_shared, t0 = t / kBRun * kBRun, ns = min(kBRun, p.T - t0);
@@ -288,7 +333,7 @@ __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanPa
     BHead h;
     h.nseg[0] = off ? 0 : (int)n_runs + n_sh;
     h.nseg[1] = off ? 0 : (int)n_runs * p.kc_r + n_sh * p.kc_s;
-    h.total[0] = t1 + (unsigned)n_sh * us1 * (p.n_shared ? p.shared_inter / 16 : 0);
+    h.total[0] = t1 + (unsigned)n_sh * cs1;
     h.total[1] = t2 + (unsigned)n_sh * cs2;
     h.off = off ? 1 : 0;
     *p.head = h;
@@ -297,28 +342,17 @@ __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanPa
 }
 
 // ---- the projections --------------------------------------------------------------------------------------
-struct BShare {  // a part of a CTA's share: row blocks first .. last - 1 of a segment
-  const uint8_t* ptr[2][4];  // [gate, up / down][MSB, LSB, scales, zero-points]
-  int first, last;
-  int n;
-  unsigned high;
-  int inter, hoff, yrow;
-  int kb0, nkb, row_kb;      // first 128-column block, their number, blocks of a whole row
-  int lsb;                   // some pair uses both slices
-  uint8_t tok[kBRun];
-};
 struct BParams {
-  const slicemoe_expert* experts;
-  const slicemoe_expert* shared;
-  const uint16_t* x;
   const BHead* head;
-  const BRun* runs;
   const BSeg* segs;
+  const uint8_t* xdig;
+  const float *xsum, *xinv;
   float* h;
   float* yrow;
   BatchControl ctl;
-  int n_experts, hidden, K, shift;  // K: widest vector of digits (hidden, or a chunk of the intermediate width)
-  int stages;                       // per group
+  int hidden, K, shift;  // K: widest vector of digits (hidden, or a chunk of the intermediate width)
+  int stages;            // per group
+  int max_segs;          // entries the list can have
 };
 template <int G, int PHASE>
 struct BSmem {
@@ -326,18 +360,18 @@ struct BSmem {
   static constexpr int kStage = kBPlane + kMeta;
   static constexpr int kMats = PHASE == 1 ? 2 : 1;
   static constexpr int kPart = kBGroupWarps * kMats * kBRun * 20;  // floats: [warp][matrix][token][16 rows, padded]
-  static constexpr int shares = 0;
-  static constexpr int ctl = shares + kBMaxSegs * (int)sizeof(BShare);  // number of shares, dead flag, wait limit
+  static constexpr int shares = 0;                                    // segments of the share ...
+  static constexpr int range = shares + kBMaxSegs * (int)sizeof(BSeg);  // ... and their first and last row block of it
+  static constexpr int ctl = range + kBMaxSegs * 8;                   // first and last segment, dead flag
   static constexpr int bars = ctl + 32;
   static constexpr int kMaxStages = 8;
   static constexpr int part = (bars + 2 * kBGroups * kMaxStages * 8 + 127) & ~127;
   static constexpr int dig = part + kBGroups * 2 * kPart * 4;
   __host__ __device__ static int tok_stride(int K) { return 3 * K + 32; }  // eight tokens' digit rows spread over the banks
-  __host__ __device__ static int sums(int K) { return dig + kBRun * tok_stride(K); }            // float [K / G][8]
-  __host__ __device__ static int inv(int K) { return sums(K) + K / G * kBRun * 4; }             // float [K / 128][8]
+  __host__ __device__ static int sums(int K) { return dig + kBRun * tok_stride(K); }            // float [K / G][digits 0 and 1, digit 2][8]
+  __host__ __device__ static int inv(int K) { return sums(K) + 2 * (K / G) * kBRun * 4; }       // float [K / 128][8]
   __host__ __device__ static int ring(int K) { return (inv(K) + K / 128 * kBRun * 4 + 127) & ~127; }
 };
-static_assert(sizeof(BShare) % 8 == 0, "alignment");
 
 struct BWait {
   volatile int* dead;
@@ -361,70 +395,210 @@ struct BWait {
 };
 
 // One 16 x 128 block for eight tokens: acc[2 row half + token] += the block's contribution (lane (g, c): rows g and
-// g + 8, tokens 2 c and 2 c + 1).  As in the batch-1 kernel the A fragment of rows g + 8 is the bytes as they are, 16 x
-// their nibble plus row g's: the difference of the accumulator rows is 16 C[g + 8], and the row's scale is divided by 16.
-template <int G, bool LSB>
+// g + 8, tokens 2 c and 2 c + 1).
+//   kModeHigh   all pairs use both slices: the nibbles are put together into 8-bit codes first, one MMA per 32 columns and
+//               digit, and nothing to add up afterwards;
+//   kModeLow    none does: the MSB nibbles alone, worth 2^shift;
+//   kModeMixed  both products, and a pair's column takes the LSB product or not.
+// Where nibbles are used as they are (low, mixed) the A fragment of rows g + 8 is the raw bytes, 16 x their nibble plus row
+// g's: the difference of the accumulator rows is 16 C[g + 8], and the row's scale is divided by 16.
+// WIDE: column n of the B operand is token n, an MMA per digit.  Otherwise, for up to two tokens, columns 4 t .. 4 t + 2 are the
+// digits of token t, one MMA for all: even lanes c hold digits 0 and 1 of token c / 2, odd ones digit 2, acc[0] and
+// acc[1] are the row halves, and the caller adds lane pairs at the end.
+enum { kModeLow = 0, kModeMixed = 1, kModeHigh = 2 };
+template <int G, int MODE, bool WIDE>
 __device__ __forceinline__ void b_block(const uint8_t* msb, const uint8_t* lsb, const uint8_t* sc, const uint8_t* zp, const uint8_t* dig,
-                                        const float* X, const float* inv, int shift, unsigned low0, unsigned low1, float (&acc)[4]) {
+                                        const float* X, const float* inv, int shift, int odd, unsigned low0, unsigned low1,
+                                        float (&acc)[4]) {
   constexpr int SG = 128 / G, KS = G / 32;
   constexpr uint32_t kLow = 0x0f0f0f0fu;
-  uint32_t a[2][8];  // [plane][words of the lane: 16 columns each]
-  {
-    const uint4 v0 = *reinterpret_cast<const uint4*>(msb), v1 = *reinterpret_cast<const uint4*>(msb + 512);
-    a[0][0] = v0.x; a[0][1] = v0.y; a[0][2] = v0.z; a[0][3] = v0.w;
-    a[0][4] = v1.x; a[0][5] = v1.y; a[0][6] = v1.z; a[0][7] = v1.w;
-  }
-  if (LSB) {
-    const uint4 v0 = *reinterpret_cast<const uint4*>(lsb), v1 = *reinterpret_cast<const uint4*>(lsb + 512);
-    a[1][0] = v0.x; a[1][1] = v0.y; a[1][2] = v0.z; a[1][3] = v0.w;
-    a[1][4] = v1.x; a[1][5] = v1.y; a[1][6] = v1.z; a[1][7] = v1.w;
-  }
-  const float2 iv = *reinterpret_cast<const float2*>(inv);
+  float2 iv;
+  if (WIDE) iv = *reinterpret_cast<const float2*>(inv);
+  else iv.x = *inv;
+  constexpr int ND = WIDE ? 3 : 1;
 #pragma unroll
   for (int sg = 0; sg < SG; ++sg) {
-    float t[4];
+    // the group's words of the lane, 16 columns each: [plane], or [row half] of the codes
+    constexpr int W = G / 16;
+    uint32_t a[2][W];
+    if (W == 2) {  // half of a 64-column tile
+      const uint2 v = *reinterpret_cast<const uint2*>(msb + (sg >> 1) * 512 + (sg & 1) * 8);
+      a[0][0] = v.x; a[0][1] = v.y;
+      if (MODE != kModeLow) {
+        const uint2 u = *reinterpret_cast<const uint2*>(lsb + (sg >> 1) * 512 + (sg & 1) * 8);
+        a[1][0] = u.x; a[1][1] = u.y;
+      }
+    } else {
 #pragma unroll
-    for (int d = 2; d >= 0; --d) {
+      for (int h = 0; h < W / 4; ++h) {
+        const uint4 v = *reinterpret_cast<const uint4*>(msb + (sg * (W / 4) + h) * 512);
+        a[0][(4 * h) % W] = v.x; a[0][(4 * h + 1) % W] = v.y; a[0][(4 * h + 2) % W] = v.z; a[0][(4 * h + 3) % W] = v.w;
+        if (MODE != kModeLow) {
+          const uint4 u = *reinterpret_cast<const uint4*>(lsb + (sg * (W / 4) + h) * 512);
+          a[1][(4 * h) % W] = u.x; a[1][(4 * h + 1) % W] = u.y; a[1][(4 * h + 2) % W] = u.z; a[1][(4 * h + 3) % W] = u.w;
+        }
+      }
+    }
+    if (MODE == kModeHigh) {
+      // a slice narrower than four bits leaves the top of its nibble zero, so what the masks let through beyond it is zero
+      const uint32_t mask = kLow << shift;
+      const int back = 4 - shift;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const uint32_t m = a[0][w], l = a[1][w];
+        a[0][w] = ((m << shift) & mask) | (l & ~mask);
+        a[1][w] = ((m >> back) & mask) | ((l >> 4) & ~mask);
+      }
+    }
+    int v[ND][4];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
       int m[4], l[4];
 #pragma unroll
       for (int s = 0; s < KS; ++s) {
         const int ks = sg * KS + s;
         const uint2 b = *reinterpret_cast<const uint2*>(dig + ks * 96 + d * 32);
-        const uint32_t w0 = a[0][2 * ks], w1 = a[0][2 * ks + 1];
-        if (s == 0) mma_u8s8_first(m, w0 & kLow, w0, w1 & kLow, w1, b.x, b.y);
-        else mma_u8s8(m, w0 & kLow, w0, w1 & kLow, w1, b.x, b.y);
-        if (LSB) {
-          const uint32_t u0 = a[1][2 * ks], u1 = a[1][2 * ks + 1];
-          if (s == 0) mma_u8s8_first(l, u0 & kLow, u0, u1 & kLow, u1, b.x, b.y);
-          else mma_u8s8(l, u0 & kLow, u0, u1 & kLow, u1, b.x, b.y);
+        const uint32_t w0 = a[0][2 * s], w1 = a[0][2 * s + 1], u0 = a[1][2 * s], u1 = a[1][2 * s + 1];
+        if (MODE == kModeHigh) {
+          if (s == 0) mma_u8s8_first(m, w0, u0, w1, u1, b.x, b.y);
+          else mma_u8s8(m, w0, u0, w1, u1, b.x, b.y);
+        } else {
+          if (s == 0) mma_u8s8_first(m, w0 & kLow, w0, w1 & kLow, w1, b.x, b.y);
+          else mma_u8s8(m, w0 & kLow, w0, w1 & kLow, w1, b.x, b.y);
+          if (MODE == kModeMixed) {
+            if (s == 0) mma_u8s8_first(l, u0 & kLow, u0, u1 & kLow, u1, b.x, b.y);
+            else mma_u8s8(l, u0 & kLow, u0, u1 & kLow, u1, b.x, b.y);
+          }
         }
       }
-      m[2] -= m[0];
-      m[3] -= m[1];
-      if (LSB) {
+      if (MODE != kModeHigh) {
+        m[2] -= m[0];
+        m[3] -= m[1];
+      }
+      if (MODE == kModeMixed) {
         l[2] -= l[0];
         l[3] -= l[1];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m[i] = (m[i] << shift) + (l[i] & ((i & 1) ? ~low1 : ~low0));
       }
 #pragma unroll
+      for (int i = 0; i < 4; ++i) v[d][i] = m[i];
+    }
+    float s0 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32)), s1 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32 + 16));
+    unsigned z0 = zp[sg * 16], z1 = zp[sg * 16 + 8];
+    if (MODE == kModeLow) {  // 2^shift (q_msb - (zp >> shift)): the power of two goes into the scale
+      const float two = (float)(1 << shift);
+      z0 >>= shift;
+      z1 >>= shift;
+      s0 *= two;
+      s1 *= two;
+    }
+    if (MODE != kModeHigh) {
+      s1 *= 0.0625f;
+      z1 <<= 4;
+    }
+    // a pair at MSB precision among others at both slices: 2^shift (zp >> shift)
+    const unsigned drop = (1u << shift) - 1u;
+    // Digits 0 and 1 go together in 32 bits: 255 x 128 x 128 x 257 at most.  Not so in the rows of a mixed run that carry a factor
+    // of 16.  Digit 2 joins in fp32.
+    if (WIDE) {
+      const float2 xl = *reinterpret_cast<const float2*>(X + sg * 2 * kBRun), xh = *reinterpret_cast<const float2*>(X + sg * 2 * kBRun + kBRun);
+      const float x0 = xl.x + xh.x, x1 = xl.y + xh.y;
+#pragma unroll
       for (int i = 0; i < 4; ++i) {
-        int v = m[i] << shift;
-        if (LSB) v += l[i] & ((i & 1) ? ~low1 : ~low0);
-        t[i] = d == 2 ? (float)v : fmaf(t[i], 256.f, (float)v);
+        const bool mixed16 = MODE == kModeMixed && i >= 2;
+        float t = mixed16 ? fmaf((float)v[ND - 1][i], 65536.f, fmaf((float)v[ND / 2][i], 256.f, (float)v[0][i]))
+                          : fmaf((float)v[ND - 1][i], 65536.f, (float)(v[0][i] + v[ND / 2][i] * 256));
+        unsigned z = i >= 2 ? z1 : z0;
+        if (MODE == kModeMixed) z &= ~(((i & 1) ? low1 : low0) & (i >= 2 ? drop << 4 : drop));
+        t = fmaf(-(float)z, (i & 1) ? x1 : x0, t);
+        acc[i] = fmaf((i >= 2 ? s1 : s0) * ((i & 1) ? iv.y : iv.x), t, acc[i]);
+      }
+    } else {
+      const float x = X[sg * 2 * kBRun];  // the lane's digits'
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const bool mixed16 = MODE == kModeMixed && r == 1;
+        float t;
+        if (mixed16) t = odd ? (float)v[0][2] * 65536.f : fmaf((float)v[0][3], 256.f, (float)v[0][2]);
+        else t = (float)(odd ? v[0][2 * r] : v[0][2 * r] + v[0][2 * r + 1] * 256) * (odd ? 65536.f : 1.f);
+        unsigned z = r ? z1 : z0;
+        if (MODE == kModeMixed) z &= ~(low0 & (r ? drop << 4 : drop));
+        t = fmaf(-(float)z, x, t);
+        acc[r] = fmaf((r ? s1 : s0) * iv.x, t, acc[r]);
       }
     }
-    const float2 xs = *reinterpret_cast<const float2*>(X + sg * kBRun);
-    const float s0 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32));
-    const float s1 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32 + 16)) * 0.0625f;
-    const unsigned z0 = zp[sg * 16], z1 = zp[sg * 16 + 8];
-    // MSB slice alone: 2^shift (zp >> shift)
-    const unsigned drop = (1u << shift) - 1u;
-    const float za = (float)(z0 & ~(low0 & drop)), zb = (float)(z0 & ~(low1 & drop));
-    const float zc = (float)((z1 & ~(low0 & drop)) << 4), zd = (float)((z1 & ~(low1 & drop)) << 4);
-    acc[0] = fmaf(s0 * iv.x, fmaf(-za, xs.x, t[0]), acc[0]);
-    acc[1] = fmaf(s0 * iv.y, fmaf(-zb, xs.y, t[1]), acc[1]);
-    acc[2] = fmaf(s1 * iv.x, fmaf(-zc, xs.x, t[2]), acc[2]);
-    acc[3] = fmaf(s1 * iv.y, fmaf(-zd, xs.y, t[3]), acc[3]);
   }
+}
+
+// A consumer warp's part of a share's row blocks `u`, u + kBGroups, ... below `last`.
+struct BState {
+  int st, half;   // stage, buffer of partial rows
+  uint32_t par;   // parity of the stage's use
+};
+template <int G, int PHASE, int MODE, bool WIDE>
+__device__ __forceinline__ void b_rows(const BParams& p, const BSeg& sh, int u, int last, uint32_t fb, const uint8_t* ring, float* part,
+                                       const uint8_t* dig, const float* X, const float* inv, int stride, int group, int gw, int lane,
+                                       const BWait& wait, BState& state) {
+  using S = BSmem<G, PHASE>;
+  constexpr int SG = 128 / G;
+  constexpr int per = MODE == kModeLow ? 8 : 4;  // blocks of a stage
+  const int g8 = lane >> 2, c = lane & 3, n = sh.n, nkb = sh.nkb, shift = p.shift;
+  // the lane's tokens: 2 c and 2 c + 1, or c / 2
+  const int tk0 = WIDE ? 2 * c : c >> 1, tk1 = WIDE ? 2 * c + 1 : c >> 1;
+  const unsigned low0 = (sh.high >> tk0) & 1u ? 0u : 0xffffffffu, low1 = (sh.high >> tk1) & 1u ? 0u : 0xffffffffu;
+  // columns without a token repeat the last one's; the narrow form's fourth column repeats a digit
+  const uint8_t* my_dig = dig + c * 8 + (WIDE ? min(g8, n - 1) * stride : min(g8 >> 2, n - 1) * stride + min(g8 & 3, 2) * 32);
+  const float* my_X = X + (WIDE ? 2 * c : (c >> 1) + (c & 1) * kBRun);
+  const float* my_inv = inv + tk0;
+  int st = state.st, half = state.half;
+  uint32_t par = state.par;
+  for (; u < last; u += kBGroups) {
+    float* pb = part + half * S::kPart;
+#pragma unroll 1
+    for (int m = 0; m < S::kMats; ++m) {
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int b0 = 0; b0 < nkb; b0 += per) {
+        wait(fb + 16 * st, par);
+        const uint8_t* stage = ring + st * S::kStage;
+        const int nb = min(per, nkb - b0);
+#pragma unroll 1
+        for (int b = gw; b < nb; b += kBGroupWarps)
+          b_block<G, MODE, WIDE>(stage + b * 1024 + lane * 16, stage + kBPlane / 2 + b * 1024 + lane * 16, stage + kBPlane + b * (SG * 32) + g8 * 2,
+                                 stage + kBPlane + 8 * SG * 32 + b * (SG * 16) + g8, my_dig + (b0 + b) * 384, my_X + (b0 + b) * SG * 2 * kBRun,
+                                 my_inv + (b0 + b) * kBRun, shift, c & 1, low0, low1, acc);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(fb + 16 * st + 8);
+        if (++st == p.stages) { st = 0; par ^= 1; }
+      }
+      float* w = pb + (gw * S::kMats + m) * (kBRun * 20);
+      if (WIDE) {
+        w[(2 * c) * 20 + g8] = acc[0];
+        w[(2 * c + 1) * 20 + g8] = acc[1];
+        w[(2 * c) * 20 + g8 + 8] = acc[2];
+        w[(2 * c + 1) * 20 + g8 + 8] = acc[3];
+      } else {
+        const float a0 = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1), a1 = acc[1] + __shfl_xor_sync(0xffffffffu, acc[1], 1);
+        w[(c >> 1) * 20 + g8 + 8 * (c & 1)] = (c & 1) ? a1 : a0;
+      }
+    }
+    // the four warps' shares of the columns, added in warp order by a thread per (token, row); two buffers take turns
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + group), "n"(32 * kBGroupWarps) : "memory");
+    const int t = (gw * 32 + lane) >> 4, row = lane & 15;
+    if (t < n) {
+      float s[2] = {0.f, 0.f};
+#pragma unroll
+      for (int w = 0; w < kBGroupWarps; ++w)
+#pragma unroll
+        for (int m = 0; m < S::kMats; ++m) s[m] += pb[(w * S::kMats + m) * (kBRun * 20) + t * 20 + row];
+      if (PHASE == 1) p.h[sh.hoff + (size_t)t * sh.inter + u * 16 + row] = s[0] / (1.f + expf(-s[0])) * s[1];  // silu(gate) * up
+      else p.yrow[(size_t)(sh.yrow + t) * p.hidden + u * 16 + row] = s[0];
+    }
+    half ^= 1;
+  }
+  state.st = st;
+  state.half = half;
+  state.par = par;
 }
 
 template <int G, int PHASE>
@@ -433,11 +607,14 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
   constexpr int SG = 128 / G;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-  BShare* shares = reinterpret_cast<BShare*>(smem + S::shares);
-  int* n_shares = reinterpret_cast<int*>(smem + S::ctl);
-  volatile int* dead = n_shares + 1;
+  BSeg* shares = reinterpret_cast<BSeg*>(smem + S::shares);
+  int2* range = reinterpret_cast<int2*>(smem + S::range);
+  int* ctl = reinterpret_cast<int*>(smem + S::ctl);
+  volatile int* dead = ctl + 2;
   const uint32_t bars = smem_u32(smem + S::bars);
   if (tid == 0) {
+    ctl[0] = 0x7fffffff;
+    ctl[1] = -1;
     *dead = 0;
     for (int i = 0; i < kBGroups * p.stages; ++i) {
       mbar_init(bars + 16 * i, 1);                // full: the producer's arrive, and the bytes
@@ -446,6 +623,7 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  __syncthreads();
   // The gate/up launch waits for the plan before it lets the next launch start.  So the down launch, when it starts, finds the
   // plan complete: it looks up its share and streams its weights while gate/up is still running, and waits only for h.
   if (PHASE == 1) {
@@ -457,65 +635,31 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
   wait.dead = dead;
   wait.limit = lim != 0ull ? lim : kWaitCycles;
   wait.status = p.ctl.status;
-  if (warp == 0) {
-    // this CTA's share: the row blocks whose start, in cost, lies in its window
+  // This CTA's share: the row blocks whose start, in cost, lies in its window.  A thread per segment; everything a role needs
+  // to know about a segment is in its entry, so the way to the first copy is two trips to L2.
+  {
+    const uint4 head = tid < p.max_segs ? __ldcg(reinterpret_cast<const uint4*>(p.segs + tid)) : make_uint4(0u, 1u, 0u, 0u);
     const int nseg = __ldcg(&p.head->nseg[PHASE - 1]);
     const unsigned long long total = __ldcg(&p.head->total[PHASE - 1]);
     const unsigned lo = (unsigned)((total * blockIdx.x + gridDim.x - 1) / gridDim.x);
     const unsigned hi = (unsigned)((total * (blockIdx.x + 1) + gridDim.x - 1) / gridDim.x);
-    int count = 0;
-    for (int s0 = 0; s0 < nseg; s0 += 32) {
-      int first = 0, last = 0;
-      BSeg g{};
-      if (s0 + lane < nseg) {
-        const uint4* src = reinterpret_cast<const uint4*>(p.segs + s0 + lane);
-        reinterpret_cast<uint4*>(&g)[0] = __ldcg(src);
-        reinterpret_cast<uint4*>(&g)[1] = __ldcg(src + 1);
-        auto ord = [&](unsigned at) { return at <= g.start ? 0 : (int)min((unsigned)g.units, (at - g.start + g.ucost - 1) / g.ucost); };
-        first = ord(lo);
-        last = ord(hi);
-      }
-      const unsigned has = __ballot_sync(0xffffffffu, last > first);
-      const int at = count + __popc(has & ((1u << lane) - 1u));
-      if (last > first && at < kBMaxSegs) {
-        BRun r;
-        const uint4* src = reinterpret_cast<const uint4*>(p.runs + g.run);
-#pragma unroll
-        for (int i = 0; i < (int)(sizeof(BRun) / 16); ++i) reinterpret_cast<uint4*>(&r)[i] = __ldcg(src + i);
-        BShare& sh = shares[at];
-        const slicemoe_expert* ex = r.expert >= p.n_experts ? p.shared + (r.expert - p.n_experts) : p.experts + r.expert;
-        sh.lsb = r.high != 0u;
-#pragma unroll
-        for (int m = 0; m < S::kMats; ++m) {
-          const slicemoe_mat* mat = PHASE == 1 ? (m ? &ex->up : &ex->gate) : &ex->down;
-          sh.ptr[m][0] = reinterpret_cast<const uint8_t*>(mat->msb);
-          sh.ptr[m][1] = reinterpret_cast<const uint8_t*>(mat->lsb);
-          sh.ptr[m][2] = reinterpret_cast<const uint8_t*>(mat->scale);
-          sh.ptr[m][3] = mat->zp;
-          if (sh.lsb && !sh.ptr[m][1]) {  // both slices asked of an expert without LSB planes: defined garbage, reported
-            sh.ptr[m][1] = sh.ptr[m][0];
-            atomicOr(p.ctl.status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
-          }
-        }
-        sh.first = first;
-        sh.last = last;
-        sh.n = r.n;
-        sh.high = r.high;
-        sh.inter = r.inter;
-        sh.hoff = r.hoff;
-        sh.yrow = g.yrow;
-        sh.row_kb = (PHASE == 1 ? p.hidden : r.inter) >> 7;
-        sh.kb0 = PHASE == 1 ? 0 : g.kc * (kBChunkK / 128);
-        sh.nkb = PHASE == 1 ? sh.row_kb : b_chunk_cols(r.inter, g.kc) >> 7;
-#pragma unroll
-        for (int i = 0; i < kBRun; ++i) sh.tok[i] = r.tok[i];
-      }
-      count += __popc(has);
+    int2 r = make_int2(0, 0);
+    if (tid < nseg) {
+      auto ord = [&](unsigned at) { return at <= head.x ? 0 : (int)min(head.z, (at - head.x + head.y - 1) / head.y); };
+      r = make_int2(ord(lo), ord(hi));
     }
-    if (lane == 0) *n_shares = min(count, kBMaxSegs);
+    if (r.y > r.x) {
+      atomicMin(&ctl[0], tid);
+      atomicMax(&ctl[1], tid);
+    }
+    __syncthreads();
+    const int s0 = ctl[0], n = min(ctl[1] - s0 + 1, kBMaxSegs);
+    if (r.y > r.x && tid - s0 < kBMaxSegs) range[tid - s0] = r;
+    for (int i = warp; i < n; i += kBThreads / 32)
+      reinterpret_cast<uint32_t*>(shares + i)[lane] = __ldcg(reinterpret_cast<const uint32_t*>(p.segs + s0 + i) + lane);
+    __syncthreads();
   }
-  __syncthreads();
-  const int ns = *n_shares;
+  const int ns = ctl[1] < 0 ? 0 : min(ctl[1] - ctl[0] + 1, kBMaxSegs);
   uint8_t* ring0 = smem + S::ring(p.K);
 
   if (warp >= kBConsumers) {
@@ -530,12 +674,13 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
     uint32_t par = 1, used = 0;
     bool ok = true;
     for (int i = 0; i < ns && ok; ++i) {
-      const BShare& sh = shares[i];
+      const BSeg& sh = shares[i];
+      const int u0 = range[i].x, u1 = range[i].y;
       const int nkb = sh.nkb, per = sh.lsb ? 4 : 8;
       const bool active = lane != 1 || sh.lsb;
       const unsigned dst0 = lane == 0 ? 0u : lane == 1 ? kBPlane / 2 : lane == 2 ? kBPlane : kBPlane + 8 * SG * 32;
       // the group's row blocks: every kBGroups-th of the share
-      for (int u = sh.first + ((group - ord) & (kBGroups - 1)); u < sh.last && ok; u += kBGroups) {
+      for (int u = u0 + ((group - ord) & (kBGroups - 1)); u < u1 && ok; u += kBGroups) {
 #pragma unroll 1
         for (int m = 0; m < S::kMats && ok; ++m) {
           const uint8_t* src = sh.ptr[m][lane] + ((size_t)u * sh.row_kb + sh.kb0) * per_block;
@@ -551,7 +696,7 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
           }
         }
       }
-      ord += sh.last - sh.first;
+      ord += u1 - u0;
     }
     // no copy may be on its way when the CTA ends (in the normal case the consumers have seen them all land)
     for (uint32_t i = used > (uint32_t)p.stages ? used - p.stages : 0; i < used; ++i) {
@@ -562,7 +707,7 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
   }
 
   // ---- consumers ----
-  const int group = warp / kBGroupWarps, gw = warp % kBGroupWarps, g8 = lane >> 2, c = lane & 3;
+  const int group = warp / kBGroupWarps, gw = warp % kBGroupWarps;
   const uint32_t fb = bars + 16 * group * p.stages;
   const uint8_t* ring = ring0 + (size_t)group * p.stages * S::kStage;
   float* part = reinterpret_cast<float*>(smem + S::part) + group * 2 * S::kPart;
@@ -574,82 +719,79 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
     b_dep_wait();  // h
     b_dep_launch();
   }
-  int st = 0, ord = 0, half = 0;
-  uint32_t par = 0;
+  BState state = {0, 0, 0u};
+  int ord = 0;
   for (int i = 0; i < ns; ++i) {
-    const BShare& sh = shares[i];
-    const int n = sh.n, nkb = sh.nkb;
+    const BSeg& sh = shares[i];
+    const int u0 = range[i].x, u1 = range[i].y, n = sh.n, nkb = sh.nkb;
     if (i > 0) asm volatile("bar.sync 1, %0;" ::"n"(32 * kBConsumers) : "memory");  // the digits of the run before have been used
-    for (int blk = warp; blk < n * nkb; blk += kBConsumers) {
-      const int t = blk / nkb, b = blk - t * nkb;
-      float v[4];
-      if (PHASE == 1) {
-        const uint2 raw = *reinterpret_cast<const uint2*>(p.x + (size_t)sh.tok[t] * p.hidden + b * 128 + 4 * lane);
-        v[0] = __uint_as_float(raw.x << 16);
-        v[1] = __uint_as_float(raw.x & 0xffff0000u);
-        v[2] = __uint_as_float(raw.y << 16);
-        v[3] = __uint_as_float(raw.y & 0xffff0000u);
-      } else {
-        const float4 raw = __ldcg(reinterpret_cast<const float4*>(p.h + sh.hoff + (size_t)t * sh.inter + (sh.kb0 + b) * 128) + lane);
-        v[0] = raw.x; v[1] = raw.y; v[2] = raw.z; v[3] = raw.w;
+    // the run's vectors as digits: x's are copied (the plan launch has worked them out), h's are worked out here.  Several
+    // loads in flight together: each is a trip to L2
+    if (PHASE == 1) {
+      const int per = 3 * p.hidden / 16, ngrp = p.hidden / G;
+      for (int at = tid; at < per; at += 32 * kBConsumers)
+        for (int t0 = 0; t0 < n; t0 += 4) {
+          uint4 raw[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (t0 + t < n) raw[t] = __ldcg(reinterpret_cast<const uint4*>(p.xdig + (size_t)sh.tok[t0 + t] * 3 * p.hidden) + at);
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (t0 + t < n) *(reinterpret_cast<uint4*>(dig + (t0 + t) * stride) + at) = raw[t];
+        }
+      for (int at = tid; at < n * 2 * ngrp; at += 32 * kBConsumers) {
+        const int t = at / (2 * ngrp), g = at - t * 2 * ngrp;
+        X[g * kBRun + t] = __ldcg(p.xsum + (size_t)sh.tok[t] * 2 * ngrp + g);
       }
-      const BlockDigits d = block_digits(v);
-      store_digits(d, b * 128 + 4 * lane, dig + t * stride);
-      int s0, s1, s2;
-      group_digit_sums<G>(d, lane, s0, s1, s2);
-      if ((lane & (G / 4 - 1)) == 0)
-        X[(b * SG + lane / (G / 4)) * kBRun + t] = fmaf(65536.f, (float)s2, fmaf(256.f, (float)s1, (float)s0));
-      if (lane == 0) inv[b * kBRun + t] = d.inv;
+      for (int at = tid; at < n * nkb; at += 32 * kBConsumers) {
+        const int t = at / nkb, b = at - t * nkb;
+        inv[b * kBRun + t] = __ldcg(p.xinv + sh.tok[t] * nkb + b);
+      }
+    } else {
+      constexpr int kAhead = 4;
+      for (int blk0 = warp; blk0 < n * nkb; blk0 += kAhead * kBConsumers) {
+        uint4 raw[kAhead];
+#pragma unroll
+        for (int a = 0; a < kAhead; ++a) {
+          const int blk = blk0 + a * kBConsumers, t = blk / nkb, b = blk - t * nkb;
+          if (blk < n * nkb) raw[a] = __ldcg(reinterpret_cast<const uint4*>(p.h + sh.hoff + (size_t)t * sh.inter + (sh.kb0 + b) * 128) + lane);
+        }
+#pragma unroll
+        for (int a = 0; a < kAhead; ++a) {
+          const int blk = blk0 + a * kBConsumers, t = blk / nkb, b = blk - t * nkb;
+          if (blk >= n * nkb) break;
+          const float v[4] = {__uint_as_float(raw[a].x), __uint_as_float(raw[a].y), __uint_as_float(raw[a].z), __uint_as_float(raw[a].w)};
+          const BlockDigits d = block_digits(v);
+          store_digits(d, b * 128 + 4 * lane, dig + t * stride);
+          int s0, s1, s2;
+          group_digit_sums<G>(d, lane, s0, s1, s2);
+          if ((lane & (G / 4 - 1)) == 0) {
+            float* x = X + (b * SG + lane / (G / 4)) * 2 * kBRun + t;
+            x[0] = fmaf(256.f, (float)s1, (float)s0);
+            x[kBRun] = 65536.f * (float)s2;
+          }
+          if (lane == 0) inv[b * kBRun + t] = d.inv;
+        }
+      }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kBConsumers) : "memory");
-    const unsigned low0 = (sh.high >> (2 * c)) & 1u ? 0u : 0xffffffffu, low1 = (sh.high >> (2 * c + 1)) & 1u ? 0u : 0xffffffffu;
-    const bool lsb = sh.lsb != 0;
-    const int per = lsb ? 4 : 8;
-    const uint8_t* my_dig = dig + min(g8, n - 1) * stride + c * 8;  // columns without a token repeat the last one's
-    for (int u = sh.first + ((group - ord) & (kBGroups - 1)); u < sh.last; u += kBGroups) {
-      float* pb = part + half * S::kPart;
-#pragma unroll 1
-      for (int m = 0; m < S::kMats; ++m) {
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int b0 = 0; b0 < nkb; b0 += per) {
-          wait(fb + 16 * st, par);
-          const uint8_t* stage = ring + st * S::kStage;
-          const int nb = min(per, nkb - b0);
-          for (int b = gw; b < nb; b += kBGroupWarps) {
-            const uint8_t* sc = stage + kBPlane + b * (SG * 32) + g8 * 2;
-            const uint8_t* zp = stage + kBPlane + 8 * SG * 32 + b * (SG * 16) + g8;
-            const uint8_t* dg = my_dig + (b0 + b) * 384;
-            const float* xp = X + (b0 + b) * SG * kBRun + 2 * c;
-            const float* ip = inv + (b0 + b) * kBRun + 2 * c;
-            const uint8_t* ap = stage + b * 1024 + lane * 16;
-            if (lsb) b_block<G, true>(ap, ap + kBPlane / 2, sc, zp, dg, xp, ip, p.shift, low0, low1, acc);
-            else b_block<G, false>(ap, nullptr, sc, zp, dg, xp, ip, p.shift, 0xffffffffu, 0xffffffffu, acc);
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(fb + 16 * st + 8);
-          if (++st == p.stages) { st = 0; par ^= 1; }
-        }
-        float* w = pb + (gw * S::kMats + m) * (kBRun * 20);
-        w[(2 * c) * 20 + g8] = acc[0];
-        w[(2 * c + 1) * 20 + g8] = acc[1];
-        w[(2 * c) * 20 + g8 + 8] = acc[2];
-        w[(2 * c + 1) * 20 + g8 + 8] = acc[3];
-      }
-      // the four warps' shares of the columns, added in warp order by a thread per (token, row); two buffers take turns
-      asm volatile("bar.sync %0, %1;" ::"r"(2 + group), "n"(32 * kBGroupWarps) : "memory");
-      const int t = (gw * 32 + lane) >> 4, row = lane & 15;
-      if (t < n) {
-        float s[2] = {0.f, 0.f};
-#pragma unroll
-        for (int w = 0; w < kBGroupWarps; ++w)
-#pragma unroll
-          for (int m = 0; m < S::kMats; ++m) s[m] += pb[(w * S::kMats + m) * (kBRun * 20) + t * 20 + row];
-        if (PHASE == 1) p.h[sh.hoff + (size_t)t * sh.inter + u * 16 + row] = s[0] / (1.f + expf(-s[0])) * s[1];  // silu(gate) * up
-        else p.yrow[(size_t)(sh.yrow + t) * p.hidden + u * 16 + row] = s[0];
-      }
-      half ^= 1;
+    const unsigned all = (1u << n) - 1u;
+    const int first = u0 + ((group - ord) & (kBGroups - 1));
+    const bool high = (sh.high & all) == all;
+    auto rows = [&](auto mode, auto wide) {
+      b_rows<G, PHASE, decltype(mode)::value, decltype(wide)::value>(p, sh, first, u1, fb, ring, part, dig, X, inv, stride, group, gw, lane, wait, state);
+    };
+    using std::integral_constant;
+    if (n > 2) {
+      if (!sh.lsb) rows(integral_constant<int, kModeLow>(), std::true_type());
+      else if (high) rows(integral_constant<int, kModeHigh>(), std::true_type());
+      else rows(integral_constant<int, kModeMixed>(), std::true_type());
+    } else {
+      if (!sh.lsb) rows(integral_constant<int, kModeLow>(), std::false_type());
+      else if (high) rows(integral_constant<int, kModeHigh>(), std::false_type());
+      else rows(integral_constant<int, kModeMixed>(), std::false_type());
     }
-    ord += sh.last - sh.first;
+    ord += u1 - u0;
   }
 }
 
@@ -668,23 +810,34 @@ __global__ void __launch_bounds__(kBCombineThreads) batch_combine_kernel(const B
   const int t = blockIdx.y, col = (blockIdx.x * kBCombineThreads + threadIdx.x) * 2, slots = p.k + p.n_shared;
   b_dep_launch();
   b_dep_wait();
-  if (col >= p.hidden || p.head->off) return;
-  float2 a = make_float2(0.f, 0.f);
-  const float gate = p.gate ? p.gate[t] : 1.f;
-#pragma unroll 4
-  for (int j = 0; j < slots; ++j) {
+  __shared__ int4 s_at[SLICEMOE_MAX_TOP_K + SLICEMOE_MAX_SHARED];  // first row, rows from chunk to chunk, chunks, weight
+  if (threadIdx.x < slots) {
+    const int j = threadIdx.x;
     const int2 at = p.pos[t * slots + j];
-    if (at.x < 0) continue;
-    const float w = j < p.k ? p.weights[t * p.k + j] : gate;
-    const int kc_n = j < p.k ? p.kc_r : p.kc_s;
-    float2 v = __ldcg(reinterpret_cast<const float2*>(p.yrow + (size_t)at.x * p.hidden + col));
-    for (int kc = 1; kc < kc_n; ++kc) {
-      const float2 u = __ldcg(reinterpret_cast<const float2*>(p.yrow + (size_t)(at.x + kc * at.y) * p.hidden + col));
-      v.x += u.x;
-      v.y += u.y;
+    const float w = j < p.k ? p.weights[t * p.k + j] : p.gate ? p.gate[t] : 1.f;
+    s_at[j] = make_int4(at.x, at.y, j < p.k ? p.kc_r : p.kc_s, __float_as_int(w));
+  }
+  const bool off = p.head->off != 0;
+  __syncthreads();
+  if (col >= p.hidden || off) return;
+  float2 a = make_float2(0.f, 0.f);
+  for (int j0 = 0; j0 < slots; j0 += 4) {
+    float2 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j0 + j < slots && s_at[j0 + j].x >= 0) v[j] = __ldcg(reinterpret_cast<const float2*>(p.yrow + (size_t)s_at[j0 + j].x * p.hidden + col));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j0 + j >= slots || s_at[j0 + j].x < 0) continue;
+      const int4 at = s_at[j0 + j];
+      for (int kc = 1; kc < at.z; ++kc) {
+        const float2 u = __ldcg(reinterpret_cast<const float2*>(p.yrow + (size_t)(at.x + kc * at.y) * p.hidden + col));
+        v[j].x += u.x;
+        v[j].y += u.y;
+      }
+      a.x = fmaf(__int_as_float(at.w), v[j].x, a.x);
+      a.y = fmaf(__int_as_float(at.w), v[j].y, a.y);
     }
-    a.x = fmaf(w, v.x, a.x);
-    a.y = fmaf(w, v.y, a.y);
   }
   *reinterpret_cast<float2*>(p.y + (size_t)t * p.hidden + col) = a;
 }
@@ -725,6 +878,14 @@ static int b_launch_ffn(BParams p, int sms, cudaStream_t st) {
                   (size_t)S::ring(p.K) + (size_t)kBGroups * p.stages * S::kStage, st, p);
 }
 
+template <int G>
+static int b_launch_all(const BPlanParams& pp, BParams p1, BParams p2, int sms, cudaStream_t st) {
+  int rc = b_launch(batch_plan_kernel<G>, dim3((unsigned)(1 + pp.T)), kBPlanThreads, 0, st, pp);
+  if (rc == SLICEMOE_OK) rc = b_launch_ffn<G, 1>(p1, sms, st);
+  if (rc == SLICEMOE_OK) rc = b_launch_ffn<G, 2>(p2, sms, st);
+  return rc;
+}
+
 int batch_layer(const slicemoe_shape* s, const slicemoe_expert* experts, const slicemoe_expert* shared, int n_shared,
                 const float* gate_vec, const uint16_t* x, int T, const int32_t* ids, const uint8_t* prec, const float* weights,
                 float* y, void* workspace, const BatchControl& ctl, int sms, void* stream) {
@@ -747,43 +908,40 @@ int batch_layer(const slicemoe_shape* s, const slicemoe_expert* experts, const s
   pp.kc_r = L.kc_r;
   pp.kc_s = L.kc_s;
   pp.head = reinterpret_cast<BHead*>(ws + L.head);
-  pp.runs = reinterpret_cast<BRun*>(ws + L.runs);
+  pp.experts = experts;
+  pp.shared = shared;
   pp.seg1 = reinterpret_cast<BSeg*>(ws + L.seg1);
   pp.seg2 = reinterpret_cast<BSeg*>(ws + L.seg2);
   pp.pos = reinterpret_cast<int2*>(ws + L.pos);
   pp.gate = reinterpret_cast<float*>(ws + L.gate);
+  pp.xdig = ws + L.xdig;
+  pp.xsum = reinterpret_cast<float*>(ws + L.xsum);
+  pp.xinv = reinterpret_cast<float*>(ws + L.xinv);
   pp.ctl = ctl;
-  int rc = b_launch(batch_plan_kernel, dim3(gated ? 1 + T : 1), kBPlanThreads, 0, st, pp);
-  if (rc != SLICEMOE_OK) return rc;
   BParams p;
-  p.experts = experts;
-  p.shared = shared;
-  p.x = x;
   p.head = pp.head;
-  p.runs = pp.runs;
   p.segs = pp.seg1;
+  p.xdig = pp.xdig;
+  p.xsum = pp.xsum;
+  p.xinv = pp.xinv;
   p.h = reinterpret_cast<float*>(ws + L.h);
   p.yrow = reinterpret_cast<float*>(ws + L.yrow);
   p.ctl = ctl;
-  p.n_experts = s->n_experts;
   p.hidden = s->hidden;
   p.K = s->hidden;
   p.shift = s->b_high - s->b_low;
   p.stages = 0;
+  const int parts = (T + kBRun - 1) / kBRun;
+  p.max_segs = T * s->top_k + n_shared * parts;
   BParams p2 = p;
   p2.segs = pp.seg2;
+  p2.max_segs = T * s->top_k * L.kc_r + n_shared * parts * L.kc_s;
+  // (widths add up to 12288 over a token's experts: never more segments than threads)
+  if (p2.max_segs > kBThreads) return SLICEMOE_E_UNSUPPORTED;
   const int widest = s->inter > pp.shared_inter ? s->inter : pp.shared_inter;
   p2.K = widest < kBChunkK ? widest : kBChunkK;
-  if (s->group == 128) {
-    rc = b_launch_ffn<128, 1>(p, sms, st);
-    if (rc == SLICEMOE_OK) rc = b_launch_ffn<128, 2>(p2, sms, st);
-  } else if (s->group == 64) {
-    rc = b_launch_ffn<64, 1>(p, sms, st);
-    if (rc == SLICEMOE_OK) rc = b_launch_ffn<64, 2>(p2, sms, st);
-  } else {
-    rc = b_launch_ffn<32, 1>(p, sms, st);
-    if (rc == SLICEMOE_OK) rc = b_launch_ffn<32, 2>(p2, sms, st);
-  }
+  const int rc = s->group == 128 ? b_launch_all<128>(pp, p, p2, sms, st)
+                 : s->group == 64 ? b_launch_all<64>(pp, p, p2, sms, st) : b_launch_all<32>(pp, p, p2, sms, st);
   if (rc != SLICEMOE_OK) return rc;
   BCombine c;
   c.head = pp.head;
