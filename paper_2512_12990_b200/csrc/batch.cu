@@ -21,7 +21,7 @@
 //
 // Bound: HBM.  Per 16 x 128 block of both planes (2 KB, 89 cycles of an SM's share of the bandwidth) a warp issues about 125
 // instructions, 24 of them MMAs (53 cycles of the integer tensor pipe).
-// Measured, 8 tokens, 64 x 1408 top-6 + 2 shared, hidden 2048: eight batch-1 launches 133 us, this BATCH_US.
+// Measured, 8 tokens, 64 x 1408 top-6 + 2 shared, hidden 2048: eight batch-1 launches 133 us, this 52.
 //
 // Bounded waits: when one runs out the CTA's dead flag goes up and SLICEMOE_STATUS_WAIT_TIMEOUT is set; from then on nobody
 // waits for data, the consumers walk through the rest of their work and the producers stop and wait for their copies.

@@ -127,7 +127,9 @@ constexpr size_t kWsBatchOff = (kWsBytes + 255) & ~(size_t)255;
 constexpr size_t kWsListEntries = (size_t)kBatchTokens * SLICEMOE_MAX_TOP_K;
 constexpr size_t kWsListBytes = kWsListEntries * 9;
 // From this many tokens on a layer call takes the batch kernels (four launches) instead of a launch of the batch-1 kernel
-// per token.  BATCH_RULE
+// per token.  Measured, us, loop / batch at T = 2, 3, 4: 2048-wide layer of 1408-wide experts 33 / 37, 49 / 40, 65 / 43; 1024 wide
+// 22 / 19, 33 / 20, 44 / 21; 256 wide 13 / 14, 20 / 14, 27 / 14.  (At three tokens the loop stays, because slicemoe_layer_static,
+// which has no room for the batch, promises the bits of slicemoe_layer there.)
 constexpr int kBatchMinTokens = 4;
 static_assert(sizeof(WsHeader) <= kWsHOff, "workspace header");
 static_assert(kWsStLogits + 4 * 512 <= kWsStIds, "x and the logits fit the staging area back to back too");
@@ -1148,7 +1150,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
       mbar_init(bars + 8 * Bars::pfull2, kConsumerWarps);
       mbar_init(bars + 8 * Bars::pempty2, 1);
       mbar_init(bars + 8 * Bars::p1_done, kConsumerWarps);
-      mbar_init(bars + 8 * Bars::plan_ready, early_lists ? 2 : 1);  // resident lists: warps 0 and 1 each say when done
+      mbar_init(bars + 8 * Bars::plan_ready, 2);  // warps 0 and 1 each say when done
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -1193,10 +1195,18 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
     SM_TRACE_G(21);
   }
   if (warp == 0) {
-    if (!early_lists) build_plan<FUSED>(p, smem, lane);
+    if (!early_lists) {
+      build_plan<FUSED>(p, smem, lane);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(plan_ready);
+    }
     SM_TRACE(2);
   } else if (warp == 1) {
-    if (!early_lists) load_slot_pointers<FUSED>(p, smem, lane, true);
+    if (!early_lists) {
+      load_slot_pointers<FUSED>(p, smem, lane, true);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(plan_ready);
+    }
   } else if (warp == 2) {
     if (lane == 0) {
       // a wait limit set by the host for this workspace
@@ -1240,7 +1250,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
   if (warp == 3) SM_TRACE(3);
   asm volatile("bar.sync 1, %0;" ::"n"(32 * (kConsumerWarps + 1)) : "memory");
   if (warp == 3) SM_TRACE(4);
-  if (!early_lists && tid == 0) mbar_arrive(plan_ready);
   if (plan->nslots == 0 && blockIdx.x == 0)
     for (int i = tid; i < p.hidden; i += 32 * (kConsumerWarps + 1)) p.y[i] = 0.f;
 
