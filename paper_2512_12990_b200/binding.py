@@ -395,11 +395,12 @@ class Dbsc:
     def assign(self, step: int, layer: int, ids, prec_req):
         """ids: numpy int32 [n]; prec_req: numpy uint8 [n] -> numpy uint8 [n]."""
         import numpy as np
-        ids = np.ascontiguousarray(ids, dtype=np.int32)
-        prec_req = np.ascontiguousarray(prec_req, dtype=np.uint8)
-        out = np.empty(ids.shape, dtype=np.uint8)
-        rc = lib().slicemoe_dbsc_assign(self._h, step, layer, ids.ctypes.data, prec_req.ctypes.data, ids.size, out.ctypes.data)
-        _check(rc, "slicemoe_dbsc_assign")
+        out = np.empty(np.shape(ids), dtype=np.uint8)
+        m = _m or _marshal()
+        if not m.dbsc_assign(self._h, step, layer, ids, prec_req, out):   # other types or layouts: converted first
+            ids = np.ascontiguousarray(ids, dtype=np.int32)
+            if not m.dbsc_assign(self._h, step, layer, ids, np.ascontiguousarray(prec_req, dtype=np.uint8), out):
+                raise SliceMoEError(E_INVALID_ARG, "slicemoe_dbsc_assign")
         return out
 
     def bias(self, layer: int, n_experts: int, delta: float):

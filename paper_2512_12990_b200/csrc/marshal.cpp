@@ -15,6 +15,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "slicemoe.h"
 
@@ -31,6 +32,7 @@ struct Entry {
   decltype(&slicemoe_layer_static) layer_static;
   decltype(&slicemoe_decode_step_host) decode_step_host;
   decltype(&slicemoe_prefill_layer) prefill_layer;
+  decltype(&slicemoe_dbsc_assign) dbsc_assign;
 } lib;
 PyObject* error_type = nullptr;  // binding.SliceMoEError(code, where)
 PyObject* s_data_ptr = nullptr;
@@ -103,6 +105,19 @@ struct ShapeArg {
 at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type, at::Device dev) {
   if (dev.is_cuda()) return at::Tensor(at::detail::empty_cuda(sizes, type, dev, std::nullopt));
   return at::empty(sizes, at::TensorOptions().dtype(type).device(dev));
+}
+// Several small outputs of one call in one allocation (an allocation costs 0.7 us, a tensor on an existing storage a
+// third of that): [rows, cols] of the given types, each on a 16-byte boundary.
+template <int N>
+void empty_together(int64_t rows, int64_t cols, const at::ScalarType (&types)[N], at::Device dev, at::Tensor (&out)[N]) {
+  int64_t at[N + 1] = {0};
+  for (int i = 0; i < N; ++i) at[i + 1] = at[i] + ((rows * cols * (int64_t)c10::elementSize(types[i]) + 15) & ~(int64_t)15);
+  const at::Tensor all = empty({std::max<int64_t>(at[N], 1)}, at::kByte, dev);
+  for (int i = 0; i < N; ++i) {
+    out[i] = at::detail::make_tensor<c10::TensorImpl>(c10::Storage(all.storage()), all.key_set(), c10::scalarTypeToTypeMeta(types[i]));
+    out[i].unsafeGetTensorImpl()->set_sizes_contiguous({rows, cols});
+    out[i].unsafeGetTensorImpl()->set_storage_offset(at[i] / (int64_t)c10::elementSize(types[i]));
+  }
 }
 PyObject* wrap(const at::Tensor& t) {
   PyObject* o = THPVariable_Wrap(t);
@@ -193,6 +208,7 @@ PyObject* py_setup(SM_ARGS) {  // (error type, dict name -> address)
     load("slicemoe_layer_static", lib.layer_static);
     load("slicemoe_decode_step_host", lib.decode_step_host);
     load("slicemoe_prefill_layer", lib.prefill_layer);
+    load("slicemoe_dbsc_assign", lib.dbsc_assign);
     Py_XSETREF(error_type, Py_NewRef(a[0]));
     Py_RETURN_NONE;
   });
@@ -207,7 +223,12 @@ PyObject* py_pack_new(SM_ARGS) {  // W, group, b_high, b_low, stream -> (msb, ls
     const int64_t nm = std::max<int64_t>(group > 0 ? (int64_t)lib.meta_count(N, K, group) : 1, 1);
     const at::Device dev = W.device();
     const at::Tensor msb = empty({nb}, at::kByte, dev), lsb = empty({nb}, at::kByte, dev);
-    const at::Tensor scale = empty({nm}, at::kShort, dev), zp = empty({nm}, at::kByte, dev);
+    // (the planes apart: either may be given up on its own)
+    at::Tensor meta[2];
+    empty_together<2>(1, nm, {at::kShort, at::kByte}, dev, meta);
+    const at::Tensor &scale = meta[0], &zp = meta[1];
+    scale.unsafeGetTensorImpl()->set_sizes_contiguous({nm});
+    zp.unsafeGetTensorImpl()->set_sizes_contiguous({nm});
     const int bh = integer32(a[2]), bl = integer32(a[3]);
     void* st = stream_of(a[4]);
     check(unlocked([&] {
@@ -230,9 +251,16 @@ PyObject* py_route_topk(SM_ARGS) {  // logits, k, bias, renorm, tau, rank_high, 
     const int64_t T = logits.size(0), E = logits.size(1);
     const int k = integer32(a[1]), kk = std::max(k, 1);
     const at::Device dev = logits.device();
-    const at::Tensor ids = empty({T, kk}, at::kInt, dev), w = empty({T, kk}, at::kFloat, dev);
-    at::Tensor prec;
-    if (truth(a[6])) prec = empty({T, kk}, at::kByte, dev);
+    at::Tensor ids, w, prec;
+    if (truth(a[6])) {
+      at::Tensor l[3];
+      empty_together<3>(T, kk, {at::kInt, at::kFloat, at::kByte}, dev, l);
+      ids = l[0], w = l[1], prec = l[2];
+    } else {
+      at::Tensor l[2];
+      empty_together<2>(T, kk, {at::kInt, at::kFloat}, dev, l);
+      ids = l[0], w = l[1];
+    }
     const float* bias = static_cast<const float*>(address(a[2]));
     const int renorm = truth(a[3]), rank_high = integer32(a[5]);
     const float tau = real(a[4]);
@@ -244,6 +272,44 @@ PyObject* py_route_topk(SM_ARGS) {  // logits, k, bias, renorm, tau, rank_high, 
           }),
           "slicemoe_route_topk");
     return tuple_of({&ids, &w, &prec});
+  });
+}
+
+// A contiguous buffer of `size`-byte items with one of the format characters in `kinds`; nothing is raised if it is not.
+bool plain_buffer(PyObject* o, Py_buffer* b, Py_ssize_t size, const char* kinds) {
+  if (PyObject_GetBuffer(o, b, PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) != 0) {
+    PyErr_Clear();
+    return false;
+  }
+  const char* f = b->format ? b->format : "B";
+  if (*f == '<' || *f == '=' || *f == '@') ++f;
+  if (b->itemsize == size && *f && strchr(kinds, *f) && !f[1]) return true;
+  PyBuffer_Release(b);
+  return false;
+}
+// handle, step, layer, ids (int32), prec_req (uint8), prec_out (uint8, written); returns False if the buffers are of other types
+PyObject* py_dbsc_assign(SM_ARGS) {
+  return guarded([&]() -> PyObject* {
+    want(n, 6);
+    auto* c = a[0] == Py_None ? nullptr : static_cast<slicemoe_dbsc*>(PyLong_AsVoidPtr(a[0]));
+    if (PyErr_Occurred()) throw Failed();
+    const int step = integer32(a[1]), layer = integer32(a[2]);
+    Py_buffer ids, req, out;
+    if (!plain_buffer(a[3], &ids, 4, "il")) Py_RETURN_FALSE;
+    int rc = 1;
+    if (plain_buffer(a[4], &req, 1, "B")) {
+      if (plain_buffer(a[5], &out, 1, "B")) {
+        if (!out.readonly && req.len >= ids.len / 4 && out.len >= ids.len / 4)
+          rc = lib.dbsc_assign(c, step, layer, static_cast<const int32_t*>(ids.buf), static_cast<const uint8_t*>(req.buf),
+                               (int)(ids.len / 4), static_cast<uint8_t*>(out.buf));
+        PyBuffer_Release(&out);
+      }
+      PyBuffer_Release(&req);
+    }
+    PyBuffer_Release(&ids);
+    if (rc == 1) Py_RETURN_FALSE;
+    check(rc, "slicemoe_dbsc_assign");
+    Py_RETURN_TRUE;
   });
 }
 
@@ -324,9 +390,9 @@ PyObject* py_layer_routed(SM_ARGS) {
     const int64_t T = x.size(0), k = s.get()->top_k;
     at::Tensor ids, prec, w;
     if (truth(a[12])) {
-      ids = empty({T, k}, at::kInt, x.device());
-      prec = empty({T, k}, at::kByte, x.device());
-      w = empty({T, k}, at::kFloat, x.device());
+      at::Tensor l[3];
+      empty_together<3>(T, k, {at::kInt, at::kFloat, at::kByte}, x.device(), l);
+      ids = l[0], w = l[1], prec = l[2];
     }
     const auto* ex = static_cast<const slicemoe_expert*>(address(a[1]));
     const auto* sh = static_cast<const slicemoe_expert*>(address(a[2]));
@@ -411,6 +477,7 @@ PyObject* py_prefill_layer(SM_ARGS) {
 PyMethodDef methods[] = {SM_METHOD(setup),        SM_METHOD(pack_new),         SM_METHOD(route_topk),
                          SM_METHOD(expert_ffn),   SM_METHOD(layer),            SM_METHOD(layer_static),
                          SM_METHOD(layer_routed), SM_METHOD(decode_step_host), SM_METHOD(prefill_layer),
+                         SM_METHOD(dbsc_assign),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
