@@ -3,10 +3,10 @@
 // that prefill wants high-bit computation; the per-expert precision flag here is this library's generalisation
 // (an expert can also be run from its MSB slice alone), which the mixed-precision prefill benchmark uses.
 //
-// Steps, all on the device, five launches chained by programmatic dependent launch:
+// Steps, all on the device, five or six launches chained by programmatic dependent launch:
 //   1. plan: count the tokens of every routed expert, give every (token, expert) pair a row - the experts' rows one
 //      after the other, without padding - and sort the experts by their number of tokens;
-//   2. gather x (bf16) into that order as fp16 (exact for every bf16 value in fp16's normal range);
+//   2. scatter x (bf16) into that order as fp16 (exact for every bf16 value in fp16's normal range);
 //   3. grouped GEMM 1: per tile  H = silu(X Wg^T) * (X Wu^T)  (fp16 out);
 //   4. grouped GEMM 2: per tile  Yrow = H Wd^T  (fp32 out, one row per (token, expert) pair);
 //   5. combine: y[t] = sum_j w[t,j] Yrow[pos(t,j)] + shared experts, in list order (deterministic).
@@ -40,10 +40,13 @@ struct PfHead {
   int next1, next2;       // next work item to hand out
 };
 
+constexpr int kPfSmemExperts = 2048;
+constexpr int kPfRankPairs = 4096;  // pairs that one block counts
+
 // ---- workspace layout (host and device agree through this one function) --------------------------------
 struct PfLayout {
-  size_t head, counts, offsets, cursor, runs, row_token, posmap, gate, xs, h, yrow, total;
-  int in_rows, out_rows, nexp_all;
+  size_t head, counts, base, hist, runs, rank, posmap, gate, xs, h, yrow, total;
+  int in_rows, out_rows, nexp_all, rank_blocks;
 };
 __host__ __device__ inline size_t pf_align(size_t v) { return (v + 255) & ~(size_t)255; }
 __host__ __device__ inline PfLayout pf_layout(int T, int E, int k, int n_shared, int hidden, int inter, int shared_inter) {
@@ -51,14 +54,16 @@ __host__ __device__ inline PfLayout pf_layout(int T, int E, int k, int n_shared,
   L.nexp_all = E + n_shared;
   L.in_rows = T * k + (n_shared ? T : 0);  // the shared experts read the same rows
   L.out_rows = T * (k + n_shared);
+  // beyond kPfSmemExperts the counters do not fit shared memory and one block counts them in the workspace
+  L.rank_blocks = E > kPfSmemExperts ? 1 : (T * k + kPfRankPairs - 1) / kPfRankPairs;
   const int wide = inter > shared_inter ? inter : shared_inter;
   size_t o = 0;
   L.head = o;         o = pf_align(o + sizeof(PfHead));
   L.counts = o;       o = pf_align(o + sizeof(int) * L.nexp_all);
-  L.offsets = o;      o = pf_align(o + sizeof(int) * L.nexp_all);
-  L.cursor = o;       o = pf_align(o + sizeof(int) * L.nexp_all);
+  L.base = o;         o = pf_align(o + sizeof(int) * L.nexp_all);
+  L.hist = o;         o = pf_align(o + sizeof(int) * (size_t)L.rank_blocks * E);
   L.runs = o;         o = pf_align(o + sizeof(PfRun) * L.nexp_all);
-  L.row_token = o;    o = pf_align(o + sizeof(int) * (size_t)T * k);
+  L.rank = o;         o = pf_align(o + sizeof(int) * (size_t)T * k);
   L.posmap = o;       o = pf_align(o + sizeof(int) * (size_t)T * (k + n_shared));
   L.gate = o;         o = pf_align(o + sizeof(float) * T);
   L.xs = o;           o = pf_align(o + sizeof(__half) * (size_t)L.in_rows * hidden);
@@ -72,21 +77,52 @@ __device__ __forceinline__ void pf_dep_wait() { asm volatile("griddepcontrol.wai
 __device__ __forceinline__ void pf_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- step 1: rows and work items ---------------------------------------------------------------------------
-// One block: the whole plan is a few passes over T k expert ids, and one block needs no grid barrier between them.
-// Counters sit in shared memory up to kPfSmemExperts experts, in the workspace beyond.  Which row a pair gets depends
-// on the order of the atomics, the values computed for it do not.
+// A pair's row is its expert's first row, plus the pairs of the expert in the blocks of pairs before, plus its rank
+// among its own block's: the rank is what the counting atomic returns.  Up to kPfRankPairs pairs the plan block counts them
+// itself; above, a launch of its own does, a block per kPfRankPairs pairs.  (One block for all: 13 us for 8,192 pairs, 58 for
+// 49,152, at the rate of one SM's shared-memory atomics.)  Which row a pair gets depends on the order of the atomics, the
+// values computed for it do not.
 constexpr int kPfPlanThreads = 1024;
-constexpr int kPfSmemExperts = 2048;
 struct PfPlanParams {
   const int32_t* ids;
   int T, k, E, n_shared;
   int per1_routed, per1_shared, per2;  // work items per tile: GEMM 1 of a routed / shared expert, GEMM 2
+  int rank_blocks;
   PfHead* head;
-  int *counts, *offsets, *cursor;
+  int *counts, *base;   // [experts]: counters that do not fit shared memory; first rows likewise
+  int* hist;            // [block][E]: pairs of the expert in the block; the plan turns them into the block's first rows
   PfRun* runs;
-  int *row_token, *posmap;
+  int* rank;            // [T k]
   unsigned* status;
 };
+// Ranks of the pairs [i0, i1) by the calling block; an id out of range gets rank -1.
+__device__ __forceinline__ void pf_rank(const int32_t* ids, int i0, int i1, int E, int* counts, int* rank) {
+  constexpr int kAhead = kPfRankPairs / kPfPlanThreads;
+  for (int b = i0; b < i1; b += kPfRankPairs) {
+    int e[kAhead];
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      const int i = b + a * kPfPlanThreads + (int)threadIdx.x;
+      e[a] = i < i1 ? ids[i] : -1;
+    }
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      const int i = b + a * kPfPlanThreads + (int)threadIdx.x;
+      if (i < i1) rank[i] = e[a] >= 0 && e[a] < E ? atomicAdd(&counts[e[a]], 1) : -1;
+    }
+  }
+}
+__global__ void __launch_bounds__(kPfPlanThreads) pf_rank_kernel(const PfPlanParams p) {
+  __shared__ int s_counts[kPfSmemExperts];
+  pf_dep_launch();
+  for (int e = threadIdx.x; e < p.E; e += kPfPlanThreads) s_counts[e] = 0;
+  pf_dep_wait();  // the ids may be the work of the kernel before, which may also still read what is now the workspace
+  __syncthreads();
+  const int i0 = blockIdx.x * kPfRankPairs;
+  pf_rank(p.ids, i0, min(i0 + kPfRankPairs, p.T * p.k), p.E, s_counts, p.rank);
+  __syncthreads();
+  for (int e = threadIdx.x; e < p.E; e += kPfPlanThreads) p.hist[(size_t)blockIdx.x * p.E + e] = s_counts[e];
+}
 __device__ __forceinline__ int pf_tiles_of(int count) { return (count + kPfTileN - 1) / kPfTileN; }
 // Exclusive block-wide scan of one value per thread; *total gets the sum.
 __device__ int pf_block_scan(int v, int* warp_sums, int* total) {
@@ -109,56 +145,55 @@ __device__ int pf_block_scan(int v, int* warp_sums, int* total) {
   return before + inc - v;
 }
 __global__ void __launch_bounds__(kPfPlanThreads) pf_plan_kernel(const PfPlanParams p) {
-  __shared__ int s_counts[kPfSmemExperts], s_offsets[kPfSmemExperts], s_cursor[kPfSmemExperts];
+  __shared__ int s_counts[kPfSmemExperts], s_base[kPfSmemExperts];
   __shared__ int s_sums[32];
   const int tid = threadIdx.x;
   const int n = p.E + p.n_shared;
   const bool fits = n <= kPfSmemExperts;
   int* counts = fits ? s_counts : p.counts;
-  int* offsets = fits ? s_offsets : p.offsets;
-  int* cursor = fits ? s_cursor : p.cursor;
+  int* base = fits ? s_base : p.base;
   pf_dep_launch();
-  pf_dep_wait();  // the ids may be the work of the kernel before, which may also still read what is now the workspace
+  pf_dep_wait();
+  const int npairs = p.T * p.k;
+  const bool alone = p.rank_blocks == 1;
   for (int e = tid; e < n; e += kPfPlanThreads) {
-    counts[e] = e < p.E ? 0 : p.T;
-    cursor[e] = 0;
+    int c = e < p.E ? 0 : p.T;
+    if (!alone && e < p.E) {
+      // the blocks' counts become the pairs before each block
+#pragma unroll 4
+      for (int b = 0; b < p.rank_blocks; ++b) {
+        const int h = p.hist[(size_t)b * p.E + e];
+        p.hist[(size_t)b * p.E + e] = c;
+        c += h;
+      }
+    }
+    counts[e] = c;
   }
   if (tid == 0) {
     *p.status = 0u;
     p.head->next1 = p.head->next2 = 0;
   }
   __syncthreads();
-  const int npairs = p.T * p.k;
-  bool bad = false;
-  for (int i = tid; i < npairs; i += kPfPlanThreads) {
-    const int e = p.ids[i];
-    if (e >= 0 && e < p.E) atomicAdd(&counts[e], 1);
-    else bad = true;
+  if (alone) {
+    pf_rank(p.ids, 0, npairs, p.E, counts, p.rank);
+    __syncthreads();
   }
-  if (bad) atomicOr(p.status, (unsigned)SLICEMOE_STATUS_BAD_EXPERT_ID);
-  __syncthreads();
   // rows: the routed experts' one after the other
-  int base = 0;
+  int rows = 0;
   for (int e0 = 0; e0 < p.E; e0 += kPfPlanThreads) {
     const int e = e0 + tid;
     int total;
     const int before = pf_block_scan(e < p.E ? counts[e] : 0, s_sums, &total);
-    if (e < p.E) offsets[e] = base + before;
-    base += total;
-  }
-  __syncthreads();
-  for (int i = tid; i < npairs; i += kPfPlanThreads) {
-    const int e = p.ids[i], t = i / p.k;
-    int pos = -1;
-    if (e >= 0 && e < p.E) {
-      pos = offsets[e] + atomicAdd(&cursor[e], 1);
-      p.row_token[pos] = t;
+    if (e < p.E) {
+      const int first = rows + before;
+      base[e] = first;
+      if (alone) {
+        p.hist[e] = first;
+      } else {
+        for (int b = 0; b < p.rank_blocks; ++b) p.hist[(size_t)b * p.E + e] += first;
+      }
     }
-    p.posmap[t * (p.k + p.n_shared) + (i - t * p.k)] = pos;
-  }
-  for (int i = tid; i < p.T * p.n_shared; i += kPfPlanThreads) {
-    const int t = i / p.n_shared, j = i - t * p.n_shared;
-    p.posmap[t * (p.k + p.n_shared) + p.k + j] = npairs + j * p.T + t;
+    rows += total;
   }
   // runs: experts with tokens, shared ones first (their contraction in GEMM 2 is usually the longest), then by
   // falling number of tokens: handed out in this order, the longest items do not come last.  rank = number of
@@ -178,8 +213,8 @@ __global__ void __launch_bounds__(kPfPlanThreads) pf_plan_kernel(const PfPlanPar
     r.expert = e;
     r.count = c;
     r.tiles = pf_tiles_of(c);
-    r.in_row = e < p.E ? offsets[e] : npairs;
-    r.out_row = e < p.E ? offsets[e] : npairs + (e - p.E) * p.T;
+    r.in_row = e < p.E ? base[e] : npairs;
+    r.out_row = e < p.E ? base[e] : npairs + (e - p.E) * p.T;
     r.items1 = r.items2 = r.pad_ = 0;
     p.runs[rank] = r;
   }
@@ -216,29 +251,49 @@ __global__ void __launch_bounds__(kPfPlanThreads) pf_plan_kernel(const PfPlanPar
   }
 }
 
-// ---- step 2: gather x into expert order, bf16 -> fp16 ----------------------------------------------------
-// A warp per row, 16 bytes per lane and step (4 where x is not 16-byte aligned).  With a gated shared expert the last
-// T rows - the tokens in their own order - also give the token's gate sigmoid(gate_vec . x): the row is being read
-// anyway.
+// ---- step 2: scatter x into expert order, bf16 -> fp16 ---------------------------------------------------
+// A block per token: the row is read once and written to the row of each of its pairs, and to the token's row for the shared
+// experts, 16 bytes per thread and step (4 where x is not 16-byte aligned).  The pairs' rows are worked out on the way, and
+// with a gated shared expert the token's gate sigmoid(gate_vec . x).  Bound: the writes.  (A warp per written row read every
+// token's row k + 1 times: 17 us for 2,048 tokens x 5 rows, 53 for 8,192 x 7.)
 constexpr int kPfGatherThreads = 256;
+constexpr int kPfMaxSlots = SLICEMOE_MAX_TOP_K + SLICEMOE_MAX_SHARED;
+struct PfGatherParams {
+  const uint16_t* x;
+  const int32_t* ids;
+  const int *rank, *first;  // rank of a pair, [block][E] first rows
+  int T, k, E, n_shared, hidden;
+  int* posmap;
+  __half* xs;
+  const float* gate_vec;  // or null
+  float* gate;
+  unsigned* status;
+};
 template <int WORDS>
-__global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const uint16_t* __restrict__ x, int hidden, int T,
-                                                                     const int* __restrict__ row_token, int routed_rows,
-                                                                     int rows, __half* __restrict__ xs,
-                                                                     const float* __restrict__ gate_vec,
-                                                                     float* __restrict__ gate) {
-  const int row = (int)(blockIdx.x * (kPfGatherThreads / 32) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const PfGatherParams p) {
+  __shared__ int s_row[SLICEMOE_MAX_TOP_K + 1];
+  __shared__ float s_part[kPfGatherThreads / 32];
+  const int t = blockIdx.x, tid = threadIdx.x, npairs = p.T * p.k;
   pf_dep_launch();
   pf_dep_wait();
-  if (row >= rows) return;
-  const int t = row < routed_rows ? row_token[row] : row - routed_rows;
-  if ((unsigned)t >= (unsigned)T) return;  // ids out of range leave rows at the end of the routed ones without a token
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(x + (size_t)t * hidden);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(xs + (size_t)row * hidden);
-  const bool gated = gate_vec != nullptr && row >= routed_rows;
+  if (tid < p.k + p.n_shared) {
+    int pos;
+    if (tid < p.k) {
+      const int i = t * p.k + tid, e = p.ids[i], r = p.rank[i];
+      pos = r >= 0 ? p.first[(size_t)(i / kPfRankPairs) * (p.E > kPfSmemExperts ? 0 : p.E) + e] + r : -1;
+      if (r < 0) atomicOr(p.status, (unsigned)SLICEMOE_STATUS_BAD_EXPERT_ID);
+      s_row[tid] = pos;
+    } else {
+      pos = npairs + (tid - p.k) * p.T + t;
+    }
+    p.posmap[t * (p.k + p.n_shared) + tid] = pos;
+  }
+  if (tid == 0 && p.n_shared > 0) s_row[p.k] = npairs + t;  // the shared experts read the same row
+  const int copies = p.k + (p.n_shared > 0 ? 1 : 0);
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(p.x + (size_t)t * p.hidden);
   float dot = 0.f;
-#pragma unroll 4
-  for (int i = lane * WORDS; i < hidden / 2; i += 32 * WORDS) {
+  __syncthreads();
+  for (int i = tid * WORDS; i < p.hidden / 2; i += kPfGatherThreads * WORDS) {
     uint32_t in[WORDS], out[WORDS];
     if (WORDS == 4) {
       const uint4 v = *reinterpret_cast<const uint4*>(src + i);
@@ -251,19 +306,30 @@ __global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const uint1
       const float lo = __uint_as_float(in[j] << 16), hi = __uint_as_float(in[j] & 0xffff0000u);
       const __half2 h = __floats2half2_rn(lo, hi);
       out[j] = *reinterpret_cast<const uint32_t*>(&h);
-      if (gated) {
-        const float2 gv = *reinterpret_cast<const float2*>(gate_vec + 2 * (i + j));
+      if (p.gate_vec) {
+        const float2 gv = *reinterpret_cast<const float2*>(p.gate_vec + 2 * (i + j));
         dot = fmaf(gv.x, lo, dot);
         dot = fmaf(gv.y, hi, dot);
       }
     }
-    if (WORDS == 4) *reinterpret_cast<uint4*>(dst + i) = make_uint4(out[0], out[WORDS / 4], out[WORDS / 2], out[WORDS - 1]);
-    else dst[i] = out[0];
+    for (int c = 0; c < copies; ++c) {
+      const int row = s_row[c];
+      if (row < 0) continue;
+      uint32_t* dst = reinterpret_cast<uint32_t*>(p.xs + (size_t)row * p.hidden) + i;
+      if (WORDS == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(out[0], out[WORDS / 4], out[WORDS / 2], out[WORDS - 1]);
+      else *dst = out[0];
+    }
   }
-  if (gated) {
+  if (p.gate_vec) {  // block sum in a fixed order: lanes by butterfly, then the warps one after the other
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    if (lane == 0) gate[t] = 1.f / (1.f + expf(-dot));
+    if ((tid & 31) == 0) s_part[tid >> 5] = dot;
+    __syncthreads();
+    if (tid == 0) {
+      float sum = 0.f;
+      for (int w = 0; w < kPfGatherThreads / 32; ++w) sum += s_part[w];
+      p.gate[t] = 1.f / (1.f + expf(-sum));
+    }
   }
 }
 
@@ -971,12 +1037,11 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
               const float v0 = half_of(acc[i], 0), v1 = half_of(acc[i], 1);
               const float got = __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 16);
               const float gate = up ? got : v0, upv = up ? v1 : got;
-              // silu: g / (1 + e^-g), the quotient by the reciprocal and one step of Newton's iteration.  Below -80 the
-              // result is zero in fp16 either way; the bound keeps 1 + e^-g finite.
+              // silu: g / (1 + e^-g), by the approximate reciprocal: its error, 2^-23, is 2^-12 of the rounding to fp16 that
+              // follows.  Below -80 the result is zero in fp16 either way; the bound keeps 1 + e^-g finite.
               const float t = 1.f + __expf(fminf(-gate, 80.f));
               float r;
               asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
-              r = fmaf(r, fmaf(-t, r, 1.f), r);
               if (2 * i + (up ? 1 : 0) < count) *dst = __float2half_rn(gate * r * upv);
               dst += two_rows;
             }
@@ -1012,7 +1077,6 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
 // ---- step 5: weighted combine in list order ---------------------------------------------------------------
 // A block per token: the token's rows and weights are read once into shared memory, then four slots' rows at a time are in
 // flight.
-constexpr int kPfMaxSlots = SLICEMOE_MAX_TOP_K + SLICEMOE_MAX_SHARED;
 __global__ void __launch_bounds__(256) pf_combine_kernel(const float* __restrict__ yrow, const int* __restrict__ posmap,
                                                          const float* __restrict__ weights, const float* __restrict__ gate, int k,
                                                          int n_shared, int hidden, float* __restrict__ y) {
@@ -1176,19 +1240,36 @@ extern "C" int slicemoe_prefill_layer(const slicemoe_shape* s, const slicemoe_ex
   pp.per2 = s->hidden / 128;
   pp.head = reinterpret_cast<PfHead*>(ws + L.head);
   pp.counts = reinterpret_cast<int*>(ws + L.counts);
-  pp.offsets = reinterpret_cast<int*>(ws + L.offsets);
-  pp.cursor = reinterpret_cast<int*>(ws + L.cursor);
+  pp.base = reinterpret_cast<int*>(ws + L.base);
+  pp.hist = reinterpret_cast<int*>(ws + L.hist);
   pp.runs = reinterpret_cast<PfRun*>(ws + L.runs);
-  pp.row_token = reinterpret_cast<int*>(ws + L.row_token);
-  pp.posmap = reinterpret_cast<int*>(ws + L.posmap);
+  pp.rank = reinterpret_cast<int*>(ws + L.rank);
+  pp.rank_blocks = L.rank_blocks;
   pp.status = reinterpret_cast<unsigned*>(status_out_device);
+  int* posmap = reinterpret_cast<int*>(ws + L.posmap);
+  if (L.rank_blocks > 1) {
+    rc = pf_launch(pf_rank_kernel, (unsigned)L.rank_blocks, (unsigned)kPfPlanThreads, 0, st, (PfPlanParams)pp);
+    if (rc != SLICEMOE_OK) return rc;
+  }
   rc = pf_launch(pf_plan_kernel, 1u, (unsigned)kPfPlanThreads, 0, st, (PfPlanParams)pp);
   if (rc != SLICEMOE_OK) return rc;
-  constexpr int kRowsPerBlock = kPfGatherThreads / 32;
-  rc = pf_launch((reinterpret_cast<uintptr_t>(x) & 15) ? pf_gather_kernel<1> : pf_gather_kernel<4>,
-                 (unsigned)((L.in_rows + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)kPfGatherThreads, 0, st,
-                 reinterpret_cast<const uint16_t*>(x), (int)s->hidden, (int)T, (const int*)pp.row_token, (int)(T * k), (int)L.in_rows, xs,
-                 gated ? shared_gate_vec : (const float*)nullptr, gate);
+  PfGatherParams pg;
+  pg.x = reinterpret_cast<const uint16_t*>(x);
+  pg.ids = ids;
+  pg.rank = pp.rank;
+  pg.first = pp.hist;
+  pg.T = T;
+  pg.k = k;
+  pg.E = E;
+  pg.n_shared = nsh;
+  pg.hidden = s->hidden;
+  pg.posmap = posmap;
+  pg.xs = xs;
+  pg.gate_vec = gated ? shared_gate_vec : nullptr;
+  pg.gate = gate;
+  pg.status = pp.status;
+  rc = pf_launch((reinterpret_cast<uintptr_t>(x) & 15) ? pf_gather_kernel<1> : pf_gather_kernel<4>, (unsigned)T, (unsigned)kPfGatherThreads, 0, st,
+                 (PfGatherParams)pg);
   if (rc != SLICEMOE_OK) return rc;
   PfGemmParams p;
   p.experts = experts;
@@ -1213,6 +1294,6 @@ extern "C" int slicemoe_prefill_layer(const slicemoe_shape* s, const slicemoe_ex
     rc = pf_launch_gemms<32>(p, xs, L.in_rows, L.out_rows, st);
   }
   if (rc != SLICEMOE_OK) return rc;
-  return pf_launch(pf_combine_kernel, (unsigned)T, 256u, 0, st, (const float*)yrow, (const int*)pp.posmap, weights,
+  return pf_launch(pf_combine_kernel, (unsigned)T, 256u, 0, st, (const float*)yrow, (const int*)posmap, weights,
                    gated ? (const float*)gate : (const float*)nullptr, (int)k, (int)nsh, (int)s->hidden, y);
 }
