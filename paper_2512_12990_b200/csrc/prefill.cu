@@ -913,6 +913,14 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
           for (int i = 0; i < 4; ++i) lv[i] = prec ? *reinterpret_cast<const uint4*>(slot + 8 * kURawBlock + 512 * i) : make_uint4(0, 0, 0, 0);
           if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
           tc_fence_after();
+          // the words are in registers: the raw stage is handed back before the conversion, not after
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&raw_free[rs]);
+          rs += kUSets;
+          if (rs >= kURawStages) {
+            rs -= kURawStages;
+            rpar ^= 1;
+          }
           const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + kUWCol0 + st * kUWCols;
 #pragma unroll
           for (int b = 0; b < 2; ++b) {
@@ -950,12 +958,6 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
           tmem_st_wait();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&raw_free[rs]);
-          rs += kUSets;
-          if (rs >= kURawStages) {
-            rs -= kURawStages;
-            rpar ^= 1;
-          }
           if (lane == 0) mbar_arrive(&full[st]);
           st += kUSets;
           if (st >= kUStages) {
