@@ -22,7 +22,7 @@
 
 namespace slicemoe {
 
-constexpr int kPfTileN = 192;  // most token rows of a tile
+constexpr int kPfTileN = 192, kPfNarrowN = 96;  // most token rows of a tile: the wide form, the narrow one
 constexpr int kPfTileB = 128;  // weight rows per tile: 64 gate + 64 up columns of h (GEMM 1), 128 columns of y (GEMM 2)
 constexpr int kPfChunkK = 128;  // contraction columns per pipeline step (two plane blocks; every width is a multiple)
 
@@ -88,6 +88,7 @@ struct PfPlanParams {
   int T, k, E, n_shared;
   int per1_routed, per1_shared, per2;  // work items per tile: GEMM 1 of a routed / shared expert, GEMM 2
   int rank_blocks;
+  int tile;             // most token rows of a tile
   PfHead* head;
   int *counts, *base;   // [experts]: counters that do not fit shared memory; first rows likewise
   int* hist;            // [block][E]: pairs of the expert in the block; the plan turns them into the block's first rows
@@ -123,7 +124,6 @@ __global__ void __launch_bounds__(kPfPlanThreads) pf_rank_kernel(const PfPlanPar
   __syncthreads();
   for (int e = threadIdx.x; e < p.E; e += kPfPlanThreads) p.hist[(size_t)blockIdx.x * p.E + e] = s_counts[e];
 }
-__device__ __forceinline__ int pf_tiles_of(int count) { return (count + kPfTileN - 1) / kPfTileN; }
 // Exclusive block-wide scan of one value per thread; *total gets the sum.
 __device__ int pf_block_scan(int v, int* warp_sums, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kPfPlanThreads) pf_plan_kernel(const PfPlanPar
     PfRun r;
     r.expert = e;
     r.count = c;
-    r.tiles = pf_tiles_of(c);
+    r.tiles = (c + p.tile - 1) / p.tile;
     r.in_row = e < p.E ? base[e] : npairs;
     r.out_row = e < p.E ? base[e] : npairs + (e - p.E) * p.T;
     r.items1 = r.items2 = r.pad_ = 0;
@@ -334,56 +334,66 @@ __global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const PfGat
 }
 
 // ---- steps 3 and 4: the grouped GEMM on the 5th-generation tensor cores ---------------------------------
-// One persistent CTA per SM takes work items (128 weight rows x up to 192 token rows) from a counter and computes the
+// One persistent CTA per SM takes work items (128 weight rows x a tile of token rows) from a counter and computes the
 // transposed product D[weight row, token].  Per 128-column step of the contraction:
-//   - the token warp brings the token tile (rows of x or h, fp16) into shared memory with TMA tiled copies of 32
-//     rows, 128-byte swizzle: the B operand;
-//   - the weight warps (two sets of four, taking the steps in turn) turn nibbles into fp16 integers d = q - zp (or
+//   - the token warp brings the token tile (rows of x or h, fp16) into shared memory with two TMA tiled copies of 64 columns,
+//     128-byte swizzle: the B operand; and the raw words of the LSB planes with cp.async.  Another warp copies the MSB
+//     planes' words, and scales and zero-points of 16 groups at a time;
+//   - the weight warps (sets of four, taking the steps in turn) turn nibbles into fp16 integers d = q - zp (or
 //     2^shift (q_msb - (zp >> shift))) and store them to tensor memory with tcgen05.st, one weight row per lane: the A
 //     operand.  Weights never pass through shared memory as fp16;
-//   - the MMA warp issues tcgen05.mma (M 128, K 16) for one quantisation group at a time, into one of two fp32
-//     accumulators in tensor memory.  A tile wider than 96 tokens is cut into two halves with an accumulator each; a
-//     narrower one uses them for alternate groups.  Either way one accumulator is read while the other is written;
-//   - the sum warps (two warpgroups) read a group's sums with tcgen05.ld and add them, times the weight row's scale of
-//     that group, to fp32 registers: 96 tokens per warpgroup, one weight row per lane.
-// After the last group the sum warps hold the item's result and write it: SwiGLU between gate and up rows (GEMM 1,
-// exchanged through shared memory), fp32 rows (GEMM 2).  A scheduler warp fetches items ahead and leaves their
-// description in a ring in shared memory.
+//   - the MMA warp issues tcgen05.mma (M 128, K 16, N the tile's tokens) for one quantisation group at a time, into the two
+//     fp32 accumulators in turn: one is read while the other is written;
+//   - the sum warps read a group's sums with tcgen05.ld and add them, times the weight row's scale of that group, to fp32
+//     registers: up to 96 tokens per warpgroup, one weight row per lane.
+// After the last group the sum warps hold the item's result and write it: SwiGLU between gate and up rows (GEMM 1, one
+// exchange between lanes), fp32 rows (GEMM 2).  A scheduler warp fetches items ahead and leaves their description in a ring in
+// shared memory.
 //
 // Why integers and a read-out per group: the dequantised weight s (q - zp) has up to 20 significant bits.  Kept as the
-// exact sum of two fp16 numbers (the version before this one) every product is issued twice and the conversion is twice
-// as long; the read-out costs half an instruction per value with packed multiply-adds.  Why 192 tokens: the conversion of a
-// weight tile is shared by all its tokens, and 96 sums per lane leave registers (61,440 at launch) for eight weight
-// warps, without which a tile of few tokens is bound by one set's latency.
+// exact sum of two fp16 numbers every product is issued twice and the conversion is twice as long; the read-out costs half
+// an instruction per value with packed multiply-adds.
+// Two forms, by the widest tile.  192 tokens: the conversion of a weight tile is shared by all its tokens, and 96 sums per
+// lane leave registers for eight weight warps.  96 tokens, where experts have few: the weights' way through the CTA bounds a
+// step, not the products, and the shared and tensor memory that a narrower tile leaves take four steps of tokens and five of
+// weights; one warpgroup reads the sums.  One accumulator for all of a tile's tokens: the MMA warp's serial path (a wait, eight
+// products, commits) bounds a wide step, and two accumulators of half the tile's tokens run through it twice per group.
+// Measured, one layer of 64 + 2 experts of 2048 x 1408 (us): 8,192 tokens 1499 -> 1425, 77 tokens 151 -> 135.5; 96 tokens
+// through the wide form 155, through the narrow one 138.
 // Every wait is bounded; a wait that runs out sets SLICEMOE_STATUS_WAIT_TIMEOUT and the CTA winds down (tensor memory is
 // freed on every path).
-constexpr int kUSumWarps = 8;                 // two warpgroups
-constexpr int kUSets = 2;                     // sets of four weight warps; the steps go round them
-constexpr int kUWarpTok = kUSumWarps + 4 * kUSets, kUWarpMma = kUWarpTok + 1, kUWarpSched = kUWarpTok + 2,
-              kUWarpMeta = kUWarpTok + 3;
-constexpr int kUThreads = 32 * (kUWarpTok + 4);
-// registers per thread at launch 96 (640 threads); the split's sum is the launch's: 256 x 152 + 256 x 72 + 128 x 32
-constexpr int kURegsSum = 152, kURegsWeight = 72, kURegsRest = 32;
-static_assert(256 * kURegsSum + 256 * kURegsWeight + 128 * kURegsRest <= kUThreads * 96, "register split");
-constexpr int kUStages = 3;                   // steps in flight: tokens in shared, weights in tensor memory
 constexpr int kUBoxRows = 32, kUBoxCols = 64; // a TMA copy brings a multiple of 32 token rows x 64 columns (128 bytes: the swizzle's span)
-constexpr int kUBoxes = kPfTileN / kUBoxRows; // heights a copy can have: a tensor map each
-constexpr int kUPanelBytes = kPfTileN * kUBoxCols * 2;  // half of a step's tile: 64 columns of all tokens
-constexpr int kUTileBytes = 2 * kUPanelBytes;
-constexpr int kURawStages = 4;                // steps of raw plane words in shared memory or on their way to it
 constexpr int kURawBlock = 1024;              // a row block's bytes of a step in one plane
 constexpr int kURawStep = 16 * kURawBlock;    // [plane][row block]
-constexpr int kURawBytes = kURawStages * kURawStep;
 constexpr int kUItemSlots = 8;
 // Scales and zero-points of 16 quantisation groups at a time: [8 row blocks][16 groups][16 rows], 512 + 256 bytes each
 constexpr int kUMetaGroups = 16, kUMetaStages = 2;
 constexpr int kUMetaScale = kUMetaGroups * 32, kUMetaZp = kUMetaGroups * 16;
 constexpr int kUMetaBytes = 8 * (kUMetaScale + kUMetaZp);
-constexpr int kUHalfMax = kPfTileN / 2;       // tokens per warpgroup
-constexpr int kUAccs = 3, kUAccCols = 96;     // accumulators, tensor-memory columns of one
-constexpr int kUWCol0 = kUAccs * kUAccCols, kUWCols = 64;  // weight stages: 128 fp16 per row
 constexpr int kUTmemCols = 512;
-static_assert(kUWCol0 + kUStages * kUWCols <= kUTmemCols && kUHalfMax <= kUAccCols, "tensor memory");
+constexpr int kUWCols = 64;                   // a step's weights in tensor memory: 128 fp16 per row
+// What the width of the widest tile decides.  (Narrow, 77 tokens, us: four steps of tokens 135, three 140, two 156; six steps of
+// raw words 138; three sets of weight warps 142, one 154; a second warpgroup for the sums 138.)
+template <int TN>
+struct UCfg {
+  static constexpr bool wide = TN > kPfNarrowN;
+  static constexpr int sum_wgs = wide ? 2 : 1;            // warpgroups that read sums, 96 tokens each
+  static constexpr int half_max = 96;
+  static constexpr int sets = 2;                          // sets of four weight warps; the steps go round them
+  static constexpr int sum_warps = 4 * sum_wgs, warp_tok = sum_warps + 4 * sets, warp_mma = warp_tok + 1,
+                       warp_sched = warp_tok + 2, warp_meta = warp_tok + 3;
+  static constexpr int threads = 32 * (warp_tok + 4);
+  // registers per thread: at launch, and the split, whose sum is at most the launch's
+  static constexpr int regs = wide ? 96 : 128;
+  static constexpr int regs_sum = 152, regs_weight = wide ? 72 : 128, regs_rest = wide ? 32 : 40;
+  static_assert(32 * sum_warps * regs_sum + 128 * sets * regs_weight + 128 * regs_rest <= threads * regs, "register split");
+  static constexpr int panel_bytes = TN * kUBoxCols * 2;  // half of a step's tile: 64 columns of all tokens
+  static constexpr int tile_bytes = 2 * panel_bytes;
+  static constexpr int accs = 2, acc_cols = TN;           // accumulators in tensor memory; the columns left take weights
+  static constexpr int w_col0 = accs * acc_cols, w_stages = (kUTmemCols - w_col0) / kUWCols;
+  static constexpr int tok_stages = wide ? 3 : 4;
+  static constexpr int raw_stages = 4;                    // steps of raw plane words in shared memory or on their way to it
+};
 constexpr uint32_t kUWaitCycles = 2000000000u;
 constexpr uint32_t kUCopyCycles = 2000000u;  // a millisecond: far more than any copy takes
 
@@ -395,7 +405,6 @@ struct __align__(16) PfItem {
   const uint8_t* zp[2];
   int nk;        // steps
   int n, n0;     // tokens of the tile, up to a multiple of 16; of the first warpgroup
-  int halves;    // accumulators of a group: 2 when the tile is cut in two
   int count;     // tokens that are there
   int in_row, out_row;
   int col;       // first column of h or of y
@@ -403,25 +412,30 @@ struct __align__(16) PfItem {
   int stop;      // no more items
 };
 
+template <int TN>
 struct USmem {
+  using C = UCfg<TN>;
   static constexpr int tok = 0;
-  static constexpr int raw = tok + kUStages * kUTileBytes;
-  static constexpr int meta = raw + kURawBytes;
+  static constexpr int raw = tok + C::tok_stages * C::tile_bytes;
+  static constexpr int meta = raw + C::raw_stages * kURawStep;
   static constexpr int items = meta + kUMetaStages * kUMetaBytes;
   static constexpr int bars = items + kUItemSlots * (int)sizeof(PfItem);
-  // barriers: tokens and weights of a step in / step done / sums there [accumulator] / sums read [accumulator] / item
+  // barriers: weights of a step in, used / its tokens in, used / sums there [accumulator] / sums read [accumulator] / item
   // there, item read / scales and zero-points in, read / raw words in, read / drained
-  static constexpr int full = 0, done = full + kUStages, acc_full = done + kUStages, acc_free = acc_full + kUAccs,
-                       item_full = acc_free + kUAccs, item_free = item_full + kUItemSlots, meta_full = item_free + kUItemSlots,
-                       meta_free = meta_full + kUMetaStages, raw_full = meta_free + kUMetaStages, raw_free = raw_full + kURawStages,
-                       drain = raw_free + kURawStages, nbars = drain + 1;
+  static constexpr int w_full = 0, w_free = w_full + C::w_stages, tok_full = w_free + C::w_stages, tok_free = tok_full + C::tok_stages,
+                       acc_full = tok_free + C::tok_stages, acc_free = acc_full + C::accs,
+                       item_full = acc_free + C::accs, item_free = item_full + kUItemSlots, meta_full = item_free + kUItemSlots,
+                       meta_free = meta_full + kUMetaStages, raw_full = meta_free + kUMetaStages, raw_free = raw_full + C::raw_stages,
+                       drain = raw_free + C::raw_stages, nbars = drain + 1;
   static constexpr int tail = bars + nbars * 8;  // tensor-memory address, abort flag
   static constexpr int total = tail + 16;
 };
-static_assert(USmem::bars % 8 == 0 && USmem::items % 16 == 0, "alignment");
-constexpr int kUSmemBytes = USmem::total + 1024 /* alignment slack */;
-static_assert(kUSmemBytes <= 227 * 1024, "shared memory budget");
+template <int TN>
+constexpr int kUSmemBytes = USmem<TN>::total + 1024 /* alignment slack */;
+static_assert(USmem<192>::bars % 8 == 0 && USmem<192>::items % 16 == 0, "alignment");
+static_assert(kUSmemBytes<192> <= 227 * 1024 && kUSmemBytes<kPfNarrowN> <= 227 * 1024, "shared memory budget");
 
+constexpr int kUBoxes = kPfTileN / kUBoxRows;
 struct PfMaps {
   CUtensorMap rows[kUBoxes];  // [i]: copies of 32 (i + 1) rows
 };
@@ -577,18 +591,21 @@ __device__ __forceinline__ void u_copy_raw(uint32_t dst, const uint8_t* first, c
   }
 }
 
-template <int G, int PHASE>
-__global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParams p, const __grid_constant__ PfMaps maps) {
+template <int G, int PHASE, int TN>
+__global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfGemmParams p, const __grid_constant__ PfMaps maps) {
+  using C = UCfg<TN>;
+  using S = USmem<TN>;
   constexpr int LG = G == 128 ? 7 : (G == 64 ? 6 : 5);
   extern __shared__ uint8_t u_smem_raw[];
   uint8_t* smem = u_smem_raw + ((1024 - (smem_u32(u_smem_raw) & 1023)) & 1023);
-  PfItem* items = reinterpret_cast<PfItem*>(smem + USmem::items);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + USmem::bars);
-  uint64_t *full = bars + USmem::full, *done = bars + USmem::done, *acc_full = bars + USmem::acc_full,
-           *acc_free = bars + USmem::acc_free, *item_full = bars + USmem::item_full, *item_free = bars + USmem::item_free,
-           *meta_full = bars + USmem::meta_full, *meta_free = bars + USmem::meta_free,
-           *raw_full = bars + USmem::raw_full, *raw_free = bars + USmem::raw_free, *drain = bars + USmem::drain;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + USmem::tail);
+  PfItem* items = reinterpret_cast<PfItem*>(smem + S::items);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::bars);
+  uint64_t *w_full = bars + S::w_full, *w_free = bars + S::w_free, *tok_full = bars + S::tok_full,
+           *tok_free = bars + S::tok_free, *acc_full = bars + S::acc_full,
+           *acc_free = bars + S::acc_free, *item_full = bars + S::item_full, *item_free = bars + S::item_free,
+           *meta_full = bars + S::meta_full, *meta_free = bars + S::meta_free,
+           *raw_full = bars + S::raw_full, *raw_free = bars + S::raw_free, *drain = bars + S::drain;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + S::tail);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   // the warp index by way of a shuffle: the compiler then knows that it is uniform across the warp, and keeps
@@ -596,23 +613,27 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   pf_dep_launch();
   if (tid == 0) {
-    for (int s = 0; s < kUStages; ++s) {
-      mbar_init(&full[s], 1 + 4);  // the token warp (and its copies' bytes) and a set's four warps
-      mbar_init(&done[s], 1);
+    for (int s = 0; s < C::w_stages; ++s) {
+      mbar_init(&w_full[s], 4);  // a set's four warps
+      mbar_init(&w_free[s], 1);
     }
-    for (int a = 0; a < kUAccs; ++a) {
+    for (int s = 0; s < C::tok_stages; ++s) {
+      mbar_init(&tok_full[s], 1);
+      mbar_init(&tok_free[s], 1);
+    }
+    for (int a = 0; a < C::accs; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_free[a], 8);  // the eight sum warps once each, or one warpgroup's four twice each
+      mbar_init(&acc_free[a], C::sum_warps);
     }
     for (int s = 0; s < kUItemSlots; ++s) {
       mbar_init(&item_full[s], 1);
-      mbar_init(&item_free[s], kUSumWarps + 4 * kUSets + 3);
+      mbar_init(&item_free[s], C::sum_warps + 4 * C::sets + 3);
     }
     for (int s = 0; s < kUMetaStages; ++s) {
       mbar_init(&meta_full[s], 1);
-      mbar_init(&meta_free[s], kUSumWarps + 4 * kUSets);
+      mbar_init(&meta_free[s], C::sum_warps + 4 * C::sets);
     }
-    for (int s = 0; s < kURawStages; ++s) {
+    for (int s = 0; s < C::raw_stages; ++s) {
       mbar_init(&raw_full[s], 64);  // the lanes of the two warps that copy, one plane each
       mbar_init(&raw_free[s], 4);  // the four warps of the set that takes the step
     }
@@ -620,7 +641,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == kUWarpMma) {
+  if (warp == C::warp_mma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kUTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -632,9 +653,9 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   bool alive = true;
   pf_dep_wait();  // the plan, the token rows and the counters are the work of the kernels before
 
-  if (warp >= kUWarpTok) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kURegsRest));
-    if (warp == kUWarpTok) {
+  if (warp >= C::warp_tok) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::regs_rest));
+    if (warp == C::warp_tok) {
       // ---- token tiles: two TMA copies of the tile's rows x 64 columns; and the raw LSB planes ----
       uint32_t st = 0, par = 1;  // stage; parity of the use before (the first one waits for nothing)
       uint32_t rs = 0, rpar = 1;
@@ -652,80 +673,82 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         for (int kc = 0; kc < nk; ++kc) {
           if (!mbar_wait(&raw_free[rs], rpar, abort_flag)) { alive = false; break; }
           if (prec) {
-            u_copy_raw<PHASE>(smem_u32(smem + USmem::raw + rs * kURawStep + 8 * kURawBlock + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
+            u_copy_raw<PHASE>(smem_u32(smem + S::raw + rs * kURawStep + 8 * kURawBlock + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
             p0 += kURawBlock;
             p1 += kURawBlock;
           }
           cp_async_arrive(&raw_full[rs]);
-          if (++rs == kURawStages) { rs = 0; rpar ^= 1; }
-          if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
+          if (++rs == C::raw_stages) { rs = 0; rpar ^= 1; }
+          if (!mbar_wait(&tok_free[st], par, abort_flag)) { alive = false; break; }
           if (elect_one()) {
-            mbar_expect_tx(&full[st], 2 * box * (kUBoxRows * kUBoxCols * 2));
+            mbar_expect_tx(&tok_full[st], 2 * box * (kUBoxRows * kUBoxCols * 2));
 #pragma unroll
             for (int panel = 0; panel < 2; ++panel)
               asm volatile(
                   "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-                      smem_u32(smem + USmem::tok + st * kUTileBytes + panel * kUPanelBytes)),
-                  "l"(&maps.rows[box - 1]), "r"(smem_u32(&full[st])), "r"(kc * kPfChunkK + panel * kUBoxCols), "r"(row)
+                      smem_u32(smem + S::tok + st * C::tile_bytes + panel * C::panel_bytes)),
+                  "l"(&maps.rows[box - 1]), "r"(smem_u32(&tok_full[st])), "r"(kc * kPfChunkK + panel * kUBoxCols), "r"(row)
                   : "memory");
           }
           __syncwarp();
-          if (++st == kUStages) { st = 0; par ^= 1; }
+          if (++st == C::tok_stages) { st = 0; par ^= 1; }
         }
         if (!alive) break;
       }
       asm volatile("cp.async.wait_all;" ::: "memory");
-      // No copy may still be on its way into shared memory when the CTA ends (only after a time-out can one be): the
-      // step's barrier also counts the weight warps, so it cannot tell; the longest a copy can take is waited out.
+      // No copy may still be on its way into shared memory when the CTA ends: only after a time-out can one be, and then the
+      // longest that a copy can take is waited out.
       if (!alive) {
         const uint32_t t0 = (uint32_t)clock64();
         while ((uint32_t)clock64() - t0 < kUCopyCycles) {}
       }
-    } else if (warp == kUWarpMma) {
+    } else if (warp == C::warp_mma) {
       // ---- MMA issue: D[weight row, token] += W[weight row, k] (tensor memory) x X[token, k] (shared memory) ----
       // The whole warp walks the loop, so that its state stays on the uniform datapath, where the tensor instructions take
       // their operands from; one elected lane issues.  (All of it in one lane: twice the time per step.)
-      uint32_t st = 0, par = 0;  // stage and parity of its use
-      uint32_t buf = 0, bpar = 1;  // accumulator of the next unit, parity of its use before
+      uint32_t st = 0, par = 0, ts = 0, tpar = 0;  // weight and token stage, parity of their use
+      uint32_t buf = 0, bpar = 1;  // accumulator of the next group, parity of its use before
       bool issued = false;
-      const uint64_t bd0 = umma_desc(smem_u32(smem + USmem::tok));
+      const uint64_t bd0 = umma_desc(smem_u32(smem + S::tok));
       constexpr int kGroups = 128 / G, kKs = G / 16;  // quantisation groups of a step, K 16 slices of a group
       for (uint32_t ni = 0; alive; ++ni) {
         const PfItem& it = items[ni % kUItemSlots];
         if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
         if (__shfl_sync(0xffffffffu, it.stop, 0)) break;
-        const int nk = __shfl_sync(0xffffffffu, it.nk, 0), halves = __shfl_sync(0xffffffffu, it.halves, 0),
-                  n0 = __shfl_sync(0xffffffffu, it.n0, 0), n = __shfl_sync(0xffffffffu, it.n, 0);
+        const int nk = __shfl_sync(0xffffffffu, it.nk, 0);
+        const uint32_t id = umma_idesc(__shfl_sync(0xffffffffu, it.n, 0));
         __syncwarp();
         if (elect_one()) mbar_arrive(&item_free[ni % kUItemSlots]);
-        const uint32_t id_first = umma_idesc(halves == 2 ? n0 : n), id_second = umma_idesc(n - n0);
         for (int kc = 0; kc < nk && alive; ++kc) {
-          if (!mbar_wait(&full[st], par, abort_flag)) { alive = false; break; }
-          const uint64_t bd_step = bd0 + (uint64_t)((st * kUTileBytes) >> 4);
-          const uint32_t a_step = tmem + kUWCol0 + st * kUWCols;
+          if (!mbar_wait(&tok_full[ts], tpar, abort_flag)) { alive = false; break; }
+          if (!mbar_wait(&w_full[st], par, abort_flag)) { alive = false; break; }
+          const uint64_t bd = bd0 + (uint64_t)((ts * C::tile_bytes) >> 4);
+          const uint32_t a_step = tmem + C::w_col0 + st * kUWCols;
+          const uint32_t st0 = st, ts0 = ts;
+          if (++st == C::w_stages) { st = 0; par ^= 1; }
+          if (++ts == C::tok_stages) { ts = 0; tpar ^= 1; }
 #pragma unroll
           for (int grp = 0; grp < kGroups; ++grp) {
-            for (int half = 0; half < halves; ++half) {
-              if (!mbar_wait(&acc_free[buf], bpar, abort_flag)) { alive = false; break; }
-              tc_fence_after();
-              const uint32_t d = tmem + buf * kUAccCols, id = half ? id_second : id_first;
-              const uint64_t bd = bd_step + (half ? (uint64_t)(n0 * 8) : 0ull);
-              if (elect_one()) {
+            if (!mbar_wait(&acc_free[buf], bpar, abort_flag)) { alive = false; break; }
+            tc_fence_after();
+            const uint32_t d = tmem + buf * C::acc_cols;
+            auto issue = [&](int ks) {
+              const int k16 = grp * kKs + ks;  // within the step; four to a panel
+              umma_f16_ts(d, a_step + 8 * k16, bd + (uint64_t)((k16 >> 2) * (C::panel_bytes >> 4) + 2 * (k16 & 3)), id, ks ? 1u : 0u);
+            };
+            if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < kKs; ++ks) {
-                  const int k16 = grp * kKs + ks;  // within the step; four to a panel
-                  umma_f16_ts(d, a_step + 8 * k16, bd + (uint64_t)((k16 >> 2) * (kUPanelBytes >> 4) + 2 * (k16 & 3)), id, ks ? 1u : 0u);
-                }
-                if (grp == kGroups - 1 && half == halves - 1) umma_commit(&done[st]);
-                umma_commit(&acc_full[buf]);
+              for (int ks = 0; ks < kKs; ++ks) issue(ks);
+              if (grp == kGroups - 1) {
+                umma_commit(&w_free[st0]);
+                umma_commit(&tok_free[ts0]);
               }
-              issued = true;
-              __syncwarp();
-              if (++buf == kUAccs) { buf = 0; bpar ^= 1; }
+              umma_commit(&acc_full[buf]);
             }
-            if (!alive) break;
+            issued = true;
+            __syncwarp();
+            if (++buf == C::accs) { buf = 0; bpar ^= 1; }
           }
-          if (++st == kUStages) { st = 0; par ^= 1; }
         }
       }
       // the last commits must have arrived before shared and tensor memory go away
@@ -736,7 +759,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         while (!mbar_try(drain, 0) && (uint32_t)clock64() - t0 < kUWaitCycles) {}
         __syncwarp();
       }
-    } else if (warp == kUWarpSched) {
+    } else if (warp == C::warp_sched) {
       // ---- scheduler: takes items from the counter and describes them ----
       int* next = PHASE == 1 ? &p.head->next1 : &p.head->next2;
       const int n_runs = p.head->runs, n_items = PHASE == 1 ? p.head->items1 : p.head->items2;
@@ -797,9 +820,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
           if (lane == 0) {
             it.nk = K / kPfChunkK;
             it.n = n;
-            it.halves = n > kUHalfMax ? 2 : 1;
-            // two accumulators: halves of a multiple of 16; one: the first warpgroup reads whole 32-column pieces
-            it.n0 = n > kUHalfMax ? ((n / 2 + 15) & ~15) : min(n, 32 * ((n + 63) / 64));
+            it.n0 = C::sum_wgs == 1 ? n : min(n, 32 * ((n + 63) / 64));  // the first warpgroup reads whole 32-column pieces
             it.count = count;
             it.in_row = (PHASE == 1 ? r.in_row : r.out_row) + t0;
             it.out_row = r.out_row + t0;
@@ -837,7 +858,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
             const uint32_t ms = m % kUMetaStages;
             if (!mbar_wait(&meta_free[ms], ((m / kUMetaStages) & 1) ^ 1, abort_flag)) { alive = false; break; }
             const int g0 = (kc * kPfChunkK) >> LG, gs = min(kUMetaGroups, ngroups - g0), bytes = gs * (second ? 16 : 32);
-            uint8_t* dst = smem + USmem::meta + ms * kUMetaBytes + (second ? 8 * kUMetaScale + rbk * kUMetaZp : rbk * kUMetaScale);
+            uint8_t* dst = smem + S::meta + ms * kUMetaBytes + (second ? 8 * kUMetaScale + rbk * kUMetaZp : rbk * kUMetaScale);
             const uint8_t* from = src + (size_t)g0 * (second ? 16 : 32);
             if (aligned) {
               if (lane == 0) mbar_expect_tx(&meta_full[ms], gs * 8 * 48);
@@ -852,11 +873,11 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
             ++m;
           }
           if (!mbar_wait(&raw_free[rs], rpar, abort_flag)) { alive = false; break; }
-          u_copy_raw<PHASE>(smem_u32(smem + USmem::raw + rs * kURawStep + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
+          u_copy_raw<PHASE>(smem_u32(smem + S::raw + rs * kURawStep + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
           p0 += kURawBlock;
           p1 += kURawBlock;
           cp_async_arrive(&raw_full[rs]);
-          if (++rs == kURawStages) { rs = 0; rpar ^= 1; }
+          if (++rs == C::raw_stages) { rs = 0; rpar ^= 1; }
         }
       }
       asm volatile("cp.async.wait_all;" ::: "memory");
@@ -865,26 +886,27 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         while (!mbar_try(&meta_full[i % kUMetaStages], (i / kUMetaStages) & 1) && (uint32_t)clock64() - t0 < kUWaitCycles) {}
       }
     }
-  } else if (warp >= kUSumWarps) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kURegsWeight));
+  } else if (warp >= C::sum_warps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::regs_weight));
     // ---- weights: sets of four warps take the steps in turn; warp q of a set owns tensor-memory lanes
     // [32 q, 32 q + 32), two row blocks, and stores their integers of the step into the stage's columns.  The planes are laid
     // out as the fragments of a 16-row store: plane lane 4 g + c holds rows g and g + 8, columns 16 w + 4 c + j, which
     // is what lane 4 g + c of tcgen05.st.16x256b gives.  So a lane reads 16 bytes of a plane block, converts and stores
     // them: both nibbles of every byte are used, and nothing is exchanged. ----
-    const int q = warp & 3, set = (warp - kUSumWarps) >> 2;
+    const int q = warp & 3, set = (warp - C::sum_warps) >> 2;
     const int g = lane >> 2;
-    const uint8_t* raw = smem + USmem::raw + 2 * q * kURawBlock + lane * 16;
+    const uint8_t* raw = smem + S::raw + 2 * q * kURawBlock + lane * 16;
     const int shift = p.shift;
     // row g's codes: MSB nibble at bit `shift`, LSB nibble below; row g + 8's the same from the high nibbles.  A slice
     // narrower than four bits leaves the top of its nibble zero, so what the second mask lets through beyond it is zero.
     const uint32_t mask = 0x0f0f0f0fu << shift;
     const int back = 4 - shift;
-    // (Steps are counted over all items; those of the set's parity are its own.)
-    uint32_t st = set, par = 1, m = 0, skip = set;  // stage of the next own step, parity of its use before; scale and zero-point
+    // (Steps are counted over all items; every C::sets-th is the set's own.)
+    int skip = set;
+    uint32_t st = set, par = 1, m = 0;  // stage of the next own step, parity of its use before; scale and zero-point
                                                     // stages; steps of the item before the first own one
     uint32_t rs = set, rpar = 0;                    // raw stage of the next own step, parity of this use
-    static_assert(kUSets < kUStages && kURawStages % kUSets == 0, "a set's next stage is at most once round the rings away");
+    static_assert(C::sets <= C::w_stages && C::raw_stages % C::sets == 0, "a set's next stage is at most once round the rings away");
     for (uint32_t ni = 0; alive; ++ni) {
       const PfItem& it = items[ni % kUItemSlots];
       if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
@@ -894,15 +916,14 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       const uint32_t zmask = prec ? 0xffu : 0xffu << shift;  // from the MSB slice alone: 2^shift (zp >> shift)
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
-      int kc = (int)skip;
-      skip = (uint32_t)(skip + nk) & 1u;
+      int kc = skip;
       constexpr int kMetaSteps = kUMetaGroups * G / 128;  // steps of a scale and zero-point stage
       for (int k0 = 0; k0 < nk && alive; k0 += kMetaSteps, ++m) {
         const uint32_t ms = m % kUMetaStages;
         if (!mbar_wait(&meta_full[ms], (m / kUMetaStages) & 1, abort_flag)) { alive = false; break; }
-        const uint8_t* zp_stage = smem + USmem::meta + ms * kUMetaBytes + 8 * kUMetaScale + 2 * q * kUMetaZp + g;
+        const uint8_t* zp_stage = smem + S::meta + ms * kUMetaBytes + 8 * kUMetaScale + 2 * q * kUMetaZp + g;
         const int k_end = min(nk, k0 + kMetaSteps);
-        for (; kc < k_end; kc += kUSets) {
+        for (; kc < k_end; kc += C::sets) {
           const uint8_t* zp = zp_stage + (kc - k0) * (128 / G * 16);
           if (!mbar_wait(&raw_full[rs], rpar, abort_flag)) { alive = false; break; }
           const uint8_t* slot = raw + rs * kURawStep;
@@ -911,17 +932,17 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
           for (int i = 0; i < 4; ++i) mv[i] = *reinterpret_cast<const uint4*>(slot + 512 * i);
 #pragma unroll
           for (int i = 0; i < 4; ++i) lv[i] = prec ? *reinterpret_cast<const uint4*>(slot + 8 * kURawBlock + 512 * i) : make_uint4(0, 0, 0, 0);
-          if (!mbar_wait(&done[st], par, abort_flag)) { alive = false; break; }
+          if (!mbar_wait(&w_free[st], par, abort_flag)) { alive = false; break; }
           tc_fence_after();
           // the words are in registers: the raw stage is handed back before the conversion, not after
           __syncwarp();
           if (lane == 0) mbar_arrive(&raw_free[rs]);
-          rs += kUSets;
-          if (rs >= kURawStages) {
-            rs -= kURawStages;
+          rs += C::sets;
+          if (rs >= C::raw_stages) {
+            rs -= C::raw_stages;
             rpar ^= 1;
           }
-          const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + kUWCol0 + st * kUWCols;
+          const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + C::w_col0 + st * kUWCols;
 #pragma unroll
           for (int b = 0; b < 2; ++b) {
             __half2 off[128 / G][2];  // 1024 + zero-point, rows g and g + 8, twice
@@ -958,18 +979,19 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
           tmem_st_wait();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&full[st]);
-          st += kUSets;
-          if (st >= kUStages) {
-            st -= kUStages;
+          if (lane == 0) mbar_arrive(&w_full[st]);
+          st += C::sets;
+          if (st >= C::w_stages) {
+            st -= C::w_stages;
             par ^= 1;
           }
         }
         if (alive && lane == 0) mbar_arrive(&meta_free[ms]);
       }
+      skip = kc - nk;
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kURegsSum));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::regs_sum));
     // ---- sums: warp (q, wg) owns weight rows [32 q, 32 q + 32) x the warpgroup's tokens, in fp32 registers ----
     const int q = warp & 3, wg = warp >> 2;
     uint32_t buf = 0, bpar = 0;  // accumulator of the next unit (a group's sums for the tile or half of it), parity of its use
@@ -978,47 +1000,41 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       const PfItem& it = items[ni % kUItemSlots];
       if (!mbar_wait(&item_full[ni % kUItemSlots], (ni / kUItemSlots) & 1, abort_flag)) { alive = false; break; }
       if (it.stop) break;
-      const int halves = it.halves, n0 = it.n0;
+      const int n0 = it.n0;
       const int cols = wg == 0 ? n0 : it.n - n0;  // tokens of this warpgroup
       const int ngroups = (it.nk * kPfChunkK) >> LG;
       const int count = wg == 0 ? min(it.count, n0) : it.count - n0, out_row = it.out_row + (wg == 0 ? 0 : n0), col = it.col;
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
-      const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16) + (halves == 1 && wg ? n0 : 0);
+      const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16) + (wg ? n0 : 0);
       auto next_unit = [&]() {
-        if (++buf == kUAccs) { buf = 0; bpar ^= 1; }
+        if (++buf == C::accs) { buf = 0; bpar ^= 1; }
       };
-      uint64_t acc[kUHalfMax / 2];
+      uint64_t acc[C::half_max / 2];
 #pragma unroll
-      for (int i = 0; i < kUHalfMax / 2; ++i) acc[i] = 0ull;
+      for (int i = 0; i < C::half_max / 2; ++i) acc[i] = 0ull;
       for (int g0 = 0; g0 < ngroups && alive; g0 += kUMetaGroups, ++m) {
         const uint32_t ms = m % kUMetaStages;
         if (!mbar_wait(&meta_full[ms], (m / kUMetaStages) & 1, abort_flag)) { alive = false; break; }
-        const uint8_t* sc = smem + USmem::meta + ms * kUMetaBytes + (2 * q + (lane >> 4)) * kUMetaScale + (lane & 15) * 2;
+        const uint8_t* sc = smem + S::meta + ms * kUMetaBytes + (2 * q + (lane >> 4)) * kUMetaScale + (lane & 15) * 2;
         for (int gi = min(kUMetaGroups, ngroups - g0); gi > 0; --gi, sc += 32) {
           const float s = __half2float(*reinterpret_cast<const __half*>(sc));
           const uint64_t ss = ((uint64_t)__float_as_uint(s) << 32) | __float_as_uint(s);
-          // (a tile in two halves has a unit for each warpgroup; the other one's is filled and read without this one)
-          if (halves == 2 && wg == 1) next_unit();
           if (!mbar_wait(&acc_full[buf], bpar, abort_flag)) { alive = false; break; }
           tc_fence_after();
 #pragma unroll
-          for (int c = 0; c < kUHalfMax / 32; ++c) {
+          for (int c = 0; c < C::half_max / 32; ++c) {
             if (32 * c < cols) {
               uint32_t v[32];
-              tmem_ld32(lane_base + buf * kUAccCols + 32 * c, v);
+              tmem_ld32(lane_base + buf * C::acc_cols + 32 * c, v);
 #pragma unroll
               for (int i = 0; i < 16; ++i) fma2(acc[16 * c + i], v[2 * i], v[2 * i + 1], ss);
             }
           }
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(&acc_free[buf]);
-            if (halves == 2) mbar_arrive(&acc_free[buf]);
-          }
+          if (lane == 0) mbar_arrive(&acc_free[buf]);
           next_unit();
-          if (halves == 2 && wg == 0) next_unit();
         }
         __syncwarp();
         if (alive && lane == 0) mbar_arrive(&meta_free[ms]);
@@ -1032,7 +1048,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
         const size_t two_rows = 2 * (size_t)p.ldh;
         // 16 tokens at a time, with a branch per 16: within them the chains of shuffle, exponential and reciprocal overlap
 #pragma unroll
-        for (int i0 = 0; i0 < kUHalfMax / 2; i0 += 8) {
+        for (int i0 = 0; i0 < C::half_max / 2; i0 += 8) {
           if (2 * i0 < count) {
 #pragma unroll
             for (int i = i0; i < i0 + 8; ++i) {
@@ -1052,7 +1068,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
       } else {
         float* dst = p.yrow + (size_t)out_row * p.hidden + col + 32 * q + lane;
 #pragma unroll
-        for (int i0 = 0; i0 < kUHalfMax / 2; i0 += 8) {
+        for (int i0 = 0; i0 < C::half_max / 2; i0 += 8) {
           if (2 * i0 < count) {
 #pragma unroll
             for (int i = 2 * i0; i < 2 * i0 + 16; ++i) {
@@ -1070,7 +1086,7 @@ __global__ void __launch_bounds__(kUThreads, 1) pf_umma_kernel(const PfGemmParam
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == kUWarpMma) {
+  if (warp == C::warp_mma) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kUTmemCols) : "memory");
   }
@@ -1161,7 +1177,7 @@ static int pf_launch(void (*kernel)(Args...), unsigned blocks, unsigned threads,
   return SLICEMOE_OK;
 }
 
-template <int G>
+template <int G, int TN>
 static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int in_rows, int out_rows, cudaStream_t st) {
   static bool attr_set[64];
   static int sm_count[64];
@@ -1169,8 +1185,8 @@ static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int in_rows,
   SM_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return SLICEMOE_E_UNSUPPORTED;
   if (!attr_set[dev]) {
-    SM_CUDA_TRY(cudaFuncSetAttribute(pf_umma_kernel<G, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUSmemBytes));
-    SM_CUDA_TRY(cudaFuncSetAttribute(pf_umma_kernel<G, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUSmemBytes));
+    SM_CUDA_TRY(cudaFuncSetAttribute(pf_umma_kernel<G, 1, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUSmemBytes<TN>));
+    SM_CUDA_TRY(cudaFuncSetAttribute(pf_umma_kernel<G, 2, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUSmemBytes<TN>));
     SM_CUDA_TRY(cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev));
     attr_set[dev] = true;
   }
@@ -1180,9 +1196,23 @@ static int pf_launch_gemms(const PfGemmParams& p, const __half* xs, int in_rows,
   rc = pf_tensor_maps(&tm_h, p.h, out_rows, p.ldh);
   if (rc != SLICEMOE_OK) return rc;
   // one persistent CTA per SM (shared memory admits one); each takes work items until there are none
-  rc = pf_launch(pf_umma_kernel<G, 1>, (unsigned)sm_count[dev], kUThreads, kUSmemBytes, st, p, tm_x);
+  rc = pf_launch(pf_umma_kernel<G, 1, TN>, (unsigned)sm_count[dev], UCfg<TN>::threads, kUSmemBytes<TN>, st, p, tm_x);
   if (rc != SLICEMOE_OK) return rc;
-  return pf_launch(pf_umma_kernel<G, 2>, (unsigned)sm_count[dev], kUThreads, kUSmemBytes, st, p, tm_h);
+  return pf_launch(pf_umma_kernel<G, 2, TN>, (unsigned)sm_count[dev], UCfg<TN>::threads, kUSmemBytes<TN>, st, p, tm_h);
+}
+
+template <int TN>
+static int pf_launch_gemms(int group, const PfGemmParams& p, const __half* xs, int in_rows, int out_rows, cudaStream_t st) {
+  if (group == 128) return pf_launch_gemms<128, TN>(p, xs, in_rows, out_rows, st);
+  if (group == 64) return pf_launch_gemms<64, TN>(p, xs, in_rows, out_rows, st);
+  return pf_launch_gemms<32, TN>(p, xs, in_rows, out_rows, st);
+}
+
+// Which form: narrow tiles where none is cut by them, or hardly any: up to 36 rows per expert on average.  (Where the two meet
+// depends on how uneven the routing is and on the shared experts' part: 30 rows for 60 experts and a shared one four
+// times as wide, 50 for 64 + 2, 64 and more for others; at 36 the narrow one is 3 to 13 % ahead or level.)
+static int pf_tile(const slicemoe_shape* s, int T) {
+  return T <= kPfNarrowN || (long long)T * (s->top_k + s->n_shared) <= 36ll * (s->n_experts + s->n_shared) ? kPfNarrowN : kPfTileN;
 }
 
 static int pf_check(const slicemoe_shape* s, int T) {
@@ -1247,6 +1277,7 @@ extern "C" int slicemoe_prefill_layer(const slicemoe_shape* s, const slicemoe_ex
   pp.runs = reinterpret_cast<PfRun*>(ws + L.runs);
   pp.rank = reinterpret_cast<int*>(ws + L.rank);
   pp.rank_blocks = L.rank_blocks;
+  pp.tile = pf_tile(s, T);
   pp.status = reinterpret_cast<unsigned*>(status_out_device);
   int* posmap = reinterpret_cast<int*>(ws + L.posmap);
   if (L.rank_blocks > 1) {
@@ -1288,13 +1319,8 @@ extern "C" int slicemoe_prefill_layer(const slicemoe_shape* s, const slicemoe_ex
   p.shared_inter = shared_inter;
   p.ldh = s->inter > shared_inter ? s->inter : shared_inter;
   p.shift = s->b_high - s->b_low;
-  if (s->group == 128) {
-    rc = pf_launch_gemms<128>(p, xs, L.in_rows, L.out_rows, st);
-  } else if (s->group == 64) {
-    rc = pf_launch_gemms<64>(p, xs, L.in_rows, L.out_rows, st);
-  } else {
-    rc = pf_launch_gemms<32>(p, xs, L.in_rows, L.out_rows, st);
-  }
+  rc = pp.tile == kPfNarrowN ? pf_launch_gemms<kPfNarrowN>(s->group, p, xs, L.in_rows, L.out_rows, st)
+                             : pf_launch_gemms<kPfTileN>(s->group, p, xs, L.in_rows, L.out_rows, st);
   if (rc != SLICEMOE_OK) return rc;
   return pf_launch(pf_combine_kernel, (unsigned)T, 256u, 0, st, (const float*)yrow, (const int*)posmap, weights,
                    gated ? (const float*)gate : (const float*)nullptr, (int)k, (int)nsh, (int)s->hidden, y);

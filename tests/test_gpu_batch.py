@@ -1,0 +1,73 @@
+"""Several tokens through slicemoe_layer and slicemoe_layer_routed in one pass of the batch kernels, against the float64 oracle,
+at the sizes where their split can go wrong: the fewest tokens that take them, runs of exactly, less and more than eight
+pairs of an expert, one token more than a pass holds, each group size, several chunks of the down projection.  Tolerance
+as for one token."""
+import numpy as np
+import pytest
+
+from oracle import moe
+from paper_2512_12990_b200 import synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,hidden,inter,group,n_shared,shared_inter,gated,bits", [
+    (4, 128, 128, 32, 0, 0, False, (8, 4)),       # the smallest layer, the fewest tokens
+    (8, 384, 640, 64, 2, 128, False, (8, 4)),     # runs of exactly eight for the shared experts
+    (9, 256, 2176, 128, 1, 256, True, (8, 4)),    # one more than a run holds; two chunks of the down projection
+    (16, 2176, 128, 128, 1, 2304, True, (6, 3)),  # a whole pass; the shared expert wider than the routed ones
+    (17, 256, 256, 32, 0, 0, False, (4, 2)),      # a pass and one token
+])
+def test_batches_against_the_oracle(T, hidden, inter, group, n_shared, shared_inter, gated, bits):
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    E, k = 6, 3
+    sh = synth.Shape("batch", hidden, inter, E, k, group, n_shared=n_shared, shared_inter=shared_inter,
+                     shared_sigmoid_gate=gated, n_layers=1, seed=7000 + T)
+    L = H.Layer(sh, range(E), b_high=bits[0], b_low=bits[1])
+    rng = np.random.default_rng(T)
+    ids = np.stack([rng.permutation(E)[:k] for _ in range(T)]).astype(np.int32)
+    ids[:, 0] = np.where(ids[:, 1:].min(axis=1) > 0, 0, ids[:, 0])  # expert 0 has many pairs
+    ids[1] = [4, 4, 2]                                              # an expert twice in a token
+    prec = rng.integers(0, 2, (T, k)).astype(np.uint8)
+    w = rng.random((T, k)).astype(np.float32)
+    xbits, x64 = H.x_inputs(sh, T, "batch-x")
+    x = H.to_dev_bf16(xbits)
+
+    def dev(a):
+        return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+    def layer(ids_, ws):
+        y = B.slicemoe_layer(L.cshape, L.experts_tbl, L.shared_tbl, L.gate_vec_dev, x, dev(ids_), dev(prec), dev(w), ws)
+        torch.cuda.synchronize()
+        return y.cpu().numpy(), B.slicemoe_get_status(ws)
+
+    def oracle(ids_, prec_, w_):
+        return moe.layer(x64, L.oracle_list(), ids_, prec_, w_.astype(np.float64), shared=L.oracle_shared, shared_gate_vec=L.gate_vec)
+
+    y_ref = oracle(ids, prec, w)
+    y, status = layer(ids, L.ws)
+    assert status == 0
+    for t in range(T):
+        H.assert_close(y[t], y_ref[t], f"token {t}")
+    # a workspace without the batch part: token after token
+    y, status = layer(ids, B.new_workspace(L.cshape)[:L.ws.numel() - 256])
+    assert status == 0
+    for t in range(T):
+        H.assert_close(y[t], y_ref[t], f"token {t} alone")
+    # an id out of range is skipped and reported; the workspace is fit for the next call
+    bad, w_ref = ids.copy(), w.copy()
+    bad[T - 1, 1], w_ref[T - 1, 1] = E, 0.0
+    y, status = layer(bad, L.ws)
+    assert status & B.STATUS_BAD_EXPERT_ID
+    H.assert_close(y, oracle(ids, prec, w_ref), "bad id skipped")
+    # routed in the same call
+    logits = synth.router_logits_normal(sh.seed, ("batch-logits",), T, E)
+    y, ids_r, prec_r, w_r = B.slicemoe_layer_routed(L.cshape, L.experts_tbl, L.shared_tbl, L.gate_vec_dev, x,
+                                                    dev(logits.astype(np.float32)), L.ws, rank_high=1)
+    torch.cuda.synchronize()
+    assert B.slicemoe_get_status(L.ws) == 0
+    ids_ref, _, _ = moe.route_topk(logits, k)
+    assert np.array_equal(ids_r.cpu().numpy(), ids_ref)
+    H.assert_close(y.cpu().numpy(), oracle(ids_ref, prec_r.cpu().numpy(), w_r.cpu().numpy()), "routed")
