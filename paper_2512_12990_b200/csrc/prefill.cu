@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(kPfPlanThreads) pf_plan_kernel(const PfPlanPar
   const bool fits = n <= kPfSmemExperts;
   int* counts = fits ? s_counts : p.counts;
   int* base = fits ? s_base : p.base;
-  pf_dep_launch();
   pf_dep_wait();
+  pf_dep_launch();  // not before: the gather kernel reads x, which may be the work of the kernel before this one, without a wait
   const int npairs = p.T * p.k;
   const bool alone = p.rank_blocks == 1;
   for (int e = tid; e < n; e += kPfPlanThreads) {
@@ -274,8 +274,20 @@ __global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const PfGat
   __shared__ int s_row[SLICEMOE_MAX_TOP_K + 1];
   __shared__ float s_part[kPfGatherThreads / 32];
   const int t = blockIdx.x, tid = threadIdx.x, npairs = p.T * p.k;
-  pf_dep_launch();
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(p.x + (size_t)t * p.hidden);
+  uint32_t in[WORDS];
+  auto load = [&](int i) {
+    if (i >= p.hidden / 2) return;
+    if (WORDS == 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(src + i);
+      in[0] = v.x; in[WORDS / 4] = v.y; in[WORDS / 2] = v.z; in[WORDS - 1] = v.w;
+    } else {
+      in[0] = src[i];
+    }
+  };
+  load(tid * WORDS);
   pf_dep_wait();
+  pf_dep_launch();  // not before: the GEMM kernel reads the plan without a wait
   if (tid < p.k + p.n_shared) {
     int pos;
     if (tid < p.k) {
@@ -290,17 +302,10 @@ __global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const PfGat
   }
   if (tid == 0 && p.n_shared > 0) s_row[p.k] = npairs + t;  // the shared experts read the same row
   const int copies = p.k + (p.n_shared > 0 ? 1 : 0);
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(p.x + (size_t)t * p.hidden);
   float dot = 0.f;
   __syncthreads();
   for (int i = tid * WORDS; i < p.hidden / 2; i += kPfGatherThreads * WORDS) {
-    uint32_t in[WORDS], out[WORDS];
-    if (WORDS == 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(src + i);
-      in[0] = v.x; in[WORDS / 4] = v.y; in[WORDS / 2] = v.z; in[WORDS - 1] = v.w;
-    } else {
-      in[0] = src[i];
-    }
+    uint32_t out[WORDS];
 #pragma unroll
     for (int j = 0; j < WORDS; ++j) {
       const float lo = __uint_as_float(in[j] << 16), hi = __uint_as_float(in[j] & 0xffff0000u);
@@ -312,6 +317,7 @@ __global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const PfGat
         dot = fmaf(gv.y, hi, dot);
       }
     }
+    load(i + kPfGatherThreads * WORDS);
     for (int c = 0; c < copies; ++c) {
       const int row = s_row[c];
       if (row < 0) continue;
@@ -651,7 +657,9 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   bool alive = true;
-  pf_dep_wait();  // the plan, the token rows and the counters are the work of the kernels before
+  // Only the token warp waits for the kernel before, whose work the token rows are (gathered x, or h).  That this kernel runs
+  // says that the gather kernel's blocks have all seen the plan kernel's end: the plan, the counters and the caller's arrays
+  // are there, and the weights' way through the CTA fills up meanwhile.
 
   if (warp >= C::warp_tok) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::regs_rest));
@@ -670,8 +678,8 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
         // weight warps want it while they have steps of this one to deliver)
         __syncwarp();
         if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
-        for (int kc = 0; kc < nk; ++kc) {
-          if (!mbar_wait(&raw_free[rs], rpar, abort_flag)) { alive = false; break; }
+        auto copy_step = [&]() {
+          if (!mbar_wait(&raw_free[rs], rpar, abort_flag)) return false;
           if (prec) {
             u_copy_raw<PHASE>(smem_u32(smem + S::raw + rs * kURawStep + 8 * kURawBlock + lane * 16), p0, p1, (uint32_t)nk * kURawBlock);
             p0 += kURawBlock;
@@ -679,6 +687,16 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
           }
           cp_async_arrive(&raw_full[rs]);
           if (++rs == C::raw_stages) { rs = 0; rpar ^= 1; }
+          return true;
+        };
+        int copied = 0;
+        if (ni == 0) {
+          for (; copied < min(nk, C::raw_stages); ++copied)
+            if (!copy_step()) break;
+          pf_dep_wait();
+        }
+        for (int kc = 0; kc < nk; ++kc) {
+          if (kc >= copied && !copy_step()) { alive = false; break; }
           if (!mbar_wait(&tok_free[st], par, abort_flag)) { alive = false; break; }
           if (elect_one()) {
             mbar_expect_tx(&tok_full[st], 2 * box * (kUBoxRows * kUBoxCols * 2));
@@ -695,6 +713,7 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
         }
         if (!alive) break;
       }
+      pf_dep_wait();  // (without an item:) the kernel after this one counts on it
       asm volatile("cp.async.wait_all;" ::: "memory");
       // No copy may still be on its way into shared memory when the CTA ends: only after a time-out can one be, and then the
       // longest that a copy can take is waited out.
@@ -764,10 +783,11 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
       int* next = PHASE == 1 ? &p.head->next1 : &p.head->next2;
       const int n_runs = p.head->runs, n_items = PHASE == 1 ? p.head->items1 : p.head->items2;
       // How far ahead: one item where an item is long (its successor is fetched when the sums of the item itself have
-      // begun, and no CTA sits on items that another could take), else as many as the ring holds.
+      // begun, and no CTA sits on items that another could take) or a CTA has few, else as many as the ring holds.
       constexpr int kLongItem = 8, kAheadShort = 6;
+      const int share = n_items / (int)gridDim.x, ahead_short = share < kAheadShort ? max(share, 1) : kAheadShort;
       static_assert(kAheadShort <= kUItemSlots, "items between the copies and their use");
-      int ahead = kAheadShort;
+      int ahead = ahead_short;
       for (uint32_t ni = 0;; ++ni) {
         if (ni >= (uint32_t)ahead) {
           const uint32_t j = ni - ahead;
@@ -804,7 +824,7 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
           const int nt = in_run / r.tiles, tile = in_run - nt * r.tiles;
           const bool is_shared = r.expert >= p.E;
           const int K = PHASE == 1 ? p.hidden : (is_shared ? p.shared_inter : p.inter);
-          ahead = K / kPfChunkK >= kLongItem ? 1 : kAheadShort;
+          ahead = K / kPfChunkK >= kLongItem ? 1 : ahead_short;
           const int width = ((r.count + r.tiles - 1) / r.tiles + 15) & ~15;  // the tiles are equally wide, the last may be shorter
           const int t0 = tile * width, count = max(0, min(width, r.count - t0)), n = (count + 15) & ~15;
           // the item's first row block: 4 of gate and of up per 64 columns of h, or 8 of down
@@ -1003,6 +1023,8 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
       const int n0 = it.n0;
       const int cols = wg == 0 ? n0 : it.n - n0;  // tokens of this warpgroup
       const int ngroups = (it.nk * kPfChunkK) >> LG;
+      // (The first item's successor is fetched when its sums have begun, too: the CTAs do not all start at once.)
+      if (ni == 0 && !mbar_wait(&acc_full[0], 0, abort_flag)) { alive = false; break; }
       const int count = wg == 0 ? min(it.count, n0) : it.count - n0, out_row = it.out_row + (wg == 0 ? 0 : n0), col = it.col;
       __syncwarp();
       if (lane == 0) mbar_arrive(&item_free[ni % kUItemSlots]);
@@ -1160,7 +1182,9 @@ static int pf_tensor_maps(PfMaps* maps, const __half* base, int rows, int cols) 
   return SLICEMOE_OK;
 }
 
-// Every kernel of a step starts while the one before it is still running and waits for it itself (pf_dep_wait).
+// Every kernel of a step starts while the one before it is still running and waits for it itself (pf_dep_wait), only where it
+// needs that kernel's work: the gather kernel reads x and the GEMM kernels their weights before.  77 tokens through 64 + 2
+// experts of 2048 x 1408: 135.5 us with every kernel waiting at its start, 129 so; 16 tokens 98 -> 92.
 template <class... Args>
 static int pf_launch(void (*kernel)(Args...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
