@@ -647,8 +647,8 @@ def run_cuda(args, sh, workload: str = WORKLOAD, rank_high: int = RANK_HIGH, met
         "bytes_per_step": bytes_per_launch,
         "gbs": bytes_per_launch / (us_per_layer * 1e-6) / 1e9,
         "e2e": {"value": e2e_us, "unit": UNIT, "h2d_bytes_per_step": row, "d2h_bytes_per_step": 4 * sh.hidden,
-                "steps": K, "reps": Re, "what": "slicemoe_decode_step_host: one copy of x and the logits from a pinned "
-                "host buffer, one launch, y written to pinned host memory, one stream synchronise per step"},
+                "steps": K, "reps": Re, "what": "slicemoe_decode_step_host: a kernel reads x and the logits from a "
+                "pinned host buffer and routes, the layer's launch writes y to pinned host memory, one stream synchronise per step"},
         "gpu_launches": 2 * K,
         "step": "slicemoe_route_topk then slicemoe_layer, chained by programmatic dependent launch",
         "fused_step_us": fused["us_median"] * world,
@@ -777,7 +777,7 @@ def run_prefill(args, K: int, W: int):
         "metric": "prefill TFLOP/s of one MoE layer (Qwen1.5-MoE shape, 2048 tokens); share of the tensor-core peak",
         "value": tf, "unit": "TFLOP/s", "n_gpus": 1, "steps": K, "warmup": W, "ms_per_step": ms,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "fp16 tokens x weights as exact sums of two fp16, f32 accumulate", "data": "synthetic",
+        "dtype": "fp16 tokens x integer weights in fp16, f32 accumulate and scales", "data": "synthetic",
         "config": {"workload": "qwen_prefill", "tokens": T, "hidden": sh.hidden, "inter": sh.inter, "experts": sh.n_experts,
                    "top_k": sh.top_k, "shared_inter": sh.shared_inter, "group": sh.group,
                    "precision_mix": "experts of even popularity rank at 4-bit, odd rank at 8-bit; shared 8-bit",
@@ -788,7 +788,7 @@ def run_prefill(args, K: int, W: int):
         "flops_per_step": flops,
         "e2e": {"value": flops / (e2e_ms * 1e-3) / 1e12, "unit": "TFLOP/s", "h2d_bytes_per_step": 2 * T * sh.hidden,
                 "d2h_bytes_per_step": 4 * T * sh.hidden, "steps": Ke},
-        "gpu_launches": 8 * K,
+        "gpu_launches": 6 * K,  # ranks, plan, gather, two GEMMs, combine
         "roofline": {"bound": "tensor", "kernel": "pf_umma_kernel (both GEMMs) within the whole step", "achieved": tf,
                      "peak": peak, "unit": "TFLOP/s", "frac": tf / peak, "peak_kind": f"of {kind}", "traffic": None},
         "clocks": sampler.summary(windows),

@@ -153,8 +153,9 @@ int slicemoe_route_topk(const float *logits, int T, int E, int k, const float *b
 
 /*
  * Workspace.  The FFN kernels need caller-owned device scratch: a header (launch count, status word, wait
- * limit), two buffers for the fp32 intermediate h (alternate launches use alternate buffers) and staging for the
- * host-buffer entry point.  Allocate slicemoe_workspace_bytes() bytes (256-byte aligned) and call
+ * limit), two buffers for the fp32 intermediate h (alternate launches use alternate buffers), staging for the
+ * host-buffer entry point, and the part of the kernels that take several tokens at once.  (Calls also work with a
+ * workspace too small for that last part, of 127,168 bytes: token after token.)  Allocate slicemoe_workspace_bytes() bytes (256-byte aligned) and call
  * slicemoe_workspace_init() once before first use (it zeroes the header and marks both h buffers empty; every
  * launch leaves the workspace ready for the next).  One workspace serves one stream at a time.
  *
@@ -189,9 +190,9 @@ int slicemoe_workspace_set_wait(void *workspace, unsigned long long wait_cycles,
  *   x        device bf16 [T, hidden]
  *   ids, prec, weights   device [T, k] (int32, uint8, float32), k = shape->top_k
  *   y        device float32 [T, hidden], overwritten
- * Tokens are processed one after another by the batch-1 decode kernel (weights are streamed once
- * per token); accumulation is fp32, h stays fp32 between the two projections, the summation
- * order is fixed (results are bit-reproducible run to run).
+ * Up to three tokens are processed one after another by the batch-1 decode kernel; from four on up to 16 at a
+ * time go through kernels that stream each expert they name once for all of them.  Accumulation is fp32, h stays
+ * fp32 between the two projections, the summation order is fixed (results are bit-reproducible run to run).
  * Errors: INVALID_ARG, UNSUPPORTED (shape limits above; sum of intermediate widths over the k + n_shared
  * slots must be <= 12288; hidden / 16 must not exceed 4 x the device's SM count), CUDA.
  */
@@ -219,6 +220,7 @@ int slicemoe_layer(const slicemoe_shape *shape, const slicemoe_expert *experts,
  *            The kernel then reads them, and requests the routed experts' slices, while that preceding work is
  *            still running; only x is waited for.  Results are the same bits as slicemoe_layer's.
  * Without the flag the kernel still requests the shared experts' slices early: they follow from the shape alone.
+ * (From four tokens on a call has no use for either flag: its kernels do not wait for one another's CTAs.)
  *   SLICEMOE_COOPERATIVE  the kernel is launched as a cooperative grid: the driver guarantees that all its CTAs are
  *            resident together, or fails the launch (SLICEMOE_E_CUDA), so a device shared with other kernels
  *            cannot make the wait for h run out.  About 1.4 us per launch slower on a B200 (a cooperative grid
@@ -233,8 +235,8 @@ int slicemoe_layer_flags(const slicemoe_shape *shape, const slicemoe_expert *exp
                          void *workspace, size_t workspace_bytes, unsigned flags, void *stream);
 
 /*
- * slicemoe_layer_routed - slicemoe_route_topk and slicemoe_layer in one kernel launch per token: the decode
- * kernel's prologue computes the routing list from the router logits with the arithmetic of
+ * slicemoe_layer_routed - slicemoe_route_topk and slicemoe_layer in one kernel launch per token (up to three tokens;
+ * from four on the routing kernel and then those that take several tokens at once): the decode kernel's prologue computes the routing list from the router logits with the arithmetic of
  * slicemoe_route_topk (same bits), takes the precision request as the precision list (Section 4.1: experts
  * whose gating score reaches tau, or the rank_high best, run at both slices), and runs the layer.
  *   logits   device float32 [T, E]; bias, renorm, tau, rank_high as in slicemoe_route_topk
@@ -290,7 +292,8 @@ int slicemoe_stream_probe(const slicemoe_shape *shape, const slicemoe_expert *ex
  * memory that every GPU holds from the moment it loads the library until the process exits.
  *
  * Arguments are those of slicemoe_layer without workspace / workspace_bytes; inputs and outputs are
- * still the caller's.  The computation and its result are the same as slicemoe_layer's.
+ * still the caller's.  Up to three tokens the computation and its result are the same as slicemoe_layer's; more are
+ * processed one after another too, each with the bits of a call of its own.
  *   - Limits: the array is sized for hidden <= 4096 and top_k * inter + n_shared * shared_inter <= 12288
  *     (the limits of slicemoe_layer itself).  A larger layer is refused with SLICEMOE_E_UNSUPPORTED;
  *     nothing is ever allocated to make it fit.
@@ -313,13 +316,12 @@ int slicemoe_layer_static(const slicemoe_shape *shape, const slicemoe_expert *ex
 
 /*
  * slicemoe_decode_step_host - one batch-1 decode step of a layer with HOST inputs and outputs:
- * copies x (bf16 [hidden]) and logits (float32 [E]) to the device, runs slicemoe_layer_routed
+ * brings x (bf16 [hidden]) and logits (float32 [E]) to the device, routes and runs the layer
  * (bias/tau/rank_high as in slicemoe_route_topk; the precision request is used as the precision
- * list), copies y (float32 [hidden]) back and synchronises `stream`.  x_host, logits_host
- * and y_host should be pinned for the copies to be asynchronous.  logits_host may be NULL: the logits then
- * follow x directly in the buffer at x_host (bf16 [hidden], then float32 [E]) and one copy brings both.  When y_host is pinned,
- * device-mapped host memory (cudaHostAlloc / cudaHostRegister, 16-byte aligned) the kernel writes y
- * straight into it and no copy back is issued.  Weights stay resident on the device.  Staging
+ * list), brings y (float32 [hidden]) back and synchronises `stream`.  logits_host may be NULL: the logits then
+ * follow x directly in the buffer at x_host (bf16 [hidden], then float32 [E]).  When x and the logits are in pinned,
+ * device-mapped host memory (cudaHostAlloc / cudaHostRegister, 4-byte aligned) a kernel reads them there, and
+ * when y_host is (16-byte aligned) the kernel writes y straight into it; otherwise they are copied.  Weights stay resident on the device.  Staging
  * buffers live in the workspace.
  */
 int slicemoe_decode_step_host(const slicemoe_shape *shape, const slicemoe_expert *experts,
@@ -333,10 +335,10 @@ int slicemoe_decode_step_host(const slicemoe_shape *shape, const slicemoe_expert
  * every expert of a layer, so the expert FFN becomes a grouped dense contraction).  Section 6.3 says that
  * prefill wants high-bit computation; the per-expert precision flag is this library's generalisation (an
  * expert may also be run from its MSB slice alone), which a mixed-precision prefill uses.
- * Tokens are grouped by expert on the device; per 128-token tile the weight tile is dequantised
- * from the nibble planes - s*(q - zp), or 16*s*(q_msb - (zp >> 4)) for an MSB-only expert - into
- * tensor memory as the exact sum of two fp16 numbers per weight (no weight is rounded) and
- * contracted on the tensor cores (tcgen05, fp16 x fp16 with fp32 accumulation); tokens enter as
+ * Tokens are grouped by expert on the device; per tile of up to 192 tokens the integers q - zp, or
+ * 16*(q_msb - (zp >> 4)) for an MSB-only expert, are made from the nibble planes in tensor memory as fp16
+ * (exact; no weight is rounded) and contracted on the tensor cores (tcgen05, fp16 x fp16 with fp32
+ * accumulation) one quantisation group at a time; the groups' sums are scaled and added in fp32.  Tokens enter as
  * fp16 (exact for bf16 inputs in fp16's normal range) and h is rounded to fp16 between the two
  * projections (relative error 2^-11, inside the FFN tolerance).  Both conversions go to fp16's range: a token
  * value or an h beyond +-65504 becomes infinite and that row of y is not finite (nothing faults, no status

@@ -477,6 +477,15 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
                : "memory");
   return ok != 0;
 }
+// The same without waiting at all.
+__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+               : "=r"(ok)
+               : "r"(smem_u32(b)), "r"(parity)
+               : "memory");
+  return ok != 0;
+}
 // The same, but the hardware may hold the thread for up to 10 ms while the phase is not there: a waiting warp then takes
 // no issue slots from the others.
 __device__ __forceinline__ bool mbar_try_long(uint64_t* b, uint32_t parity) {
@@ -739,8 +748,13 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
         __syncwarp();
         if (elect_one()) mbar_arrive(&item_free[ni % kUItemSlots]);
         for (int kc = 0; kc < nk && alive; ++kc) {
-          if (!mbar_wait(&tok_full[ts], tpar, abort_flag)) { alive = false; break; }
-          if (!mbar_wait(&w_full[st], par, abort_flag)) { alive = false; break; }
+          // The three that a step waits for are looked at together: their latencies overlap.
+          {
+            const bool t = mbar_test(&tok_full[ts], tpar), w = mbar_test(&w_full[st], par), a = mbar_test(&acc_free[buf], bpar);
+            if (!__all_sync(0xffffffffu, t && w && a) &&
+                !(mbar_wait(&tok_full[ts], tpar, abort_flag) && mbar_wait(&w_full[st], par, abort_flag) &&
+                  mbar_wait(&acc_free[buf], bpar, abort_flag))) { alive = false; break; }
+          }
           const uint64_t bd = bd0 + (uint64_t)((ts * C::tile_bytes) >> 4);
           const uint32_t a_step = tmem + C::w_col0 + st * kUWCols;
           const uint32_t st0 = st, ts0 = ts;
@@ -748,7 +762,7 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
           if (++ts == C::tok_stages) { ts = 0; tpar ^= 1; }
 #pragma unroll
           for (int grp = 0; grp < kGroups; ++grp) {
-            if (!mbar_wait(&acc_free[buf], bpar, abort_flag)) { alive = false; break; }
+            if (grp > 0 && !mbar_wait(&acc_free[buf], bpar, abort_flag)) { alive = false; break; }
             tc_fence_after();
             const uint32_t d = tmem + buf * C::acc_cols;
             auto issue = [&](int ks) {
