@@ -218,15 +218,7 @@ class PackedMat:
 
 def slicemoe_pack(W, group: int, b_high: int = 8, b_low: int = 4, stream=None, out: PackedMat | None = None) -> PackedMat:
     """W: CUDA float32 [N, K] contiguous.  Allocates the outputs with torch unless `out` is given."""
-    import torch
-    assert W.is_cuda and W.dtype == torch.float32 and W.is_contiguous() and W.dim() == 2
-    N, K = W.shape
-    if out is None:
-        return PackedMat(N, K, group, *(_m or _marshal()).pack_new(W, group, b_high, b_low, stream))
-    rc = lib().slicemoe_pack(_ptr(W), N, K, group, b_high, b_low, _ptr(out.msb), _ptr(out.lsb), _ptr(out.scale),
-                             _ptr(out.zp), _stream(stream))
-    _check(rc, "slicemoe_pack")
-    return out
+    return (_m or _marshal()).pack(PackedMat, W, group, b_high, b_low, stream, out)
 
 
 def slicemoe_unpack_plane(plane, N: int, K: int, stream=None):

@@ -214,11 +214,40 @@ PyObject* py_setup(SM_ARGS) {  // (error type, dict name -> address)
   });
 }
 
-PyObject* py_pack_new(SM_ARGS) {  // W, group, b_high, b_low, stream -> (msb, lsb, scale, zp)
+PyObject* py_pack(SM_ARGS) {  // PackedMat, W, group, b_high, b_low, stream, out -> out, or a new PackedMat
   return guarded([&]() -> PyObject* {
-    want(n, 5);
-    const at::Tensor& W = tensor(a[0], "W");
-    const int N = (int)W.size(0), K = (int)W.size(1), group = integer32(a[1]);
+    want(n, 7);
+    if (!THPVariable_Check(a[1])) {
+      PyErr_Format(PyExc_AttributeError, "W: a tensor is wanted, got %s", Py_TYPE(a[1])->tp_name);
+      throw Failed();
+    }
+    const at::Tensor& W = THPVariable_Unpack(a[1]);
+    if (!(W.is_cuda() && W.scalar_type() == at::kFloat && W.is_contiguous() && W.dim() == 2)) {
+      PyErr_SetString(PyExc_AssertionError, "W: a contiguous CUDA float32 matrix is wanted");
+      throw Failed();
+    }
+    const int N = (int)W.size(0), K = (int)W.size(1), group = integer32(a[2]), bh = integer32(a[3]), bl = integer32(a[4]);
+    void* st = stream_of(a[5]);
+    auto call = [&](void* msb, void* lsb, void* scale, void* zp) {
+      check(unlocked([&] {
+              return lib.pack(static_cast<const float*>(W.data_ptr()), N, K, group, bh, bl, msb, lsb, static_cast<uint16_t*>(scale),
+                              static_cast<uint8_t*>(zp), st);
+            }),
+            "slicemoe_pack");
+    };
+    if (a[6] != Py_None) {
+      void* p[4];
+      const char* names[4] = {"msb", "lsb", "scale", "zp"};
+      for (int i = 0; i < 4; ++i) {
+        PyObject* o = PyObject_GetAttrString(a[6], names[i]);
+        if (!o) throw Failed();
+        const at::Tensor* t = THPVariable_Check(o) ? &THPVariable_Unpack(o) : nullptr;
+        p[i] = t ? t->data_ptr() : o == Py_None ? nullptr : address(o);
+        Py_DECREF(o);
+      }
+      call(p[0], p[1], p[2], p[3]);
+      return Py_NewRef(a[6]);
+    }
     const int64_t nb = std::max<int64_t>((int64_t)lib.plane_bytes(N, K), 1);
     const int64_t nm = std::max<int64_t>(group > 0 ? (int64_t)lib.meta_count(N, K, group) : 1, 1);
     const at::Device dev = W.device();
@@ -229,14 +258,19 @@ PyObject* py_pack_new(SM_ARGS) {  // W, group, b_high, b_low, stream -> (msb, ls
     const at::Tensor &scale = meta[0], &zp = meta[1];
     scale.unsafeGetTensorImpl()->set_sizes_contiguous({nm});
     zp.unsafeGetTensorImpl()->set_sizes_contiguous({nm});
-    const int bh = integer32(a[2]), bl = integer32(a[3]);
-    void* st = stream_of(a[4]);
-    check(unlocked([&] {
-            return lib.pack(static_cast<const float*>(W.data_ptr()), N, K, group, bh, bl, msb.data_ptr(), lsb.data_ptr(),
-                            static_cast<uint16_t*>(scale.data_ptr()), static_cast<uint8_t*>(zp.data_ptr()), st);
-          }),
-          "slicemoe_pack");
-    return tuple_of({&msb, &lsb, &scale, &zp});
+    call(msb.data_ptr(), lsb.data_ptr(), scale.data_ptr(), zp.data_ptr());
+    PyObject* args[7] = {};
+    PyObject* r = nullptr;
+    args[0] = PyLong_FromLong(N);
+    args[1] = PyLong_FromLong(K);
+    args[2] = Py_NewRef(a[2]);
+    const at::Tensor* t[4] = {&msb, &lsb, &scale, &zp};
+    bool ok = args[0] && args[1];
+    for (int i = 0; i < 4 && ok; ++i) ok = (args[3 + i] = THPVariable_Wrap(*t[i])) != nullptr;
+    if (ok) r = PyObject_Vectorcall(a[0], args, 7, nullptr);
+    for (PyObject* o : args) Py_XDECREF(o);
+    if (!r) throw Failed();
+    return r;
   });
 }
 
@@ -474,7 +508,7 @@ PyObject* py_prefill_layer(SM_ARGS) {
 }
 
 #define SM_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_##name)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {SM_METHOD(setup),        SM_METHOD(pack_new),         SM_METHOD(route_topk),
+PyMethodDef methods[] = {SM_METHOD(setup),        SM_METHOD(pack),         SM_METHOD(route_topk),
                          SM_METHOD(expert_ffn),   SM_METHOD(layer),            SM_METHOD(layer_static),
                          SM_METHOD(layer_routed), SM_METHOD(decode_step_host), SM_METHOD(prefill_layer),
                          SM_METHOD(dbsc_assign),
