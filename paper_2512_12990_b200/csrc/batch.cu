@@ -839,7 +839,13 @@ __global__ void __launch_bounds__(kBCombineThreads) batch_combine_kernel(const B
       a.y = fmaf(__int_as_float(at.w), v[j].y, a.y);
     }
   }
-  *reinterpret_cast<float2*>(p.y + (size_t)t * p.hidden + col) = a;
+  float* y = p.y + (size_t)t * p.hidden + col;
+  if ((reinterpret_cast<uintptr_t>(y) & 7) == 0) {
+    *reinterpret_cast<float2*>(y) = a;
+  } else {  // a caller's y that starts on any float, as the batch-1 kernel takes it
+    y[0] = a.x;
+    y[1] = a.y;
+  }
 }
 
 // ---- host side ---------------------------------------------------------------------------------------------

@@ -71,3 +71,26 @@ def test_batches_against_the_oracle(T, hidden, inter, group, n_shared, shared_in
     ids_ref, _, _ = moe.route_topk(logits, k)
     assert np.array_equal(ids_r.cpu().numpy(), ids_ref)
     H.assert_close(y.cpu().numpy(), oracle(ids_ref, prec_r.cpu().numpy(), w_r.cpu().numpy()), "routed")
+
+
+def _random_lists(rng, T, E, k):
+    ids = np.stack([rng.permutation(E)[:k] for _ in range(T)]).astype(np.int32)
+    return ids, rng.integers(0, 2, (T, k)).astype(np.uint8), rng.random((T, k)).astype(np.float32)
+
+
+def test_a_result_buffer_may_start_on_any_float():
+    """As for one token, nothing is asked of y's alignment: a view one float into a buffer gets the same bits."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    T, E, k = 4, 6, 3
+    sh = synth.Shape("batch", 256, 128, E, k, 64, n_shared=0, shared_inter=0, shared_sigmoid_gate=False, n_layers=1, seed=7100)
+    L = H.Layer(sh, range(E))
+    ids, prec, w = (torch.from_numpy(a).cuda() for a in _random_lists(np.random.default_rng(1), T, E, k))
+    x = H.to_dev_bf16(H.x_inputs(sh, T, "batch-y")[0])
+    want = B.slicemoe_layer(L.cshape, L.experts_tbl, None, None, x, ids, prec, w, L.ws)
+    buf = torch.full((T * sh.hidden + 2,), 7.0, device="cuda")
+    y = buf[1:-1].view(T, sh.hidden)
+    assert y.data_ptr() % 8 == 4
+    B.slicemoe_layer(L.cshape, L.experts_tbl, None, None, x, ids, prec, w, L.ws, y=y)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want) and buf[0] == 7.0 and buf[-1] == 7.0
