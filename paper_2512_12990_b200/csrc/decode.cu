@@ -1370,6 +1370,22 @@ struct FusedRouting {
   float* weights_out;
 };
 
+// What a layer call refuses beyond missing arguments, of a checked shape; the device's index and number of SMs.
+static int check_layer(const slicemoe_shape* shape, const slicemoe_expert* shared, int n_shared, const float* gate_vec, const void* x,
+                       const void* workspace, size_t workspace_bytes, int* dev, int* sms) {
+  if (n_shared > 0 && !shared) return SLICEMOE_E_INVALID_ARG;
+  if (n_shared > 0 && shape->shared_sigmoid_gate && !gate_vec) return SLICEMOE_E_INVALID_ARG;
+  if (workspace_bytes < kWsBytes || (reinterpret_cast<uintptr_t>(workspace) & 255)) return SLICEMOE_E_INVALID_ARG;
+  if (reinterpret_cast<uintptr_t>(x) & 15) return SLICEMOE_E_INVALID_ARG;
+  const long long hsum = (long long)shape->top_k * shape->inter + (long long)n_shared * shape->shared_inter;
+  if (hsum > kHCap) return SLICEMOE_E_UNSUPPORTED;
+  const int rc = device_setup(dev, sms);
+  if (rc != SLICEMOE_OK) return rc;
+  // at most 4 output row blocks per CTA: what the consumer groups' phase-2 chunk lists are sized for
+  if ((shape->hidden / 16 + *sms - 1) / *sms > 4) return SLICEMOE_E_UNSUPPORTED;
+  return SLICEMOE_OK;
+}
+
 static int run_layer(const slicemoe_shape* shape, const slicemoe_expert* experts, const slicemoe_expert* shared,
                      int n_shared, const float* gate_vec, const void* x, int T, const int32_t* ids,
                      const uint8_t* prec, const float* weights, float* y, void* workspace, size_t workspace_bytes,
@@ -1381,17 +1397,9 @@ static int run_layer(const slicemoe_shape* shape, const slicemoe_expert* experts
   if (fused && shape->n_experts > 32 * ROUTE_MAX_VPT) return SLICEMOE_E_UNSUPPORTED;
   if ((flags & ~(unsigned)(SLICEMOE_LISTS_RESIDENT | SLICEMOE_COOPERATIVE)) != 0u || (fused && flags != 0u)) return SLICEMOE_E_INVALID_ARG;
   const bool coop = (flags & SLICEMOE_COOPERATIVE) != 0u;
-  if (n_shared > 0 && !shared) return SLICEMOE_E_INVALID_ARG;
-  if (n_shared > 0 && shape->shared_sigmoid_gate && !gate_vec) return SLICEMOE_E_INVALID_ARG;
-  if (workspace_bytes < kWsBytes || (reinterpret_cast<uintptr_t>(workspace) & 255)) return SLICEMOE_E_INVALID_ARG;
-  if (reinterpret_cast<uintptr_t>(x) & 15) return SLICEMOE_E_INVALID_ARG;
-  const long long hsum = (long long)shape->top_k * shape->inter + (long long)n_shared * shape->shared_inter;
-  if (hsum > kHCap) return SLICEMOE_E_UNSUPPORTED;
   int dev, sms;
-  rc = device_setup(&dev, &sms);
+  rc = check_layer(shape, shared, n_shared, gate_vec, x, workspace, workspace_bytes, &dev, &sms);
   if (rc != SLICEMOE_OK) return rc;
-  // at most 4 output row blocks per CTA: what the consumer groups' phase-2 chunk lists are sized for
-  if ((shape->hidden / 16 + sms - 1) / sms > 4) return SLICEMOE_E_UNSUPPORTED;
 
   DecodeParams p;
   p.experts = experts;
@@ -1583,15 +1591,12 @@ extern "C" int slicemoe_layer_routed(const slicemoe_shape* shape, const slicemoe
                    workspace_bytes, stream, &f);
 }
 
-extern "C" int slicemoe_decode_step_host(const slicemoe_shape* shape, const slicemoe_expert* experts,
-                                         const slicemoe_expert* shared, const float* shared_gate_vec,
-                                         const void* x_host, const float* logits_host, const float* bias, int renorm,
-                                         float tau, int rank_high, float* y_host, void* workspace,
-                                         size_t workspace_bytes, void* stream) {
-  int rc = check_shape(shape);
-  if (rc != SLICEMOE_OK) return rc;
-  if (!x_host || !y_host || !workspace || workspace_bytes < kWsBytes) return SLICEMOE_E_INVALID_ARG;
-  if (shape->n_experts > 512) return SLICEMOE_E_UNSUPPORTED;
+namespace slicemoe {
+// Everything of a host step but its last synchronisation, on checked arguments.
+static int enqueue_host_step(const slicemoe_shape* shape, const slicemoe_expert* experts, const slicemoe_expert* shared,
+                             const float* shared_gate_vec, const void* x_host, const float* logits_host, const float* bias,
+                             int renorm, float tau, int rank_high, float* y_host, void* workspace, size_t workspace_bytes,
+                             void* stream) {
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   cudaStream_t st = (cudaStream_t)stream;
   void* dx = ws + kWsStX;
@@ -1622,7 +1627,6 @@ extern "C" int slicemoe_decode_step_host(const slicemoe_shape* shape, const slic
                                                         logits_host ? static_cast<const void*>(logits_host)
                                                                     : static_cast<const uint8_t*>(x_host) + 2 * (size_t)shape->hidden, 4));
   if (logits_mapped) {
-    if (!experts || (shape->n_shared > 0 && (!shared || (shape->shared_sigmoid_gate && !shared_gate_vec)))) return SLICEMOE_E_INVALID_ARG;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1);
     cfg.blockDim = dim3(kStageThreads);
@@ -1635,10 +1639,9 @@ extern "C" int slicemoe_decode_step_host(const slicemoe_shape* shape, const slic
     SM_CUDA_TRY(cudaLaunchKernelEx(&cfg, stage_step_kernel, reinterpret_cast<const uint32_t*>(x_mapped), logits_mapped, (int)shape->hidden,
                                    (int)shape->n_experts, (int)shape->top_k, bias, renorm, tau, rank_high,
                                    reinterpret_cast<uint32_t*>(dx), dids, dw, dprec));
-    rc = slicemoe_layer(shape, experts, shared, shared_gate_vec, dx, 1, dids, dprec, dw, dy, workspace, workspace_bytes, stream);
+    const int rc = slicemoe_layer(shape, experts, shared, shared_gate_vec, dx, 1, dids, dprec, dw, dy, workspace, workspace_bytes, stream);
     if (rc != SLICEMOE_OK) return rc;
     if (!y_direct) SM_CUDA_TRY(cudaMemcpyAsync(y_host, dy, 4 * (size_t)shape->hidden, cudaMemcpyDeviceToHost, st));
-    SM_CUDA_TRY(cudaStreamSynchronize(st));
     return SLICEMOE_OK;
   }
   if (logits_host) {
@@ -1648,12 +1651,35 @@ extern "C" int slicemoe_decode_step_host(const slicemoe_shape* shape, const slic
     SM_CUDA_TRY(cudaMemcpyAsync(dx, x_host, 2 * (size_t)shape->hidden + 4 * (size_t)shape->n_experts,
                                 cudaMemcpyHostToDevice, st));
   }
-  rc = slicemoe_layer_routed(shape, experts, shared, shared_gate_vec, dx, 1, dlogits, bias, renorm, tau, rank_high, dids,
-                             dprec, dw, dy, workspace, workspace_bytes, stream);
+  const int rc = slicemoe_layer_routed(shape, experts, shared, shared_gate_vec, dx, 1, dlogits, bias, renorm, tau, rank_high, dids,
+                                       dprec, dw, dy, workspace, workspace_bytes, stream);
   if (rc != SLICEMOE_OK) return rc;
   if (!y_direct) SM_CUDA_TRY(cudaMemcpyAsync(y_host, dy, 4 * (size_t)shape->hidden, cudaMemcpyDeviceToHost, st));
-  SM_CUDA_TRY(cudaStreamSynchronize(st));
   return SLICEMOE_OK;
+}
+}  // namespace slicemoe
+
+extern "C" int slicemoe_decode_step_host(const slicemoe_shape* shape, const slicemoe_expert* experts,
+                                         const slicemoe_expert* shared, const float* shared_gate_vec,
+                                         const void* x_host, const float* logits_host, const float* bias, int renorm,
+                                         float tau, int rank_high, float* y_host, void* workspace,
+                                         size_t workspace_bytes, void* stream) {
+  int rc = check_shape(shape);
+  if (rc != SLICEMOE_OK) return rc;
+  if (!x_host || !y_host || !workspace || workspace_bytes < kWsBytes) return SLICEMOE_E_INVALID_ARG;
+  if (shape->n_experts > 512) return SLICEMOE_E_UNSUPPORTED;
+  if (!experts) return SLICEMOE_E_INVALID_ARG;
+  // all that the layer call would refuse is refused before a kernel that reads the caller's buffers is enqueued
+  int dev, sms;
+  rc = check_layer(shape, shared, shape->n_shared, shared_gate_vec, static_cast<uint8_t*>(workspace) + kWsStX, workspace, workspace_bytes,
+                   &dev, &sms);
+  if (rc != SLICEMOE_OK) return rc;
+  rc = enqueue_host_step(shape, experts, shared, shared_gate_vec, x_host, logits_host, bias, renorm, tau, rank_high, y_host, workspace,
+                         workspace_bytes, stream);
+  // also after an error: the caller may free its buffers when the call returns, and part of the step may be enqueued
+  const cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
+  if (rc == SLICEMOE_OK) SM_CUDA_TRY(e);
+  return rc;
 }
 
 // ---- entry point for callers that cannot allocate -----------------------------------------------------

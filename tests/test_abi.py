@@ -81,3 +81,26 @@ def test_argument_errors_are_codes_not_faults():
     assert L.slicemoe_workspace_set_wait(ctypes.c_void_p(8), 1000, 0, None) == B.E_INVALID_ARG   # not 256-byte aligned
     assert L.slicemoe_dbsc_create(-1, 1, 1, -1.0, 10) is None
     assert L.slicemoe_dbsc_request(None, 0, 0, 0, 0, None, None, None) == B.E_INVALID_ARG
+
+
+def test_a_refused_host_step_has_enqueued_nothing():
+    """What the layer call inside would refuse, slicemoe_decode_step_host refuses before its first CUDA call (a kernel
+    that read the caller's pinned buffers would still be running when the call returns): the codes below, and not a CUDA
+    error, also where there is no GPU."""
+    import ctypes
+    L = B.lib()
+    one, ws, big = ctypes.c_void_p(16), ctypes.c_void_p(4096), 1 << 24
+    x = (ctypes.c_uint8 * 8192)()
+    logits, y = (ctypes.c_float * 64)(), (ctypes.c_float * 2048)()
+
+    def step(sh, experts=one, shared=one, gate=one, workspace=ws):
+        return L.slicemoe_decode_step_host(ctypes.byref(sh), experts, shared, gate, ctypes.addressof(x), ctypes.addressof(logits), None, 0,
+                                           2.0, 0, ctypes.addressof(y), workspace, big, None)
+
+    assert step(B.make_shape(2048, 2048, 64, 7, 128)) == B.E_UNSUPPORTED           # widths add up to more than 12288
+    gated = B.make_shape(2048, 1408, 64, 4, 128, 1, 1408, True)
+    assert step(gated, experts=None) == B.E_INVALID_ARG
+    assert step(gated, shared=None) == B.E_INVALID_ARG
+    assert step(gated, gate=None) == B.E_INVALID_ARG
+    assert step(gated, workspace=ctypes.c_void_p(4096 + 2)) == B.E_INVALID_ARG
+    assert step(B.make_shape(8192, 1408, 64, 4, 128)) == B.E_UNSUPPORTED
