@@ -321,7 +321,7 @@ int slicemoe_layer_static(const slicemoe_shape *shape, const slicemoe_expert *ex
  * list), brings y (float32 [hidden]) back and synchronises `stream`.  logits_host may be NULL: the logits then
  * follow x directly in the buffer at x_host (bf16 [hidden], then float32 [E]).  When x and the logits are in pinned,
  * device-mapped host memory (cudaHostAlloc / cudaHostRegister, 4-byte aligned) a kernel reads them there, and
- * when y_host is (16-byte aligned) the kernel writes y straight into it; otherwise they are copied.  Weights stay resident on the device.  Staging
+ * when y_host is (16-byte aligned) the kernel writes y straight into it; otherwise they are copied.  A buffer that is registered in part is refused (INVALID_ARG).  Weights stay resident on the device.  Staging
  * buffers live in the workspace.
  */
 int slicemoe_decode_step_host(const slicemoe_shape *shape, const slicemoe_expert *experts,

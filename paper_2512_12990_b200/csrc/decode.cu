@@ -1592,6 +1592,25 @@ extern "C" int slicemoe_layer_routed(const slicemoe_shape* shape, const slicemoe
 }
 
 namespace slicemoe {
+// A caller's host buffer and where the device sees it.  Every page is asked about: of a buffer that is registered in part a
+// kernel would touch pages that the device does not have (a copy of it fails as well, so such a call is refused).
+struct HostBuffer {
+  uint8_t* dev = nullptr;  // null: not registered
+  bool look(const void* host, size_t bytes) {
+    constexpr uintptr_t kPage = 4096;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(host);
+    for (uintptr_t p = at; p < at + bytes; p = (p | (kPage - 1)) + 1) {
+      cudaPointerAttributes attr;
+      uint8_t* d = nullptr;
+      if (cudaPointerGetAttributes(&attr, reinterpret_cast<const void*>(p)) != cudaSuccess) (void)cudaGetLastError();  // not registered
+      else if (attr.type == cudaMemoryTypeHost && attr.devicePointer) d = static_cast<uint8_t*>(attr.devicePointer);
+      if (p == at) dev = d;
+      else if (d != (dev ? dev + (p - at) : nullptr)) return false;
+    }
+    return true;
+  }
+  bool mapped(unsigned align) const { return dev && (reinterpret_cast<uintptr_t>(dev) & (align - 1)) == 0; }
+};
 // Everything of a host step but its last synchronisation, on checked arguments.
 static int enqueue_host_step(const slicemoe_shape* shape, const slicemoe_expert* experts, const slicemoe_expert* shared,
                              const float* shared_gate_vec, const void* x_host, const float* logits_host, const float* bias,
@@ -1608,24 +1627,17 @@ static int enqueue_host_step(const slicemoe_shape* shape, const slicemoe_expert*
   uint8_t* dprec = ws + kWsStPrec;
   float* dy = reinterpret_cast<float*>(ws + kWsStY);
   // y_host in pinned (device-mapped) host memory: the kernel writes its 16 output rows per CTA straight
-  // into it and the copy back falls away; otherwise y goes through the staging area.
-  auto mapped = [](const void* host, unsigned align) -> void* {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, host) == cudaSuccess && attr.type == cudaMemoryTypeHost && attr.devicePointer &&
-        (reinterpret_cast<uintptr_t>(attr.devicePointer) & (align - 1)) == 0)
-      return attr.devicePointer;
-    (void)cudaGetLastError();  // an unregistered pointer is not an error here
-    return nullptr;
-  };
-  void* y_mapped = mapped(y_host, 16);
-  const bool y_direct = y_mapped != nullptr;
-  if (y_direct) dy = reinterpret_cast<float*>(y_mapped);
-  // x and the logits likewise are read where they are
-  const void* x_mapped = mapped(x_host, 4);
-  const float* logits_mapped = x_mapped == nullptr ? nullptr
-                                                  : reinterpret_cast<const float*>(mapped(
-                                                        logits_host ? static_cast<const void*>(logits_host)
-                                                                    : static_cast<const uint8_t*>(x_host) + 2 * (size_t)shape->hidden, 4));
+  // into it and the copy back falls away; otherwise y goes through the staging area.  x and the logits likewise are read
+  // where they are.
+  const size_t x_bytes = 2 * (size_t)shape->hidden, logits_bytes = 4 * (size_t)shape->n_experts;
+  HostBuffer hy, hx, hl;
+  if (!hy.look(y_host, 4 * (size_t)shape->hidden) || !hx.look(x_host, x_bytes) ||
+      !hl.look(logits_host ? static_cast<const void*>(logits_host) : static_cast<const uint8_t*>(x_host) + x_bytes, logits_bytes))
+    return SLICEMOE_E_INVALID_ARG;
+  const bool y_direct = hy.mapped(16);
+  if (y_direct) dy = reinterpret_cast<float*>(hy.dev);
+  const void* x_mapped = hx.dev;
+  const float* logits_mapped = hx.mapped(4) && hl.mapped(4) ? reinterpret_cast<const float*>(hl.dev) : nullptr;
   if (logits_mapped) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1);

@@ -393,3 +393,43 @@ def test_narrower_slice_formats_decode(name, b_high, b_low):
         refs[label] = y_ref
     # the low-bit result really is a different (coarser) model
     assert np.linalg.norm(refs["both slices"] - refs["MSB only"]) > 2e-2 * np.linalg.norm(refs["both slices"])
+
+
+def test_host_step_refuses_a_buffer_that_is_registered_in_part():
+    """A kernel reads and writes registered host buffers in place, so all of their pages have to be registered: where only
+    some are, the call is refused on the host with nothing enqueued, and the next call works."""
+    import ctypes
+    import mmap
+    torch = _torch()
+    from paper_2512_12990_b200 import binding as B
+    sh = synth.Shape("host", 2048, 128, 8, 2, 128, n_layers=1, seed=4711)
+    L = H.Layer(sh, range(sh.n_experts))
+    xbits, _ = H.x_inputs(sh, 1)
+    xh = torch.from_numpy(xbits.view(np.int16).copy()).view(torch.bfloat16)[0].pin_memory()
+    lh = torch.randn(sh.n_experts).pin_memory()
+    yh = torch.empty(sh.hidden).pin_memory()
+
+    def step(x, y):
+        return B.slicemoe_decode_step_host(L.cshape, L.experts_tbl, None, None, x, lh, y, L.ws, rank_high=1)
+
+    want = step(xh, yh).clone()
+    pages = mmap.mmap(-1, 6 * 4096)
+    raw = torch.frombuffer(pages, dtype=torch.uint8)
+    x = raw[2048:2048 + 4096].view(torch.bfloat16)                  # pages 0 and 1
+    y = raw[3 * 4096:5 * 4096].view(torch.float32)                  # pages 3 and 4
+    x.copy_(xh)
+    rt = torch.cuda.cudart()
+    try:
+        for first in (0, 4):                                        # the first page of x, the last of y
+            assert int(rt.cudaHostRegister(raw.data_ptr() + first * 4096, 4096, 0)) == 0
+        for args in ((x, yh), (xh, y)):
+            with pytest.raises(B.SliceMoEError) as e:
+                step(*args)
+            assert e.value.code == B.E_INVALID_ARG
+        assert int(rt.cudaHostRegister(raw.data_ptr() + 4096, 4096, 0)) == 0
+        assert int(rt.cudaHostRegister(raw.data_ptr() + 3 * 4096, 4096, 0)) == 0
+        assert torch.equal(step(x, y), want)                        # whole, if in pieces
+    finally:
+        for page in (0, 1, 3, 4):
+            rt.cudaHostUnregister(raw.data_ptr() + page * 4096)
+    assert torch.equal(step(xh, yh), want)
