@@ -176,8 +176,9 @@ int slicemoe_get_status(void *workspace, int *status_out, void *stream);
  * and a switch that makes the kernels treat h as never complete.  extra_arrivals is 0 in any real use; a
  * non-zero value makes the wait for h run out by construction, which is how the time-out path
  * is exercised without faulting or hanging anything: the kernel returns by itself after `wait_cycles`,
- * SLICEMOE_STATUS_WAIT_TIMEOUT is set and y is not valid.  slicemoe_workspace_init resets both.  Enqueued
- * on `stream`.
+ * SLICEMOE_STATUS_WAIT_TIMEOUT is set and y is not valid.  (In a call of four and more tokens the weights are never
+ * brought then, and the waits for them run out, once in either projection of a pass.)  slicemoe_workspace_init resets
+ * both.  Enqueued on `stream`.
  */
 int slicemoe_workspace_set_wait(void *workspace, unsigned long long wait_cycles, unsigned extra_arrivals,
                                 void *stream);

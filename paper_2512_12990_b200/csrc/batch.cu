@@ -24,7 +24,9 @@
 // Measured, 8 tokens, 64 x 1408 top-6 + 2 shared, hidden 2048: eight batch-1 launches 133 us, this 52.
 //
 // Bounded waits: when one runs out the CTA's dead flag goes up and SLICEMOE_STATUS_WAIT_TIMEOUT is set; from then on nobody
-// waits for data, the consumers walk through the rest of their work and the producers stop and wait for their copies.
+// waits for data, the consumers walk through the rest of their work and the producers - their four lanes together, so that
+// every copy that one of them asks for is one that its barrier counts - stop and wait for the copies on their way, for a
+// millisecond at least whatever the limit.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -61,9 +63,9 @@ struct __align__(16) BSeg {
 };
 static_assert(sizeof(BSeg) == 128, "a lane per word copies a segment");
 struct BHead {
-  int nseg[2];
+  int nseg[2];               // negative: see `off`
   unsigned total[2];
-  int off;                   // nothing is to be computed
+  int off;                   // the time-out exercise: no weights are brought, y is not written
 };
 
 struct BLayout {
@@ -331,13 +333,13 @@ __global__ void __launch_bounds__(kBPlanThreads) batch_plan_kernel(const BPlanPa
   }
   if (tid == 0) {
     BHead h;
-    h.nseg[0] = off ? 0 : (int)n_runs + n_sh;
-    h.nseg[1] = off ? 0 : (int)n_runs * p.kc_r + n_sh * p.kc_s;
+    const int sign = off ? -1 : 1;
+    h.nseg[0] = sign * ((int)n_runs + n_sh);
+    h.nseg[1] = sign * ((int)n_runs * p.kc_r + n_sh * p.kc_s);
     h.total[0] = t1 + (unsigned)n_sh * cs1;
     h.total[1] = t2 + (unsigned)n_sh * cs2;
     h.off = off ? 1 : 0;
     *p.head = h;
-    if (off) atomicOr(p.ctl.status, (unsigned)SLICEMOE_STATUS_WAIT_TIMEOUT);
   }
 }
 
@@ -373,26 +375,35 @@ struct BSmem {
   __host__ __device__ static int ring(int K) { return (inv(K) + K / 128 * kBRun * 4 + 127) & ~127; }
 };
 
+constexpr unsigned long long kBCopyCycles = 2000000ull;  // a millisecond: far more than any copy takes
 struct BWait {
   volatile int* dead;
   unsigned long long limit;
   unsigned* status;
   // true: the phase is there; false: it is not, and nobody waits any more
-  __device__ __forceinline__ bool operator()(uint32_t bar, uint32_t parity) const {
-    if (mbar_try(bar, parity)) return true;
+  __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) const {
     const long long t0 = clock64();
-    for (;;) {
+    while (!*dead) {
       for (int i = 0; i < 64; ++i)
         if (mbar_try(bar, parity)) return true;
-      if (*dead) return false;
       if ((unsigned long long)(clock64() - t0) > limit) {
         *dead = 1;
         atomicOr(status, (unsigned)SLICEMOE_STATUS_WAIT_TIMEOUT);
-        return false;
       }
     }
+    return false;
   }
 };
+// The consumers' wait: a call where the first look fails, not six copies of the loop (8 tokens of a 512-wide layer of 512-wide
+// experts, top-4, G 64: 19.8 us, in line 20.7).
+__device__ __noinline__ void b_wait_slow(uint32_t bar, uint32_t parity, BWait w) { w.wait(bar, parity); }
+__device__ __forceinline__ void b_wait(uint32_t bar, uint32_t parity, const BWait& w) {
+  if (!mbar_try(bar, parity)) b_wait_slow(bar, parity, w);
+}
+// The producers': their four lanes go on together or stop together.
+__device__ __forceinline__ bool b_wait_lanes(uint32_t bar, uint32_t parity, const BWait& w) {
+  return __all_sync(0xfu, mbar_try(bar, parity)) || __all_sync(0xfu, w.wait(bar, parity));
+}
 
 // One 16 x 128 block for eight tokens: acc[2 row half + token] += the block's contribution (lane (g, c): rows g and
 // g + 8, tokens 2 c and 2 c + 1).
@@ -559,7 +570,7 @@ __device__ __forceinline__ void b_rows(const BParams& p, const BSeg& sh, int u, 
     for (int m = 0; m < S::kMats; ++m) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
       for (int b0 = 0; b0 < nkb; b0 += per) {
-        wait(fb + 16 * st, par);
+        b_wait(fb + 16 * st, par, wait);
         const uint8_t* stage = ring + st * S::kStage;
         const int nb = min(per, nkb - b0);
 #pragma unroll 1
@@ -635,11 +646,13 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
   wait.dead = dead;
   wait.limit = lim != 0ull ? lim : kWaitCycles;
   wait.status = p.ctl.status;
+  bool off;
   // This CTA's share: the row blocks whose start, in cost, lies in its window.  A thread per segment; everything a role needs
   // to know about a segment is in its entry, so the way to the first copy is two trips to L2.
   {
     const uint4 head = tid < p.max_segs ? __ldcg(reinterpret_cast<const uint4*>(p.segs + tid)) : make_uint4(0u, 1u, 0u, 0u);
-    const int nseg = __ldcg(&p.head->nseg[PHASE - 1]);
+    const int said = __ldcg(&p.head->nseg[PHASE - 1]), nseg = abs(said);
+    off = said < 0;
     const unsigned long long total = __ldcg(&p.head->total[PHASE - 1]);
     const unsigned lo = (unsigned)((total * blockIdx.x + gridDim.x - 1) / gridDim.x);
     const unsigned hi = (unsigned)((total * (blockIdx.x + 1) + gridDim.x - 1) / gridDim.x);
@@ -665,6 +678,7 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
   if (warp >= kBConsumers) {
     // ---- producer of a group: lane 0 the MSB plane, 1 the LSB plane, 2 the scales, 3 the zero-points ----
     if (lane >= 4) return;
+    if (off) return;  // the time-out exercise: nothing is asked for, and the consumers' waits run out
     const int group = warp - kBConsumers;
     const uint32_t fb = bars + 16 * group * p.stages;
     const uint32_t ring = smem_u32(ring0 + (size_t)group * p.stages * S::kStage);
@@ -686,7 +700,8 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
           const uint8_t* src = sh.ptr[m][lane] + ((size_t)u * sh.row_kb + sh.kb0) * per_block;
           for (int b0 = 0; b0 < nkb; b0 += per) {
             const unsigned nb = (unsigned)min(per, nkb - b0);
-            if (!wait(fb + 16 * st + 8, par)) { ok = false; break; }
+            ok = b_wait_lanes(fb + 16 * st + 8, par, wait);
+            if (!ok) break;
             if (lane == 0) mbar_arrive_expect_tx(fb + 16 * st, nb * ((sh.lsb ? 2048u : 1024u) + SG * 48u));
             __syncwarp(0xfu);
             if (active) bulk_g2s(ring + st * S::kStage + dst0, src, nb * per_block, fb + 16 * st, pol);
@@ -699,9 +714,10 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
       ord += u1 - u0;
     }
     // no copy may be on its way when the CTA ends (in the normal case the consumers have seen them all land)
+    const unsigned long long drain = wait.limit > kBCopyCycles ? wait.limit : kBCopyCycles;
     for (uint32_t i = used > (uint32_t)p.stages ? used - p.stages : 0; i < used; ++i) {
       const long long t0 = clock64();
-      while (!mbar_try(fb + 16 * (i % p.stages), (i / p.stages) & 1) && (unsigned long long)(clock64() - t0) < wait.limit) {}
+      while (!mbar_try(fb + 16 * (i % p.stages), (i / p.stages) & 1) && (unsigned long long)(clock64() - t0) < drain) {}
     }
     return;
   }

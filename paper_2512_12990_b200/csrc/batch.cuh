@@ -14,7 +14,7 @@ constexpr int kBatchTokens = 16;
 // What the workspace header offers to the batch kernels.
 struct BatchControl {
   unsigned* status;
-  const unsigned* extra_arrivals;         // != 0: nothing is computed, the time-out status is set
+  const unsigned* extra_arrivals;         // != 0: no weights are brought, so that the waits for them run out, and y is not written
   const unsigned long long* wait_cycles;  // limit of the device-side waits, 0 = the default
 };
 

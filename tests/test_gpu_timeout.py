@@ -51,3 +51,35 @@ def test_wait_timeout_is_reported_and_the_workspace_recovers():
     torch.cuda.synchronize()
     assert B.slicemoe_get_status(layer.ws) == 0
     assert torch.equal(y2, y), "same bits as before the time-out"
+
+
+@pytest.mark.parametrize("T,limit", [(4, 2_000_000), (17, 200_000)])
+def test_wait_timeout_of_several_tokens(T, limit):
+    """The same for the kernels that take several tokens at once, in one pass and in two: their waits for the weights run
+    out, y stays as it was, and the workspace works again.  (200,000 cycles: less than what the producers give copies on
+    their way, which is a floor of their own.)"""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    sh = synth.Shape("batch-timeout", 512, 384, 12, 3, 64, n_shared=1, shared_inter=256, n_layers=1, seed=7300)
+    layer = H.Layer(sh, range(sh.n_experts))
+    rng = np.random.default_rng(T)
+    ids = np.stack([rng.permutation(sh.n_experts)[:sh.top_k] for _ in range(T)]).astype(np.int32)
+    lists = [torch.from_numpy(a).cuda() for a in (ids, rng.integers(0, 2, ids.shape).astype(np.uint8), rng.random(ids.shape).astype(np.float32))]
+    x = H.to_dev_bf16(H.x_inputs(sh, T, "batch-timeout-x")[0])
+
+    def call(y=None):
+        y = B.slicemoe_layer(layer.cshape, layer.experts_tbl, layer.shared_tbl, None, x, *lists, layer.ws, y=y)
+        torch.cuda.synchronize()
+        return y
+
+    y = call()
+    assert B.slicemoe_get_status(layer.ws) == 0
+    B.slicemoe_workspace_set_wait(layer.ws, limit, extra_arrivals=1)
+    y_bad = torch.full((T, sh.hidden), 7.0, device="cuda")
+    t0 = time.time()
+    call(y_bad)
+    assert time.time() - t0 < 5.0, "the kernels must return by themselves"
+    assert B.slicemoe_get_status(layer.ws) == B.STATUS_WAIT_TIMEOUT
+    assert torch.all(y_bad == 7.0)
+    B.lib().slicemoe_workspace_init(layer.ws.data_ptr(), layer.ws.numel(), None)
+    assert torch.equal(call(), y) and B.slicemoe_get_status(layer.ws) == 0
