@@ -700,6 +700,9 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
           const uint8_t* src = sh.ptr[m][lane] + ((size_t)u * sh.row_kb + sh.kb0) * per_block;
           for (int b0 = 0; b0 < nkb; b0 += per) {
             const unsigned nb = (unsigned)min(per, nkb - b0);
+            // the down launch's first lap round the ring finds it empty; after that space is the consumers' doing, who wait for
+            // the gate/up launch first: that is no part of the limit on this wait
+            if (PHASE == 2 && used == (uint32_t)p.stages) b_dep_wait();
             ok = b_wait_lanes(fb + 16 * st + 8, par, wait);
             if (!ok) break;
             if (lane == 0) mbar_arrive_expect_tx(fb + 16 * st, nb * ((sh.lsb ? 2048u : 1024u) + SG * 48u));

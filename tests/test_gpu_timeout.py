@@ -83,3 +83,24 @@ def test_wait_timeout_of_several_tokens(T, limit):
     assert torch.all(y_bad == 7.0)
     B.lib().slicemoe_workspace_init(layer.ws.data_ptr(), layer.ws.numel(), None)
     assert torch.equal(call(), y) and B.slicemoe_get_status(layer.ws) == 0
+
+
+def test_a_short_limit_is_not_spent_on_the_launch_before():
+    """The down projection of several tokens starts while gate/up still runs.  Its waits are counted from the end of that
+    launch: a limit of 40,000 cycles, 20 us, lets a pass through whose gate/up alone takes longer."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    E, k, T, h, inter = 16, 4, 16, 4096, 1408
+    g = torch.Generator(device="cuda").manual_seed(5)
+    pack = lambda n, c: B.slicemoe_pack(torch.randn((n, c), generator=g, device="cuda").mul_(0.02), 32)
+    experts = [dict(gate=pack(inter, h), up=pack(inter, h), down=pack(h, inter)) for _ in range(E)]
+    table, shape = B.expert_table(experts), B.make_shape(h, inter, E, k, 32)
+    ws = B.new_workspace(shape)
+    ids = torch.stack([torch.randperm(E, generator=g, device="cuda")[:k] for _ in range(T)]).to(torch.int32)
+    prec = torch.randint(0, 2, (T, k), generator=g, device="cuda").to(torch.uint8)
+    w, x = torch.rand((T, k), generator=g, device="cuda"), torch.randn((T, h), generator=g, device="cuda").bfloat16()
+    want = B.slicemoe_layer(shape, table, None, None, x, ids, prec, w, ws)
+    B.slicemoe_workspace_set_wait(ws, 40_000)
+    for _ in range(20):
+        assert torch.equal(B.slicemoe_layer(shape, table, None, None, x, ids, prec, w, ws), want)
+    assert B.slicemoe_get_status(ws) == 0
