@@ -193,7 +193,9 @@ int slicemoe_workspace_set_wait(void *workspace, unsigned long long wait_cycles,
  *   y        device float32 [T, hidden], overwritten
  * Up to three tokens are processed one after another by the batch-1 decode kernel; from four on up to 16 at a
  * time go through kernels that stream each expert they name once for all of them.  Accumulation is fp32, h stays
- * fp32 between the two projections, the summation order is fixed (results are bit-reproducible run to run).
+ * fp32 between the two projections, the summation order is fixed (results are bit-reproducible run to run).  A token's
+ * result does not depend on the other tokens of the call, bit for bit; that of a call of up to three tokens and that of
+ * a larger one differ in the last bits, by the order in which fp32 sums are added up.
  * Errors: INVALID_ARG, UNSUPPORTED (shape limits above; sum of intermediate widths over the k + n_shared
  * slots must be <= 12288; hidden / 16 must not exceed 4 x the device's SM count), CUDA.
  */

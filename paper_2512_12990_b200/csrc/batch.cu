@@ -414,8 +414,10 @@ __device__ __forceinline__ bool b_wait_lanes(uint32_t bar, uint32_t parity, cons
 // Where nibbles are used as they are (low, mixed) the A fragment of rows g + 8 is the raw bytes, 16 x their nibble plus row
 // g's: the difference of the accumulator rows is 16 C[g + 8], and the row's scale is divided by 16.
 // WIDE: column n of the B operand is token n, an MMA per digit.  Otherwise, for up to two tokens, columns 4 t .. 4 t + 2 are the
-// digits of token t, one MMA for all: even lanes c hold digits 0 and 1 of token c / 2, odd ones digit 2, acc[0] and
-// acc[1] are the row halves, and the caller adds lane pairs at the end.
+// digits of token t, one MMA for all: even lanes c get digits 0 and 1 of token c / 2, odd ones digit 2.  The two exchange a
+// row half's, so that an even lane finishes row g in acc[0] and an odd one row g + 8; `sc` and `zp` are at that row.
+// Every form gives a token the same bits: the same exact integers (times a power of two that the row's scale takes back), rounded
+// at the same points, blocks in the same order.  So what else is in a run does not show in a token's result.
 enum { kModeLow = 0, kModeMixed = 1, kModeHigh = 2 };
 template <int G, int MODE, bool WIDE>
 __device__ __forceinline__ void b_block(const uint8_t* msb, const uint8_t* lsb, const uint8_t* sc, const uint8_t* zp, const uint8_t* dig,
@@ -495,8 +497,9 @@ __device__ __forceinline__ void b_block(const uint8_t* msb, const uint8_t* lsb, 
 #pragma unroll
       for (int i = 0; i < 4; ++i) v[d][i] = m[i];
     }
-    float s0 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32)), s1 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32 + 16));
-    unsigned z0 = zp[sg * 16], z1 = zp[sg * 16 + 8];
+    // rows g and g + 8; in the narrow form the lane's own row, twice
+    float s0 = __half2float(*reinterpret_cast<const __half*>(sc + sg * 32)), s1 = WIDE ? __half2float(*reinterpret_cast<const __half*>(sc + sg * 32 + 16)) : s0;
+    unsigned z0 = zp[sg * 16], z1 = WIDE ? zp[sg * 16 + 8] : z0;
     if (MODE == kModeLow) {  // 2^shift (q_msb - (zp >> shift)): the power of two goes into the scale
       const float two = (float)(1 << shift);
       z0 >>= shift;
@@ -526,18 +529,17 @@ __device__ __forceinline__ void b_block(const uint8_t* msb, const uint8_t* lsb, 
         acc[i] = fmaf((i >= 2 ? s1 : s0) * ((i & 1) ? iv.y : iv.x), t, acc[i]);
       }
     } else {
-      const float x = X[sg * 2 * kBRun];  // the lane's digits'
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const bool mixed16 = MODE == kModeMixed && r == 1;
-        float t;
-        if (mixed16) t = odd ? (float)v[0][2] * 65536.f : fmaf((float)v[0][3], 256.f, (float)v[0][2]);
-        else t = (float)(odd ? v[0][2 * r] : v[0][2 * r] + v[0][2 * r + 1] * 256) * (odd ? 65536.f : 1.f);
-        unsigned z = r ? z1 : z0;
-        if (MODE == kModeMixed) z &= ~(low0 & (r ? drop << 4 : drop));
-        t = fmaf(-(float)z, x, t);
-        acc[r] = fmaf((r ? s1 : s0) * iv.x, t, acc[r]);
-      }
+      // digits 0 and 1 of both row halves in an even lane, digit 2 of both in an odd one
+      const float f0 = (float)(odd ? v[0][0] : v[0][0] + v[0][1] * 256);
+      const float f1 = odd ? (float)v[0][2]
+                           : MODE == kModeMixed ? fmaf((float)v[0][3], 256.f, (float)v[0][2]) : (float)(v[0][2] + v[0][3] * 256);
+      const float got = __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
+      const float x = X[sg * 2 * kBRun] + X[sg * 2 * kBRun + kBRun];
+      float t = odd ? fmaf(f1, 65536.f, got) : fmaf(got, 65536.f, f0);
+      unsigned z = odd ? z1 : z0;
+      if (MODE == kModeMixed) z &= ~(low0 & (odd ? drop << 4 : drop));
+      t = fmaf(-(float)z, x, t);
+      acc[0] = fmaf((odd ? s1 : s0) * iv.x, t, acc[0]);
     }
   }
 }
@@ -560,7 +562,8 @@ __device__ __forceinline__ void b_rows(const BParams& p, const BSeg& sh, int u, 
   const unsigned low0 = (sh.high >> tk0) & 1u ? 0u : 0xffffffffu, low1 = (sh.high >> tk1) & 1u ? 0u : 0xffffffffu;
   // columns without a token repeat the last one's; the narrow form's fourth column repeats a digit
   const uint8_t* my_dig = dig + c * 8 + (WIDE ? min(g8, n - 1) * stride : min(g8 >> 2, n - 1) * stride + min(g8 & 3, 2) * 32);
-  const float* my_X = X + (WIDE ? 2 * c : (c >> 1) + (c & 1) * kBRun);
+  const float* my_X = X + (WIDE ? 2 * c : c >> 1);
+  const int my_row = WIDE ? g8 : g8 + 8 * (c & 1);  // first row of the lane
   const float* my_inv = inv + tk0;
   int st = state.st, half = state.half;
   uint32_t par = state.par;
@@ -575,8 +578,8 @@ __device__ __forceinline__ void b_rows(const BParams& p, const BSeg& sh, int u, 
         const int nb = min(per, nkb - b0);
 #pragma unroll 1
         for (int b = gw; b < nb; b += kBGroupWarps)
-          b_block<G, MODE, WIDE>(stage + b * 1024 + lane * 16, stage + kBPlane / 2 + b * 1024 + lane * 16, stage + kBPlane + b * (SG * 32) + g8 * 2,
-                                 stage + kBPlane + 8 * SG * 32 + b * (SG * 16) + g8, my_dig + (b0 + b) * 384, my_X + (b0 + b) * SG * 2 * kBRun,
+          b_block<G, MODE, WIDE>(stage + b * 1024 + lane * 16, stage + kBPlane / 2 + b * 1024 + lane * 16, stage + kBPlane + b * (SG * 32) + my_row * 2,
+                                 stage + kBPlane + 8 * SG * 32 + b * (SG * 16) + my_row, my_dig + (b0 + b) * 384, my_X + (b0 + b) * SG * 2 * kBRun,
                                  my_inv + (b0 + b) * kBRun, shift, c & 1, low0, low1, acc);
         __syncwarp();
         if (lane == 0) mbar_arrive(fb + 16 * st + 8);
@@ -589,8 +592,7 @@ __device__ __forceinline__ void b_rows(const BParams& p, const BSeg& sh, int u, 
         w[(2 * c) * 20 + g8 + 8] = acc[2];
         w[(2 * c + 1) * 20 + g8 + 8] = acc[3];
       } else {
-        const float a0 = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1), a1 = acc[1] + __shfl_xor_sync(0xffffffffu, acc[1], 1);
-        w[(c >> 1) * 20 + g8 + 8 * (c & 1)] = (c & 1) ? a1 : a0;
+        w[(c >> 1) * 20 + my_row] = acc[0];
       }
     }
     // the four warps' shares of the columns, added in warp order by a thread per (token, row); two buffers take turns

@@ -94,3 +94,42 @@ def test_a_result_buffer_may_start_on_any_float():
     B.slicemoe_layer(L.cshape, L.experts_tbl, None, None, x, ids, prec, w, L.ws, y=y)
     torch.cuda.synchronize()
     assert torch.equal(y, want) and buf[0] == 7.0 and buf[-1] == 7.0
+
+
+@pytest.mark.parametrize("group,bits", [(128, (8, 4)), (64, (6, 3)), (32, (8, 4)), (32, (4, 2))])
+def test_a_token_does_not_depend_on_the_others_of_its_batch(group, bits):
+    """The form of the arithmetic follows from the run that a token's pair falls into: alone or with one other pair, among
+    up to eight, at one precision or both.  None of that shows in the token's result, bit for bit."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    E, k, hidden = 12, 3, 640
+    sh = synth.Shape("batch", hidden, 384, E, k, group, n_shared=1, shared_inter=256, shared_sigmoid_gate=True, n_layers=1, seed=7200 + group)
+    L = H.Layer(sh, range(E), b_high=bits[0], b_low=bits[1])
+    x_all = H.to_dev_bf16(H.x_inputs(sh, 16, "batch-alone")[0])
+    mine, mine_w = np.array([3, 7, 5], np.int32), np.array([0.5, 0.3, 0.2], np.float32)
+
+    def call(others, others_prec, my_prec):
+        """Token 0 keeps its list; the others' lists [T - 1, k] vary."""
+        T = len(others) + 1
+        ids = np.concatenate([mine[None], others]).astype(np.int32)
+        prec = np.concatenate([my_prec[None], others_prec]).astype(np.uint8)
+        w = np.concatenate([mine_w[None], np.full((T - 1, k), 0.25, np.float32)])
+        y = B.slicemoe_layer(L.cshape, L.experts_tbl, L.shared_tbl, L.gate_vec_dev, x_all[:T].contiguous(),
+                             *(torch.from_numpy(a).cuda() for a in (ids, prec, w)), L.ws)
+        torch.cuda.synchronize()
+        assert B.slicemoe_get_status(L.ws) == 0
+        return y[0].cpu()
+
+    for my_prec in (np.array([1, 0, 1], np.uint8), np.array([0, 1, 0], np.uint8)):
+        elsewhere = np.array([0, 1, 2])                                   # none of the token's experts: it is alone with each
+        want = call(np.tile(elsewhere, (3, 1)), np.zeros((3, k)), my_prec)
+        assert want.abs().max() > 0
+        for T in (4, 5, 9, 16):
+            for shared_with in (1, T - 1):                                # one other pair, or all of them
+                for p in (0, 1):
+                    others = np.tile(elsewhere, (T - 1, 1))
+                    others[:shared_with] = mine[None]
+                    got = call(others, np.full((T - 1, k), p), my_prec)
+                    assert torch.equal(got, want), f"T {T}, {shared_with} others at precision {p}"
+        got = call(np.tile(mine, (7, 1)), np.arange(7)[:, None] % 2 * np.ones((1, k)), my_prec)
+        assert torch.equal(got, want), "others at either precision"
