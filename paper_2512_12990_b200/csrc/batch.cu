@@ -38,14 +38,12 @@
 
 namespace slicemoe {
 
-constexpr int kBRun = 8;                 // pairs of a run: the columns of an MMA
 constexpr int kBGroups = 4, kBGroupWarps = 4, kBConsumers = kBGroups * kBGroupWarps;
 constexpr int kBThreads = 32 * (kBConsumers + kBGroups);
-constexpr int kBChunkK = 2048;           // columns of a down projection's task; wider experts are several
 constexpr int kBPlane = 8192;            // plane bytes of a stage: 4 blocks of both slices or 8 of the MSB slice
-constexpr int kBMaxSegs = 40;            // runs that a CTA's share can touch
 constexpr int kBPlanThreads = 256;
 static_assert(kBatchTokens * SLICEMOE_MAX_TOP_K <= kBPlanThreads, "a thread per pair");
+static_assert(kBMaxTasks <= kBThreads, "a thread per segment");
 
 // The row blocks of a run - up to eight pairs of one expert - in one projection (down: for one chunk of columns).
 struct __align__(16) BSeg {
@@ -115,14 +113,6 @@ struct BPlanParams {
   float *xsum, *xinv;     // their group sums [T][hidden / G][2], block scales [T][hidden / 128]
   BatchControl ctl;
 };
-// What a 16 x 128 block of a run costs a CTA: the bytes it brings (an MSB tile 2, both slices 4) and its instructions - by
-// measurement about half as much again for up to two pairs, the same for more, twice that where pairs of either precision
-// meet.  (By bytes alone, CTAs with both-slice runs were done in 21,000 cycles and those with MSB runs in 34,000.)
-__device__ __forceinline__ unsigned b_block_cost(int n, unsigned high) {
-  const unsigned all = (1u << n) - 1u, compute = (n <= 2 ? 1u : 2u) << (high != 0u && (high & all) != all ? 1 : 0);
-  return (high ? 4u : 2u) + compute;
-}
-constexpr unsigned kBFixedCost = 12;  // a row block's own: hand-shakes and the exchange between the four warps
 __device__ __forceinline__ int b_chunk_cols(int inter, int kc) { return min(kBChunkK, inter - kc * kBChunkK); }
 // Block-wide exclusive scans of four values, in place; `total` gets the sums.
 __device__ void b_scan(unsigned (&v)[4], unsigned (*sums)[kBPlanThreads / 32], unsigned (&total)[4]) {
@@ -369,10 +359,10 @@ struct BSmem {
   static constexpr int kMaxStages = 8;
   static constexpr int part = (bars + 2 * kBGroups * kMaxStages * 8 + 127) & ~127;
   static constexpr int dig = part + kBGroups * 2 * kPart * 4;
-  __host__ __device__ static int tok_stride(int K) { return 3 * K + 32; }  // eight tokens' digit rows spread over the banks
-  __host__ __device__ static int sums(int K) { return dig + kBRun * tok_stride(K); }            // float [K / G][digits 0 and 1, digit 2][8]
-  __host__ __device__ static int inv(int K) { return sums(K) + 2 * (K / G) * kBRun * 4; }       // float [K / 128][8]
-  __host__ __device__ static int ring(int K) { return (inv(K) + K / 128 * kBRun * 4 + 127) & ~127; }
+  __host__ __device__ static constexpr int tok_stride(int K) { return 3 * K + 32; }  // eight tokens' digit rows spread over the banks
+  __host__ __device__ static constexpr int sums(int K) { return dig + kBRun * tok_stride(K); }            // float [K / G][digits 0 and 1, digit 2][8]
+  __host__ __device__ static constexpr int inv(int K) { return sums(K) + 2 * (K / G) * kBRun * 4; }       // float [K / 128][8]
+  __host__ __device__ static constexpr int ring(int K) { return (inv(K) + K / 128 * kBRun * 4 + 127) & ~127; }
 };
 
 constexpr unsigned long long kBCopyCycles = 2000000ull;  // a millisecond: far more than any copy takes
@@ -887,6 +877,7 @@ static int b_launch(void (*kernel)(P), dim3 grid, unsigned threads, size_t smem,
 }
 
 constexpr int kBSmemMax = 227 * 1024;
+constexpr int kBMaxHidden = 4096;
 template <int G, int PHASE>
 static int b_launch_ffn(BParams p, int sms, cudaStream_t st) {
   static bool attr_set[64];
@@ -898,7 +889,10 @@ static int b_launch_ffn(BParams p, int sms, cudaStream_t st) {
     attr_set[dev] = true;
   }
   using S = BSmem<G, PHASE>;
-  // as many stages as shared memory holds: bytes in flight are what the bandwidth needs
+  // As many stages as shared memory holds beside the digits of eight tokens: bytes in flight are what the bandwidth needs.
+  // Gate/up: three per group at hidden 2048, two at 4096, one at 4096 with G 32, where copy and arithmetic take turns (four
+  // tokens that share none of their experts of 1408: 84 us, token after token 89).
+  static_assert(S::ring(PHASE == 1 ? kBMaxHidden : kBChunkK) + kBGroups * S::kStage <= kBSmemMax, "one stage at least");
   p.stages = (kBSmemMax - S::ring(p.K)) / (kBGroups * S::kStage);
   if (p.stages > S::kMaxStages) p.stages = S::kMaxStages;
   return b_launch(batch_ffn_kernel<G, PHASE>, dim3((unsigned)sms), kBThreads,
@@ -963,8 +957,6 @@ int batch_layer(const slicemoe_shape* s, const slicemoe_expert* experts, const s
   BParams p2 = p;
   p2.segs = pp.seg2;
   p2.max_segs = T * s->top_k * L.kc_r + n_shared * parts * L.kc_s;
-  // (widths add up to 12288 over a token's experts: never more segments than threads)
-  if (p2.max_segs > kBThreads) return SLICEMOE_E_UNSUPPORTED;
   const int widest = s->inter > pp.shared_inter ? s->inter : pp.shared_inter;
   p2.K = widest < kBChunkK ? widest : kBChunkK;
   const int rc = s->group == 128 ? b_launch_all<128>(pp, p, p2, sms, st)

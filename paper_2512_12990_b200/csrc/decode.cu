@@ -1432,7 +1432,8 @@ static int run_layer(const slicemoe_shape* shape, const slicemoe_expert* experts
   // A small batch: every expert is streamed once for all of a pass' tokens.  (A workspace of the batch-1 kernel's size, as
   // slicemoe_layer_static's, has no room for that: token after token then.)
   const size_t batch_bytes = batch_workspace_bytes(shape, n_shared);
-  if (T >= kBatchMinTokens && workspace_bytes >= kWsBatchOff + batch_bytes + kWsListBytes) {
+  if (T >= kBatchMinTokens && workspace_bytes >= kWsBatchOff + batch_bytes + kWsListBytes &&
+      batch_fits(shape, n_shared, T < kBatchTokens ? T : kBatchTokens, sms)) {
     uint8_t* bws = reinterpret_cast<uint8_t*>(workspace) + kWsBatchOff;
     uint8_t* lists = bws + batch_bytes;
     const BatchControl ctl = {&p.ws->status, &p.ws->extra_arrivals, &p.ws->wait_cycles};

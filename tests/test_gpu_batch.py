@@ -133,3 +133,22 @@ def test_a_token_does_not_depend_on_the_others_of_its_batch(group, bits):
                     assert torch.equal(got, want), f"T {T}, {shared_with} others at precision {p}"
         got = call(np.tile(mine, (7, 1)), np.arange(7)[:, None] % 2 * np.ones((1, k)), my_prec)
         assert torch.equal(got, want), "others at either precision"
+
+
+@pytest.mark.parametrize("T", [4, 16])
+def test_the_widest_hidden_with_the_smallest_groups(T):
+    """Hidden 4096 at group 32: the digits of eight tokens leave the gate/up kernel one ring stage per group."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    E, k = 6, 3
+    sh = synth.Shape("batch", 4096, 128, E, k, 32, n_shared=1, shared_inter=256, shared_sigmoid_gate=True, n_layers=1, seed=7400 + T)
+    L = H.Layer(sh, range(E))
+    ids, prec, w = _random_lists(np.random.default_rng(T), T, E, k)
+    xbits, x64 = H.x_inputs(sh, T, "batch-wide")
+    y = B.slicemoe_layer(L.cshape, L.experts_tbl, L.shared_tbl, L.gate_vec_dev, H.to_dev_bf16(xbits),
+                         *(torch.from_numpy(a).cuda() for a in (ids, prec, w)), L.ws)
+    torch.cuda.synchronize()
+    assert B.slicemoe_get_status(L.ws) == 0
+    y_ref = moe.layer(x64, L.oracle_list(), ids, prec, w.astype(np.float64), shared=L.oracle_shared, shared_gate_vec=L.gate_vec)
+    for t in range(T):
+        H.assert_close(y[t].cpu().numpy(), y_ref[t], f"token {t}")
