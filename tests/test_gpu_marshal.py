@@ -62,3 +62,22 @@ def test_errors_are_exceptions():
     with pytest.raises((TypeError, BufferError)):
         B.slicemoe_layer(None, None, None, None, x, logits, logits, logits, ws)
     assert np.isfinite(x.float().cpu().numpy()).all()
+
+
+def test_outputs_have_storages_of_their_own():
+    """A packed matrix and a routing list can be saved and loaded, and an output that is kept keeps nothing else."""
+    import io
+    import torch
+    m = B.slicemoe_pack(torch.randn((32, 256), device="cuda"), 64)
+    routed = B.slicemoe_route_topk(torch.randn((3, 8), device="cuda"), 2)
+    shape = B.make_shape(256, 128, 8, 2, 64)
+    layer = H.Layer(synth.SHAPES["tiny"], range(8))
+    x = torch.zeros((1, 256), dtype=torch.bfloat16, device="cuda")
+    out = B.slicemoe_layer_routed(shape, layer.experts_tbl, None, None, x, torch.randn((1, 8), device="cuda"), B.new_workspace(shape))
+    for group in ([m.msb, m.lsb, m.scale, m.zp], routed, out):
+        assert len({t.untyped_storage().data_ptr() for t in group}) == len(group)
+        assert all(t.storage_offset() == 0 and t.untyped_storage().nbytes() == t.numel() * t.element_size() for t in group)
+        f = io.BytesIO()
+        torch.save(list(group), f)
+        f.seek(0)
+        assert all(torch.equal(a, b) for a, b in zip(torch.load(f), group))
