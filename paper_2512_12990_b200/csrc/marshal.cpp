@@ -12,6 +12,7 @@
 #include <ATen/cuda/EmptyTensor.h>
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
@@ -164,8 +165,8 @@ PyObject* guarded(F&& f) {
   try {
     return f();
   } catch (const Failed&) {
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
+  } catch (const std::exception&) {  // torch's own kinds stay what they are: out of memory, an index out of range
+    torch::translate_exception_to_python(std::current_exception());
   }
   return nullptr;
 }

@@ -104,3 +104,11 @@ def test_a_refused_host_step_has_enqueued_nothing():
     assert step(gated, gate=None) == B.E_INVALID_ARG
     assert step(gated, workspace=ctypes.c_void_p(4096 + 2)) == B.E_INVALID_ARG
     assert step(B.make_shape(8192, 1408, 64, 4, 128)) == B.E_UNSUPPORTED
+
+
+def test_a_tensor_without_dimensions_is_an_index_error():
+    """An exception out of torch keeps its kind on the way through the native marshalling."""
+    import torch
+    sh = B.make_shape(256, 128, 8, 2, 64)
+    with pytest.raises(IndexError):
+        B.slicemoe_layer(sh, None, None, None, torch.tensor(1.0), None, None, None, torch.zeros(8, dtype=torch.uint8))

@@ -81,3 +81,18 @@ def test_outputs_have_storages_of_their_own():
         torch.save(list(group), f)
         f.seek(0)
         assert all(torch.equal(a, b) for a, b in zip(torch.load(f), group))
+
+
+def test_running_out_of_memory_is_torchs_own_error():
+    import torch
+    W = torch.zeros((16384, 4096), device="cuda")          # 256 MB; its planes take 32 MB each
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (8 << 20)) / total)
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            B.slicemoe_pack(W, 128)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert B.slicemoe_pack(W, 128).N == 16384
