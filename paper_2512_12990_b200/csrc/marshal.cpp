@@ -324,8 +324,10 @@ PyObject* py_dbsc_assign(SM_ARGS) {
     if (plain_buffer(a[4], &req, 1, "B")) {
       if (plain_buffer(a[5], &out, 1, "B")) {
         if (!out.readonly && req.len >= ids.len / 4 && out.len >= ids.len / 4)
-          rc = lib.dbsc_assign(c, step, layer, static_cast<const int32_t*>(ids.buf), static_cast<const uint8_t*>(req.buf),
-                               (int)(ids.len / 4), static_cast<uint8_t*>(out.buf));
+          rc = unlocked([&] {
+            return lib.dbsc_assign(c, step, layer, static_cast<const int32_t*>(ids.buf), static_cast<const uint8_t*>(req.buf),
+                                   (int)(ids.len / 4), static_cast<uint8_t*>(out.buf));
+          });
         PyBuffer_Release(&out);
       }
       PyBuffer_Release(&req);

@@ -89,3 +89,27 @@ def test_eviction_log_names_exactly_what_left_the_cache():
                 m_, l_ = c.contains(ll, ee)
                 assert ((ll, ee, 0) in held) == m_ and ((ll, ee, 1) in held) == l_
     assert B.lib().slicemoe_dbsc_drain_evicted(None, None, None, None, 0) == B.E_INVALID_ARG
+
+
+def test_assign_lets_other_threads_run():
+    """A long call of the cache does not hold the interpreter lock."""
+    import threading
+    import time
+    c = B.Dbsc(1000 * (M + L), M, L)
+    ids = np.random.default_rng(0).integers(0, 4000, 3_000_000).astype(np.int32)
+    req, seen, stop = np.ones(ids.size, np.uint8), [], threading.Event()
+
+    def other():
+        while not stop.is_set():
+            seen.append(time.perf_counter())
+            time.sleep(0.001)
+
+    t = threading.Thread(target=other)
+    t.start()
+    a = time.perf_counter()
+    c.assign(0, 0, ids, req)
+    b = time.perf_counter()
+    stop.set()
+    t.join()
+    assert b - a > 0.02, "long enough to tell"
+    assert any(a + 0.25 * (b - a) < s < a + 0.75 * (b - a) for s in seen)
