@@ -387,7 +387,7 @@ class Dbsc:
     def assign(self, step: int, layer: int, ids, prec_req):
         """ids: numpy int32 [n]; prec_req: numpy uint8 [n] -> numpy uint8 [n]."""
         import numpy as np
-        out = np.empty(np.shape(ids), dtype=np.uint8)
+        out = np.empty(np.shape(ids) or (1,), dtype=np.uint8)
         m = _m or _marshal()
         if not m.dbsc_assign(self._h, step, layer, ids, prec_req, out):   # other types or layouts: converted first
             ids = np.ascontiguousarray(ids, dtype=np.int32)

@@ -113,3 +113,12 @@ def test_assign_lets_other_threads_run():
     t.join()
     assert b - a > 0.02, "long enough to tell"
     assert any(a + 0.25 * (b - a) < s < a + 0.75 * (b - a) for s in seen)
+
+
+def test_assign_of_one_id_without_a_list():
+    """A scalar id is a list of one, as any other type or layout is converted."""
+    c = B.Dbsc(4 * (M + L), M, L)
+    assert c.assign(0, 0, np.int32(3), np.uint8(1)).tolist() == [1]
+    assert c.assign(1, 0, [[3, 1], [2, 0]], [[0, 1], [1, 0]]).tolist() == [[0, 1], [1, 0]]
+    with pytest.raises(B.SliceMoEError):
+        c.assign(2, 0, np.arange(4, dtype=np.int32), np.ones(3, np.uint8))
