@@ -164,6 +164,9 @@ def _marshal():
         L = lib()
         import torch  # noqa: F401  (its libraries are what the module links to)
         from . import _marshal as m
+        from .build import marshal_tag
+        if m.built_for != marshal_tag():
+            raise ImportError(f"_marshal.so was built for {m.built_for}, this is {marshal_tag()}: build it again")
         m.setup(SliceMoEError, {n: ctypes.cast(getattr(L, n), c_void_p).value for n in EXPORTS})
         _m = m
     return _m

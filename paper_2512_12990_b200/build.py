@@ -40,25 +40,40 @@ def build(force: bool = False, verbose: bool = False, trace: bool = False) -> st
             _build_library(lib, force, verbose, trace)
         finally:
             out, _ = marshal.communicate()
+            if marshal.returncode != 0:
+                sys.stderr.write(out)
         if marshal.returncode != 0:
-            sys.stderr.write(out)
             raise RuntimeError("the compiler failed on marshal.cpp")
         os.replace(MARSHAL + ".new", MARSHAL)
         return lib
     return _build_library(lib, force, verbose, trace)
 
 
-def _start_marshal(force: bool):
-    """Starts the compiler on marshal.cpp when _marshal.so is older than its sources."""
+def marshal_tag() -> str:
+    """What _marshal.so is compiled against besides its sources: the layouts of torch's and Python's objects."""
+    import sysconfig
+    import torch
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _marshal_is_current() -> bool:
     deps = (MARSHAL_SRC, os.path.join(ROOT, "include", "slicemoe.h"))
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(map(os.path.getmtime, deps)):
+    if not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < max(map(os.path.getmtime, deps)):
+        return False
+    with open(MARSHAL, "rb") as f:
+        return marshal_tag().encode() + b"\0" in f.read()
+
+
+def _start_marshal(force: bool):
+    """Starts the compiler on marshal.cpp when _marshal.so is older than its sources or made for another torch or Python."""
+    if not force and _marshal_is_current():
         return None
     import sysconfig
     import torch
     t = os.path.dirname(torch.__file__)
     cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", os.path.join(ROOT, "include"),
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DSLICEMOE_BUILT_FOR="{marshal_tag()}"', "-I", os.path.join(ROOT, "include"),
            "-isystem", os.path.join(t, "include"), "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"),
            "-isystem", cuda, "-isystem", sysconfig.get_paths()["include"], MARSHAL_SRC, "-o", MARSHAL + ".new",
            "-L", os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"]

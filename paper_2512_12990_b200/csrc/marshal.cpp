@@ -513,5 +513,7 @@ PyMODINIT_FUNC PyInit__marshal() {
   s_data_ptr = PyUnicode_InternFromString("data_ptr");
   s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
   if (!s_data_ptr || !s_cuda_stream) return nullptr;
-  return PyModule_Create(&module);
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "built_for", SLICEMOE_BUILT_FOR) < 0) Py_CLEAR(m);
+  return m;
 }

@@ -112,3 +112,17 @@ def test_a_tensor_without_dimensions_is_an_index_error():
     sh = B.make_shape(256, 128, 8, 2, 64)
     with pytest.raises(IndexError):
         B.slicemoe_layer(sh, None, None, None, torch.tensor(1.0), None, None, None, torch.zeros(8, dtype=torch.uint8))
+
+
+def test_the_native_marshalling_belongs_to_this_torch(monkeypatch):
+    """_marshal.so uses torch's and Python's objects by their layout: made for others it is built again and not loaded."""
+    import torch
+    from paper_2512_12990_b200 import build
+    build.build()
+    assert build._marshal_is_current()
+    assert B._marshal().built_for == build.marshal_tag()
+    monkeypatch.setattr(torch, "__version__", "0.0")
+    assert not build._marshal_is_current()
+    monkeypatch.setattr(B, "_m", None)
+    with pytest.raises(ImportError):
+        B._marshal()
