@@ -17,6 +17,7 @@
 // multiply-add by the scale.  No weight is rounded anywhere.
 #include <cuda.h>  // CUtensorMap (types only; the encoder is fetched through the runtime)
 #include <cuda_fp16.h>
+#include <stddef.h>
 
 #include "common.cuh"
 
@@ -279,10 +280,10 @@ __global__ void __launch_bounds__(kPfGatherThreads) pf_gather_kernel(const PfGat
   auto load = [&](int i) {
     if (i >= p.hidden / 2) return;
     if (WORDS == 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(src + i);
+      const uint4 v = __ldcg(reinterpret_cast<const uint4*>(src + i));
       in[0] = v.x; in[WORDS / 4] = v.y; in[WORDS / 2] = v.z; in[WORDS - 1] = v.w;
     } else {
-      in[0] = src[i];
+      in[0] = __ldcg(src + i);
     }
   };
   load(tid * WORDS);
@@ -579,6 +580,9 @@ __device__ __forceinline__ void fma2(uint64_t& acc, uint32_t v0, uint32_t v1, ui
 }
 __device__ __forceinline__ float half_of(uint64_t v, int i) { return __uint_as_float((uint32_t)(v >> (32 * i))); }
 
+__device__ __forceinline__ PfRun pf_load_run(const PfRun* at) {
+  return {__ldcg(&at->expert), __ldcg(&at->count), __ldcg(&at->tiles), __ldcg(&at->in_row), __ldcg(&at->out_row), __ldcg(&at->items1), __ldcg(&at->items2), 0};
+}
 // The run that a work item belongs to: the last one whose first item is not above it.  Whole warp, 32 runs a step.
 template <int PHASE>
 __device__ __forceinline__ int u_find_run(const PfRun* runs, int n, int item, int lane) {
@@ -587,7 +591,7 @@ __device__ __forceinline__ int u_find_run(const PfRun* runs, int n, int item, in
   while (step * 32 < n) step *= 32;
   for (; step >= 1; step >>= 5) {
     const int r = lo + lane * step;
-    const bool below = r < n && (PHASE == 1 ? runs[r].items1 : runs[r].items2) <= item;
+    const bool below = r < n && __ldcg(PHASE == 1 ? &runs[r].items1 : &runs[r].items2) <= item;
     lo += (__popc(__ballot_sync(0xffffffffu, below)) - 1) * step;
     if (step == 1) break;
   }
@@ -668,7 +672,8 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
   bool alive = true;
   // Only the token warp waits for the kernel before, whose work the token rows are (gathered x, or h).  That this kernel runs
   // says that the gather kernel's blocks have all seen the plan kernel's end: the plan, the counters and the caller's arrays
-  // are there, and the weights' way through the CTA fills up meanwhile.
+  // are there, and the weights' way through the CTA fills up meanwhile.  They are there in L2: what is read without the wait is
+  // read past L1, where an SM may still hold a line of the call before (same workspace, same tables).
 
   if (warp >= C::warp_tok) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::regs_rest));
@@ -795,7 +800,7 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
     } else if (warp == C::warp_sched) {
       // ---- scheduler: takes items from the counter and describes them ----
       int* next = PHASE == 1 ? &p.head->next1 : &p.head->next2;
-      const int n_runs = p.head->runs, n_items = PHASE == 1 ? p.head->items1 : p.head->items2;
+      const int n_runs = __ldcg(&p.head->runs), n_items = __ldcg(PHASE == 1 ? &p.head->items1 : &p.head->items2);
       // How far ahead: one item where an item is long (its successor is fetched when the sums of the item itself have
       // begun, and no CTA sits on items that another could take) or a CTA has few, else as many as the ring holds.
       constexpr int kLongItem = 8, kAheadShort = 6;
@@ -818,15 +823,16 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
         const void* ptr = nullptr;
         if (item < n_items) {
           const int run = u_find_run<PHASE>(p.runs, n_runs, item, lane);
-          r = p.runs[run];
+          r = pf_load_run(p.runs + run);
           in_run = item - (PHASE == 1 ? r.items1 : r.items2);
           const bool is_shared = r.expert >= p.E;
           ex = is_shared ? p.shared + (r.expert - p.E) : p.experts + r.expert;
-          prec = is_shared || p.expert_prec[r.expert] != 0;
+          prec = is_shared || __ldcg(p.expert_prec + r.expert) != 0;
           // lanes 0 .. 7: MSB, LSB, scales, zero-points of the first and of the second matrix
           const slicemoe_mat* m = PHASE == 1 ? ((lane & 1) ? &ex->up : &ex->gate) : &ex->down;
           const int what = (lane >> 1) & 3;
-          ptr = what == 0 ? m->msb : what == 1 ? m->lsb : what == 2 ? (const void*)m->scale : (const void*)m->zp;
+          static_assert(offsetof(slicemoe_mat, lsb) == 8 && offsetof(slicemoe_mat, scale) == 16 && offsetof(slicemoe_mat, zp) == 24, "in this order");
+          ptr = reinterpret_cast<const void*>(__ldcg(reinterpret_cast<const unsigned long long*>(m) + what));
           const bool no_lsb = __any_sync(0xffffffffu, what == 1 && ptr == nullptr);
           if (prec && no_lsb) {  // both slices were asked for but the LSB planes are absent
             if (lane == 0) atomicOr(p.status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
@@ -898,7 +904,7 @@ __global__ void __launch_bounds__(UCfg<TN>::threads, 1) pf_umma_kernel(const PfG
               if (lane == 0) mbar_expect_tx(&meta_full[ms], gs * 8 * 48);
               __syncwarp();
               if (lane < 16) bulk_copy(dst, from, bytes, &meta_full[ms]);
-            } else {  // a caller's array that does not start on 16 bytes: byte by byte
+            } else {  // a caller's array that does not start on 16 bytes: byte by byte (weights: no call before has them otherwise)
               if (lane < 16)
                 for (int i = 0; i < bytes; ++i) dst[i] = from[i];
               __syncwarp();

@@ -58,3 +58,35 @@ def test_tile_edges(T, E, k, group, n_shared):
         assert H.errors(y2, y)[0] <= 1e-4
     else:
         assert np.array_equal(y2, y)
+
+
+def test_calls_in_a_row_through_the_same_buffers():
+    """Kernels of a call start before the one ahead has ended and read the plan, x and the tables then: prompts that take
+    turns in one workspace, with nothing in between, each give what they give alone."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    E, k, hidden = 12, 3, 512
+    sh = synth.Shape("edges", hidden, 256, E, k, 128, n_shared=1, shared_inter=256, shared_sigmoid_gate=True, n_layers=1, seed=8900)
+    L = H.Layer(sh, range(E))
+    rng = np.random.default_rng(9)
+    prompts = []
+    for T in (5, 300, 40):
+        ids = np.stack([rng.permutation(E)[:k] for _ in range(T)]).astype(np.int32)
+        if T == 40:
+            ids[:] = [1, 2, 3]
+        prompts.append((H.to_dev_bf16(H.x_inputs(sh, T, f"row-{T}")[0]), torch.from_numpy(ids).cuda(), torch.rand((T, k), device="cuda"),
+                        torch.from_numpy(rng.integers(0, 2, E).astype(np.uint8)).cuda()))
+    ws = B.new_prefill_workspace(L.cshape, 300)
+
+    def call(p):
+        return B.slicemoe_prefill_layer(L.cshape, L.experts_tbl, L.shared_tbl, L.gate_vec_dev, *p, ws)
+
+    alone = []
+    for p in prompts:
+        ws.fill_(0)
+        alone.append(call(p)[0])
+        torch.cuda.synchronize()
+    out = [call(p) for _ in range(20) for p in prompts]
+    torch.cuda.synchronize()
+    for i, (y, status) in enumerate(out):
+        assert int(status) == 0 and torch.equal(y, alone[i % 3]), f"call {i}"
