@@ -17,7 +17,7 @@ Reported (one JSON line on rank 0):
   e2e        the same through slicemoe_decode_step_host: one pinned host buffer (x, logits) in, host y out, every step
   roofline   the decode kernel alone: algorithmic bytes (slice planes read + scales + zero-points)
              per launch / its average duration, against the measured HBM copy bandwidth; `traffic` comes from the
-             tracked ncu record under profiles/ and is null when decode.cu has changed since the capture
+             tracked ncu record under profiles/ and is null when the kernel's sources have changed since the capture
   stream_only_us   the same bytes through the same bulk copies with no arithmetic (slicemoe_stream_probe)
   cpu_baseline   the CPU oracle timed on this host on a few steps of the same workload
   workloads  (one GPU, default workload) short legs of the Qwen-shaped decode layer, the 26-layer decode stack and
@@ -361,14 +361,16 @@ def n_reps(k_steps: int, est_us_per_step: float) -> int:
 
 def decode_traffic_record(workload: str):
     """DRAM bytes per launch of the decode kernel from the tracked ncu record under profiles/, or None when
-    there is none for this workload or decode.cu has changed since the capture (the record stores its hash)."""
+    there is none for this workload or the kernel's sources have changed since the capture (the record stores their hash)."""
     import hashlib
     try:
         with open(os.path.join(ROOT, "profiles", "decode_layer_kernel_traffic.json")) as f:
             rec = json.load(f)
-        with open(os.path.join(ROOT, "paper_2512_12990_b200", "csrc", "decode.cu"), "rb") as f:
-            digest = hashlib.sha256(f.read()).hexdigest()
-        if rec.get("decode_cu_sha256") != digest:
+        digest = hashlib.sha256()
+        for name in ("decode.cu", "decode_common.cuh", "route.cuh", "common.cuh"):
+            with open(os.path.join(ROOT, "paper_2512_12990_b200", "csrc", name), "rb") as f:
+                digest.update(f.read())
+        if rec.get("sources_sha256") != digest.hexdigest():
             return None
         v = rec.get("dram_bytes_per_launch", {}).get(workload)
         return None if v is None else int(v)

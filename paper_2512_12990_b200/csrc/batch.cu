@@ -9,7 +9,7 @@
 //   gate/up  h = silu(gate x) * (up x) of every pair, fp32;
 //   down     result row of every pair, fp32;
 //   combine  y[t] = sum of the token's rows times their weights, slots in list order, then the shared experts.
-// The two projections are one kernel.  A CTA (one per SM) takes an equal share, by bytes, of the row blocks of all runs.
+// The two projections are one kernel.  A CTA (one per SM) takes an equal share, by measured cost, of the row blocks of all runs.
 // Four groups of a producer warp and four consumer warps each take the share's row blocks in turn: the producer
 // streams the planes, scales and zero-points through the group's own ring with bulk copies, never waiting for anything but
 // space; the consumers split a row block's 128-column blocks.  The arithmetic is the batch-1 kernel's: activations
@@ -21,7 +21,8 @@
 //
 // Bound: HBM.  Per 16 x 128 block of both planes (2 KB, 89 cycles of an SM's share of the bandwidth) a warp issues about 125
 // instructions, 24 of them MMAs (53 cycles of the integer tensor pipe).
-// Measured, 8 tokens, 64 x 1408 top-6 + 2 shared, hidden 2048: eight batch-1 launches 133 us, this 52.
+// Measured, 8 tokens, 64 x 1408 top-6 + 2 shared, hidden 2048: eight batch-1 launches 133 us, this 53.6 (where the
+// tokens' experts overlap as by Zipf(1.1) popularity: 195 MB, 30 us at the copy bandwidth).
 //
 // Bounded waits: when one runs out the CTA's dead flag goes up and SLICEMOE_STATUS_WAIT_TIMEOUT is set; from then on nobody
 // waits for data, the consumers walk through the rest of their work and the producers - their four lanes together, so that

@@ -128,8 +128,10 @@ constexpr size_t kWsListEntries = (size_t)kBatchTokens * SLICEMOE_MAX_TOP_K;
 constexpr size_t kWsListBytes = kWsListEntries * 9;
 // From this many tokens on a layer call takes the batch kernels (four launches) instead of a launch of the batch-1 kernel
 // per token.  Measured, us, loop / batch at T = 2, 3, 4: 2048-wide layer of 1408-wide experts 33 / 37, 49 / 40, 65 / 43; 1024 wide
-// 22 / 19, 33 / 20, 44 / 21; 256 wide 13 / 14, 20 / 14, 27 / 14.  (At three tokens the loop stays, because slicemoe_layer_static,
-// which has no room for the batch, promises the bits of slicemoe_layer there.)
+// 22 / 19, 33 / 20, 44 / 21; 256 wide 13 / 14, 20 / 14, 27 / 14; from four tokens on the batch was ahead at every one of 75
+// shapes, groups, T and overlaps of the lists, by least at hidden 4096 and group 32: 84 / 89.  By time alone the line would lie
+// at three; it lies at four because slicemoe_layer_static, which has no room for the batch, gives the bits of
+// slicemoe_layer up to three tokens, as its header says.
 constexpr int kBatchMinTokens = 4;
 static_assert(sizeof(WsHeader) <= kWsHOff, "workspace header");
 static_assert(kWsStLogits + 4 * 512 <= kWsStIds, "x and the logits fit the staging area back to back too");
