@@ -100,13 +100,13 @@ size_t slicemoe_meta_count(int N, int K, int group); /* number of (scale, zp) en
 /*
  * slicemoe_pack - offline preparation of one weight matrix: quantise (Table 1 fn. 1, Section 6.1:
  * grouped asymmetric codes) and split into MSB / LSB slice planes (Sections 4.1, 4.2).
- *   W      device, float32 [N, K] row-major (read only)
+ *   W      device, float32 [N, K] row-major (read only), 16-byte aligned
  *   msb, lsb, scale, zp   device outputs in the physical layout; sizes from the functions above
  * Per (row, group), in float32, with Q = 2^b_high - 1: lo = min(min w, 0), hi = max(max w, 0),
  * s = fp16((hi - lo)/Q) (round to nearest even; a group with hi == lo or s in {0, inf} gets s = 1, zp = 0),
  * zp = clamp(rint(-lo/s), 0, Q), q = clamp(rint(w/s) + zp, 0, Q) with IEEE division and
  * round-half-even.  Bit-exact and deterministic.
- * Errors: INVALID_ARG (null, N % 16, K % 128, K % group), UNSUPPORTED ((b_high, b_low) not one of (8,4), (6,3),
+ * Errors: INVALID_ARG (null, N % 16, K % 128, K % group, W off its alignment), UNSUPPORTED ((b_high, b_low) not one of (8,4), (6,3),
  * (4,2); group not in {32,64,128}), CUDA.
  */
 int slicemoe_pack(const float *W, int N, int K, int group, int b_high, int b_low, void *msb,

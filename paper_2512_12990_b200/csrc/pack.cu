@@ -199,6 +199,10 @@ extern "C" int slicemoe_pack(const float* W, int N, int K, int group, int b_high
   const int qmax = (1 << b_high) - 1, shift = b_high - b_low;
   const int rc = check_dims(N, K, group);
   if (rc != SLICEMOE_OK) return rc;
+  // four columns of W a load, a word of a plane a store: elsewhere the kernel would fault
+  if ((reinterpret_cast<uintptr_t>(W) & 15) || ((reinterpret_cast<uintptr_t>(msb) | reinterpret_cast<uintptr_t>(lsb)) & 3) ||
+      (reinterpret_cast<uintptr_t>(scale) & 1))
+    return SLICEMOE_E_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const long long blocks = (long long)(N / 16) * ((K / 128 + kPackBlocks - 1) / kPackBlocks);
   if (blocks > 0x7fffffffll) return SLICEMOE_E_INVALID_ARG;

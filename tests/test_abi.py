@@ -126,3 +126,13 @@ def test_the_native_marshalling_belongs_to_this_torch(monkeypatch):
     monkeypatch.setattr(B, "_m", None)
     with pytest.raises(ImportError):
         B._marshal()
+
+
+@pytest.mark.parametrize("which,off", [(0, 4), (1, 2), (2, 1), (3, 1)])
+def test_pack_refuses_pointers_off_their_alignment(which, off):
+    """W on 16 bytes, planes on words, scales on theirs: the kernel's loads and stores would fault elsewhere."""
+    import ctypes
+    p = [64, 64, 64, 64, 64]
+    p[which] += off
+    W, msb, lsb, scale, zp = map(ctypes.c_void_p, p)
+    assert B.lib().slicemoe_pack(W, 16, 128, 128, 8, 4, msb, lsb, scale, zp, None) == B.E_INVALID_ARG
