@@ -929,7 +929,7 @@ __device__ __forceinline__ Routed read_routing(const DecodeParams& p, int lane, 
   rt.w = 0.f;
   if (FUSED) {
     // same arithmetic as the stand-alone routing kernel; the precision request is the precision
-    const RouteSel sel = route_warp(p.logits, p.n_experts, p.k, p.bias, p.renorm, p.tau, p.rank_high, lane);
+    const RouteSel sel = route_warp(RouteGlobal{p.logits}, p.n_experts, p.k, p.bias, p.renorm, p.tau, p.rank_high, lane);
     if (lane < p.k) {
       rt.e = sel.id;
       rt.pr = sel.prec_req;
@@ -1287,7 +1287,7 @@ __global__ void __launch_bounds__(kStageThreads) stage_step_kernel(const uint32_
   for (int i = 0; i < kWords; ++i)
     if (i * kStageThreads + tid < hidden / 2) x[i * kStageThreads + tid] = v[i];
   if (tid < 32) {
-    const RouteSel sel = route_warp(row, E, k, bias, renorm, tau, rank_high, lane);
+    const RouteSel sel = route_warp(RouteShared{row}, E, k, bias, renorm, tau, rank_high, lane);
     if (lane < k) {
       ids[lane] = sel.id;
       weights[lane] = sel.w;

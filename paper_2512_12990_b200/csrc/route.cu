@@ -16,7 +16,7 @@ __global__ void route_topk_kernel(const float* __restrict__ logits, int T, int E
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= T) return;
-  const RouteSel sel = route_warp(logits + (size_t)warp * E, E, k, bias, renorm, tau, rank_high, lane);
+  const RouteSel sel = route_warp(RouteGlobal{logits + (size_t)warp * E}, E, k, bias, renorm, tau, rank_high, lane);
   if (lane < k) {
     const size_t o = (size_t)warp * k + lane;
     ids[o] = sel.id;

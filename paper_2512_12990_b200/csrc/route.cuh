@@ -23,12 +23,21 @@ struct RouteSel {  // lane j < k holds selection j
   uint8_t prec_req;
 };
 
+// Where a token's logits are: in global memory, read past L1 (a kernel that is launched early may run on an SM whose L1 still
+// holds what the addresses held before), or in shared memory.
+struct RouteGlobal {
+  const float* row;
+  __device__ __forceinline__ float operator[](int e) const { return __ldcg(row + e); }
+};
+struct RouteShared {
+  const float* row;
+  __device__ __forceinline__ float operator[](int e) const { return row[e]; }
+};
+
 // VPT: values per lane, a compile-time bound with 32 VPT >= E.  The result does not depend on it: a lane's
 // values are visited in the same order, only the unrolled loops over absent values are shorter.
-template <int VPT>
-__device__ __forceinline__ RouteSel route_warp_vpt(const float* __restrict__ row, int E, int k,
-                                                   const float* __restrict__ bias, int renorm, float tau, int rank_high,
-                                                   int lane) {
+template <int VPT, class Row>
+__device__ __forceinline__ RouteSel route_warp_vpt(const Row row, int E, int k, const float* bias, int renorm, float tau, int rank_high, int lane) {
   uint32_t key[VPT];  // ordered like the float keys; 0: no such expert, or taken
   float val[VPT];
   float vmax = -CUDART_INF_F;
@@ -40,7 +49,7 @@ __device__ __forceinline__ RouteSel route_warp_vpt(const float* __restrict__ row
     if (e < E) {
       const float raw = row[e];
       l = isnan(raw) ? -CUDART_INF_F : raw;
-      float kk = bias ? __fadd_rn(raw, bias[e]) : raw;
+      float kk = bias ? __fadd_rn(raw, __ldcg(bias + e)) : raw;
       if (isnan(kk)) kk = -CUDART_INF_F;
       const uint32_t b = __float_as_uint(kk + 0.0f);  // both zeros are one key
       key[v] = b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
@@ -77,11 +86,13 @@ __device__ __forceinline__ RouteSel route_warp_vpt(const float* __restrict__ row
       if (e == v * 32 + lane) key[v] = 0u;
     if (lane == j) idsel = e;
   }
-  float p = 0.0f;
-  if (lane < k) {
-    const float raw = row[idsel];
-    p = expf((isnan(raw) ? -CUDART_INF_F : raw) - vmax) * inv_sum;
+  float sel_val = 0.0f;  // the selection's logit, from the lane that holds it
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const float got = __shfl_sync(0xffffffffu, val[v], idsel & 31);
+    if ((idsel >> 5) == v) sel_val = got;
   }
+  const float p = lane < k ? expf(sel_val - vmax) * inv_sum : 0.0f;
   float total = 1.0f;
   if (renorm) {  // added up in selection order
     total = 0.0f;
@@ -94,8 +105,8 @@ __device__ __forceinline__ RouteSel route_warp_vpt(const float* __restrict__ row
   return sel;
 }
 
-__device__ __forceinline__ RouteSel route_warp(const float* __restrict__ row, int E, int k, const float* __restrict__ bias,
-                                               int renorm, float tau, int rank_high, int lane) {
+template <class Row>
+__device__ __forceinline__ RouteSel route_warp(const Row row, int E, int k, const float* bias, int renorm, float tau, int rank_high, int lane) {
   if (E <= 64) return route_warp_vpt<2>(row, E, k, bias, renorm, tau, rank_high, lane);
   if (E <= 128) return route_warp_vpt<4>(row, E, k, bias, renorm, tau, rank_high, lane);
   return route_warp_vpt<ROUTE_MAX_VPT>(row, E, k, bias, renorm, tau, rank_high, lane);
