@@ -4,13 +4,13 @@
 // The work is a pure weight stream: every plane byte is used once, so the bound is HBM bandwidth and
 // everything else is arranged so that the stream never stops.
 //   * One CTA per SM: 16 consumer warps in 4 groups, one epilogue warp, two producer warps (6 lanes each,
-//     one per bulk copy of a chunk).  The 4 warps of a group split a chunk's 128-column blocks, so the
+//     one per bulk copy of a chunk) and a warp that requests the down tiles.  The 4 warps of a group split a chunk's 128-column blocks, so the
 //     per-chunk bookkeeping is paid by 4 warps, not 16, while 4 chunks are in work at any time.  The
 //     schedule is a pure function of the slot table, so every role enumerates it for itself and only
 //     data and barrier phases pass between them.  The producer streams chunks - 16 rows x <=2048 columns: the MSB plane tile,
 //     the LSB plane tile when the expert runs at 8 bits (<=16 KB each, one contiguous run thanks to the
 //     tiled layout), scales and zero-points - into a ring of eight 19 KB units with cp.async.bulk +
-//     mbarriers.  They never wait for the gate/up -> down dependency, so down-projection tiles are
+//     mbarriers.  Nobody waits for the gate/up -> down dependency to request tiles, so down-projection tiles are
 //     already in flight (up to the whole ring) while the grid exchanges h.
 //   * Integer arithmetic on the tensor pipe.  The activation vector (x, later h) is converted once,
 //     per 128-element block, to fixed point relative to the block's largest magnitude and split into
@@ -23,8 +23,11 @@
 //        sum_k x_k s (q_k - zp) = s (sum_k q_k x_k - zp sum_{k in group} x_k).
 //     The plain ALUs could not unpack + convert + FMA two weights per byte at HBM rate; this costs
 //     about seven instructions per 512 weights.
-//   * Phase 1 (gate/up + SwiGLU): tasks are (expert slot, 16-row block), split over the CTAs by
-//     bytes.  The epilogue warp adds the warps' partial rows, applies SwiGLU and writes h (fp32) to
+//   * Phase 1 (gate/up + SwiGLU): tasks are (expert slot, 16-row block), dealt to the CTAs one by one in slot order, so that h is
+//     complete slot after slot and part of it is in digits before the last of it is written.  (A window of consecutive
+//     tasks per CTA - all slots complete at the end - and all of h converted then: a launch of a 2048-wide layer of 1408-wide
+//     experts, top-6 + 2 shared, 16.4 us; dealt, with the warp that requests the down tiles at once: 15.8; with a gated shared
+//     expert of 5632, 18.5 / 16.1; 1024-wide, top-8 of 512, 11.1 / 9.6; 256-wide, 6.45 / 5.9.)  The epilogue warp adds the warps' partial rows, applies SwiGLU and writes h (fp32) to
 //     the workspace.  There is no barrier between the phases: readers poll the h words themselves (two
 //     buffers used by alternate launches, each left "empty" by the launch before; every wait bounded).
 //   * Phase 2 (down + weighted combine): a task is a 16-row block of the OUTPUT over ALL slots, so
@@ -46,10 +49,11 @@ constexpr int kGroupWarps = 4;   // warps of a group; they split the 128-column 
 static_assert(kGroups * kGroupWarps == kConsumerWarps, "groups");
 constexpr int kEpilogueWarp = kConsumerWarps;
 constexpr int kProducerWarp = kConsumerWarps + 1;  // first of kProducers producer warps
-constexpr int kProducers = 2;                      // they take alternate tasks (phase 1) / chunks (phase 2)
-constexpr int kThreads = 32 * (kConsumerWarps + 1 + kProducers);
+constexpr int kProducers = 2;                      // see TaskPlace
+constexpr int kDownWarp = kProducerWarp + kProducers;  // fetches the routed experts' pointers, then requests the down tiles
+constexpr int kThreads = 32 * (kDownWarp + 1);
 constexpr int kUnits2 = 16;                        // at most this many (smaller) units in phase 2
-constexpr int kFull2PerGroup = 8;  // >= chunks one producer can have in flight in phase 2 (kUnits2 / 2 units)
+constexpr int kFull2PerGroup = 8;  // >= chunks that a group can have in flight in phase 2 (of kUnits2 units)
 constexpr int kUnits = 8;                                 // ring units; a chunk takes one per plane
 constexpr int kChunkK = 2048;                             // K columns per chunk (16 blocks of 128)
 constexpr int kBlocksPerWarp = kChunkK / 128 / kGroupWarps;
@@ -88,13 +92,12 @@ __device__ __forceinline__ long long trace_gtime() {
 #define SM_TRACE(i) do { } while (0)
 #define SM_TRACE_G(i) do { } while (0)
 #endif
-// stamp numbers (clock64 unless noted): 1 dependency wait over, 2 plan built (warp 0), 3 x as digits (warp 3),
+// stamp numbers (clock64 unless noted): 1 dependency wait over, 2 plan built, 3 x as digits (warp 3),
 // 4 prologue barrier passed, 5-8 gate/up phase done (consumer groups 0-3), 9 list of down chunks built (warp 0),
-// 10 own h blocks in digits (warp 0), 11 down phase done (warp 0), 12 last h value written, 13 y written;
-// 14-17 own h blocks in digits (first warp of consumer groups 0-3), 23-26 the h blocks of the group's last down chunk
-// flagged, 27-30 down phase done (first warp of groups 0-3), 31 producer 0 begins the down tiles, 18-19 producer 0 / 1
-// has requested all its down tiles, 32-39 producer 0 has requested its gate/up chunk 0-7, 40-43 / 44-47 the down
-// chunks of producer 0 / 1 have landed (in the order it waits for them); global timer: 20 kernel entry, 21 dependency
+// 10 no block of h left to take on (warp 0), 11 down phase done (warp 0), 12 last h value written, 13 y written;
+// 14-17 no block of h left (first warp of consumer groups 0-3), 23-26 the h blocks of the group's last down chunk
+// flagged, 27-30 down phase done (first warp of groups 0-3), 31 the request of the down tiles begins, 18 all down tiles
+// requested, 32-39 producer 0 has requested its gate/up chunk 0-7; global timer: 20 kernel entry, 21 dependency
 // wait over, 22 y written
 
 // ---- workspace --------------------------------------------------------------------------------
@@ -177,29 +180,29 @@ struct Slot {
 };
 
 // The schedule of a CTA.
-//   phase 1: tasks n = 0 .. count1-1 are (slot, 16-row block) pairs: first count_s tasks of the shared experts,
-//     from (slot_s, idx_s) on - this part follows from the shape alone, so its tiles can be requested before the
-//     routing list is known - then the routed tasks from (first_slot, first_idx) on.  A
-//     task of an 8-bit slot is 2 * nch chunks (gate then up; nch = 2048-column chunks of hidden), each two
-//     units (MSB tile, LSB tile); a task of a 4-bit slot is nch chunks, each two units (the gate's MSB tile
-//     and the up's).  Every phase-1 chunk takes two units.  Task n is consumed by group n % kGroups and
-//     produced by producer n % kProducers; which units and barriers a chunk uses is stated at `struct Bars`.
+//   phase 1: tasks are 16-row blocks of gate and up, numbered slot after slot - shared, routed from both slices, routed from the
+//     MSB slice alone - so that task o of the grid writes h[16 o ..].  Both-slice tasks go to CTA o mod P; of the MSB-only ones,
+//     half as long, the CTAs short of a both-slice task get two first, and the rest is dealt out (task_ordinal()): the CTAs
+//     differ by a task at most.  How many tasks of the shared experts a CTA has (count_s) follows from the shape alone, so their
+//     tiles are requested before the routing list is known.  A
+//     both-slice task is 2 * nch chunks (gate then up; nch = 2048-column chunks of hidden), each two
+//     units (MSB tile, LSB tile); an MSB-only task is nch chunks, each two units (the gate's MSB tile
+//     and the up's).  Every phase-1 chunk takes two units.  Which producer and which group a task goes to says TaskPlace;
+//     which units and barriers a chunk uses is stated at `struct Bars`.
 //   phase 2: tasks m = 0 .. count2-1 are the output row blocks blockIdx.x + m * gridDim.x; each is one run of
 //     chunks over the slots in order (p2c[j] chunks and p2u[j] units come before slot j), two units per
-//     chunk for 8-bit slots and one for 4-bit slots.  Chunk number c is consumed by group c % kGroups and
-//     produced by producer c % kProducers.
+//     chunk for 8-bit slots and one for 4-bit slots.  Chunk number c is consumed by group c % kGroups.
 //     Phase 2 re-cuts the ring into nunits2 units of unit2_bytes, just large enough for the widest down
 //     chunk (plane area, then scales at scale2_off, zero-points at zp2_off), so that more - for the
 //     benchmark shapes all - of the phase's tiles are in shared memory before h arrives.
 struct Plan {
-  int slot_s, idx_s, count_s;
+  int count_s, count_both, count1;  // phase-1 tasks of this CTA: of the shared experts, from both slices (with those), in all
+  int light, count_light, ord_light, ord_rest;  // its MSB-only tasks: see task_ordinal()
   int hpar;         // which h buffer this launch uses
   int never_ready;  // the time-out exercise: treat h as never complete
-  int first_slot, first_idx, count1;
   int count2;
   int nslots;
   int htotal;   // sum of the slots' intermediate widths
-  float gate;   // sigmoid(gate_vec . x) when the shared experts are gated
   int unit2_bytes, nunits2, scale2_off, zp2_off;
   short p2c[kMaxSlots + 1], p2u[kMaxSlots + 1];
 };
@@ -218,10 +221,12 @@ struct SmemLayout {
   static constexpr int slots = p2list + kConsumerWarps * kMaxMine * 16;
   static constexpr int plan = slots + kMaxSlots * (int)sizeof(Slot);
   static constexpr int bars = (plan + (int)sizeof(Plan) + 15) & ~15;  // uint64 barriers
-  static constexpr int nbars = 2 * kUnits + kGroups * kFull2PerGroup + kUnits2 + 2 * kGroups + 6;
+  static constexpr int nbars = 2 * kUnits + kGroups * kFull2PerGroup + kUnits2 + 2 * kGroups + 5;
   static constexpr int dead = bars + nbars * 8;  // int dead flag; 8 bytes on, the wait limit in cycles
   static constexpr int hready = dead + 16;       // uint8 [kHCap / 128]: the 128-block of h is in shared memory as digits
-  static constexpr int total = hready + kHCap / 128;
+  static constexpr int hnext = hready + kHCap / 128;  // int: the next block of h that nobody has taken on
+  static constexpr int gate = hnext + 16;            // float [kMaxHidden / 128]: a block's share of gate_vec . x
+  static constexpr int total = gate + kMaxHidden / 128 * 4;
 };
 static_assert(SmemLayout::total <= 227 * 1024, "shared memory budget");
 static_assert(sizeof(Slot) % 8 == 0, "slot alignment");
@@ -232,20 +237,21 @@ static_assert(SmemLayout::slots % 8 == 0 && SmemLayout::hdig % 16 == 0 && SmemLa
 // Barriers.  Every barrier has ONE waiter that meets its phases strictly in order, so a parity wait can never
 // be a phase off (mbarrier.try_wait.parity only tells the current phase from the one before it):
 //   - a chunk's "full" barrier belongs to the consumer group that consumes it: group g's i-th chunk of a phase
-//     uses full[g][i % 2] in phase 1 and full2[g][i % kFull2PerGroup] in phase 2, armed with the chunk's bytes by
-//     the producer that serves the group (group g is served by producer g % kProducers in both phases);
-//   - an "empty" barrier belongs to the producer that refills the space: producer P owns half of the ring and
-//     walks it in order.  Phase 1: P's j-th chunk takes the unit pair (4 P + 2 (j % 2), + 1) and waits on
-//     empty[2 P + j % 2]; phase 2: P's units are [P h, P h + h), h = nunits2 / 2, taken in running order, one
+//     uses full[g][i % 2] in phase 1, armed with the chunk's bytes by producer g % kProducers, and
+//     full2[g][i % kFull2PerGroup] in phase 2, armed by the down warp;
+//   - an "empty" barrier belongs to the warp that refills the space.  Phase 1: producer P owns half of the ring and
+//     walks it in order: its j-th chunk takes the unit pair (4 P + 2 (j % 2), + 1) and waits on
+//     empty[2 P + j % 2]; phase 2: the down warp takes the nunits2 units in running order, one
 //     empty2 barrier per unit (an arrive from each warp of the group that consumed it).
 // pfull1 / pempty1 per group (phase-1 partial rows to the epilogue warp and back), pfull2 / pempty2 (phase-2
 // partial rows of all warps), p1_done (every consumer warp is through with phase 1, so the ring may be re-cut), plan_ready (the
-// routed part of the plan and the routed slots stand: the producers wait for it after the shared experts' tasks).
+// routed part of the plan and the routed slots stand: waited for after the shared experts' tasks), head_ready (what the workspace
+// header says is in the plan).  The last two have one phase, and several waiters.
 struct Bars {
   static constexpr int full = 0, empty = kUnits, full2 = 2 * kUnits, empty2 = full2 + kGroups * kFull2PerGroup,
                        pfull1 = empty2 + kUnits2,
-                       pempty1 = pfull1 + kGroups, pfull2 = pempty1 + kGroups, pempty2 = pfull2 + 1, hx_go = pfull2 + 2,
-                       hs_ready = pfull2 + 3, p1_done = pfull2 + 4, plan_ready = pfull2 + 5, count = pfull2 + 6;
+                       pempty1 = pfull1 + kGroups, pfull2 = pempty1 + kGroups, pempty2 = pfull2 + 1, head_ready = pfull2 + 2,
+                       p1_done = pfull2 + 3, plan_ready = pfull2 + 4, count = pfull2 + 5;
 };
 
 static_assert(Bars::count <= SmemLayout::nbars, "barrier storage");
@@ -272,75 +278,92 @@ __device__ __forceinline__ void block_to_digits(const float (&v)[4], int k0, int
 __device__ __forceinline__ int nchunks_of(int K) { return (K + kChunkK - 1) / kChunkK; }
 enum ChunkMode { kModeSingle = 0, kModeBoth = 1, kModePair = 2 };
 
-// The phase-1 tasks of a CTA in order: `slot`, `idx` name task n once at(n) has been called for it.
-struct TaskWalk {
-  int slot, idx;
-  __device__ __forceinline__ void start(const Plan& plan) {
-    slot = plan.slot_s;
-    idx = plan.idx_s;
-  }
-  __device__ __forceinline__ void at(const Plan& plan, int n) {
-    if (n == plan.count_s) {  // the routed run begins
-      slot = plan.first_slot;
-      idx = plan.first_idx;
+// The number in the grid of this CTA's phase-1 task n.
+__device__ __forceinline__ int task_ordinal(const Plan& plan, int n) {
+  const int c = (int)blockIdx.x, P = (int)gridDim.x;
+  if (n < plan.count_s || n < plan.count_both) return c + n * P;
+  n -= plan.count_both;
+  return n < plan.count_light ? plan.ord_light + n * plan.light : plan.ord_rest + (n - plan.count_light) * P;
+}
+
+// Which producer a task goes to and which of that producer's tasks it is; the producer's groups take its tasks in turn.  The
+// tasks of both slices alternate; where their number is odd, the first two of the MSB-only ones, half as long, go to the
+// producer that got one less, the rest alternates again.
+struct TaskPlace {
+  int producer, turn;
+  __device__ __forceinline__ TaskPlace(int count_both, int n) {
+    const int k = n - count_both;  // among the MSB-only tasks
+    if (k >= 0 && (count_both & 1)) {
+      producer = k < 2 ? 1 : k & 1;
+      turn = (count_both >> 1) + (k < 2 ? k : producer ? 2 + ((k - 2) >> 1) : 1 + ((k - 2) >> 1));
+    } else {
+      producer = n & 1;
+      turn = n >> 1;
     }
   }
-  __device__ __forceinline__ void next(const Slot* slots) {
-    if (++idx >= slots[slot].inter / 16) {
-      idx = 0;
-      ++slot;
-    }
-  }
+  __device__ __forceinline__ int group() const { return producer + kProducers * (turn & 1); }
+  __device__ __forceinline__ int round() const { return turn >> 1; }  // which of its group's tasks it is
 };
+static_assert(kProducers == 2 && kGroups == 4, "two groups to a producer");
 
 // ---- consumers -----------------------------------------------------------------------------------
-// Phase change: every consumer warp polls its 128-blocks of the grid's h in the workspace until all of a block's
-// values have been written (see kHEmpty), and turns the block into digits at once: blocks whose CTAs finished early
-// are done before the last CTA's values arrive.  A block's flag in `hready` tells the other warps that its digits
+// Phase change: the consumer warps take 128-blocks of the grid's h on, a few at a time in order, poll them in the
+// workspace until all of a block's values have been written (see kHEmpty), and turn the block into digits at once.  The tasks are
+// dealt so that h is complete slot after slot, and a warp whose group is through with phase 1 early begins with the early slots.
+// A block's flag in `hready` tells the other warps that its digits
 // stand; nobody waits for the whole of h (see wait_h_blocks).  Returns false if the (bounded) wait ran out.
+// (Four warps that did nothing else than this while gate/up ran took its issue slots: 20.8 -> 23.9 us where groups are 32 wide.
+// Chunks that were ready consumed before more of h was taken on: 15.9 -> 17.0, a look at h is a trip of over a microsecond.)
 template <int G>
-__device__ bool fetch_h(const DecodeParams& p, uint8_t* smem, int warp, int lane, int htotal, const float* hbuf,
-                        bool never_ready, volatile int* dead, unsigned* status, uint32_t bars) {
+__device__ bool fetch_h(const DecodeParams& p, uint8_t* smem, int lane, int htotal, const float* hbuf, bool never_ready,
+                        volatile int* dead, unsigned* status) {
   const int nblk = htotal >> 7;
-  constexpr int kMaxIt = (kHCap / 128 + kConsumerWarps - 1) / kConsumerWarps;
-  unsigned pending = 0u;  // warp-uniform
-#pragma unroll
-  for (int it = 0; it < kMaxIt; ++it)
-    if (it * kConsumerWarps + warp < nblk) pending |= 1u << it;
+  // Loads in flight together, fewer where there would not be some for every warp.  (2048-wide layer, two shared experts, us: four
+  // 15.9, two 16.2, six 16.0; with groups of 32, whose digit sums take longer: 22.4, 21.2, 22.7.)
+  constexpr int kTake = G == 128 ? 4 : 2;
+  const int take = max(1, min(kTake, nblk / kConsumerWarps));
   const long long t0 = clock64();
-  while (pending != 0u) {
-    float4 v[kMaxIt];
+  for (;;) {
+    int b0 = 0;
+    if (lane == 0) b0 = atomicAdd(reinterpret_cast<int*>(smem + SmemLayout::hnext), take);
+    b0 = __shfl_sync(0xffffffffu, b0, 0);
+    if (b0 >= nblk) return true;
+    unsigned pending = (1u << min(take, nblk - b0)) - 1u, before = 0u;  // warp-uniform
+    while (pending != 0u) {
+      if (pending == before) __nanosleep(100);  // (others are still at work on phase 1, whose way to memory this is, too)
+      before = pending;
+      float4 v[kTake];
 #pragma unroll
-    for (int it = 0; it < kMaxIt; ++it)  // all of the warp's open blocks in flight together; L2 is the point of coherence
-      if ((pending >> it) & 1u) v[it] = __ldcg(reinterpret_cast<const float4*>(hbuf) + (it * kConsumerWarps + warp) * 32 + lane);
+      for (int i = 0; i < kTake; ++i)  // L2 is the point of coherence
+        if ((pending >> i) & 1u) v[i] = __ldcg(reinterpret_cast<const float4*>(hbuf) + (b0 + i) * 32 + lane);
 #pragma unroll
-    for (int it = 0; it < kMaxIt; ++it) {
-      if ((pending >> it) & 1u) {
-        const bool mine = __float_as_uint(v[it].x) != kHEmpty && __float_as_uint(v[it].y) != kHEmpty &&
-                          __float_as_uint(v[it].z) != kHEmpty && __float_as_uint(v[it].w) != kHEmpty;
-        if (__all_sync(0xffffffffu, mine) && !never_ready) {
-          const float q[4] = {v[it].x, v[it].y, v[it].z, v[it].w};
-          block_to_digits<G>(q, (it * kConsumerWarps + warp) * 128, lane, smem + SmemLayout::hdig,
-                             reinterpret_cast<float*>(smem + SmemLayout::hsumw), reinterpret_cast<float*>(smem + SmemLayout::hinv));
-          pending &= ~(1u << it);
-          __syncwarp();  // every lane's digits of the block are written ...
-          if (lane == 0) {
-            __threadfence_block();  // ... and visible before the flag is
-            *reinterpret_cast<volatile uint8_t*>(smem + SmemLayout::hready + it * kConsumerWarps + warp) = 1;
+      for (int i = 0; i < kTake; ++i) {
+        if ((pending >> i) & 1u) {
+          const bool mine = __float_as_uint(v[i].x) != kHEmpty && __float_as_uint(v[i].y) != kHEmpty &&
+                            __float_as_uint(v[i].z) != kHEmpty && __float_as_uint(v[i].w) != kHEmpty;
+          if (__all_sync(0xffffffffu, mine) && !never_ready) {
+            const float q[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+            block_to_digits<G>(q, (b0 + i) * 128, lane, smem + SmemLayout::hdig, reinterpret_cast<float*>(smem + SmemLayout::hsumw),
+                               reinterpret_cast<float*>(smem + SmemLayout::hinv));
+            pending &= ~(1u << i);
+            __syncwarp();  // every lane's digits of the block are written ...
+            if (lane == 0) {
+              __threadfence_block();  // ... and visible before the flag is
+              *reinterpret_cast<volatile uint8_t*>(smem + SmemLayout::hready + b0 + i) = 1;
+            }
           }
         }
       }
-    }
-    if (pending != 0u) {
-      if (*dead) return false;
-      if ((unsigned long long)(clock64() - t0) > wait_limit(dead)) {
-        *dead = 1;
-        atomicOr(status, (unsigned)SLICEMOE_STATUS_WAIT_TIMEOUT);
-        return false;
+      if (pending != 0u) {
+        if (*dead) return false;
+        if ((unsigned long long)(clock64() - t0) > wait_limit(dead)) {
+          *dead = 1;
+          atomicOr(status, (unsigned)SLICEMOE_STATUS_WAIT_TIMEOUT);
+          return false;
+        }
       }
     }
   }
-  return true;
 }
 
 // Waits (bounded) until the `n` (<= 32) 128-blocks of h from block `b0` on are in shared memory as digits.
@@ -494,16 +517,21 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
   const int nch = nchunks_of(p.hidden);
   const int prod = group % kProducers;  // the producer that serves this group
   {
-    TaskWalk tw;
-    tw.start(plan);
-    int cn = 0;
+    int cn = 0, end = plan.count_s;  // the shared experts' tasks are known from the start, the others once the plan stands
     int jp = 0;  // chunks of this group's producer so far (they fix the unit pair)
     int ig = 0;  // chunks of this group so far (they fix the full barrier)
-    for (int n = 0; n < plan.count1; ++n) {
-      tw.at(plan, n);
-      const Slot& sl = slots[tw.slot];
-      const int nchunks = sl.prec ? 2 * nch : nch;
-      if (n % kGroups == group) {
+    for (int n = 0;; ++n) {
+      if (n == plan.count_s) {
+        if (!mbar_wait(bars + 8 * Bars::plan_ready, 0, dead, status)) return;
+        end = plan.count1;
+        if (plan.nslots == 0 && blockIdx.x == 0)
+          for (int i = threadIdx.x; i < p.hidden; i += 32 * kConsumerWarps) p.y[i] = 0.f;
+      }
+      if (n >= end) break;
+      const bool shared = n < plan.count_s, both = shared || n < plan.count_both;
+      const int nchunks = both ? 2 * nch : nch;
+      const TaskPlace at(shared ? n + 1 : plan.count_both, n);
+      if (at.group() == group) {
         float part0 = 0.f, part1 = 0.f, unused = 0.f;
         for (int q = 0; q < nchunks; ++q, ++jp, ++ig) {
           const int c = cn + q;
@@ -515,7 +543,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
           const float* sumw = reinterpret_cast<const float*>(smem + SmemLayout::xsumw) + kc * (kChunkK >> LG) * 2;
           const float* binv = reinterpret_cast<const float*>(smem + SmemLayout::xinv) + kc * (kChunkK >> 7);
           const uint8_t* unit0 = smem + SmemLayout::ring + u0 * kUnitBytes;
-          if (sl.prec) {
+          if (both) {
             consume_chunk<G>(lr, lane, gw, c % kGroupWarps, kModeBoth, nblocks, unit0, unit0 + kUnitBytes, kPlaneUnitBytes,
                              kPlaneUnitBytes + kScaleUnitBytes, dig, sumw, binv, q < nch ? &part0 : &part1, &unused, p.shift);
           } else {
@@ -528,16 +556,15 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
         // hand the four warps' shares of the K split to the epilogue warp
         part0 += __shfl_xor_sync(0xffffffffu, part0, 1);  // digits 0,1 (even c) + digit 2 (odd c)
         part1 += __shfl_xor_sync(0xffffffffu, part1, 1);
-        const int round = n / kGroups;
+        const int round = at.round();
         if (!mbar_wait(bars + 8 * (Bars::pempty1 + group), (round & 1) ^ 1, dead, status)) return;
         if (lr.cq == 0) partial[warp * 16 + lr.r] = make_float2(part0, part1);
         __syncwarp();
         if (lane == 0) mbar_arrive(bars + 8 * (Bars::pfull1 + group));
-      } else if (n % kProducers == prod) {
+      } else if (at.producer == prod) {
         jp += nchunks;  // the other group this producer serves
       }
       cn += nchunks;
-      tw.next(slots);
     }
   }
   __syncwarp();
@@ -551,8 +578,8 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
   int nmine = 0;
   {
     const int chunks2 = plan.p2c[plan.nslots];
-    const int half = plan.nunits2 / kProducers;  // units of one producer
-    int xp = 0;                                   // units this group's producer has handed out so far
+    const int units = plan.nunits2;
+    int u = 0;                                    // the next chunk's first unit
     for (int m = 0; m < plan.count2; ++m) {
       for (int j = 0; j < plan.nslots; ++j) {
         const int nchj = plan.p2c[j + 1] - plan.p2c[j];
@@ -560,9 +587,9 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
         const int wu = sl.prec ? 2 : 1;
         for (int kc = 0; kc < nchj; ++kc) {
           const int c = m * chunks2 + plan.p2c[j] + kc;  // chunk number within the phase
-          if (c % kProducers != prod) continue;
-          const int x0 = xp;
-          xp += wu;
+          const int u0 = u, u1 = u + 1 == units ? 0 : u + 1;
+          u += wu;
+          if (u >= units) u -= units;
           if (c % kGroups != group) continue;
           const int ig = c / kGroups;  // this group's ordinal of the chunk
           if (lane == 0 && nmine < kMaxMine) {
@@ -570,7 +597,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
             // both slices? | first column of the chunk in h
             const int k0 = kc * kChunkK;
             mylist[nmine] = make_uint4((unsigned)j | (unsigned)m << 16 | (unsigned)(ig % kGroupWarps) << 24,
-                                       (unsigned)(prod * half + x0 % half) | (unsigned)(prod * half + (x0 + 1) % half) << 8 |
+                                       (unsigned)u0 | (unsigned)u1 << 8 |
                                            (unsigned)(ig % kFull2PerGroup) << 16 | (unsigned)((ig / kFull2PerGroup) & 1) << 24,
                                        (unsigned)(min(kChunkK, sl.inter - k0) >> 7) | (sl.prec ? 256u : 0u),
                                        (unsigned)(sl.hoff + k0));
@@ -585,14 +612,20 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
   if (warp == 0) SM_TRACE(9);
 
   // ---- the grid's h ----
-  if (!fetch_h<G>(p, smem, warp, lane, plan.htotal, p.ws_h + (size_t)plan.hpar * kHCap, plan.never_ready != 0, dead, status,
-                  bars))
-    return;
+  if (!mbar_wait(bars + 8 * Bars::head_ready, 0, dead, status)) return;
+  if (!fetch_h<G>(p, smem, lane, plan.htotal, p.ws_h + (size_t)plan.hpar * kHCap, plan.never_ready != 0, dead, status)) return;
   if (warp == 0) SM_TRACE(10);
   if (gw == 0) SM_TRACE(14 + group);
 
   // ---- phase 2: chunks round-robin over the groups, all warps contribute to every task ----
   const uint32_t full2 = bars + 8 * Bars::full2, empty2 = bars + 8 * Bars::empty2;
+  float gate = 1.f;
+  if (p.sigmoid_gate && p.n_shared > 0) {  // Qwen-style shared-expert gate: sigmoid(v . x)
+    float dot = lane < (p.hidden >> 7) ? reinterpret_cast<const float*>(smem + SmemLayout::gate)[lane] : 0.f;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+    gate = 1.f / (1.f + expf(-dot));
+  }
   int i = 0;
   for (int m = 0; m < plan.count2; ++m) {
     float part = 0.f, unused = 0.f, sacc = 0.f;
@@ -602,7 +635,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
       if ((int)((d.x >> 16) & 0xffu) != m) break;
       const int j = d.x & 0xffffu, rot = d.x >> 24;
       if (j != jcur) {  // weighted combine, in slot order
-        if (jcur >= 0) part = fmaf(slots[jcur].gated ? plan.gate : slots[jcur].coef, sacc, part);
+        if (jcur >= 0) part = fmaf(slots[jcur].gated ? gate : slots[jcur].coef, sacc, part);
         jcur = j;
         sacc = 0.f;
       }
@@ -624,7 +657,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
         if (p8) mbar_arrive(empty2 + 8 * u1);
       }
     }
-    if (jcur >= 0) part = fmaf(slots[jcur].gated ? plan.gate : slots[jcur].coef, sacc, part);
+    if (jcur >= 0) part = fmaf(slots[jcur].gated ? gate : slots[jcur].coef, sacc, part);
     part += __shfl_xor_sync(0xffffffffu, part, 1);
     if (!mbar_wait(bars + 8 * Bars::pempty2, (m & 1) ^ 1, dead, status)) return;
     if (lr.cq == 0) partial[warp * 16 + lr.r] = make_float2(0.f, part);
@@ -637,7 +670,6 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
 
 // ---- epilogue warp ---------------------------------------------------------------------------------
 __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
-  const Slot* slots = reinterpret_cast<const Slot*>(smem + SmemLayout::slots);
   const Plan& plan = *reinterpret_cast<const Plan*>(smem + SmemLayout::plan);
   const float2* partial = reinterpret_cast<const float2*>(smem + SmemLayout::partial);
   volatile int* dead = reinterpret_cast<volatile int*>(smem + SmemLayout::dead);
@@ -655,12 +687,10 @@ __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
   float* hbuf = p.ws_h + (size_t)plan.hpar * kHCap;
   // phase 1: one group's four partial rows per task -> SwiGLU -> h
   {
-    TaskWalk tw;
-    tw.start(plan);
     for (int n = 0; n < plan.count1; ++n) {
-      tw.at(plan, n);
-      const int slot = tw.slot, idx = tw.idx;
-      const int group = n % kGroups, round = n / kGroups;
+      const int ord = task_ordinal(plan, n);
+      const TaskPlace place(plan.count_both, n);
+      const int group = place.group(), round = place.round();
       if (!mbar_wait(bars + 8 * (Bars::pfull1 + group), round & 1, dead, status)) return;
       float a = 0.f, b = 0.f;
       if (lane < 16) {
@@ -673,8 +703,7 @@ __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bars + 8 * (Bars::pempty1 + group));
-      if (lane < 16) hbuf[slots[slot].hoff + idx * 16 + lane] = a / (1.f + expf(-a)) * b;  // silu(gate) * up
-      tw.next(slots);
+      if (lane < 16) hbuf[ord * 16 + lane] = a / (1.f + expf(-a)) * b;  // silu(gate) * up
     }
   }
   SM_TRACE(12);
@@ -695,7 +724,7 @@ __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
 }
 
 // ---- producer --------------------------------------------------------------------------------------
-// What a producer lane copies, for a chunk of matrix A (and, in a pair chunk, matrix B):
+// What a producer lane copies, for a phase-1 chunk of matrix A (and, in a pair chunk, matrix B):
 //   lane 0  A's MSB tile            -> first unit, plane area
 //   lane 1  A's LSB tile (8-bit) or B's MSB tile (pair) -> second unit, plane area
 //   lane 2  A's scales, lane 3 A's zero-points          -> first unit, after the plane area
@@ -709,18 +738,6 @@ struct ProducerLane {
   int field;                 // which of the matrix' four pointers
   bool second_unit;
 };
-// The ring as a phase sees it.
-struct RingView {
-  uint32_t unit_bytes, scale_off, zp_off;
-};
-// Where one chunk goes: its two units, the barrier that says its space is free (with the parity to wait for)
-// and the barrier its bytes complete.
-struct ChunkSpace {
-  int u0, u1;
-  uint32_t empty_bar, empty_parity, full_bar;
-  uint32_t empty_bar_first, empty_parity_first;  // phase 2, two-unit chunks: the first unit has a barrier of its own
-};
-
 // What a producer needs to wait: it starts before the kernels ahead of this one in the stream have completed, so
 // a wait that does not pass at once is first the moment to wait for those (the consumers, on whom all of a
 // producer's barriers depend, do not start earlier; and a bounded wait's clock must not run while an earlier
@@ -739,49 +756,44 @@ struct ProducerWait {
   }
 };
 
-// One chunk of matrix A - or of matrices A and B side by side - of (slot, row block rb), columns from k0, into
-// the space `cs`.  Run by the first kProducerLanes lanes of a producer warp together.  Returns false if a
-// wait ran out.
+// One phase-1 chunk of (slot, row block rb), columns from k0: both slices of matrix `mat`, or (mode kModePair) the MSB tiles of gate
+// and up side by side, into the unit pair from `u` on, once it is empty.  Run by the first kProducerLanes lanes of a producer warp
+// together.  Returns false if a wait ran out.
 template <int G>
-__device__ __forceinline__ bool produce_chunk(uint8_t* smem, const RingView& rv, const ChunkSpace& cs, int lane,
-                                              const ProducerLane& pl, const Slot& s, int matA, int matB, int mode, int K,
-                                              int rb, int k0, ProducerWait& pw, uint64_t pol) {
-  constexpr int LG = G == 128 ? 7 : (G == 64 ? 6 : 5);
-  const bool two = mode != kModeSingle;
-  bool active;
+__device__ __forceinline__ bool produce_chunk(uint8_t* smem, int u, uint32_t empty_bar, uint32_t empty_parity, uint32_t bar, int lane,
+                                              const ProducerLane& pl, const Slot& s, int mat, int mode, int K, int rb, int k0,
+                                              ProducerWait& pw, uint64_t pol) {
+  constexpr int SG = 128 / G;
+  const bool pair = mode == kModePair;
   const uint8_t* src;
   if (lane == 1) {
-    active = two;
-    src = mode == kModePair ? s.ptr[matB][0] : s.ptr[matA][1];
-    if (mode == kModeBoth && src == nullptr) {  // 8 bits asked of an expert without LSB planes: defined garbage, reported
-      src = s.ptr[matA][0];
+    src = pair ? s.ptr[1][0] : s.ptr[mat][1];
+    if (!pair && src == nullptr) {  // 8 bits asked of an expert without LSB planes: defined garbage, reported
+      src = s.ptr[mat][0];
       atomicOr(pw.status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
     }
-  } else if (lane >= 4) {
-    active = mode == kModePair;
-    src = s.ptr[active ? matB : matA][pl.field];
   } else {
-    active = true;
-    src = s.ptr[matA][pl.field];
+    src = s.ptr[lane >= 4 ? 1 : mat][pl.field];
   }
   src += (size_t)((unsigned)rb * (unsigned)(K >> 7) + (unsigned)(k0 >> 7)) * pl.bytes_per_block;
   const uint32_t nblk = (uint32_t)(min(kChunkK, K - k0) >> 7);
-  // The two units of a phase-2 chunk may last have held chunks of different consumer groups: both must be free.
-  if (cs.empty_bar_first != 0u && !pw(cs.empty_bar_first, cs.empty_parity_first)) return false;
-  if (!pw(cs.empty_bar, cs.empty_parity)) return false;
-  const uint32_t bar = cs.full_bar;
-  if (lane == 0)
-    mbar_arrive_expect_tx(bar, nblk * ((two ? 2048u : 1024u) + (mode == kModePair ? 2u : 1u) * ((128u >> LG) * 48u)));
+  if (!pw(empty_bar, empty_parity)) return false;
+  if (lane == 0) mbar_arrive_expect_tx(bar, nblk * (2048u + (pair ? 2u : 1u) * (SG * 48u)));
   __syncwarp((1u << kProducerLanes) - 1u);
-  if (active) {
-    const uint32_t u = (uint32_t)(pl.second_unit ? cs.u1 : cs.u0);
-    const uint32_t dst_in_unit = pl.field < 2 ? 0u : (pl.field == 2 ? rv.scale_off : rv.zp_off);
-    bulk_g2s(smem_u32(smem + SmemLayout::ring) + u * rv.unit_bytes + dst_in_unit, src, nblk * pl.bytes_per_block, bar, pol);
+  if (lane < 4 || pair) {
+    const uint32_t at = pl.field < 2 ? 0u : pl.field == 2 ? kPlaneUnitBytes : kPlaneUnitBytes + kScaleUnitBytes;
+    bulk_g2s(smem_u32(smem + SmemLayout::ring) + (uint32_t)(pl.second_unit ? u + 1 : u) * kUnitBytes + at, src, nblk * pl.bytes_per_block, bar, pol);
   }
   return true;
 }
 
-// Producer warp `which` of kProducers: every producer walks the whole schedule and issues its share.
+// Whether a copy that was asked for before `t0` is not going to land any more: a millisecond is far more than any takes.
+__device__ __forceinline__ bool copy_overdue(long long t0, volatile int* dead) {
+  const unsigned long long waited = (unsigned long long)(clock64() - t0);
+  return waited > 2000000ull && (*dead || waited > wait_limit(dead));
+}
+
+// Producer warp `which` of kProducers (phase 1): every producer walks the whole schedule and issues its share.
 template <int G>
 __device__ void producer_loop(const DecodeParams& p, uint8_t* smem, int lane, int which) {
   constexpr int LG = G == 128 ? 7 : (G == 64 ? 6 : 5);
@@ -799,17 +811,12 @@ __device__ void producer_loop(const DecodeParams& p, uint8_t* smem, int lane, in
   pl.bytes_per_block = lane < 2 ? 1024u : (pl.field == 2 ? (128u >> LG) * 32u : (128u >> LG) * 16u);
   pl.second_unit = lane == 1 || lane >= 4;
   bool ok = true;
-  // phase 1: gate and up of (slot, row block) tasks; two units per chunk
-  RingView r1;
-  r1.unit_bytes = kUnitBytes;
-  r1.scale_off = kPlaneUnitBytes;
-  r1.zp_off = kPlaneUnitBytes + kScaleUnitBytes;
   const int nch = nchunks_of(p.hidden);
   static_assert(kGroups == 2 * kProducers, "a producer serves the groups `which` and `which + kProducers`");
   int ig_lo = 0, ig_hi = 0;  // chunks armed so far for group `which` and for group `which + kProducers`
   {
-    TaskWalk tw;
-    tw.start(plan);
+    const int per_s = p.shared_inter / 16, per_r = p.inter / 16, shared_tasks = p.n_shared * per_s;  // tasks of a slot
+    const float inv_r = 1.f / (float)per_r;
     int jp = 0;  // this warp's chunks so far
     // The shared experts' tasks are known from the start; what follows them - and how many tasks there are - once
     // the plan stands.
@@ -821,69 +828,34 @@ __device__ void producer_loop(const DecodeParams& p, uint8_t* smem, int lane, in
         n_end = plan.count1;
       }
       if (n >= n_end) break;
-      tw.at(plan, n);
-      const int slot = tw.slot, idx = tw.idx;
-      const Slot& s = slots[slot];
-      const int nchunks = s.prec ? 2 * nch : nch;
-      if (n % kProducers == which) {
-        const int g = n % kGroups;
+      const TaskPlace place(n < plan.count_s ? n + 1 : plan.count_both, n);
+      if (place.producer == which) {
+        const int ord = task_ordinal(plan, n), routed = ord - shared_tasks;
+        int slot, idx;
+        if (routed < 0) {
+          slot = ord / per_s;
+          idx = ord - slot * per_s;
+        } else {  // (the first request waits for this: no integer division)
+          slot = (int)((float)routed * inv_r);
+          idx = routed - slot * per_r;
+          if (idx < 0) --slot, idx += per_r;
+          if (idx >= per_r) ++slot, idx -= per_r;
+          slot += p.n_shared;
+        }
+        const Slot& s = slots[slot];
+        const int nchunks = s.prec ? 2 * nch : nch;
+        const int g = place.group();
         for (int q = 0; q < nchunks && ok; ++q, ++jp) {
-          const int mat = s.prec ? q / nch : 0;
-          ChunkSpace cs;
-          cs.u0 = 4 * which + 2 * (jp & 1);
-          cs.u1 = cs.u0 + 1;
-          cs.empty_bar = bars + 8 * (Bars::empty + 2 * which + (jp & 1));
-          cs.empty_parity = ((jp >> 1) & 1) ^ 1;
-          cs.empty_bar_first = 0u;  // a phase-1 unit pair always holds one chunk: one barrier
-          cs.empty_parity_first = 0u;
           int& igg = g == which ? ig_lo : ig_hi;
-          cs.full_bar = bars + 8 * (Bars::full + 2 * g + (igg & 1));
+          ok = produce_chunk<G>(smem, 4 * which + 2 * (jp & 1), bars + 8 * (Bars::empty + 2 * which + (jp & 1)), ((jp >> 1) & 1) ^ 1,
+                                bars + 8 * (Bars::full + 2 * g + (igg & 1)), lane, pl, s, s.prec ? q / nch : 0,
+                                s.prec ? kModeBoth : kModePair, p.hidden, idx, (q % nch) * kChunkK, pw, pol);
           ++igg;
-          ok = produce_chunk<G>(smem, r1, cs, lane, pl, s, mat, s.prec ? mat : 1, s.prec ? kModeBoth : kModePair, p.hidden,
-                                idx, (q % nch) * kChunkK, pw, pol);
           if (which == 0 && lane == 0 && jp < 8) SM_TRACE(32 + jp);
         }
       }
-      tw.next(slots);
     }
   }
-  // phase 2: down rows of every slot for the output row blocks of this CTA, in the re-cut ring
-  RingView r2;
-  r2.unit_bytes = (uint32_t)plan.unit2_bytes;
-  r2.scale_off = (uint32_t)plan.scale2_off;
-  r2.zp_off = (uint32_t)plan.zp2_off;
-  // The re-cut units lie over the phase-1 units: nothing of phase 2 lands before phase 1 has been consumed.
-  // (From then until h has crossed the grid the memory system has nothing else to do.)
-  if (ok && plan.count2 > 0) ok = pw(bars + 8 * Bars::p1_done, 0);
-  if (which == 0 && lane == 0 && plan.count2 > 0) SM_TRACE(31);
-  const int half = plan.nunits2 / kProducers;  // this warp's units are [which * half, which * half + half)
-  int c2 = 0, xp = 0;                           // chunks of the phase so far, units this warp has handed out
-  for (int m = 0; m < plan.count2 && ok; ++m) {
-    const int rb = blockIdx.x + m * gridDim.x;
-    for (int slot = 0; slot < plan.nslots && ok; ++slot) {
-      const Slot& s = slots[slot];
-      const int w = s.prec ? 2 : 1;
-      for (int k0 = 0; k0 < s.inter && ok; k0 += kChunkK, ++c2) {
-        if (c2 % kProducers != which) continue;
-        const int g = c2 % kGroups, ig = c2 / kGroups;
-        const int xl = xp + w - 1;  // the chunk's last unit
-        ChunkSpace cs;
-        cs.u0 = which * half + xp % half;
-        cs.u1 = which * half + (xp + 1) % half;
-        cs.empty_bar = bars + 8 * (Bars::empty2 + which * half + xl % half);
-        cs.empty_parity = ((xl / half) & 1) ^ 1;
-        cs.empty_bar_first = w == 2 ? bars + 8 * (Bars::empty2 + which * half + xp % half) : 0u;
-        cs.empty_parity_first = ((xp / half) & 1) ^ 1;
-        cs.full_bar = bars + 8 * (Bars::full2 + kFull2PerGroup * g + ig % kFull2PerGroup);
-        xp += w;
-        ok = produce_chunk<G>(smem, r2, cs, lane, pl, s, 2, 2, s.prec ? kModeBoth : kModeSingle, s.inter, rb, k0, pw, pol);
-      }
-    }
-  }
-  if (lane == 0 && plan.count2 > 0) SM_TRACE(18 + which);
-#ifdef SLICEMOE_TRACE
-  int landed = 0;
-#endif
   // Never leave the CTA with bulk copies still landing in its shared memory: wait (bounded) until every
   // barrier this warp may have armed has completed its last phase.  In the normal path they have long ago.
   for (int g = which; g < kGroups; g += kProducers) {
@@ -891,27 +863,85 @@ __device__ void producer_loop(const DecodeParams& p, uint8_t* smem, int lane, in
     for (int i = max(0, n1 - 2); i < n1; ++i) {
       const long long t0 = clock64();
       while (!mbar_try(bars + 8 * (Bars::full + 2 * g + (i & 1)), (i >> 1) & 1)) {
-        if (*dead || (unsigned long long)(clock64() - t0) > wait_limit(dead)) break;
+        if (copy_overdue(t0, dead)) break;
       }
     }
-    const int n2 = c2 > g ? (c2 - 1 - g) / kGroups + 1 : 0;  // chunks of the phase that went to group g
-    for (int i = max(0, n2 - kFull2PerGroup); i < n2; ++i) {
-      const long long t0 = clock64();
-      while (!mbar_try(bars + 8 * (Bars::full2 + kFull2PerGroup * g + i % kFull2PerGroup), (i / kFull2PerGroup) & 1)) {
-        if (*dead || (unsigned long long)(clock64() - t0) > wait_limit(dead)) break;
-      }
-#ifdef SLICEMOE_TRACE
-      if (lane == 0 && landed < 4) SM_TRACE(40 + 4 * which + landed);
-      ++landed;
-#endif
+  }
+}
+
+// The down tiles: rows of every slot for the output row blocks of this CTA, in the re-cut ring.  Nothing else is left to bring
+// by then and everybody waits for these, so a lane asks for one array of one chunk: what it copies is worked out while phase 1
+// still runs, and up to eight chunks are asked for by one instruction (a warp issues copies lane by lane, 60 cycles each; chunk
+// after chunk, with what goes into one worked out in between, was 1700 cycles a chunk).
+template <int G>
+__device__ void down_loop(const DecodeParams& p, uint8_t* smem, int lane) {
+  constexpr int SG = 128 / G;
+  const Slot* slots = reinterpret_cast<const Slot*>(smem + SmemLayout::slots);
+  const Plan& plan = *reinterpret_cast<const Plan*>(smem + SmemLayout::plan);
+  volatile int* dead = reinterpret_cast<volatile int*>(smem + SmemLayout::dead);
+  const uint32_t bars = smem_u32(smem + SmemLayout::bars);
+  unsigned* status = &p.ws->status;
+  if (!mbar_wait(bars + 8 * Bars::plan_ready, 0, dead, status) || plan.count2 == 0) return;
+  const uint64_t pol = l2_evict_first_policy();
+  const int units = plan.nunits2, chunks = plan.p2c[plan.nslots], chunk_units = plan.p2u[plan.nslots], total = plan.count2 * chunks;
+  const int array = lane & 3;  // MSB plane, LSB plane, scales, zero-points
+  const uint32_t block_bytes = array < 2 ? 1024u : array == 2 ? SG * 32u : SG * 16u;
+  int done = 0;  // chunks asked for
+  bool ok = true;
+  while (done < total && ok) {
+    // Up to eight chunks at a time.  A lane's chunk: row block m, slot j, columns from k0 on, first unit x of a running count.
+    const int at = lane >> 2, base = done, c = base + at, n = min(8, total - base);
+    const int m = c / chunks, r = c - m * chunks;
+    int j = 0;
+    while (j + 1 < plan.nslots && plan.p2c[j + 1] <= r) ++j;
+    const Slot& s = slots[j];
+    const int w = s.prec ? 2 : 1, k0 = (r - plan.p2c[j]) * kChunkK, x = m * chunk_units + plan.p2u[j] + (r - plan.p2c[j]) * w;
+    const int nblk = min(kChunkK, s.inter - k0) >> 7;
+    const uint8_t* src = s.ptr[2][array];
+    if (at < n && array == 1 && s.prec && src == nullptr) {  // 8 bits asked of an expert without LSB planes: defined garbage, reported
+      src = s.ptr[2][0];
+      atomicOr(status, (unsigned)SLICEMOE_STATUS_MISSING_LSB);
     }
+    src += (size_t)((unsigned)(blockIdx.x + m * gridDim.x) * (unsigned)(s.inter >> 7) + (unsigned)(k0 >> 7)) * block_bytes;
+    const int lap0 = x / units, u0 = x - lap0 * units, u1 = u0 + 1 == units ? 0 : u0 + 1, lap1 = u1 == 0 ? lap0 + 1 : lap0;
+    const uint32_t dst = smem_u32(smem + SmemLayout::ring) + (uint32_t)(array == 1 ? u1 : u0) * (uint32_t)plan.unit2_bytes +
+                         (array < 2 ? 0u : (uint32_t)(array == 2 ? plan.scale2_off : plan.zp2_off));
+    const uint32_t bar = bars + 8 * (Bars::full2 + kFull2PerGroup * (c % kGroups) + c / kGroups % kFull2PerGroup);
+    const uint32_t bytes = (uint32_t)nblk * block_bytes, all_bytes = (uint32_t)nblk * ((w == 2 ? 2048u : 1024u) + SG * 48u);
+    if (base == 0) {
+      // The re-cut units lie over the phase-1 units: nothing of phase 2 lands before phase 1 has been consumed.
+      ok = mbar_wait(bars + 8 * Bars::p1_done, 0, dead, status);
+      SM_TRACE(31);
+    }
+    // what finds its units empty goes at once, the rest chunk by chunk as units become free
+    const int fresh = __popc(__ballot_sync(0xffffffffu, at < n && x + w <= units)) >> 2;
+    for (int q = 0; q < n; q = max(q + 1, fresh)) {
+      const int end = max(q + 1, fresh);
+      const bool mine = at >= q && at < end;
+      if (ok && mine && lap0 > 0) ok = mbar_wait(bars + 8 * (Bars::empty2 + u0), (lap0 & 1) ^ 1, dead, status);
+      if (ok && mine && w == 2 && lap1 > 0) ok = mbar_wait(bars + 8 * (Bars::empty2 + u1), (lap1 & 1) ^ 1, dead, status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      if (mine && array == 0) mbar_arrive_expect_tx(bar, all_bytes);
+      __syncwarp();
+      if (mine && (array != 1 || w == 2)) bulk_g2s(dst, src, bytes, bar, pol);
+      done += end - q;
+    }
+  }
+  SM_TRACE(18);
+  // no copy may still be landing when the CTA ends (in the normal path they have all been consumed); at most as many are on
+  // their way as there are units
+  const int c = done - 1 - lane;
+  if (lane < kUnits2 && c >= 0) {
+    const long long t0 = clock64();
+    while (!mbar_try(bars + 8 * (Bars::full2 + kFull2PerGroup * (c % kGroups) + c / kGroups % kFull2PerGroup), (c / kGroups / kFull2PerGroup) & 1))
+      if (copy_overdue(t0, dead)) break;
   }
 }
 
 // ---- prologue pieces ---------------------------------------------------------------------------------
 // Slot order: shared experts, then the routed experts that run at 8 bits, then those that run at 4 bits,
-// each group in list order.  With the larger tasks first, windows of a multiple of the larger task size cut
-// the phase-1 unit sequence at task boundaries, so every CTA gets the same number of units.
+// each group in list order.
 //
 // The routing list as one warp sees it: lane j < k holds entry j; out-of-range ids are dropped.
 struct Routed {
@@ -941,9 +971,9 @@ __device__ __forceinline__ Routed read_routing(const DecodeParams& p, int lane, 
       }
     }
   } else if (lane < p.k) {
-    rt.e = p.ids[lane];
-    rt.pr = p.prec[lane];
-    rt.w = p.weights[lane];
+    rt.e = __ldcg(p.ids + lane);
+    rt.pr = __ldcg(p.prec + lane);
+    rt.w = __ldcg(p.weights + lane);
   }
   rt.valid = lane < p.k && rt.e >= 0 && rt.e < p.n_experts;
   const unsigned vmask = __ballot_sync(0xffffffffu, rt.valid);
@@ -953,6 +983,30 @@ __device__ __forceinline__ Routed read_routing(const DecodeParams& p, int lane, 
   rt.nsmall = __popc(vmask) - rt.nbig;
   rt.pos = p.n_shared + (rt.pr != 0 ? __popc(bigmask & below) : rt.nbig + __popc(vmask & ~bigmask & below));
   return rt;
+}
+
+// The plane pointers of `count` slots from `first` on; each slot's expert is shared + slot, or what the slot table's first pointer
+// names.  A slot's twelve pointers sit in slicemoe_expert in the order the slot table keeps them.
+__device__ __forceinline__ void load_slot_pointers(const DecodeParams& p, Slot* slots, int lane, int first, int count, bool routed) {
+  constexpr int kRounds = (kMaxSlots * 12 + 31) / 32;
+  unsigned long long val[kRounds];
+#pragma unroll
+  for (int rd = 0; rd < kRounds; ++rd) {  // all loads in flight together
+    if (rd * 32 >= count * 12) break;
+    const int i = rd * 32 + lane;
+    if (i < count * 12) {
+      const int sl = first + i / 12, q = i % 12;
+      const slicemoe_expert* ex = routed ? reinterpret_cast<const slicemoe_expert*>(slots[sl].ptr[0][0]) : p.shared + sl;
+      val[rd] = __ldcg(reinterpret_cast<const unsigned long long*>(reinterpret_cast<const slicemoe_mat*>(ex) + (q >> 2)) + (q & 3));
+    }
+  }
+  __syncwarp();  // every lane has read the experts' addresses before the first slot pointer overwrites one
+#pragma unroll
+  for (int rd = 0; rd < kRounds; ++rd) {
+    if (rd * 32 >= count * 12) break;
+    const int i = rd * 32 + lane;
+    if (i < count * 12) slots[first + i / 12].ptr[(i % 12) >> 2][i & 3] = reinterpret_cast<const uint8_t*>(val[rd]);
+  }
 }
 
 // What of the plan depends on the shape and the grid alone; one lane computes it while the kernel still waits
@@ -971,11 +1025,9 @@ __device__ __forceinline__ void plan_units2(const DecodeParams& p, Plan* plan, i
   plan->unit2_bytes = (maxblk * (1024 + meta_blk * 3) + 127) & ~127;
   plan->nunits2 = min(kUnits2, (kUnits * kUnitBytes) / plan->unit2_bytes);
 }
-// Shared-expert tasks before CTA c when the grid's T1 of them are dealt out evenly.
-__device__ __forceinline__ unsigned shared_before(unsigned c, unsigned T1, unsigned P) {
-  return (unsigned)((unsigned long long)c * T1 / P);
-}
-// Run by warp 0.
+// How many of n things, dealt to P CTAs one by one, go to CTA c.
+__device__ __forceinline__ int dealt(int n, int c, int P) { return n > c ? (n - c + P - 1) / P : 0; }
+// Run by the epilogue warp, as what follows.
 __device__ void build_plan_static(const DecodeParams& p, uint8_t* smem, int lane) {
   Slot* slots = reinterpret_cast<Slot*>(smem + SmemLayout::slots);
   Plan* plan = reinterpret_cast<Plan*>(smem + SmemLayout::plan);
@@ -991,22 +1043,15 @@ __device__ void build_plan_static(const DecodeParams& p, uint8_t* smem, int lane
   const int nrb = p.hidden / 16;
   plan->count2 = (int)blockIdx.x < nrb ? (nrb - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   plan_units2(p, plan, phase2_unit_blocks(p, p.k > 0));
-  // this CTA's share of the shared experts' phase-1 tasks
-  const unsigned nts = p.n_shared ? (unsigned)p.shared_inter / 16u : 0u, T1 = (unsigned)p.n_shared * nts;
-  const unsigned lo = shared_before(blockIdx.x, T1, gridDim.x), hi = shared_before(blockIdx.x + 1u, T1, gridDim.x);
-  plan->slot_s = nts ? (int)(lo / nts) : 0;
-  plan->idx_s = nts ? (int)(lo % nts) : 0;
-  plan->count_s = (int)(hi - lo);
+  plan->count_s = dealt(p.n_shared * (p.shared_inter / 16), (int)blockIdx.x, (int)gridDim.x);
 }
 
-// Warp 0: slot table (all but the pointers) and the static partition, in closed form: the phase-1 unit
-// sequence is three runs of equal tasks (shared, routed 8-bit, routed 4-bit).
+// The routed slots (all but the pointers) and the partition, in closed form.
 template <bool FUSED>
-__device__ void build_plan(const DecodeParams& p, uint8_t* smem, int lane) {
+__device__ __forceinline__ void build_plan(const DecodeParams& p, uint8_t* smem, int lane) {
   Slot* slots = reinterpret_cast<Slot*>(smem + SmemLayout::slots);
   Plan* plan = reinterpret_cast<Plan*>(smem + SmemLayout::plan);
   const Routed rt = read_routing<FUSED>(p, lane, true);
-  if (lane < p.k && !rt.valid) atomicOr(&p.ws->status, (unsigned)SLICEMOE_STATUS_BAD_EXPERT_ID);
   if (rt.valid) {
     Slot& s = slots[rt.pos];
     s.inter = p.inter;
@@ -1014,102 +1059,68 @@ __device__ void build_plan(const DecodeParams& p, uint8_t* smem, int lane) {
     s.coef = rt.w;
     s.gated = 0;
     s.hoff = p.n_shared * p.shared_inter + (rt.pos - p.n_shared) * p.inter;
+  } else if (lane < p.k) {
+    atomicOr(&p.ws->status, (unsigned)SLICEMOE_STATUS_BAD_EXPERT_ID);
   }
-  const int nslots = p.n_shared + rt.nbig + rt.nsmall;
-  // phase-2 chunk and unit counts before each slot: lane j handles slot j (8-bit: shared and the first nbig routed)
+  __syncwarp();
   {
-    int cj = 0, uj = 0;
-    if (lane < nslots) {
-      const int inter = lane < p.n_shared ? p.shared_inter : p.inter;
-      const bool p8 = lane < p.n_shared + rt.nbig;
-      cj = nchunks_of(inter);
-      uj = p8 ? 2 * cj : cj;
-    }
-    int ci = cj, ui = uj;  // inclusive scans
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int a = __shfl_up_sync(0xffffffffu, ci, off), b = __shfl_up_sync(0xffffffffu, ui, off);
-      if (lane >= off) {
-        ci += a;
-        ui += b;
+    const int nslots = p.n_shared + rt.nbig + rt.nsmall;
+    // phase-2 chunk and unit counts before each slot: lane j handles slot j (8-bit: shared and the first nbig routed)
+    {
+      int cj = 0, uj = 0;
+      if (lane < nslots) {
+        const int inter = lane < p.n_shared ? p.shared_inter : p.inter;
+        const bool p8 = lane < p.n_shared + rt.nbig;
+        cj = nchunks_of(inter);
+        uj = p8 ? 2 * cj : cj;
       }
+      int ci = cj, ui = uj;  // inclusive scans
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, ci, off), b = __shfl_up_sync(0xffffffffu, ui, off);
+        if (lane >= off) {
+          ci += a;
+          ui += b;
+        }
+      }
+      if (lane < nslots) {
+        plan->p2c[lane + 1] = (short)ci;
+        plan->p2u[lane + 1] = (short)ui;
+      }
+      if (lane == 0) plan->p2c[0] = plan->p2u[0] = 0;
     }
-    if (lane < nslots) {
-      plan->p2c[lane + 1] = (short)ci;
-      plan->p2u[lane + 1] = (short)ui;
+    if (lane == 0) {
+      const int c = (int)blockIdx.x, P = (int)gridDim.x, per = p.inter / 16;
+      const int nboth = p.n_shared * (p.shared_inter / 16) + rt.nbig * per, nmsb = rt.nsmall * per;  // tasks
+      const int q = nboth / P, r = nboth - q * P, light = r ? P - r : 0, first = min(nmsb, 2 * light), rest = nmsb - first;
+      const int at = c - r, rest_q = rest / P;  // (the two divisions of this chain)
+      plan->count_both = q + (c < r ? 1 : 0);
+      plan->light = light;
+      plan->count_light = at >= 0 ? (at < first ? 1 : 0) + (at + light < first ? 1 : 0) : 0;
+      plan->count1 = plan->count_both + plan->count_light + rest_q + (c < rest - rest_q * P ? 1 : 0);
+      plan->ord_light = nboth + at;
+      plan->ord_rest = nboth + first + c;
+      if (nslots == 0) plan->count2 = 0;  // otherwise as build_plan_static left it
+      plan->nslots = nslots;
+      plan->htotal = p.n_shared * p.shared_inter + (rt.nbig + rt.nsmall) * p.inter;
+      // phase-2 units: as large as the widest down chunk of any slot (set ahead of time for the usual case)
+      if (rt.nbig + rt.nsmall == 0 && p.k > 0) plan_units2(p, plan, phase2_unit_blocks(p, false));
     }
-    if (lane == 0) plan->p2c[0] = plan->p2u[0] = 0;
   }
-  {
-    const unsigned nsh = (unsigned)p.n_shared, nbig = (unsigned)rt.nbig, nsmall = (unsigned)rt.nsmall;
-    const unsigned nts = nsh ? (unsigned)p.shared_inter / 16u : 0u, ntr = (unsigned)p.inter / 16u;
-    const unsigned nch = (unsigned)nchunks_of(p.hidden);
-    const unsigned spb = 4u * nch, sps = 2u * nch;  // units per 8-bit / 4-bit task (shared tasks are 8-bit)
-    const unsigned T1 = nsh * nts, T2 = nbig * ntr, T3 = nsmall * ntr;  // tasks per run
-    const unsigned U1 = T1 * spb, U2 = T2 * spb, S = U1 + U2 + T3 * sps;
-    const unsigned spmax = (nsh + nbig) ? spb : sps;
-    // Every CTA gets T units of work: its shared tasks (dealt out evenly, build_plan_static) and a window of the
-    // routed unit sequence that fills the rest.  T and every shared share are multiples of the larger task size,
-    // and the larger routed tasks come first, so the windows are cut at task boundaries.
-    const unsigned T = ((S + gridDim.x - 1) / gridDim.x + spmax - 1) / spmax * spmax;
-    const unsigned UR = U2 + T3 * sps;  // the routed sequence
-    // ordinal of the first routed task that starts at or after a unit offset of the routed sequence
-    auto ord_of = [&](unsigned bound) -> unsigned {
-      if (bound >= UR) return T2 + T3;
-      if (bound < U2) return (bound + spb - 1) / spb;
-      return T2 + (bound - U2 + sps - 1) / sps;
-    };
-    // both ends of this CTA's window at once: lane 1 takes the upper one
-    const unsigned cc = blockIdx.x + (unsigned)(lane & 1);
-    const unsigned o = ord_of(cc * T - spb * shared_before(cc, T1, gridDim.x));
-    const unsigned o0 = __shfl_sync(0xffffffffu, o, 0), o1 = __shfl_sync(0xffffffffu, o, 1);
-    if (lane != 0) return;
-    plan->first_slot = (int)(nsh + o0 / ntr);
-    plan->first_idx = (int)(o0 % ntr);
-    plan->count1 = plan->count_s + (int)(o1 - o0);
-    if (nslots == 0) plan->count2 = 0;  // otherwise as build_plan_static left it
-    plan->nslots = nslots;
-    plan->htotal = (int)(nsh * (unsigned)p.shared_inter + (nbig + nsmall) * (unsigned)p.inter);
-    // phase-2 units: as large as the widest down chunk of any slot (set ahead of time for the usual case)
-    if (nbig + nsmall == 0 && p.k > 0) plan_units2(p, plan, phase2_unit_blocks(p, false));
-  }
+  __syncwarp();
+  if (lane == 0) mbar_arrive(smem_u32(smem + SmemLayout::bars) + 8 * Bars::plan_ready);
 }
-
-// Warp 1: the routed slots' plane pointers.  Warp 2: the shared slots' (they do not depend on the list).
-// Each slot's twelve pointers sit in slicemoe_expert in the order the slot table keeps them.
+// The routed slots' pointers.
 template <bool FUSED>
-__device__ void load_slot_pointers(const DecodeParams& p, uint8_t* smem, int lane, bool routed) {
+__device__ __forceinline__ void routed_pointers(const DecodeParams& p, uint8_t* smem, int lane) {
   Slot* slots = reinterpret_cast<Slot*>(smem + SmemLayout::slots);
-  constexpr int kRounds = (kMaxSlots * 12 + 31) / 32;
-  const uint8_t* const* src[kRounds];
-  int first = 0, count = p.n_shared;
-  if (routed) {
-    const Routed rt = read_routing<FUSED>(p, lane, false);
-    first = p.n_shared;
-    count = rt.nbig + rt.nsmall;
-    // lane j knows its entry's slot; every lane needs every slot's expert: pass them through the slot table
-    if (rt.valid) slots[rt.pos].ptr[0][0] = reinterpret_cast<const uint8_t*>(p.experts + rt.e);
-    __syncwarp();
-  }
-#pragma unroll
-  for (int rd = 0; rd < kRounds; ++rd) {
-    const int i = rd * 32 + lane;
-    src[rd] = nullptr;
-    if (i < count * 12) {
-      const int sl = first + i / 12, q = i % 12;
-      const slicemoe_expert* ex = routed ? reinterpret_cast<const slicemoe_expert*>(slots[sl].ptr[0][0]) : p.shared + sl;
-      src[rd] = reinterpret_cast<const uint8_t* const*>(reinterpret_cast<const slicemoe_mat*>(ex) + (q >> 2)) + (q & 3);
-    }
-  }
-  __syncwarp();  // every lane has read the experts' addresses before the first slot pointer overwrites one
-  const uint8_t* val[kRounds];
-#pragma unroll
-  for (int rd = 0; rd < kRounds; ++rd) val[rd] = src[rd] ? *src[rd] : nullptr;  // all loads in flight together
-#pragma unroll
-  for (int rd = 0; rd < kRounds; ++rd) {
-    const int i = rd * 32 + lane;
-    if (i < count * 12) slots[first + i / 12].ptr[(i % 12) >> 2][(i % 12) & 3] = val[rd];
-  }
+  const Routed rt = read_routing<FUSED>(p, lane, false);
+  // lane j knows its entry's slot; every lane needs every slot's expert: passed through the slot table
+  if (rt.valid) slots[rt.pos].ptr[0][0] = reinterpret_cast<const uint8_t*>(p.experts + rt.e);
+  __syncwarp();
+  load_slot_pointers(p, slots, lane, p.n_shared, rt.nbig + rt.nsmall, true);
+  __syncwarp();
+  if (lane == 0) mbar_arrive(smem_u32(smem + SmemLayout::bars) + 8 * Bars::plan_ready);
 }
 
 // ---- the kernel ------------------------------------------------------------------------------------
@@ -1136,6 +1147,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
   if (warp == kProducerWarp) {
     if (lane == 0) {
       *reinterpret_cast<int*>(smem + SmemLayout::dead) = 0;
+      *reinterpret_cast<int*>(smem + SmemLayout::hnext) = 0;
       *reinterpret_cast<unsigned long long*>(smem + SmemLayout::dead + 8) = kWaitCycles;
       for (int i = 0; i < kHCap / 128; i += 8) *reinterpret_cast<unsigned long long*>(smem + SmemLayout::hready + i) = 0ull;
       const uint32_t bars = smem_u32(smem + SmemLayout::bars);
@@ -1152,7 +1164,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
       mbar_init(bars + 8 * Bars::pfull2, kConsumerWarps);
       mbar_init(bars + 8 * Bars::pempty2, 1);
       mbar_init(bars + 8 * Bars::p1_done, kConsumerWarps);
-      mbar_init(bars + 8 * Bars::plan_ready, 2);  // warps 0 and 1 each say when done
+      mbar_init(bars + 8 * Bars::plan_ready, 2);  // the plan, the pointers
+      mbar_init(bars + 8 * Bars::head_ready, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -1160,106 +1173,105 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
   // Ahead of the wait: what follows from the shape alone - the shared experts' slots, pointers and this CTA's share
   // of their tasks - and the routed experts' pointer table on its way into L2 (its entries are read right after the
   // wait).
-  if (warp == 0) {
+  if (warp == kEpilogueWarp) {
     build_plan_static(p, smem, lane);
+  } else if (warp == kDownWarp) {
+    if (p.n_shared > 0) load_slot_pointers(p, reinterpret_cast<Slot*>(smem + SmemLayout::slots), lane, 0, p.n_shared, false);
   } else if (warp == 1 && p.experts != nullptr && p.k > 0 && !early_lists) {
     const char* tab = reinterpret_cast<const char*>(p.experts);
     const size_t bytes = (size_t)p.n_experts * sizeof(slicemoe_expert);
     for (size_t off = (size_t)lane * 128; off < bytes; off += 32 * 128)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(tab + off));
-  } else if (warp == 2) {
-    if (p.n_shared > 0) load_slot_pointers<FUSED>(p, smem, lane, false);
   }
   __syncthreads();
-  const uint32_t plan_ready = smem_u32(smem + SmemLayout::bars) + 8 * Bars::plan_ready;
-  if (warp >= kProducerWarp) {
+  if (warp >= kProducerWarp && warp < kDownWarp) {
     // The producers start on the shared experts' tiles (and, with resident lists, go on to the routed experts')
     // while the kernels ahead are still running; see ProducerWait for where they wait for those.
     if (lane < kProducerLanes) producer_loop<G>(p, smem, lane, warp - kProducerWarp);
     return;
   }
 
-  // Everyone else waits here.  Then, in parallel and with one barrier (of these 17 warps) at the end: warp 0 reads
-  // the routing list and builds the routed slots and the partition, warp 1 fetches the routed experts' plane
-  // pointers, warp 2 takes the wait limit and the shared-expert gate, the other 14 warps turn x into digits, one
-  // 128-element block at a time.
-  // (With resident lists warps 0 and 1 do their part first, while the producers are already busy with the shared
-  // experts' tiles, and tell the producers themselves.)
-  if (early_lists && warp < 2) {
-    if (warp == 0) build_plan<FUSED>(p, smem, lane);
-    else load_slot_pointers<FUSED>(p, smem, lane, true);
+  // Everyone else waits here.  Then the consumer warps turn x into digits, one or two 128-element blocks each, and go on to
+  // the shared experts' tiles, while the epilogue warp reads the routing list, builds the routed slots and the partition and
+  // tells everybody.  (With resident lists it does so first, while the producers are already busy with the shared experts'
+  // tiles.)  What a kernel ahead may have written is read past L1: it may have run on this SM after this CTA began.
+  if (warp == kDownWarp) {
+    if (early_lists) routed_pointers<FUSED>(p, smem, lane);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // readers, epoch, status, extra_arrivals; a wait limit set by the host for this workspace
+    const uint4 head = __ldcg(reinterpret_cast<const uint4*>(p.ws));
+    const unsigned long long lim = __ldcg(&p.ws->wait_cycles);
+    if (!early_lists) routed_pointers<FUSED>(p, smem, lane);
+    if (lane == 0) {
+      if (lim != 0ull) *reinterpret_cast<unsigned long long*>(smem + SmemLayout::dead + 8) = lim;
+      // Which h buffer: the parity of the launch count.  The count moves on once every CTA of this launch has
+      // read it (the last reader does it), so all of them see the same value, and the next launch the next.
+      plan->hpar = (int)(head.y & 1u);
+      plan->never_ready = head.w != 0u ? 1 : 0;
+      mbar_arrive(smem_u32(smem + SmemLayout::bars) + 8 * Bars::head_ready);
+      if (atomicAdd(&p.ws->readers, 1u) == gridDim.x - 1u) {
+        p.ws->readers = 0u;
+        p.ws->epoch = head.y + 1u;
+        __threadfence();
+      }
+    }
     __syncwarp();
-    if (lane == 0) mbar_arrive(plan_ready);
+    down_loop<G>(p, smem, lane);
+    return;
+  }
+  if (warp == kEpilogueWarp) {
+    if (!early_lists) asm volatile("griddepcontrol.wait;" ::: "memory");
+    build_plan<FUSED>(p, smem, lane);
+    if (early_lists) asm volatile("griddepcontrol.wait;" ::: "memory");
+    SM_TRACE(2);
+    if (mbar_wait(smem_u32(smem + SmemLayout::bars) + 8 * Bars::head_ready, 0, reinterpret_cast<volatile int*>(smem + SmemLayout::dead), &p.ws->status))
+      epilogue_loop(p, smem, lane);
+    return;
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 3) {
     SM_TRACE(1);
     SM_TRACE_G(21);
   }
-  if (warp == 0) {
-    if (!early_lists) {
-      build_plan<FUSED>(p, smem, lane);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(plan_ready);
-    }
-    SM_TRACE(2);
-  } else if (warp == 1) {
-    if (!early_lists) {
-      load_slot_pointers<FUSED>(p, smem, lane, true);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(plan_ready);
-    }
-  } else if (warp == 2) {
-    if (lane == 0) {
-      // a wait limit set by the host for this workspace
-      const unsigned long long lim = p.ws->wait_cycles;
-      if (lim != 0ull) *reinterpret_cast<unsigned long long*>(smem + SmemLayout::dead + 8) = lim;
-      // Which h buffer: the parity of the launch count.  The count moves on once every CTA of this launch has
-      // read it (the last reader does it), so all of them see the same value, and the next launch the next.
-      const unsigned epoch = p.ws->epoch;
-      plan->hpar = (int)(epoch & 1u);
-      plan->never_ready = p.ws->extra_arrivals != 0u ? 1 : 0;
-      if (atomicAdd(&p.ws->readers, 1u) == gridDim.x - 1u) {
-        p.ws->readers = 0u;
-        p.ws->epoch = epoch + 1u;
-        __threadfence();
-      }
-    }
-    if (p.sigmoid_gate && p.n_shared > 0) {
-      // Qwen-style shared-expert gate: sigmoid(v . x)
-      float dot = 0.f;
-      for (int i = lane; i < p.hidden / 2; i += 32) {
-        const uint32_t raw = *reinterpret_cast<const uint32_t*>(p.x + 2 * i);
-        const float2 gv = __ldg(reinterpret_cast<const float2*>(p.gate_vec) + i);
-        dot = fmaf(gv.x, __uint_as_float(raw << 16), dot);
-        dot = fmaf(gv.y, __uint_as_float(raw & 0xffff0000u), dot);
-      }
+  {
+    constexpr int kMine = kMaxHidden / 128 / kConsumerWarps;
+    const bool gated = p.sigmoid_gate && p.n_shared > 0;
+    uint2 raw[kMine];
+    float gv[kMine][4];
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-      if (lane == 0) plan->gate = 1.f / (1.f + expf(-dot));
+    for (int i = 0; i < kMine; ++i)
+      if ((warp + kConsumerWarps * i) * 128 < p.hidden)
+        raw[i] = __ldcg(reinterpret_cast<const uint2*>(p.x + (warp + kConsumerWarps * i) * 128) + lane);
+    if (gated) {
+#pragma unroll
+      for (int i = 0; i < kMine; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          gv[i][j] = (warp + kConsumerWarps * i) * 128 < p.hidden ? __ldg(p.gate_vec + (warp + kConsumerWarps * i) * 128 + 4 * lane + j) : 0.f;
     }
-  } else {
-    // warps 3 .. 16
-    constexpr int nw = kConsumerWarps + 1 - 3;
-    for (int blk = warp - 3; blk < p.hidden / 128; blk += nw) {
-      const uint2 raw = *reinterpret_cast<const uint2*>(p.x + blk * 128 + 4 * lane);
-      const float v[4] = {__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
-                          __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u)};
-      block_to_digits<G>(v, blk * 128, lane, smem + SmemLayout::xdig, reinterpret_cast<float*>(smem + SmemLayout::xsumw),
-                         reinterpret_cast<float*>(smem + SmemLayout::xinv));
+#pragma unroll
+    for (int i = 0; i < kMine; ++i) {
+      const int blk = warp + kConsumerWarps * i;
+      if (blk * 128 < p.hidden) {
+        const float v[4] = {__uint_as_float(raw[i].x << 16), __uint_as_float(raw[i].x & 0xffff0000u),
+                            __uint_as_float(raw[i].y << 16), __uint_as_float(raw[i].y & 0xffff0000u)};
+        block_to_digits<G>(v, blk * 128, lane, smem + SmemLayout::xdig, reinterpret_cast<float*>(smem + SmemLayout::xsumw),
+                           reinterpret_cast<float*>(smem + SmemLayout::xinv));
+        if (gated) {
+          float dot = 0.f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) dot = fmaf(gv[i][j], v[j], dot);
+#pragma unroll
+          for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+          if (lane == 0) reinterpret_cast<float*>(smem + SmemLayout::gate)[blk] = dot;
+        }
+      }
     }
   }
   if (warp == 3) SM_TRACE(3);
-  asm volatile("bar.sync 1, %0;" ::"n"(32 * (kConsumerWarps + 1)) : "memory");
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * kConsumerWarps) : "memory");
   if (warp == 3) SM_TRACE(4);
-  if (plan->nslots == 0 && blockIdx.x == 0)
-    for (int i = tid; i < p.hidden; i += 32 * (kConsumerWarps + 1)) p.y[i] = 0.f;
-
-  if (warp < kConsumerWarps) {
-    consumer_loop<G>(p, smem, warp, lane);
-  } else {
-    epilogue_loop(p, smem, lane);
-  }
+  consumer_loop<G>(p, smem, warp, lane);
 }
 
 // ---- inputs in host memory ---------------------------------------------------------------------------

@@ -14,20 +14,15 @@ from ctypes import c_void_p
 
 import numpy as np
 
-NAMES = {1: "dependency wait over", 2: "plan built (warp 0)", 3: "x as digits (warp 3)", 4: "prologue barrier passed",
+NAMES = {1: "dependency wait over", 2: "plan built", 3: "x as digits (warp 3)", 4: "prologue barrier passed",
          5: "gate/up phase done, group 0", 6: "gate/up phase done, group 1", 7: "gate/up phase done, group 2",
          8: "gate/up phase done, group 3", 12: "last h value written", 9: "list of down chunks built (warp 0)",
-         10: "own h blocks in digits (warp 0)", 11: "down phase done (warp 0)", 13: "y written"}
-NAMES[31] = "producer 0 begins the down tiles"
-NAMES[18] = "producer 0 has requested all down tiles"
-NAMES[19] = "producer 1 has requested all down tiles"
+         10: "no h left to take on (warp 0)", 11: "down phase done (warp 0)", 13: "y written", 18: "all down tiles requested",
+         31: "request of the down tiles begins"}
 for _j in range(8):
     NAMES[32 + _j] = f"producer 0 requests gate/up chunk {_j}"
-for _j in range(4):
-    NAMES[40 + _j] = f"producer 0: down chunk landed, #{_j} it waits for"
-    NAMES[44 + _j] = f"producer 1: down chunk landed, #{_j} it waits for"
 for _g in range(4):
-    NAMES[14 + _g] = f"own h blocks in digits, group {_g}"
+    NAMES[14 + _g] = f"no h left to take on, group {_g}"
     NAMES[23 + _g] = f"last down chunk's h flagged, group {_g}"
     NAMES[27 + _g] = f"down phase done, group {_g}"
 
@@ -100,8 +95,8 @@ def main(argv):
     clk = float(getattr(props, "clock_rate", 1965000)) / 1e3      # SM cycles per microsecond at the maximum clock
     dep = out[:, 1] / clk
     print("microseconds after the CTA's own dependency wait returned: mean / min / max over CTAs")
-    order = [32, 33, 34, 35, 36, 37, 38, 39, 2, 3, 4, 5, 6, 7, 8, 12, 31, 18, 19, 40, 41, 42, 43, 44, 45, 46, 47, 9, 10, 14, 15, 16, 17, 23, 24, 25, 26, 11, 27, 28, 29, 30, 13]
-    order += [k for k in range(48, out.shape[1])]   # stamps a working copy of the kernel may add
+    order = [32, 33, 34, 35, 36, 37, 38, 39, 2, 3, 4, 5, 6, 7, 8, 12, 31, 18, 9, 10, 14, 15, 16, 17, 23, 24, 25, 26, 11, 27, 28, 29, 30, 13]
+    order += [k for k in range(40, out.shape[1])]   # stamps a working copy of the kernel may add
     for k in order:
         sel = out[:, k] != 0
         if sel.any():

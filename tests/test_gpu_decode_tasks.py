@@ -1,0 +1,43 @@
+"""How the batch-1 decode kernel deals its gate/up tasks (16 rows of a slot) to the CTAs: both-slice tasks one by one, then two
+MSB-only ones to each CTA that got one less, then the rest.  Shapes at the edges of that rule on a device of 148 SMs, against
+the float64 oracle; and down projections whose chunks go several times round the ring."""
+import numpy as np
+import pytest
+
+from oracle import moe
+from paper_2512_12990_b200 import synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # hidden, inter, top_k, both-slice entries, group, shared inter
+    (256, 4736, 2, 1, 128, 0),      # 296 both-slice tasks: every CTA has two, nobody is short; 296 MSB-only ones
+    (256, 4736, 2, 1, 128, 128),    # 304: 140 CTAs are short of one; more MSB-only tasks than their two each
+    (128, 1280, 2, 1, 64, 0),       # 80 and 80: 68 CTAs are short, and get one or two
+    (128, 128, 2, 1, 32, 0),        # 8 and 8: most CTAs have nothing to do
+    (128, 128, 1, 0, 128, 0),       # MSB-only tasks alone
+    (256, 1280, 8, 2, 128, 0),      # one or two both-slice tasks and many MSB-only ones: an odd number of the former
+    (256, 1280, 8, 8, 64, 128),     # both-slice tasks alone
+    (4096, 1152, 8, 5, 32, 2176),   # two output row blocks per CTA, 34 units of down tiles a row in a ring of 8
+    (2304, 2176, 4, 2, 128, 2176),  # two chunks to a slot, the second one block wide
+]
+
+
+@pytest.mark.parametrize("hidden,inter,k,n_both,group,shared_inter", CASES)
+def test_task_dealing_and_ring_laps(hidden, inter, k, n_both, group, shared_inter):
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    sh = synth.Shape("deal", hidden, inter, k + 1, k, group, n_shared=1 if shared_inter else 0, shared_inter=shared_inter, seed=9100 + inter + k)
+    layer = H.Layer(sh, range(sh.n_experts))
+    ids = np.array([np.random.default_rng(k).permutation(sh.n_experts)[:k]], dtype=np.int32)
+    prec = (np.arange(k) < n_both).astype(np.uint8)[None, ::-1].copy()
+    w = np.linspace(0.4, 0.1, k)[None]
+    xbits, x64 = H.x_inputs(sh, 1)
+    want = moe.layer(x64, layer.oracle_list(), ids, prec, w, shared=layer.oracle_shared)
+    args = (H.to_dev_bf16(xbits), torch.from_numpy(ids).cuda(), torch.from_numpy(prec).cuda(), torch.from_numpy(w.astype(np.float32)).cuda(), layer.ws)
+    y = [B.slicemoe_layer(layer.cshape, layer.experts_tbl, layer.shared_tbl, None, *args) for _ in range(4)]
+    torch.cuda.synchronize()
+    assert B.slicemoe_get_status(layer.ws) == 0
+    H.assert_close(y[0].cpu().numpy(), want, f"{hidden} x {inter}, {n_both} of {k} from both slices")
+    assert all(torch.equal(y[0], v) for v in y[1:])
