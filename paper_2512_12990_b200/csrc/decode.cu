@@ -428,13 +428,15 @@ __device__ __forceinline__ void pass_mma(int (&acc)[128 / G][4], const uint8_t* 
   }
 }
 
-template <int G>
-__device__ __forceinline__ void consume_chunk(const LaneRole& lr, int lane, int gw, int rot, int mode, int nblocks,
+// (The mode is a template argument: with one body for down's two modes a 2048-wide layer took 15.8 us instead of 15.5, of groups of
+// 32 21.1 instead of 20.3, 512-wide ones 15.8 instead of 14.95.)
+template <int G, int MODE>
+__device__ __forceinline__ void consume_chunk(const LaneRole& lr, int lane, int gw, int rot, int nblocks,
                                               const uint8_t* unit0, const uint8_t* unit1, int scale_off, int zp_off,
                                               const uint8_t* dig, const float* sumw, const float* binv, float* out0,
                                               float* out1, int shift) {
   constexpr int SG = 128 / G;
-  const bool p8 = mode == kModeBoth, pair = mode == kModePair;
+  constexpr bool p8 = MODE == kModeBoth, pair = MODE == kModePair;
   const float pfix = p8 ? 1.f : (float)(1 << shift);
   const int zsh = p8 ? 0 : shift;
   const bool hi = (lr.c >> 1) != 0;
@@ -450,7 +452,7 @@ __device__ __forceinline__ void consume_chunk(const LaneRole& lr, int lane, int 
       const uint2 bv3 = *reinterpret_cast<const uint2*>(bp + 288);
       int m[SG][4], l[SG][4];
       pass_mma<G>(m, unit0 + b * 1024 + lane * 16, bv0, bv1, bv2, bv3);
-      if (mode != kModeSingle) pass_mma<G>(l, unit1 + b * 1024 + lane * 16, bv0, bv1, bv2, bv3);
+      if (MODE != kModeSingle) pass_mma<G>(l, unit1 + b * 1024 + lane * 16, bv0, bv1, bv2, bv3);
       const float sfix = pfix * binv[b];
       const uint16_t* ms = reinterpret_cast<const uint16_t*>(unit0 + scale_off) + (b * SG) * 16 + lr.r;
       const uint8_t* mz = unit0 + zp_off + (b * SG) * 16 + lr.r;
@@ -460,7 +462,7 @@ __device__ __forceinline__ void consume_chunk(const LaneRole& lr, int lane, int 
         int ca = hi ? m[sg][2] - m[sg][0] : m[sg][0];
         int cb = hi ? m[sg][3] - m[sg][1] : m[sg][1];
         int ca1 = 0, cb1 = 0;
-        if (mode != kModeSingle) {
+        if (MODE != kModeSingle) {
           ca1 = hi ? l[sg][2] - l[sg][0] : l[sg][0];
           cb1 = hi ? l[sg][3] - l[sg][1] : l[sg][1];
         }
@@ -544,10 +546,10 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
           const float* binv = reinterpret_cast<const float*>(smem + SmemLayout::xinv) + kc * (kChunkK >> 7);
           const uint8_t* unit0 = smem + SmemLayout::ring + u0 * kUnitBytes;
           if (both) {
-            consume_chunk<G>(lr, lane, gw, c % kGroupWarps, kModeBoth, nblocks, unit0, unit0 + kUnitBytes, kPlaneUnitBytes,
+            consume_chunk<G, kModeBoth>(lr, lane, gw, c % kGroupWarps, nblocks, unit0, unit0 + kUnitBytes, kPlaneUnitBytes,
                              kPlaneUnitBytes + kScaleUnitBytes, dig, sumw, binv, q < nch ? &part0 : &part1, &unused, p.shift);
           } else {
-            consume_chunk<G>(lr, lane, gw, c % kGroupWarps, kModePair, nblocks, unit0, unit0 + kUnitBytes, kPlaneUnitBytes,
+            consume_chunk<G, kModePair>(lr, lane, gw, c % kGroupWarps, nblocks, unit0, unit0 + kUnitBytes, kPlaneUnitBytes,
                              kPlaneUnitBytes + kScaleUnitBytes, dig, sumw, binv, &part0, &part1, p.shift);
           }
           __syncwarp();
@@ -648,9 +650,9 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
       const uint8_t* dig = smem + SmemLayout::hdig + col * 3;
       const float* sumw = reinterpret_cast<const float*>(smem + SmemLayout::hsumw) + (col >> LG) * 2;
       const float* binv = reinterpret_cast<const float*>(smem + SmemLayout::hinv) + (col >> 7);
-      consume_chunk<G>(lr, lane, gw, rot, p8 ? kModeBoth : kModeSingle, nblocks,
-                       smem + SmemLayout::ring + u0 * plan.unit2_bytes, smem + SmemLayout::ring + u1 * plan.unit2_bytes,
-                       plan.scale2_off, plan.zp2_off, dig, sumw, binv, &sacc, &unused, p.shift);
+      const uint8_t *unit0 = smem + SmemLayout::ring + u0 * plan.unit2_bytes, *unit1 = smem + SmemLayout::ring + u1 * plan.unit2_bytes;
+      if (p8) consume_chunk<G, kModeBoth>(lr, lane, gw, rot, nblocks, unit0, unit1, plan.scale2_off, plan.zp2_off, dig, sumw, binv, &sacc, &unused, p.shift);
+      else consume_chunk<G, kModeSingle>(lr, lane, gw, rot, nblocks, unit0, unit1, plan.scale2_off, plan.zp2_off, dig, sumw, binv, &sacc, &unused, p.shift);
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(empty2 + 8 * u0);
