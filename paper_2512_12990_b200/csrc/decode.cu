@@ -39,17 +39,17 @@
 #include "batch.cuh"
 #include "common.cuh"
 #include "decode_common.cuh"
+#include "decode_schedule.cuh"
 #include "route.cuh"
 
 namespace slicemoe {
 
 constexpr int kConsumerWarps = 16;
-constexpr int kGroups = 4;       // consumer groups: a phase-1 task belongs to one group, phase-2 chunks go round-robin
+// kGroups consumer groups: a phase-1 task belongs to one group, phase-2 chunks go round-robin
 constexpr int kGroupWarps = 4;   // warps of a group; they split the 128-column blocks of the chunk
 static_assert(kGroups * kGroupWarps == kConsumerWarps, "groups");
 constexpr int kEpilogueWarp = kConsumerWarps;
 constexpr int kProducerWarp = kConsumerWarps + 1;  // first of kProducers producer warps
-constexpr int kProducers = 2;                      // see TaskPlace
 constexpr int kDownWarp = kProducerWarp + kProducers;  // fetches the routed experts' pointers, then requests the down tiles
 constexpr int kThreads = 32 * (kDownWarp + 1);
 constexpr int kUnits2 = 16;                        // at most this many (smaller) units in phase 2
@@ -181,10 +181,8 @@ struct Slot {
 
 // The schedule of a CTA.
 //   phase 1: tasks are 16-row blocks of gate and up, numbered slot after slot - shared, routed from both slices, routed from the
-//     MSB slice alone - so that task o of the grid writes h[16 o ..].  Both-slice tasks go to CTA o mod P; of the MSB-only ones,
-//     half as long, the CTAs short of a both-slice task get two first, and the rest is dealt out (task_ordinal()): the CTAs
-//     differ by a task at most.  How many tasks of the shared experts a CTA has (count_s) follows from the shape alone, so their
-//     tiles are requested before the routing list is known.  A
+//     MSB slice alone - so that task o of the grid writes h[16 o ..].  Deal says which of them a CTA has.  How many tasks of the
+//     shared experts a CTA has (count_s) follows from the shape alone, so their tiles are requested before the routing list is known.  A
 //     both-slice task is 2 * nch chunks (gate then up; nch = 2048-column chunks of hidden), each two
 //     units (MSB tile, LSB tile); an MSB-only task is nch chunks, each two units (the gate's MSB tile
 //     and the up's).  Every phase-1 chunk takes two units.  Which producer and which group a task goes to says TaskPlace;
@@ -196,8 +194,8 @@ struct Slot {
 //     chunk (plane area, then scales at scale2_off, zero-points at zp2_off), so that more - for the
 //     benchmark shapes all - of the phase's tiles are in shared memory before h arrives.
 struct Plan {
-  int count_s, count_both, count1;  // phase-1 tasks of this CTA: of the shared experts, from both slices (with those), in all
-  int light, count_light, ord_light, ord_rest;  // its MSB-only tasks: see task_ordinal()
+  int count_s;      // phase-1 tasks of this CTA of the shared experts
+  Deal deal;        // its phase-1 tasks
   int hpar;         // which h buffer this launch uses
   int never_ready;  // the time-out exercise: treat h as never complete
   int count2;
@@ -217,7 +215,11 @@ struct SmemLayout {
   static constexpr int hinv = xsumw + (kMaxHidden / 32) * 8;  // float [kHCap/128]: 2^-e of each 128-block of h
   static constexpr int xinv = hinv + (kHCap / 128) * 4;       // float [kMaxHidden/128]
   static constexpr int partial = xinv + (kMaxHidden / 128) * 4;  // float2 [warps][16]
-  static constexpr int p2list = partial + kConsumerWarps * 16 * 2 * 4;  // uint4 [warps][kMaxMine]: a warp's phase-2 chunks
+  // float [warps][16], phase 2's, apart from phase 1's: the epilogue warp takes a CTA's tasks in order and may still be at another
+  // group's when a group without a chunk in the first row block, and without a block of h to take on, writes its share of it.
+  // (A wait for that instead cost 0.1 us a launch.)
+  static constexpr int partial2 = partial + kConsumerWarps * 16 * 2 * 4;
+  static constexpr int p2list = partial2 + kConsumerWarps * 16 * 4;  // uint4 [warps][kMaxMine]: a warp's phase-2 chunks
   static constexpr int slots = p2list + kConsumerWarps * kMaxMine * 16;
   static constexpr int plan = slots + kMaxSlots * (int)sizeof(Slot);
   static constexpr int bars = (plan + (int)sizeof(Plan) + 15) & ~15;  // uint64 barriers
@@ -231,7 +233,7 @@ struct SmemLayout {
 static_assert(SmemLayout::total <= 227 * 1024, "shared memory budget");
 static_assert(sizeof(Slot) % 8 == 0, "slot alignment");
 static_assert(SmemLayout::slots % 8 == 0 && SmemLayout::hdig % 16 == 0 && SmemLayout::xdig % 16 == 0 &&
-                  SmemLayout::plan % 8 == 0 && SmemLayout::partial % 8 == 0 && SmemLayout::p2list % 16 == 0,
+                  SmemLayout::plan % 8 == 0 && SmemLayout::partial % 8 == 0 && SmemLayout::partial2 % 4 == 0 && SmemLayout::p2list % 16 == 0,
               "alignment");
 
 // Barriers.  Every barrier has ONE waiter that meets its phases strictly in order, so a parity wait can never
@@ -277,34 +279,6 @@ __device__ __forceinline__ void block_to_digits(const float (&v)[4], int k0, int
 // ---- schedule enumeration (identical in every role) ----------------------------------------------------
 __device__ __forceinline__ int nchunks_of(int K) { return (K + kChunkK - 1) / kChunkK; }
 enum ChunkMode { kModeSingle = 0, kModeBoth = 1, kModePair = 2 };
-
-// The number in the grid of this CTA's phase-1 task n.
-__device__ __forceinline__ int task_ordinal(const Plan& plan, int n) {
-  const int c = (int)blockIdx.x, P = (int)gridDim.x;
-  if (n < plan.count_s || n < plan.count_both) return c + n * P;
-  n -= plan.count_both;
-  return n < plan.count_light ? plan.ord_light + n * plan.light : plan.ord_rest + (n - plan.count_light) * P;
-}
-
-// Which producer a task goes to and which of that producer's tasks it is; the producer's groups take its tasks in turn.  The
-// tasks of both slices alternate; where their number is odd, the first two of the MSB-only ones, half as long, go to the
-// producer that got one less, the rest alternates again.
-struct TaskPlace {
-  int producer, turn;
-  __device__ __forceinline__ TaskPlace(int count_both, int n) {
-    const int k = n - count_both;  // among the MSB-only tasks
-    if (k >= 0 && (count_both & 1)) {
-      producer = k < 2 ? 1 : k & 1;
-      turn = (count_both >> 1) + (k < 2 ? k : producer ? 2 + ((k - 2) >> 1) : 1 + ((k - 2) >> 1));
-    } else {
-      producer = n & 1;
-      turn = n >> 1;
-    }
-  }
-  __device__ __forceinline__ int group() const { return producer + kProducers * (turn & 1); }
-  __device__ __forceinline__ int round() const { return turn >> 1; }  // which of its group's tasks it is
-};
-static_assert(kProducers == 2 && kGroups == 4, "two groups to a producer");
 
 // ---- consumers -----------------------------------------------------------------------------------
 // Phase change: the consumer warps take 128-blocks of the grid's h on, a few at a time in order, poll them in the
@@ -503,6 +477,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
   const Slot* slots = reinterpret_cast<const Slot*>(smem + SmemLayout::slots);
   const Plan& plan = *reinterpret_cast<const Plan*>(smem + SmemLayout::plan);
   float2* partial = reinterpret_cast<float2*>(smem + SmemLayout::partial);
+  float* partial2 = reinterpret_cast<float*>(smem + SmemLayout::partial2);
   volatile int* dead = reinterpret_cast<volatile int*>(smem + SmemLayout::dead);
   const uint32_t bars = smem_u32(smem + SmemLayout::bars);
   const uint32_t full0 = bars + 8 * Bars::full, empty0 = bars + 8 * Bars::empty;
@@ -529,14 +504,14 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
     for (int n = 0;; ++n) {
       if (n == plan.count_s) {
         if (!mbar_wait(bars + 8 * Bars::plan_ready, 0, dead, status)) return;
-        end = plan.count1;
+        end = plan.deal.count1;
         if (plan.nslots == 0 && blockIdx.x == 0)
           for (int i = threadIdx.x; i < p.hidden; i += 32 * kConsumerWarps) p.y[i] = 0.f;
       }
       if (n >= end) break;
-      const bool shared = n < plan.count_s, both = shared || n < plan.count_both;
+      const bool shared = n < plan.count_s, both = shared || n < plan.deal.count_both;
       const int nchunks = both ? 2 * nch : nch;
-      const TaskPlace at(shared ? n + 1 : plan.count_both, n);
+      const TaskPlace at(shared ? n + 1 : plan.deal.count_both, n);
       if (at.group() == group) {
         float part0 = 0.f, part1 = 0.f, unused = 0.f;
         for (int q = 0; q < nchunks; ++q, ++jp, ++ig) {
@@ -666,7 +641,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
     if (jcur >= 0) part = fmaf(slots[jcur].gated ? gate : slots[jcur].coef, sacc, part);
     part += __shfl_xor_sync(0xffffffffu, part, 1);
     if (!mbar_wait(bars + 8 * Bars::pempty2, (m & 1) ^ 1, dead, status)) return;
-    if (lr.cq == 0) partial[warp * 16 + lr.r] = make_float2(0.f, part);
+    if (lr.cq == 0) partial2[warp * 16 + lr.r] = part;
     __syncwarp();
     if (lane == 0) mbar_arrive(bars + 8 * Bars::pfull2);
   }
@@ -678,6 +653,7 @@ __device__ void consumer_loop(const DecodeParams& p, uint8_t* smem, int warp, in
 __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
   const Plan& plan = *reinterpret_cast<const Plan*>(smem + SmemLayout::plan);
   const float2* partial = reinterpret_cast<const float2*>(smem + SmemLayout::partial);
+  const float* partial2 = reinterpret_cast<const float*>(smem + SmemLayout::partial2);
   volatile int* dead = reinterpret_cast<volatile int*>(smem + SmemLayout::dead);
   const uint32_t bars = smem_u32(smem + SmemLayout::bars);
   unsigned* status = &p.ws->status;
@@ -693,9 +669,9 @@ __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
   float* hbuf = p.ws_h + (size_t)plan.hpar * kHCap;
   // phase 1: one group's four partial rows per task -> SwiGLU -> h
   {
-    for (int n = 0; n < plan.count1; ++n) {
-      const int ord = task_ordinal(plan, n);
-      const TaskPlace place(plan.count_both, n);
+    for (int n = 0; n < plan.deal.count1; ++n) {
+      const int ord = plan.deal.ordinal(plan.count_s, n, (int)blockIdx.x, (int)gridDim.x);
+      const TaskPlace place(plan.deal.count_both, n);
       const int group = place.group(), round = place.round();
       if (!mbar_wait(bars + 8 * (Bars::pfull1 + group), round & 1, dead, status)) return;
       float a = 0.f, b = 0.f;
@@ -719,7 +695,7 @@ __device__ void epilogue_loop(const DecodeParams& p, uint8_t* smem, int lane) {
     float b = 0.f;
     if (lane < 16) {
 #pragma unroll
-      for (int w = 0; w < kConsumerWarps; ++w) b += partial[w * 16 + lane].y;
+      for (int w = 0; w < kConsumerWarps; ++w) b += partial2[w * 16 + lane];
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(bars + 8 * Bars::pempty2);
@@ -831,12 +807,12 @@ __device__ void producer_loop(const DecodeParams& p, uint8_t* smem, int lane, in
       if (n == plan.count_s) {
         ok = pw(bars + 8 * Bars::plan_ready, 0);
         if (!ok) break;
-        n_end = plan.count1;
+        n_end = plan.deal.count1;
       }
       if (n >= n_end) break;
-      const TaskPlace place(n < plan.count_s ? n + 1 : plan.count_both, n);
+      const TaskPlace place(n < plan.count_s ? n + 1 : plan.deal.count_both, n);
       if (place.producer == which) {
-        const int ord = task_ordinal(plan, n), routed = ord - shared_tasks;
+        const int ord = plan.deal.ordinal(plan.count_s, n, (int)blockIdx.x, (int)gridDim.x), routed = ord - shared_tasks;
         int slot, idx;
         if (routed < 0) {
           slot = ord / per_s;
@@ -1031,8 +1007,6 @@ __device__ __forceinline__ void plan_units2(const DecodeParams& p, Plan* plan, i
   plan->unit2_bytes = (maxblk * (1024 + meta_blk * 3) + 127) & ~127;
   plan->nunits2 = min(kUnits2, (kUnits * kUnitBytes) / plan->unit2_bytes);
 }
-// How many of n things, dealt to P CTAs one by one, go to CTA c.
-__device__ __forceinline__ int dealt(int n, int c, int P) { return n > c ? (n - c + P - 1) / P : 0; }
 // Run by the epilogue warp, as what follows.
 __device__ void build_plan_static(const DecodeParams& p, uint8_t* smem, int lane) {
   Slot* slots = reinterpret_cast<Slot*>(smem + SmemLayout::slots);
@@ -1096,16 +1070,8 @@ __device__ __forceinline__ void build_plan(const DecodeParams& p, uint8_t* smem,
       if (lane == 0) plan->p2c[0] = plan->p2u[0] = 0;
     }
     if (lane == 0) {
-      const int c = (int)blockIdx.x, P = (int)gridDim.x, per = p.inter / 16;
-      const int nboth = p.n_shared * (p.shared_inter / 16) + rt.nbig * per, nmsb = rt.nsmall * per;  // tasks
-      const int q = nboth / P, r = nboth - q * P, light = r ? P - r : 0, first = min(nmsb, 2 * light), rest = nmsb - first;
-      const int at = c - r, rest_q = rest / P;  // (the two divisions of this chain)
-      plan->count_both = q + (c < r ? 1 : 0);
-      plan->light = light;
-      plan->count_light = at >= 0 ? (at < first ? 1 : 0) + (at + light < first ? 1 : 0) : 0;
-      plan->count1 = plan->count_both + plan->count_light + rest_q + (c < rest - rest_q * P ? 1 : 0);
-      plan->ord_light = nboth + at;
-      plan->ord_rest = nboth + first + c;
+      const int per = p.inter / 16;  // tasks of a routed slot
+      plan->deal.set(p.n_shared * (p.shared_inter / 16) + rt.nbig * per, rt.nsmall * per, (int)blockIdx.x, (int)gridDim.x);
       if (nslots == 0) plan->count2 = 0;  // otherwise as build_plan_static left it
       plan->nslots = nslots;
       plan->htotal = p.n_shared * p.shared_inter + (rt.nbig + rt.nsmall) * p.inter;

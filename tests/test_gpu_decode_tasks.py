@@ -41,3 +41,33 @@ def test_task_dealing_and_ring_laps(hidden, inter, k, n_both, group, shared_inte
     assert B.slicemoe_get_status(layer.ws) == 0
     H.assert_close(y[0].cpu().numpy(), want, f"{hidden} x {inter}, {n_both} of {k} from both slices")
     assert all(torch.equal(y[0], v) for v in y[1:])
+
+
+@pytest.mark.parametrize("hidden,inter,k,n_both,group,shared_inter", [
+    (2048, 2048, 3, 1, 128, 0),     # 68 CTAs with a group that has a gate/up task and no chunk of the first output rows
+    (2560, 2048, 1, 0, 128, 4096),  # 40
+    (2048, 1024, 2, 1, 64, 0),
+])
+def test_rows_between_the_phases(hidden, inter, k, n_both, group, shared_inter):
+    """A group's rows of partial sums belong to gate/up until the epilogue has taken them: also where the group has nothing to wait
+    for in the down projection.  Many launches back to back and with another kernel between them, all of one result."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    sh = synth.Shape("rows", hidden, inter, k + 1, k, group, n_shared=1 if shared_inter else 0, shared_inter=shared_inter, seed=9300 + inter + k)
+    layer = H.Layer(sh, range(sh.n_experts))
+    ids = np.arange(k, dtype=np.int32)[None]
+    prec = (np.arange(k) < n_both).astype(np.uint8)[None]
+    w = np.linspace(0.4, 0.1, k)[None]
+    xbits, x64 = H.x_inputs(sh, 1)
+    want = moe.layer(x64, layer.oracle_list(), ids, prec, w, shared=layer.oracle_shared)
+    args = (H.to_dev_bf16(xbits), torch.from_numpy(ids).cuda(), torch.from_numpy(prec).cuda(), torch.from_numpy(w.astype(np.float32)).cuda(), layer.ws)
+    y = torch.empty((400, 1, hidden), device="cuda")
+    other = torch.zeros(1 << 20, device="cuda")
+    for i in range(400):
+        B.slicemoe_layer(layer.cshape, layer.experts_tbl, layer.shared_tbl, None, *args, y=y[i])
+        if i % 3 == 2:
+            other.add_(1.0)
+    torch.cuda.synchronize()
+    assert B.slicemoe_get_status(layer.ws) == 0
+    H.assert_close(y[0].cpu().numpy(), want, f"{hidden} x {inter}")
+    assert torch.equal(y, y[:1].expand_as(y))
