@@ -346,9 +346,6 @@ struct BParams {
   int hidden, K, shift;  // K: widest vector of digits (hidden, or a chunk of the intermediate width)
   int stages;            // per group
   int max_segs;          // entries the list can have
-  const slicemoe_expert* shared;
-  int n_shared;
-  size_t shared_plane;   // bytes of a shared expert's plane
 };
 template <int G, int PHASE>
 struct BSmem {
@@ -634,8 +631,6 @@ __global__ void __launch_bounds__(kBThreads, 1) batch_ffn_kernel(const __grid_co
   // The gate/up launch waits for the plan before it lets the next launch start.  So the down launch, when it starts, finds the
   // plan complete: it looks up its share and streams its weights while gate/up is still running, and waits only for h.
   if (PHASE == 1) {
-    // HBM has nothing to do until the plan stands: the shared experts' planes, which are needed whatever it says, on their way to L2
-    if (p.n_shared > 0) prefetch_shared(p.shared, p.n_shared, p.shared_plane, (int)(threadIdx.x * gridDim.x + blockIdx.x), (int)(gridDim.x * kBThreads));
     b_dep_wait();
     b_dep_launch();
   }
@@ -958,9 +953,6 @@ int batch_layer(const slicemoe_shape* s, const slicemoe_expert* experts, const s
   p.K = s->hidden;
   p.shift = s->b_high - s->b_low;
   p.stages = 0;
-  p.shared = shared;
-  p.n_shared = n_shared;
-  p.shared_plane = (size_t)s->hidden * pp.shared_inter / 2;
   const int parts = (T + kBRun - 1) / kBRun;
   p.max_segs = T * s->top_k + n_shared * parts;
   BParams p2 = p;

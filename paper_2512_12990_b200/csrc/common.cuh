@@ -54,29 +54,6 @@ __host__ __device__ inline size_t meta_index(int ngroups, int n, int g) {
   return ((size_t)(n >> 4) * ngroups + g) * 16 + (n & 15);
 }
 
-#ifdef __CUDACC__
-// Asks for the shared experts' planes ([inter, hidden] gate and up, [hidden, inter] down, `plane_bytes` each) to be brought to L2,
-// for a kernel that routing work is ahead of: which experts a token names is not known yet, but these are used in any case,
-// and HBM has nothing else to do.  Not more than a part of L2's 126 MB, gate and up before down.  Thread `index` of `count`
-// threads that call it.
-constexpr size_t kPrefetchPiece = 32768, kPrefetchMost = 48u << 20;
-__device__ __forceinline__ void prefetch_shared(const slicemoe_expert* shared, int n_shared, size_t plane_bytes, int index, int count) {
-  const int pieces = (int)((plane_bytes + kPrefetchPiece - 1) / kPrefetchPiece);
-  const int most = (int)(kPrefetchMost / kPrefetchPiece), all = 6 * n_shared * pieces;
-  for (int i = index; i < all && i < most; i += count) {
-    const int plane = i / pieces, which = plane / (2 * n_shared), e = (plane >> 1) % n_shared;
-    const slicemoe_expert* ex = shared + e;
-    const slicemoe_mat* m = which == 0 ? &ex->gate : which == 1 ? &ex->up : &ex->down;
-    const uint8_t* from = reinterpret_cast<const uint8_t*>((plane & 1) ? m->lsb : m->msb);
-    if (!from) continue;
-    const size_t at = (size_t)(i - plane * pieces) * kPrefetchPiece;
-    const size_t left = plane_bytes - at;
-    const uint32_t bytes = (uint32_t)(left < kPrefetchPiece ? left : kPrefetchPiece);
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(from + at), "r"(bytes) : "memory");
-  }
-}
-#endif
-
 inline bool valid_group(int g) { return g == 32 || g == 64 || g == 128; }
 // The slice widths of Table 1: MAT84, MAT63, MAT42 (b_high-bit codes, the top b_low bits form the MSB slice).
 inline bool valid_widths(int b_high, int b_low) {
