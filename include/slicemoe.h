@@ -12,6 +12,13 @@
  *     host memory.  `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Unless
  *     stated, calls only enqueue work and do not synchronise.
  *   - The library allocates no device memory.
+ *   - Order: calls on one stream, and the caller's own work there, take effect one after the other, although kernels overlap.
+ *     One kind of work is excepted.  A layer call of up to three tokens reads the shared experts' table and slices - with
+ *     SLICEMOE_LISTS_RESIDENT all experts' - ahead of the end of a kernel that lets its dependents start early (programmatic
+ *     dependent launch: griddepcontrol.launch_dependents, cudaTriggerProgrammaticLaunchCompletion).  A kernel of the caller's that
+ *     does so must not write expert tables or weights, unless other work is enqueued between it and the call: a kernel
+ *     that does not, a copy, or slicemoe_pack (not slicemoe_route_topk or another layer call).  Ordinary kernels, copies
+ *     and slicemoe_pack may write them directly ahead of the call.
  *   - Weight matrices are row-major [N, K] (N outputs, K inputs = contraction axis); quantisation
  *     groups run along K.
  *

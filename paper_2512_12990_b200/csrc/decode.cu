@@ -1108,8 +1108,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_layer_kernel(const __grid_
   // of this grid has got here (its CTAs find room only where one of ours has exited), and this kernel does
   // all it can before it waits for the grids before it.  Nothing an earlier kernel may write is touched
   // before that wait: x and the workspace always, and the routing lists unless the caller has promised that
-  // they were complete earlier (lists_resident).  The weights, the expert tables and the shape are never written
-  // by a kernel in flight.
+  // they were complete earlier (lists_resident).  The weights and expert tables are not written by a kernel in flight that
+  // lets this one start: pack_kernel does not, and a caller's own kernels must not (slicemoe.h, "Order").
 #ifdef SLICEMOE_TRACE
   if (tid == 0) s_trace_t0 = clock64();
   if (tid == 0 && blockIdx.x < 256) g_trace[blockIdx.x][20] = trace_gtime();

@@ -3,7 +3,7 @@ through the C ABI; plus the physical plane layout the header documents."""
 import numpy as np
 import pytest
 
-from oracle import amat
+from oracle import amat, moe
 from paper_2512_12990_b200 import synth
 
 pytestmark = pytest.mark.gpu
@@ -172,3 +172,56 @@ def test_pack_bit_exact_at_half_integers(group, b_high, b_low):
     W[5, 7] = np.inf
     with np.errstate(all="ignore"):
         _check(W, group, b_high, b_low)
+
+
+@pytest.mark.parametrize("call", ["layer", "routed", "batch", "resident", "prefill"])
+def test_repacked_in_place_directly_ahead_of_the_layer(call):
+    """An expert packed again into planes that a table names already, and the layer behind it on the same stream: the layer sees
+    the new weights, shared and routed, whatever it reads ahead of its own turn."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    from tests import helpers as H
+    T = {"batch": 8, "prefill": 24}.get(call, 1)
+    sh = synth.Shape("repack", 1024, 512, 4, 2, 128, n_shared=1, shared_inter=2048, seed=9400)
+    layer = H.Layer(sh, range(4))
+    mats = [layer.packed_shared[0][n] for n in ("gate", "up", "down")] + [layer.packed[1]["down"]]
+    W = [[torch.from_numpy(synth.normal_f32(v, ("repack", i), (m.N, m.K), 0.02)).cuda() for i, m in enumerate(mats)] for v in range(2)]
+    xbits, x64 = H.x_inputs(sh, T)
+    x = H.to_dev_bf16(xbits)
+    logits = np.zeros((T, 4), dtype=np.float32)
+    logits[:, 1], logits[:, 3] = 2.0, 1.0
+    dl = torch.from_numpy(logits).cuda()
+    ids, w, pr = B.slicemoe_route_topk(dl, 2, rank_high=1)
+    high, pws, status = torch.ones(4, dtype=torch.uint8, device="cuda"), B.new_prefill_workspace(layer.cshape, T), torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def step(v, i, y, apart=False):
+        for m, Wm in zip(mats, W[v]):
+            B.slicemoe_pack(Wm, 128, out=m)
+        if apart:
+            torch.cuda.synchronize()
+        a, b, c = B.slicemoe_route_topk(dl, 2, rank_high=1) if i % 2 and call != "resident" else (ids, w, pr)
+        if call == "routed":
+            B.slicemoe_layer_routed(layer.cshape, layer.experts_tbl, layer.shared_tbl, None, x, dl, layer.ws, rank_high=1, y=y)
+        elif call == "prefill":
+            B.slicemoe_prefill_layer(layer.cshape, layer.experts_tbl, layer.shared_tbl, None, x, a, b, high, pws, y=y, status=status)
+        else:
+            B.slicemoe_layer(layer.cshape, layer.experts_tbl, layer.shared_tbl, None, x, a, c, b, layer.ws, y=y,
+                             flags=B.LISTS_RESIDENT if call == "resident" else 0)
+
+    y = torch.empty((41, T, 1024), device="cuda")
+    for i in range(41):
+        step(i % 2, i, y[i])
+    ref = torch.empty((2, T, 1024), device="cuda")
+    for v in range(2):
+        step(v, 0, ref[v], apart=True)
+        torch.cuda.synchronize()
+        shared = {n: H.oracle_mat_from_device(m) for n, m in zip(("gate", "up", "down"), mats)}
+        routed = dict(layer.oracle_list())
+        routed[1] = dict(routed[1], down=H.oracle_mat_from_device(mats[3]))
+        prec = np.ones_like(pr.cpu().numpy()) if call == "prefill" else pr.cpu().numpy()
+        want = moe.layer(x64, routed, ids.cpu().numpy(), prec, w.cpu().numpy().astype(np.float64), shared=[shared])
+        H.assert_close(ref[v].cpu().numpy(), want, f"{call}, weights {v}")
+    assert B.slicemoe_get_status(layer.ws) == 0 and int(status) == 0
+    assert not torch.equal(ref[0], ref[1])
+    for i in range(41):
+        assert torch.equal(y[i], ref[i % 2]), i

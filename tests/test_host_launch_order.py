@@ -22,3 +22,10 @@ def test_batch_projections_know_the_experts_from_the_plan_alone():
     plan = text[text.index("batch_plan_kernel(const BPlanParams"):]
     before = plan[:plan.index("b_dep_wait();")]
     assert re.findall(r"\bp\.\w+", before) == []
+
+
+def test_weights_are_complete_before_a_layer_kernel_starts():
+    """The decode kernel streams the shared experts' slices ahead of its wait.  So a kernel that writes slices lets nobody start
+    while it runs: neither pack nor those that expand a slice for the second tier."""
+    for name in ("pack.cu", "tier.cu"):
+        assert "launch_dependents" not in _source(name), name
