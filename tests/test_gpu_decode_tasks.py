@@ -19,7 +19,7 @@ CASES = [
     (128, 128, 1, 0, 128, 0),       # MSB-only tasks alone
     (256, 1280, 8, 2, 128, 0),      # one or two both-slice tasks and many MSB-only ones: an odd number of the former
     (256, 1280, 8, 8, 64, 128),     # both-slice tasks alone
-    (4096, 1152, 8, 5, 32, 2176),   # two output row blocks per CTA, 34 units of down tiles a row in a ring of 8
+    (4096, 1152, 8, 5, 32, 2176),   # 17 units of down tiles a row block, 34 for the CTAs with two, in a ring of 8
     (2304, 2176, 4, 2, 128, 2176),  # two chunks to a slot, the second one block wide
 ]
 
@@ -71,3 +71,48 @@ def test_rows_between_the_phases(hidden, inter, k, n_both, group, shared_inter):
     assert B.slicemoe_get_status(layer.ws) == 0
     H.assert_close(y[0].cpu().numpy(), want, f"{hidden} x {inter}")
     assert torch.equal(y, y[:1].expand_as(y))
+
+
+@pytest.mark.parametrize("hidden,inter,k,n_both,group,shared_inter", [
+    (2048, 2048, 3, 1, 128, 0),
+    (2560, 2048, 1, 0, 128, 4096),
+    (4096, 1152, 8, 5, 32, 2176),
+    (256, 1280, 8, 2, 64, 128),
+])
+def test_the_same_tasks_by_every_way_to_the_list(hidden, inter, k, n_both, group, shared_inter):
+    """The list read behind the wait, ahead of it (resident), or worked out in the kernel: one plan, the same bits.  And lists of
+    which some or all entries name no expert, for which the plan and the ring of the down projection are cut anew."""
+    import torch
+    from paper_2512_12990_b200 import binding as B
+    n_shared = 1 if shared_inter else 0
+    sh = synth.Shape("ways", hidden, inter, k + 2, k, group, n_shared=n_shared, shared_inter=shared_inter, seed=9500 + inter + k)
+    layer = H.Layer(sh, range(sh.n_experts))
+    xbits, x64 = H.x_inputs(sh, 1)
+    x = H.to_dev_bf16(xbits)
+    logits = torch.from_numpy(np.random.default_rng(k).standard_normal((1, k + 2)).astype(np.float32)).cuda()
+    tables = (layer.cshape, layer.experts_tbl, layer.shared_tbl, None, x)
+    for _ in range(20):
+        routed, ids, prec, w = B.slicemoe_layer_routed(*tables, logits, layer.ws, rank_high=n_both)
+        assert prec.sum() == n_both
+        plain = B.slicemoe_layer(*tables, ids, prec, w, layer.ws)
+        torch.cuda.synchronize()  # the lists are complete before what precedes the next call begins
+        resident = [B.slicemoe_layer(*tables, ids, prec, w, layer.ws, flags=B.LISTS_RESIDENT) for _ in range(4)]
+        assert torch.equal(plain, routed) and all(torch.equal(plain, r) for r in resident)
+    assert B.slicemoe_get_status(layer.ws) == 0
+    n_ids, n_prec, n_w = ids.cpu().numpy(), prec.cpu().numpy(), w.cpu().numpy().astype(np.float64)
+    for dropped in {(0,), (k - 1,), tuple(range(k))}:
+        kept = [j for j in range(k) if j not in dropped]
+        some = ids.clone()
+        some[:, list(dropped)] = torch.tensor([-1, k + 2] * k, dtype=torch.int32, device="cuda")[:len(dropped)]
+        torch.cuda.synchronize()
+        y = [B.slicemoe_layer(*tables, some, prec, w, layer.ws, flags=f) for f in (0, B.LISTS_RESIDENT) for _ in range(3)]
+        assert B.slicemoe_get_status(layer.ws) == 1
+        if kept:
+            want = moe.layer(x64, layer.oracle_list(), n_ids[:, kept], n_prec[:, kept], n_w[:, kept], shared=layer.oracle_shared)
+        else:
+            want = sum((moe.expert_ffn_one(x64[0], e, 1) for e in layer.oracle_shared), np.zeros(hidden))[None]
+        if np.any(want):
+            H.assert_close(y[0].cpu().numpy(), want, f"without entries {dropped}")
+        else:
+            assert not y[0].any()
+        assert all(torch.equal(y[0], v) for v in y[1:])
