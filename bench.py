@@ -367,7 +367,7 @@ def decode_traffic_record(workload: str):
         with open(os.path.join(ROOT, "profiles", "decode_layer_kernel_traffic.json")) as f:
             rec = json.load(f)
         digest = hashlib.sha256()
-        for name in ("decode.cu", "decode_common.cuh", "route.cuh", "common.cuh"):
+        for name in ("decode.cu", "decode_schedule.cuh", "decode_common.cuh", "route.cuh", "common.cuh"):
             with open(os.path.join(ROOT, "paper_2512_12990_b200", "csrc", name), "rb") as f:
                 digest.update(f.read())
         if rec.get("sources_sha256") != digest.hexdigest():

@@ -13,12 +13,13 @@
  *     stated, calls only enqueue work and do not synchronise.
  *   - The library allocates no device memory.
  *   - Order: calls on one stream, and the caller's own work there, take effect one after the other, although kernels overlap.
- *     One kind of work is excepted.  A layer call of up to three tokens reads the shared experts' table and slices - with
- *     SLICEMOE_LISTS_RESIDENT all experts' - ahead of the end of a kernel that lets its dependents start early (programmatic
- *     dependent launch: griddepcontrol.launch_dependents, cudaTriggerProgrammaticLaunchCompletion).  A kernel of the caller's that
- *     does so must not write expert tables or weights, unless other work is enqueued between it and the call: a kernel
- *     that does not, a copy, or slicemoe_pack (not slicemoe_route_topk or another layer call).  Ordinary kernels, copies
- *     and slicemoe_pack may write them directly ahead of the call.
+ *     One kind of work is excepted.  A layer call of up to three tokens (slicemoe_decode_step_host's too) reads the shared
+ *     experts' table and slices - with SLICEMOE_LISTS_RESIDENT all experts' - without waiting for a kernel that lets its
+ *     dependents start early (programmatic dependent launch: griddepcontrol.launch_dependents,
+ *     cudaTriggerProgrammaticLaunchCompletion).  A kernel of the caller's that does so must not write expert tables or
+ *     weights, unless other work is enqueued between it and the call: a kernel that does not, a copy, or slicemoe_pack
+ *     (not slicemoe_route_topk or another layer call).  Ordinary kernels, copies and slicemoe_pack may write them
+ *     directly ahead of the call.
  *   - Weight matrices are row-major [N, K] (N outputs, K inputs = contraction axis); quantisation
  *     groups run along K.
  *
@@ -233,8 +234,9 @@ int slicemoe_layer(const slicemoe_shape *shape, const slicemoe_expert *experts,
  * (From four tokens on a call has no use for either flag: its kernels do not wait for one another's CTAs.)
  *   SLICEMOE_COOPERATIVE  the kernel is launched as a cooperative grid: the driver guarantees that all its CTAs are
  *            resident together, or fails the launch (SLICEMOE_E_CUDA), so a device shared with other kernels
- *            cannot make the wait for h run out.  About 1.4 us per launch slower on a B200 (a cooperative grid
- *            starts as a whole, without the CTA-by-CTA hand-over from the launch before).  Same bits.
+ *            cannot make the wait for h run out.  Slower on a B200 by 0.7 to 1.8 us per launch in a CUDA graph and 3 to
+ *            4 us as a plain launch (a cooperative grid starts as a whole, without the CTA-by-CTA hand-over from the launch
+ *            before).  Same bits.
  * flags = 0 is slicemoe_layer.  Errors: as slicemoe_layer; INVALID_ARG for an unknown flag.
  */
 #define SLICEMOE_LISTS_RESIDENT 1u

@@ -130,11 +130,12 @@ constexpr size_t kWsBatchOff = (kWsBytes + 255) & ~(size_t)255;
 constexpr size_t kWsListEntries = (size_t)kBatchTokens * SLICEMOE_MAX_TOP_K;
 constexpr size_t kWsListBytes = kWsListEntries * 9;
 // From this many tokens on a layer call takes the batch kernels (four launches) instead of a launch of the batch-1 kernel
-// per token.  Measured, us, loop / batch at T = 2, 3, 4: 2048-wide layer of 1408-wide experts 33 / 37, 49 / 40, 65 / 43; 1024 wide
-// 22 / 19, 33 / 20, 44 / 21; 256 wide 13 / 14, 20 / 14, 27 / 14; from four tokens on the batch was ahead at every one of 75
-// shapes, groups, T and overlaps of the lists, by least at hidden 4096 and group 32: 84 / 89.  By time alone the line would lie
-// at three; it lies at four because slicemoe_layer_static, which has no room for the batch, gives the bits of
-// slicemoe_layer up to three tokens, as its header says.
+// per token.  Measured, us, loop / batch at T = 4, 8 with tokens that share no expert until all are named: 2048-wide layer of
+// 1408-wide experts 62 / 45, 123 / 60; 1024 wide 33 / 19, 66 / 23; 256 wide 24 / 14, 47 / 16; groups of 32, 2048 wide 82 / 51, 163 / 69.
+// Of 30 shapes, widths 256 to 4096 and all groups, the batch was ahead from four tokens on at all but one: 4096 wide, groups
+// of 32, four experts of 1408 a token 79.5 / 83.6 (T = 5 99 / 103, T = 8 159 / 134), where its ring has one stage a group.  By time
+// alone the line would lie at three (the first three shapes, let in there: 47 / 40, 25 / 20, 18 / 14); it lies at four because
+// slicemoe_layer_static, which has no room for the batch, gives the bits of slicemoe_layer up to three tokens, as its header says.
 constexpr int kBatchMinTokens = 4;
 static_assert(sizeof(WsHeader) <= kWsHOff, "workspace header");
 static_assert(kWsStLogits + 4 * 512 <= kWsStIds, "x and the logits fit the staging area back to back too");
@@ -292,8 +293,11 @@ template <int G>
 __device__ bool fetch_h(const DecodeParams& p, uint8_t* smem, int lane, int htotal, const float* hbuf, bool never_ready,
                         volatile int* dead, unsigned* status) {
   const int nblk = htotal >> 7;
-  // Loads in flight together, fewer where there would not be some for every warp.  (2048-wide layer, two shared experts, us: four
-  // 15.9, two 16.2, six 16.0; with groups of 32, whose digit sums take longer: 22.4, 21.2, 22.7.)
+  // Loads in flight together, fewer where there would not be some for every warp.  The line lies where the digit sums of a block
+  // begin to cost.  Four / two, us a launch, the layer alone: groups of 128, 2048-wide with two shared experts 15.67 / 15.95, with a
+  // gated one of 5632 15.93 / 16.31, 1024-wide 9.58 / 9.47; groups of 64, 4096-wide 16.8 / 16.65 (experts of 1024), 29.85 / 29.83
+  // (of 1408), 2048-wide 18.6 / 18.67, 1024-wide 11.05 / 10.73 (top-8 of 512), 19.78 / 19.85 (of 1408); groups of 32, 2048-wide
+  // 22.4 / 21.64, 2688-wide 16.86 / 16.77.
   constexpr int kTake = G == 128 ? 4 : 2;
   const int take = max(1, min(kTake, nblk / kConsumerWarps));
   const long long t0 = clock64();
@@ -404,10 +408,12 @@ __device__ __forceinline__ void pass_mma(int (&acc)[128 / G][4], const uint8_t* 
 
 // (The mode is a template argument: with one body for down's two modes a 2048-wide layer took 15.8 us instead of 15.5, of groups of
 // 32 21.1 instead of 20.3, 512-wide ones 15.8 instead of 14.95.)
-// Blocks of two planes one after the other in a loop, not unrolled: what a launch stalls for most, by the counters, is instructions,
-// and another kernel between two launches - the routing - leaves fewer of them in the caches.  With the routing launch, unrolled /
-// as a loop, us: 2048-wide, top-6 + 2 shared 18.1 / 17.5, gated shared expert 19.0 / 18.0, groups of 32 23.4 / 22.6; the layer
-// alone 15.55 / 15.65, 15.85 / 15.95, 20.4 / 20.55.
+// Blocks of two planes one after the other in a loop, not unrolled: another kernel between two launches - the routing - leaves fewer
+// of this one's instructions in the caches, and a launch runs most of them once.  With the routing launch, unrolled / as a loop, us:
+// 2048-wide, top-6 + 2 shared 18.15 / 17.43, gated shared expert 19.07 / 17.97, groups of 64 21.1 / 20.85, of 32 24.5 / 23.5;
+// 4096-wide 18.75 / 18.4.  Where no other kernel comes between, the loop costs up to 0.9 % of some and saves others more: the layer
+// alone 15.55 / 15.66, 15.85 / 15.92, 18.66 / 18.66, 21.42 / 21.64, 16.59 / 16.63 (2688-wide, groups of 32: 17.17 / 16.77), with resident
+// lists 15.21 / 15.35, 15.87 / 15.96, 18.22 / 18.26, 21.29 / 21.29, 15.53 / 15.58 (16.37 / 15.91).
 template <int G, int MODE>
 __device__ __forceinline__ void consume_chunk(const LaneRole& lr, int lane, int gw, int rot, int nblocks,
                                               const uint8_t* unit0, const uint8_t* unit1, int scale_off, int zp_off,
